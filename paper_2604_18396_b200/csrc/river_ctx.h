@@ -91,7 +91,7 @@ struct river_ctx {
     cudaEvent_t off_ready[2] = {nullptr, nullptr}, off_freed[2] = {nullptr, nullptr};
     int off_slot_layer[2] = {-1, -1};
 
-    // per-context launch bookkeeping: the largest dynamic shared memory size set per kernel, and the launch geometry
+    // per-context launch bookkeeping: the dynamic shared memory limit of every kernel that was set up, and the launch geometry
     // of the streaming kernels per (kernel, task count, K)
     struct SmemAttr { const void *fn; size_t bytes; };
     std::vector<SmemAttr> smem_attr;
@@ -157,19 +157,24 @@ cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
     return launch_kc(kern, grid, block, smem, st, pdl, 1, std::forward<Args>(args)...);
 }
 
-// cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the context's device: remembered per context, raised when
-// a launch needs more than any earlier one.
+// cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the device, not to a context: a context that set it to what its
+// own launches need would lower it under another context's larger launches (which then fail as invalid).  So every kernel's
+// limit goes straight to the most the device allows beside its static shared memory - the same value whoever sets it - and
+// a context only remembers that it has done so.
 template <class Kern>
 cudaError_t ensure_smem(river_ctx *c, Kern kern, size_t bytes) {
     const void *fn = reinterpret_cast<const void *>(kern);
     for (auto &a : c->smem_attr)
-        if (a.fn == fn) {
-            if (a.bytes >= bytes) return cudaSuccess;
-            a.bytes = bytes;
-            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        }
-    c->smem_attr.push_back({fn, bytes});
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (a.fn == fn) return bytes <= a.bytes ? cudaSuccess : cudaErrorInvalidValue;
+    cudaFuncAttributes fa;
+    int most = 0;
+    cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device);
+    if (e != cudaSuccess) return e;
+    most -= (int)fa.sharedSizeBytes;
+    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess) return e;
+    c->smem_attr.push_back({fn, (size_t)most});
+    return bytes <= (size_t)most ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 inline KvAddr kv_addr(const river_ctx *c, int layer0) {

@@ -1,0 +1,26 @@
+"""Two contexts on one device: what one context sets up for a kernel must not take anything from the other's launches."""
+import pytest
+import torch
+
+from paper_2604_18396_b200 import River, make_config
+from tests.gpu_harness import draw_model
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def test_contexts_with_other_prompt_lengths_do_not_disturb_each_other():
+    # the shared memory a projection launch asks for does not grow with the rows of the chunk: 200 rows ask for more than 256
+    shape, _, (bb, rv) = draw_model("mini8")
+    cfg = make_config(shape, max_seqs=1, max_pages_per_seq=32, n_pages=32, max_batch=8, prefill_chunk=256)
+    a, b = River(cfg, bb, rv), River(cfg, bb, rv)
+    tok = synth.tokens(3, 0, 256, shape.V).cuda()
+    out = [torch.empty((1, shape.V), device="cuda") for _ in range(2)]
+    a.prefill([0], tok[:200].contiguous(), [0, 200], None, out[0])
+    b.prefill([0], tok, [0, 256])
+    a.release(0)
+    a.prefill([0], tok[:200].contiguous(), [0, 200], None, out[1])
+    torch.cuda.synchronize()
+    assert torch.equal(out[0], out[1])
+    a.close()
+    b.close()
