@@ -69,8 +69,10 @@ typedef struct river_config {
     uint32_t page_shuffle_seed;/* != 0: hand pages out in a seeded shuffled order */
     uint32_t flags;
     int32_t prefill_chunk;     /* prompt positions river_prefill runs per pass through the blocks (0 = max_batch, at most
-                                  256): every pass streams the weights once, so larger chunks make prefill cheaper; the
-                                  workspace grows with max(max_batch, prefill_chunk) */
+                                  256): every pass streams the weights once, so larger chunks make prefill cheaper; from
+                                  128 on (RIVER_KV_RIVER, shapes of the tensor-core paths) a pass takes up to four chunks,
+                                  at most 1024 positions; the workspace grows with max(max_batch, prefill_chunk) and with
+                                  the rows of a pass */
     int32_t kv_strategy;       /* what happens in the blocks a token skips (Section 3; RIVER_KV_*): the method's KV-Shared
                                   Exit River, or one of the strategies it is compared with, on the same kernels */
 } river_config;

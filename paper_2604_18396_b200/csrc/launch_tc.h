@@ -2,6 +2,7 @@
 #pragma once
 #include "river_ctx.h"
 #include "gemm_tc.cuh"
+#include "gemm_tc_wide.cuh"
 
 namespace river {
 
@@ -46,5 +47,21 @@ cudaError_t launch_tc_w4(river_ctx *c, const ProjIn &in, const CUtensorMap *cons
                                                 int, bool, bool);
 RIVER_TCW4_DECL(TcQkvEpi) RIVER_TCW4_DECL(TcResidEpi) RIVER_TCW4_DECL(TcGateUpEpi)
 #undef RIVER_TCW4_DECL
+
+// launch_tc_wide.cu: the projections of a long prefill pass (up to wide_rows rows) on CTA pairs.  The row lists' lengths
+// are known on the host there (n_list >= the device's count).  launch_wide_operand writes the operand rows (bf16 or f16
+// high and low parts); launch_w4_expand the f16 form of up to three exit-layer matrices, one after the other, in wide_w.
+inline uint16_t *wide_operand(const river_ctx *c, bool alt) { return alt ? c->wide_xalt : c->wide_x; }
+cudaError_t launch_wide_operand(river_ctx *c, const ProjIn &in, int K, int n_list, const int32_t *rows, const int32_t *cnt, bool f16);
+cudaError_t launch_w4_expand(river_ctx *c, const river_w4 *const (&w)[3], const int (&rows)[3], int K);
+template <class Epi>
+cudaError_t launch_tc_wide(river_ctx *c, const CUtensorMap &a0, const CUtensorMap &a1, const CUtensorMap &a2, int K, int tiles,
+                           int n_list, int q_tiles, int k_tiles, int run_step, int head_step, const int32_t *rows, const int32_t *cnt,
+                           const Epi &epi, bool f16, bool alt_operand);
+#define RIVER_TCWIDE_DECL(E) \
+    extern template cudaError_t launch_tc_wide<E>(river_ctx *, const CUtensorMap &, const CUtensorMap &, const CUtensorMap &, int, int, \
+                                                  int, int, int, int, int, const int32_t *, const int32_t *, const E &, bool, bool);
+RIVER_TCWIDE_DECL(WdQkvEpi) RIVER_TCWIDE_DECL(WdResidEpi) RIVER_TCWIDE_DECL(WdGateUpEpi)
+#undef RIVER_TCWIDE_DECL
 
 }  // namespace river

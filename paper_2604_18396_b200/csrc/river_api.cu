@@ -90,41 +90,67 @@ river_config effective(const river_config *cfg, int *user_max_batch) {
     return e;
 }
 
+// The shapes the tensor-core paths take: every output dimension in whole 128-feature tiles; for the exit layers also one
+// scale / zero per row and 64-input k-block, and raw code tiles of 256 inputs.
+bool tc_shape_ok(const river_config &g) {
+    return g.d % 128 == 0 && (g.Hq * g.dh) % 128 == 0 && (g.Hkv * g.dh) % 128 == 0 && g.F % 64 == 0 && g.V % 128 == 0 &&
+           g.d % 64 == 0 && g.F % 64 == 0 && (g.Hq * g.dh) % 64 == 0;
+}
+bool w4_shape_ok(const river_config &g) { return g.group == 64 && g.d % 256 == 0 && g.F % 256 == 0 && (g.Hq * g.dh) % 256 == 0; }
+
+constexpr int kWideMin = 128;  // a pass of up to this many rows takes the batch kernels, which split K where tiles are few
+// Rows of a long prefill pass (0: this configuration has none).  A pass streams every weight once and its projections run
+// on CTA pairs at about the tensor-core rate only when there are tiles for all of them, so prompts go through in passes of
+// up to 1024 rows wherever the caller allows chunks of 128 and more (8B-class shape, 1024 positions, per block: four passes of
+// 256 rows through the batch kernels 1.87 ms, one pass 0.9 ms).  The workspace pays for it: about 0.2 MB per
+// row of the 8B-class shape plus one projection's exit-layer weights in f16.
+int wide_rows_for(const river_config &c) {
+    if (c.max_batch < 128 || c.kv_strategy != RIVER_KV_RIVER || (c.flags & (RIVER_F_NO_TC | RIVER_F_NO_W4TC)) || !tc_shape_ok(c) ||
+        !w4_shape_ok(c))
+        return 0;
+    return std::min(kMaxBatch, (4 * c.max_batch + 127) / 128 * 128);
+}
+
+// (c: the effective configuration, whose max_batch is the rows of a decode step or a short prefill pass)
 size_t carve(const river_config *c, river_ctx *x, char *base, int head_rows) {
     Carver cv{base};
-    const size_t B = c->max_batch, d = c->d, L = c->L;
+    const size_t Bs = c->max_batch, d = c->d, L = c->L, W = wide_rows_for(*c), B = std::max(Bs, W);
     float *h0 = cv.take<float>(B * d), *h1 = cv.take<float>(B * d), *h2 = cv.take<float>(B * d);
     float *qb = cv.take<float>(B * c->Hq * c->dh), *ob = cv.take<float>(B * c->Hq * c->dh);
-    float *act = cv.take<float>(B * c->F);
-    float *pv = cv.take<float>(B * (size_t)head_parts_for(c));
-    int32_t *pi = cv.take<int32_t>(B * (size_t)head_parts_for(c));
+    float *act = cv.take<float>(Bs * c->F);  // (a long pass hands the activation on as operand rows only)
+    float *pv = cv.take<float>(Bs * (size_t)head_parts_for(c));
+    int32_t *pi = cv.take<int32_t>(Bs * (size_t)head_parts_for(c));
     float *tau = cv.take<float>(B);
     float *lg = cv.take<float>((size_t)head_rows * (size_t)c->V);
-    float *sc = cv.take<float>(B * L);
+    float *sc = cv.take<float>(Bs * L);
     float2 *cs = cv.take<float2>(B * (c->dh / 2));
     double *fr = cv.take<double>(c->dh / 2);
     int32_t *ai = cv.take<int32_t>((L + 1) * B), *ri = cv.take<int32_t>((L + 1) * B);
     int32_t *na = cv.take<int32_t>(L + 1), *nr = cv.take<int32_t>(L + 1);
     int32_t *pt = cv.take<int32_t>((size_t)c->max_seqs * c->max_pages_per_seq);
     int32_t *tk = cv.take<int32_t>(B), *fo = cv.take<int32_t>(B), *ex = cv.take<int32_t>(B), *nx = cv.take<int32_t>(B);
-    int32_t *md = cv.take<int32_t>(kMetaHdr + 11 * B);
+    int32_t *md = cv.take<int32_t>(kMetaHdr + 11 * B);  // (meta_rows entries per array: Bs or W)
     int32_t *pff = cv.take<int32_t>((size_t)c->max_seqs * (L + 1));
-    float *po = cv.take<float>((B + 600) * (size_t)c->Hq * c->dh);
-    float2 *pml = cv.take<float2>((B + 600) * (size_t)c->Hq);
+    float *po = cv.take<float>((Bs + 600) * (size_t)c->Hq * c->dh);
+    float2 *pml = cv.take<float2>((Bs + 600) * (size_t)c->Hq);
     const size_t sstride = (B + 15) / 16 * 16;
     uint8_t *exd = cv.take<uint8_t>((L + 1) * sstride), *ps = cv.take<uint8_t>(B);
     int *de = cv.take<int>(1);
-    unsigned *atk = cv.take<unsigned>(B * (size_t)c->Hkv), *tk4 = cv.take<unsigned>(4);
+    unsigned *atk = cv.take<unsigned>(Bs * (size_t)c->Hkv), *tk4 = cv.take<unsigned>(4);
     int32_t *hint = md ? md + 5 : nullptr;  // StepMeta::hint_act
     int32_t *scap = cv.take<int32_t>((size_t)c->max_seqs);
     uint8_t *pdep = cv.take<uint8_t>((size_t)c->max_seqs * c->max_pages_per_seq * kPage);
     unsigned long long *ehist = cv.take<unsigned long long>((size_t)c->L + 1);
-    const size_t tc_pad = std::min<size_t>(256, (B + 15) / 16 * 16);
+    const size_t tc_pad = std::min<size_t>(256, (Bs + 15) / 16 * 16);
     const size_t tc_kmax = std::max<size_t>(std::max<size_t>(c->d, c->F), (size_t)c->Hq * c->dh);
     // one allocation: lo rows may start right behind the hi rows in use (launch_tc.cu: tc_bmap)
     __nv_bfloat16 *txh = cv.take<__nv_bfloat16>(2 * tc_pad * tc_kmax), *txl = txh ? txh + tc_pad * tc_kmax : nullptr;
     __nv_bfloat16 *tx4 = cv.take<__nv_bfloat16>(2 * tc_pad * tc_kmax);
     __nv_bfloat16 *txa = cv.take<__nv_bfloat16>(2 * tc_pad * tc_kmax), *tx4a = cv.take<__nv_bfloat16>(2 * tc_pad * tc_kmax);
+    const size_t qdim = (size_t)c->Hq * c->dh, kvdim = (size_t)c->Hkv * c->dh;
+    const size_t w_most = std::max(std::max((qdim + 2 * kvdim) * d, qdim * d), 2 * (size_t)c->F * d);
+    uint16_t *wx = W ? cv.take<uint16_t>(2 * W * std::max(d, qdim)) : nullptr, *wxa = W ? cv.take<uint16_t>(2 * W * c->F) : nullptr;
+    __half *ww = W ? cv.take<__half>(w_most) : nullptr;
 
     if (x) {
         x->h[0] = h0; x->h[1] = h1; x->h[2] = h2; x->qbuf = qb; x->obuf = ob; x->act = act;
@@ -133,6 +159,8 @@ size_t carve(const river_config *c, river_ctx *x, char *base, int head_rows) {
         x->tok_i = tk; x->forced_i = fo; x->exit_i = ex; x->next_i = nx; x->meta_dev = md; x->state = exd; x->state_stride = (int)sstride; x->prefill_fail = pff;
         x->pass = ps; x->dev_err = de; x->part_o = po; x->part_ml = pml; x->attn_tickets = atk; x->tickets = tk4; x->hint_act = hint;
         x->slot_cap = scap; x->pos_depth = pdep; x->exit_hist = ehist;
+        x->wide_rows = (int)W; x->wide_x = wx; x->wide_xalt = wxa; x->wide_w = ww;
+        x->meta_rows = (int)Bs; x->list_rows = (int)B;
         x->tc_xhi = txh; x->tc_xlo = txl; x->tc_x4 = tx4; x->tc_xalt = txa; x->tc_x4alt = tx4a; x->tc_max_pad = (int)tc_pad; x->tc_kmax = (int)tc_kmax;
     }
     return (cv.off + 255) & ~(size_t)255;
@@ -153,7 +181,7 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
     int max_pos = 0;
     double total = 0.0;
     for (int i = 0; i < n; ++i) {
-        const int pos = mh[kMetaHdr + g.max_batch + i];
+        const int pos = mh[kMetaHdr + c->meta_rows + i];
         max_pos = std::max(max_pos, pos);
         total += pos + 1;
     }
@@ -173,7 +201,7 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
         int ch = (max_pos + 1 + s - 1) / s;
         ch = std::max(2 * kAttnTile, (ch + kAttnTile - 1) / kAttnTile * kAttnTile);
         double items = 0.0;
-        for (int i = 0; i < n; ++i) items += (mh[kMetaHdr + g.max_batch + i] + ch) / ch;  // ceil((pos + 1) / ch)
+        for (int i = 0; i < n; ++i) items += (mh[kMetaHdr + c->meta_rows + i] + ch) / ch;  // ceil((pos + 1) / ch)
         items *= g.Hkv;
         const int longest = std::min(ch, max_pos + 1);
         // whole waves of items of the mean length bound it from below as well (equal lengths: 1.3 waves cost 2)
@@ -192,10 +220,10 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
     mh[5] = n;  // hint_act: every row starts in the backbone
     // the attention grid takes its rows longest context first: CTA slots are handed out in launch order, and a long
     // item that starts last is what the step ends on
-    int32_t *order = mh + kMetaHdr + 10 * g.max_batch;
+    int32_t *order = mh + kMetaHdr + 10 * c->meta_rows;
     for (int i = 0; i < n; ++i) order[i] = i;
     std::stable_sort(order, order + n, [&](int32_t x, int32_t y) {
-        return mh[kMetaHdr + g.max_batch + x] > mh[kMetaHdr + g.max_batch + y];
+        return mh[kMetaHdr + c->meta_rows + x] > mh[kMetaHdr + c->meta_rows + y];
     });
     // the small-step kernel: one CTA per (row, kv head, split), chunks in whole pages
     const int Sc = small_attn_splits(c->num_sms, n, g.Hkv);
@@ -218,11 +246,6 @@ void set_io_meta(int32_t *mh, const int32_t *tok, const float *tau, const int32_
 }
 
 // ---- tensor maps of the weights for the tensor-core projections
-// The shapes the tensor-core path takes: every output dimension in whole 128-feature tiles.
-bool tc_shape_ok(const river_config &g) {
-    return g.d % 128 == 0 && (g.Hq * g.dh) % 128 == 0 && (g.Hkv * g.dh) % 128 == 0 && g.F % 64 == 0 && g.V % 128 == 0 &&
-           g.d % 64 == 0 && g.F % 64 == 0 && (g.Hq * g.dh) % 64 == 0;
-}
 bool make_tc_maps(river_ctx *c) {
     const river_config &g = c->cfg;
     const int qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
@@ -243,7 +266,7 @@ bool make_tc_maps(river_ctx *c) {
 bool make_w4_maps(river_ctx *c) {
     const river_config &g = c->cfg;
     const int qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
-    if (g.group != 64 || g.d % 256 || g.F % 256 || qdim % 256) return false;
+    if (!w4_shape_ok(g)) return false;
     c->w4_maps.resize(g.L);
     for (int l = 0; l < g.L; ++l) {
         const river_layer_weights &w = c->layers[l];
@@ -256,6 +279,31 @@ bool make_w4_maps(river_ctx *c) {
             return false;
     }
     return true;
+}
+
+// The maps of the pair kernel, over the backbone's matrices and over the buffer that holds ONE projection's exit-layer
+// weights in f16 at a time (q, k, v one after the other; o; gate and up; down).  LayerMaps::g covers gate and up together.
+bool make_wide_maps(river_ctx *c) {
+    const river_config &g = c->cfg;
+    const uint64_t qdim = (uint64_t)g.Hq * g.dh, kvdim = (uint64_t)g.Hkv * g.dh, d = g.d, F = g.F, half = g.dh / 2;
+    auto heads = [&](CUtensorMap *m, const void *w, uint64_t n) {
+        return make_map_paired(m, w, d, half * d * 2, half / 16, n, 2 * half * d * 2, (uint32_t)half / 16, kTcBM / g.dh);
+    };
+    auto make = [&](river_ctx::LayerMaps &m, const void *q, const void *k, const void *v, const void *o, const void *wg, const void *wu,
+                    const void *dn) {
+        const char *a = static_cast<const char *>(wg), *b = static_cast<const char *>(wu);
+        return heads(&m.q, q, g.Hq) && heads(&m.k, k, g.Hkv) && heads(&m.v, v, g.Hkv) && make_map_bf16(&m.o, o, qdim, d, 128) &&
+               make_map_paired(&m.g, std::min(a, b), d, (uint64_t)(a < b ? b - a : a - b), F / 16, 1, F * d * 2, 4, 1) &&
+               make_map_bf16(&m.d, dn, F, d, 128);
+    };
+    c->wide_bmaps.resize(g.L);
+    for (int l = 0; l < g.L; ++l) {
+        const river_layer_weights &w = c->layers[l];
+        if (!make(c->wide_bmaps[l], w.wq, w.wk, w.wv, w.wo, w.wg, w.wu, w.wd)) return false;
+    }
+    const __half *w = c->wide_w;
+    c->wide_wmaps.resize(1);
+    return make(c->wide_wmaps[0], w, w + qdim * d, w + (qdim + kvdim) * d, w, w, w + F * d, w);
 }
 
 // 2-D tiled tensor map over the KV pool seen as [all cache rows][dh] bf16, box = 16 rows x 64 elements (128 bytes),
@@ -290,13 +338,13 @@ int ensure_page(river_ctx *c, int slot, int pos, int32_t *mh, int &n_upd) {
     int32_t &e = c->page_tbl[(size_t)slot * g.max_pages_per_seq + pi];
     if (e >= 0) return 0;
     if (c->free_pages.empty()) return fail(c, RIVER_E_NOPAGE, "KV pool exhausted");
-    if (n_upd >= g.max_batch) return fail(c, RIVER_E_NOPAGE, "too many new pages in one step");
+    if (n_upd >= c->meta_rows) return fail(c, RIVER_E_NOPAGE, "too many new pages in one step");
     e = c->free_pages.back();
     c->free_pages.pop_back();
-    int32_t *u = mh + kMetaHdr + 2 * g.max_batch;
+    int32_t *u = mh + kMetaHdr + 2 * c->meta_rows;
     u[n_upd] = slot;
-    u[g.max_batch + n_upd] = pi;
-    u[2 * g.max_batch + n_upd] = e;
+    u[c->meta_rows + n_upd] = pi;
+    u[2 * c->meta_rows + n_upd] = e;
     ++n_upd;
     return 0;
 }
@@ -305,6 +353,10 @@ int32_t *next_meta(river_ctx *c) {
     const int i = c->meta_next;
     c->meta_next = (i + 1) % kStaging;
     cudaEventSynchronize(c->meta_ev[i]);
+    if (c->meta_host_rows[i] != c->meta_rows) {  // laid out for another row count: entries past a step's rows are valid ids again
+        std::memset(c->meta_host[i], 0, sizeof(int32_t) * c->meta_ints());
+        c->meta_host_rows[i] = c->meta_rows;
+    }
     return c->meta_host[i];
 }
 
@@ -417,7 +469,7 @@ cudaError_t tc_pair(river_ctx *c, bool with_river, const ProjIn &in, int K, int 
 // lists name (small steps: from the exit flags).
 cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const DecideArgs &dec, double kv_write) {
     const river_config &g = c->cfg;
-    const int d = g.d, B = g.max_batch, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
+    const int d = g.d, B = c->list_rows, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
     const double w4f = 0.25 + 2.0 / g.group;
     const river_layer_weights &w = c->layers[l - 1];
     const int strat = g.kv_strategy;
@@ -480,6 +532,35 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
     return err;
 }
 
+// a8: final norm + LM head + greedy token for the n_head rows that need logits.
+cudaError_t launch_head(river_ctx *c, const float *h, int n_head) {
+    const river_config &g = c->cfg;
+    const int d = g.d;
+    cudaError_t err = cudaSuccess;
+    auto note = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
+    HeadArgs a{};
+    a.w = c->lm_head;
+    a.in = ProjIn{h, c->final_norm, g.rms_eps};
+    a.d = d; a.V = g.V; a.rows = c->head_rows(); a.meta = c->meta();
+    a.part_val = c->part_val; a.part_idx = c->part_idx;
+    int n_parts = c->head_grid;
+    if (c->tc_ok && n_head >= 5 && n_head <= c->tc_max_pad) {
+        LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
+        n_parts = g.V / kTcBM;
+        TcHeadEpi e{c->meta(), g.V, c->part_val, c->part_idx, n_parts};
+        note(launch_tc(c, a.in, c->tc_map_head, c->tc_map_head, c->tc_map_head, d, n_parts, n_head, 0, 0, 0,
+                       c->head_rows(), c->meta_dev + 2 /* StepMeta::n_head_rows */, e, false, nullptr));
+    } else {
+        LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
+        note(launch_head_stream(c, a, n_head));
+    }
+    {
+        LaunchScope ls(c, K_ARGMAX, 0, 0, -1);
+        note(launch_argmax_final(c, n_head, n_parts));
+    }
+    return err;
+}
+
 // The launch sequence of one step over the rows described in the device metadata (rows, positions, caller buffers).
 //
 // Steps of up to four rows: per block QKV, attention, O, gate/up, down - the exit decision of block l is taken by the
@@ -489,7 +570,7 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
 // variant, and the score / compaction kernel after every block.
 int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool record_fail = false) {
     const river_config &g = c->cfg;
-    const int L = g.L, d = g.d, B = g.max_batch;
+    const int L = g.L, d = g.d, B = c->list_rows;
     int32_t *fail_buf = record_fail ? c->prefill_fail : nullptr;
     c->st.launches_last_step = 0;
     Lists lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, B};
@@ -509,7 +590,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     {
         LaunchScope ls(c, K_BEGIN, (double)n * d * 2.0, 0, -1);
         note(launch_k(step_begin_kernel, dim3(std::max(n, 1)), dim3(128), 0, c->stream, false, c->meta(), c->upd(),
-                      c->page_tbl_dev, g.max_pages_per_seq, B, c->embed, d, g.V, c->h[0], c->row_pos(), c->inv_freq,
+                      c->page_tbl_dev, g.max_pages_per_seq, c->meta_rows, c->embed, d, g.V, c->h[0], c->row_pos(), c->inv_freq,
                       g.dh / 2, c->rope_cs, L, g.entry_layer, c->state_at(0), c->dev_err, lists, c->hint_act, c->tickets));
     }
     auto launch_score = [&](int l, const float *h_in, const float *h_out) {
@@ -656,28 +737,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         prev_in = h_in;
         hi = (hi + 2) % 3;
     }
-    if (n_head > 0) {
-        HeadArgs a{};
-        a.w = c->lm_head;
-        a.in = ProjIn{c->h[hi], c->final_norm, g.rms_eps};
-        a.d = d; a.V = g.V; a.rows = c->head_rows(); a.meta = c->meta();
-        a.part_val = c->part_val; a.part_idx = c->part_idx;
-        int n_parts = c->head_grid;
-        if (c->tc_ok && n_head >= 5 && n_head <= c->tc_max_pad) {
-            LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
-            n_parts = g.V / kTcBM;
-            TcHeadEpi e{c->meta(), g.V, c->part_val, c->part_idx, n_parts};
-            note(launch_tc(c, a.in, c->tc_map_head, c->tc_map_head, c->tc_map_head, d, n_parts, n_head, 0, 0, 0,
-                           c->head_rows(), c->meta_dev + 2 /* StepMeta::n_head_rows */, e, false, nullptr));
-        } else {
-            LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
-            note(launch_head_stream(c, a, n_head));
-        }
-        {
-            LaunchScope ls(c, K_ARGMAX, 0, 0, -1);
-            note(launch_argmax_final(c, n_head, n_parts));
-        }
-    }
+    if (n_head > 0) note(launch_head(c, c->h[hi], n_head));
     // small steps: the last block's score (a diagnostic: no exit is taken after block L) and the final row lists
     if (fold) launch_score(L, prev_in, c->h[hi]);
     if (strat == RIVER_KV_MASK) {  // what the later tokens' attention may see of this step's positions
@@ -685,6 +745,110 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         note(launch_k(depth_note_kernel, dim3((n + 127) / 128), dim3(128), 0, c->stream, true, c->meta(),
                       (const int32_t *)c->row_slot(), (const int32_t *)c->row_pos(), c->pos_depth, g.max_pages_per_seq * kPage));
     }
+    if (err == cudaSuccess) err = cudaGetLastError();
+    if (err != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(err));
+    c->st.launches_total += c->st.launches_last_step;
+    if (c->profiling) return profile_collect(c);
+    return 0;
+}
+
+// The launch sequence of a long prefill pass: more rows than one launch of the batch kernels takes, depths known on the
+// host.  depth[i]: backbone blocks row i runs; so every block's row counts are known here, an empty list launches nothing,
+// and the score / compaction kernel runs only after a block some row leaves at (or, record_fail, after every block: the
+// pass that looks for the unified depth).  Both weight sets go through tc_gemm_wide_kernel, one after the other.
+int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *row_pos_host, const int32_t *depth, bool record_fail) {
+    const river_config &g = c->cfg;
+    const int L = g.L, d = g.d, F = g.F, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
+    c->st.launches_last_step = 0;
+    cudaError_t err = cudaSuccess;
+    auto note = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
+    std::vector<int> leave(L + 1, 0);  // rows that leave after block l
+    for (int i = 0; i < n; ++i) leave[depth[i]] += 1;
+    double kv_read = 0.0;
+    for (int i = 0; i < n; ++i) kv_read += (double)(row_pos_host[i] + 1) * 4.0 * kvdim;
+    Lists lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, c->list_rows};
+    {
+        LaunchScope ls(c, K_BEGIN, (double)n * d * 2.0, 0, -1);
+        note(launch_k(step_begin_kernel, dim3(n), dim3(128), 0, c->stream, false, c->meta(), c->upd(), c->page_tbl_dev,
+                      g.max_pages_per_seq, c->meta_rows, c->embed, d, g.V, c->h[0], c->row_pos(), c->inv_freq, g.dh / 2,
+                      c->rope_cs, L, g.entry_layer, c->state_at(0), c->dev_err, lists, c->hint_act, c->tickets));
+    }
+    c->attn_skip = nullptr;
+    c->attn_layer1 = 0;
+    int hi = 0, at = 0;          // h[hi] = block input; entry `at` of the row lists / exit flags describes the rows of this block
+    int n_riv = leave[0];
+    for (int l = 1; l <= L && err == cudaSuccess; ++l) {
+        const river_layer_weights &w = c->layers[l - 1];
+        const river_ctx::LayerMaps &bm = c->wide_bmaps[l - 1], &rm = c->wide_wmaps[0];
+        float *h_in = c->h[hi], *h_mid = c->h[(hi + 1) % 3], *h_out = c->h[(hi + 2) % 3];
+        const int n_of[2] = {n - n_riv, n_riv};
+        const int32_t *rows_of[2] = {c->act_idx + (size_t)at * c->list_rows, c->riv_idx + (size_t)at * c->list_rows};
+        const int32_t *cnt_of[2] = {c->n_act + at, c->n_riv + at};
+        auto ceil_rows = [&](int set) { return 2.0 * (set ? 0.25 + 2.0 / g.group : 1.0) * (n_of[set] ? 1.0 : 0.0); };
+        const double wsum = ceil_rows(0) + ceil_rows(1);  // bytes per weight this block streams
+        // one projection on the weight set(s) that have rows: the operand rows (unless the projection before wrote them),
+        // the f16 weights of the exit layer, the GEMM
+        auto project = [&](const ProjIn *in, int K, int tiles, int q_tiles, int k_tiles, int run_step, int head_step, int set, const CUtensorMap &m0,
+                           const CUtensorMap &m1, const CUtensorMap &m2, const river_w4 *const (&w4)[3], const int (&w4_rows)[3],
+                           const auto &epi) {
+            if (set == 1) note(launch_w4_expand(c, w4, w4_rows, K));
+            if (in) note(launch_wide_operand(c, *in, K, n_of[set], rows_of[set], cnt_of[set], set == 1));
+            note(launch_tc_wide(c, m0, m1, m2, K, tiles, n_of[set], q_tiles, k_tiles, run_step, head_step, rows_of[set], cnt_of[set], epi,
+                                set == 1, in == nullptr));
+        };
+        {
+            LaunchScope ls(c, K_QKV, wsum * (qdim + 2.0 * kvdim) * d + (double)n * 4.0 * kvdim, 0, -1);
+            const WdQkvEpi e{g.Hq, g.Hkv, g.dh, c->rope_cs, c->qbuf, kv_addr(c, l - 1), c->dev_err};
+            const ProjIn in{h_in, (const uint16_t *)w.attn_norm, g.rms_eps};
+            for (int set = 0; set < 2; ++set)
+                if (n_of[set]) {
+                    const river_ctx::LayerMaps &m = set ? rm : bm;
+                    project(&in, d, (qdim + 2 * kvdim) / kTcBM, qdim / kTcBM, kvdim / kTcBM, 0, kTcBM / g.dh, set, m.q, m.k, m.v, {&w.rq, &w.rk, &w.rv},
+                            {qdim, kvdim, kvdim}, e);
+                }
+        }
+        {
+            LaunchScope ls(c, K_PREFILL_ATTN, kv_read, 0, -1);
+            note(launch_attention_prefill(c, n_tiles, l - 1));
+        }
+        {
+            LaunchScope ls(c, K_OPROJ, wsum * qdim * d, 0, -1);
+            const WdResidEpi e{h_in, h_mid, d};
+            const ProjIn in{c->obuf, nullptr, 0.f};
+            for (int set = 0; set < 2; ++set)
+                if (n_of[set]) {
+                    const CUtensorMap &m = set ? rm.o : bm.o;
+                    project(&in, qdim, d / kTcBM, 0, 0, 0, 0, set, m, m, m, {&w.ro, &w.ro, &w.ro}, {d, 0, 0}, e);
+                }
+        }
+        const ProjIn ffn_in{h_mid, (const uint16_t *)w.ffn_norm, g.rms_eps};
+        const WdResidEpi down_e{h_mid, h_out, d};
+        for (int set = 0; set < 2; ++set) {
+            if (!n_of[set]) continue;
+            const river_ctx::LayerMaps &m = set ? rm : bm;
+            {
+                LaunchScope ls(c, K_GATEUP, ceil_rows(set) * 2.0 * F * d, 0, -1);
+                uint16_t *const op = wide_operand(c, true);
+                const WdGateUpEpi e{F, op, op + (size_t)c->wide_rows * F, set, !set && w.wu < w.wg};
+                project(&ffn_in, d, F / 64, 0, 0, 4, 0, set, m.g, m.g, m.g, {&w.rg, &w.ru, &w.ru}, {F, F, 0}, e);
+            }
+            {
+                LaunchScope ls(c, K_DOWN, ceil_rows(set) * (double)F * d, 0, -1);
+                project(nullptr, F, d / kTcBM, 0, 0, 0, 0, set, m.d, m.d, m.d, {&w.rd, &w.rd, &w.rd}, {d, 0, 0}, down_e);
+            }
+        }
+        if (record_fail || (l < L && leave[l])) {
+            LaunchScope ls(c, K_SCORE, (double)n * d * 8.0, 0, -1);
+            note(launch_k(score_compact_kernel, dim3(n), dim3(256), 0, c->stream, true, c->meta(), l, L, g.entry_layer, g.exit_mode,
+                          (const float *)h_in, (const float *)h_out, d, c->pass, (const uint8_t *)c->state_at(at), c->state_at(l),
+                          lists, c->hint_act, c->tickets + 1, record_fail ? c->prefill_fail : (int32_t *)nullptr,
+                          (const int32_t *)c->row_slot(), (int32_t *)nullptr));
+            at = l;
+            n_riv += l < L ? leave[l] : 0;
+        }
+        hi = (hi + 2) % 3;
+    }
+    if (n_head > 0) note(launch_head(c, c->h[hi], n_head));
     if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(err));
     c->st.launches_total += c->st.launches_last_step;
@@ -742,24 +906,32 @@ int refuse_if_flagged(river_ctx *c) {
 // reverse order, so that the retry finds the state it would have found at first.
 void rollback_pages(river_ctx *c, const int32_t *mh, int n_upd) {
     const river_config &g = c->cfg;
-    const int32_t *u = mh + kMetaHdr + 2 * g.max_batch;
+    const int32_t *u = mh + kMetaHdr + 2 * c->meta_rows;
     for (int i = n_upd - 1; i >= 0; --i) {
-        const int slot = u[i], pi = u[g.max_batch + i], page = u[2 * g.max_batch + i];
+        const int slot = u[i], pi = u[c->meta_rows + i], page = u[2 * c->meta_rows + i];
         c->page_tbl[(size_t)slot * g.max_pages_per_seq + pi] = -1;
         c->free_pages.push_back(page);
     }
 }
 
 
-// One pass of the prompts through the decode kernels in chunks of rows (slot, position): rows of a chunk are
+// One pass of the prompts through the blocks in chunks of rows (slot, position; long chunks on the pair kernels, the rest
+// on the decode kernels): rows of a chunk are
 // consecutive prompt positions, possibly of several sequences; K/V of the whole chunk are written before its attention
 // runs, and a row attends to positions <= its own, so causality holds inside a chunk.  depth[s]: the unified exit depth
 // of sequence s (L = the whole backbone).  record_fail: note per (sequence, block) whether some position failed Eq. 1.
 int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *tok, const int32_t *offsets,
                  const int32_t *depth, float tau, bool record_fail, float *logits_last, int32_t *next_tok) {
     const river_config &g = c->cfg;
+    const bool wide = c->wide_rows > 0 && !c->off_first;
+    const int max_rows = wide ? c->wide_rows : g.max_batch;
+    struct MetaRows {  // the metadata block is laid out for a chunk of this pass while it runs
+        river_ctx *c; int keep;
+        MetaRows(river_ctx *c_, int rows) : c(c_), keep(c_->meta_rows) { c->meta_rows = rows; }
+        ~MetaRows() { c->meta_rows = keep; }
+    } meta_rows(c, max_rows);
     {
-        std::vector<float> ta(g.max_batch, tau);
+        std::vector<float> ta(max_rows, tau);
         CUDA_TRY(c, cudaMemcpyAsync(c->tau_i, ta.data(), sizeof(float) * ta.size(), cudaMemcpyHostToDevice, c->stream));
         CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     }
@@ -769,16 +941,16 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         int n = 0, n_upd = 0, n_head = 0;
         const int tok0 = offsets[s] + p;
         int head_seq[kMaxBatch];
-        while (s < n_seqs && n < g.max_batch && n_head < c->user_max_batch) {
+        while (s < n_seqs && n < max_rows && n_head < c->user_max_batch) {
             const int len = offsets[s + 1] - offsets[s];
             if (offsets[s] + p != tok0 + n) break;  // token ids of a chunk must be contiguous in tok
             if (int rc = ensure_page(c, slots[s], p, mh, n_upd)) { rollback_pages(c, mh, n_upd); return rc; }
             mh[kMetaHdr + n] = slots[s];
-            mh[kMetaHdr + g.max_batch + n] = p;
-            mh[kMetaHdr + 6 * g.max_batch + n] = c->page_tbl[(size_t)slots[s] * g.max_pages_per_seq + p / kPage];
-            mh[kMetaHdr + 7 * g.max_batch + n] = depth[s];
+            mh[kMetaHdr + max_rows + n] = p;
+            mh[kMetaHdr + 6 * max_rows + n] = c->page_tbl[(size_t)slots[s] * g.max_pages_per_seq + p / kPage];
+            mh[kMetaHdr + 7 * max_rows + n] = depth[s];
             if (p == len - 1) {
-                mh[kMetaHdr + 5 * g.max_batch + n_head] = n;
+                mh[kMetaHdr + 5 * max_rows + n_head] = n;
                 head_seq[n_head++] = s;
             }
             ++n;
@@ -791,10 +963,10 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         for (int i = 0; i < n;) {
             int j = i + 1;
             while (j < n && j - i < kPfBM && mh[kMetaHdr + j] == mh[kMetaHdr + i] &&
-                   mh[kMetaHdr + g.max_batch + j] == mh[kMetaHdr + g.max_batch + i] + (j - i))
+                   mh[kMetaHdr + max_rows + j] == mh[kMetaHdr + max_rows + i] + (j - i))
                 ++j;
-            mh[kMetaHdr + 8 * g.max_batch + n_tiles] = i;
-            mh[kMetaHdr + 9 * g.max_batch + n_tiles] = j - i;
+            mh[kMetaHdr + 8 * max_rows + n_tiles] = i;
+            mh[kMetaHdr + 9 * max_rows + n_tiles] = j - i;
             ++n_tiles;
             i = j;
         }
@@ -805,7 +977,10 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
                     nullptr);
         if (int rc = push_meta(c, mh)) return rc;
         c->rows_distinct = false;  // consecutive positions of one sequence share a chunk
-        const int rc_rows = run_rows(c, n, n_head, mh + kMetaHdr + g.max_batch, record_fail);
+        // (a short rest of at most kWideMin rows takes the batch kernels: they split K where tiles are few)
+        const int32_t *pos = mh + kMetaHdr + max_rows;
+        const int rc_rows = wide && n > kWideMin ? run_rows_wide(c, n, n_tiles, n_head, pos, mh + kMetaHdr + 7 * max_rows, record_fail)
+                                                 : run_rows(c, n, n_head, pos, record_fail);
         c->rows_distinct = true;
         c->prefill_attn_now = false;
         if (rc_rows) return rc_rows;
@@ -889,9 +1064,12 @@ int river_init(const river_config *cfg, const river_weights *w, void *kv_pool, s
     if (make_kv_tensor_map(c)) { river_destroy(c); return RIVER_E_DEVICE; }
     c->tc_ok = !(cfg->flags & RIVER_F_NO_TC) && tc_shape_ok(*cfg) && make_tc_maps(c);
     c->w4tc_ok = c->tc_ok && !(cfg->flags & RIVER_F_NO_W4TC) && make_w4_maps(c);
+    if (c->wide_rows && !(c->w4tc_ok && make_wide_maps(c))) c->wide_rows = 0;
     for (int i = 0; i < kStaging; ++i) {
-        if (cudaMallocHost((void **)&c->meta_host[i], sizeof(int32_t) * c->meta_ints()) != cudaSuccess) return bail("cudaMallocHost failed");
-        std::memset(c->meta_host[i], 0, sizeof(int32_t) * c->meta_ints());  // entries past a step's rows stay valid row ids
+        const size_t bytes = sizeof(int32_t) * (kMetaHdr + 11 * (size_t)c->list_rows);
+        if (cudaMallocHost((void **)&c->meta_host[i], bytes) != cudaSuccess) return bail("cudaMallocHost failed");
+        std::memset(c->meta_host[i], 0, bytes);
+        c->meta_host_rows[i] = c->meta_rows;  // entries past a step's rows stay valid row ids
         if (cudaEventCreateWithFlags(&c->meta_ev[i], cudaEventDisableTiming) != cudaSuccess) return bail("cudaEventCreate failed");
     }
     c->pin_io_bytes = (size_t)cfg->max_batch * (4 * sizeof(int32_t) + sizeof(float)) + sizeof(int32_t);
@@ -956,9 +1134,9 @@ int river_decode_step(river_ctx *c, int batch, const int32_t *slots, const int32
         const int pos = c->seq_len[slots[b]];
         if (int rc = ensure_page(c, slots[b], pos, mh, n_upd)) { rollback_pages(c, mh, n_upd); return rc; }
         mh[kMetaHdr + b] = slots[b];
-        mh[kMetaHdr + g.max_batch + b] = pos;
-        mh[kMetaHdr + 5 * g.max_batch + b] = b;
-        mh[kMetaHdr + 6 * g.max_batch + b] = c->page_tbl[(size_t)slots[b] * g.max_pages_per_seq + pos / kPage];
+        mh[kMetaHdr + c->meta_rows + b] = pos;
+        mh[kMetaHdr + 5 * c->meta_rows + b] = b;
+        mh[kMetaHdr + 6 * c->meta_rows + b] = c->page_tbl[(size_t)slots[b] * g.max_pages_per_seq + pos / kPage];
         c->last_pos[b] = pos;
     }
     mh[0] = batch; mh[1] = n_upd; mh[2] = batch;
@@ -1075,15 +1253,15 @@ static int stage_rows(river_ctx *c, int layer, int n_rows, const int32_t *slots,
     for (int b = 0; b < n_rows; ++b) {
         const int pos = c->seq_len[slots[b]] - 1;
         mh[kMetaHdr + b] = slots[b];
-        mh[kMetaHdr + g.max_batch + b] = pos;
-        mh[kMetaHdr + 6 * g.max_batch + b] = c->page_tbl[(size_t)slots[b] * g.max_pages_per_seq + pos / kPage];
+        mh[kMetaHdr + c->meta_rows + b] = pos;
+        mh[kMetaHdr + 6 * c->meta_rows + b] = c->page_tbl[(size_t)slots[b] * g.max_pages_per_seq + pos / kPage];
         c->last_pos[b] = pos;
     }
     mh[0] = n_rows; mh[1] = 0; mh[2] = 0;
     set_attn_meta(c, mh, n_rows);
     set_io_meta(mh, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr);
     if (int rc = push_meta(c, mh)) return rc;
-    Lists lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, g.max_batch};
+    Lists lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, c->list_rows};
     stage_begin_kernel<<<n_rows, 64, 0, c->stream>>>(c->meta(), c->row_pos(), c->inv_freq, g.dh / 2, c->rope_cs,
                                                       c->state_at(layer - 1), lists, layer - 1, on_exit_layer, c->hint_act);
     CUDA_TRY(c, cudaGetLastError());
@@ -1271,7 +1449,7 @@ int river_last_lists(river_ctx *c, int32_t *act_idx, int32_t *n_act, int32_t *ri
     const river_config &g = c->cfg;
     const int B = c->st.batch_last, L = g.L;
     if (B <= 0) return fail(c, RIVER_E_BADARG, "no decode step has run");
-    std::vector<int32_t> a((size_t)(L + 1) * g.max_batch), r((size_t)(L + 1) * g.max_batch);
+    std::vector<int32_t> a((size_t)(L + 1) * c->list_rows), r((size_t)(L + 1) * c->list_rows);
     CUDA_TRY(c, cudaMemcpyAsync(a.data(), c->act_idx, sizeof(int32_t) * a.size(), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(r.data(), c->riv_idx, sizeof(int32_t) * r.size(), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(n_act, c->n_act, sizeof(int32_t) * (L + 1), cudaMemcpyDeviceToHost, c->stream));
@@ -1279,8 +1457,8 @@ int river_last_lists(river_ctx *c, int32_t *act_idx, int32_t *n_act, int32_t *ri
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     for (int l = 0; l <= L; ++l)
         for (int i = 0; i < B; ++i) {
-            act_idx[(size_t)l * B + i] = i < n_act[l] ? a[(size_t)l * g.max_batch + i] : -1;
-            riv_idx[(size_t)l * B + i] = i < n_riv[l] ? r[(size_t)l * g.max_batch + i] : -1;
+            act_idx[(size_t)l * B + i] = i < n_act[l] ? a[(size_t)l * c->list_rows + i] : -1;
+            riv_idx[(size_t)l * B + i] = i < n_riv[l] ? r[(size_t)l * c->list_rows + i] : -1;
         }
     return RIVER_OK;
 }

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -49,6 +50,14 @@ struct river_ctx {
     // in one buffer (`lo_ptr` = tc_xhi + np K) and `hi` covers both (one copy per k-block); beyond, two buffers
     struct BMap { int K, np; bool w4, alt, one; __nv_bfloat16 *base, *lo_ptr; CUtensorMap hi, lo; };
     std::vector<BMap> tc_bmaps;
+    // long prefill passes (launch_tc_wide.cu): rows per pass (0: not for this context), operand rows (high parts, low parts
+    // behind them) of the projections that read h / the attention output, and of the down projection; f16 exit-layer weights
+    int wide_rows = 0;
+    uint16_t *wide_x = nullptr, *wide_xalt = nullptr;
+    __half *wide_w = nullptr;
+    std::vector<LayerMaps> wide_bmaps, wide_wmaps;  // the pair kernel's maps of the backbone and (one entry) over wide_w
+    struct WMap { int K, bn; bool alt; CUtensorMap hi, lo; };
+    std::vector<WMap> wide_maps;
     int32_t *hint_act;
     const uint8_t *attn_skip = nullptr;  // exit flags of the block whose attention is being launched (strategies that run nothing for rows that left), else null
     uint8_t *pos_depth = nullptr;  // [max_seqs][max_pages_per_seq * 16] KV Mask: backbone blocks the token at each position ran
@@ -61,7 +70,7 @@ struct river_ctx {
     std::vector<GraphEntry> graphs;
     double *inv_freq;
     int32_t *act_idx, *riv_idx, *n_act, *n_riv, *page_tbl_dev, *part_idx, *tok_i, *forced_i, *exit_i, *next_i;
-    int32_t *meta_dev;  // [kMetaHdr + 11*max_batch]: StepMeta, row_slot, row_pos, upd[3], head_rows, row_page, row_forced,
+    int32_t *meta_dev;  // [kMetaHdr + 11*meta_rows]: StepMeta, row_slot, row_pos, upd[3], head_rows, row_page, row_forced,
                         // tile_row0, tile_rows (query tiles of a prefill chunk), attn_order
     int32_t *prefill_fail;  // [max_seqs][L+1]: 1 where some prompt position of the sequence failed Eq. 1 after block l
     uint8_t *state;     // [(L+1)][state_stride]: sticky exit flags of the rows entering block l + 1 (entry L: at the LM head)
@@ -73,6 +82,7 @@ struct river_ctx {
     // host state
     std::vector<int32_t> page_tbl, seq_len, free_pages;
     int32_t *meta_host[kStaging] = {nullptr, nullptr, nullptr, nullptr};
+    int meta_host_rows[kStaging] = {0};  // the meta_rows each was last laid out for
     cudaEvent_t meta_ev[kStaging];
     int meta_next = 0;
     void *pin_io = nullptr;  // pinned staging for the *_host entry point
@@ -106,17 +116,21 @@ struct river_ctx {
     double prof_ms[kNumClasses] = {0}, prof_bytes[kNumClasses] = {0};
     int64_t prof_launches[kNumClasses] = {0};
 
-    int meta_ints() const { return river::kMetaHdr + 11 * cfg.max_batch; }
+    // The metadata block holds 11 arrays of meta_rows entries behind its header: cfg.max_batch for decode steps and short
+    // prefill passes, wide_rows for a long pass.
+    int meta_rows = 0;
+    int list_rows = 0;  // entries per block of the row lists: max(cfg.max_batch, wide_rows)
+    int meta_ints() const { return river::kMetaHdr + 11 * meta_rows; }
     river::StepMeta *meta() const { return reinterpret_cast<river::StepMeta *>(meta_dev); }
     int32_t *row_slot() const { return meta_dev + river::kMetaHdr; }
-    int32_t *row_pos() const { return meta_dev + river::kMetaHdr + cfg.max_batch; }
-    int32_t *upd() const { return meta_dev + river::kMetaHdr + 2 * cfg.max_batch; }
-    int32_t *head_rows() const { return meta_dev + river::kMetaHdr + 5 * cfg.max_batch; }
-    int32_t *row_page() const { return meta_dev + river::kMetaHdr + 6 * cfg.max_batch; }  // page of each row's new position
-    int32_t *row_forced() const { return meta_dev + river::kMetaHdr + 7 * cfg.max_batch; }  // prefill: forced exit per row
-    int32_t *tile_row0() const { return meta_dev + river::kMetaHdr + 8 * cfg.max_batch; }
-    int32_t *tile_rows() const { return meta_dev + river::kMetaHdr + 9 * cfg.max_batch; }
-    int32_t *attn_order() const { return meta_dev + river::kMetaHdr + 10 * cfg.max_batch; }  // rows, longest context first
+    int32_t *row_pos() const { return meta_dev + river::kMetaHdr + meta_rows; }
+    int32_t *upd() const { return meta_dev + river::kMetaHdr + 2 * meta_rows; }
+    int32_t *head_rows() const { return meta_dev + river::kMetaHdr + 5 * meta_rows; }
+    int32_t *row_page() const { return meta_dev + river::kMetaHdr + 6 * meta_rows; }  // page of each row's new position
+    int32_t *row_forced() const { return meta_dev + river::kMetaHdr + 7 * meta_rows; }  // prefill: forced exit per row
+    int32_t *tile_row0() const { return meta_dev + river::kMetaHdr + 8 * meta_rows; }
+    int32_t *tile_rows() const { return meta_dev + river::kMetaHdr + 9 * meta_rows; }
+    int32_t *attn_order() const { return meta_dev + river::kMetaHdr + 10 * meta_rows; }  // rows, longest context first
     uint8_t *state_at(int l) const { return state + (size_t)l * state_stride; }
 };
 
