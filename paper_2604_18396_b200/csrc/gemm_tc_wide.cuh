@@ -17,7 +17,7 @@
 //
 // What bounds it: the tensor pipe and, when passes follow each other, the power cap.  8B-class shape, 1024 rows, operand
 // kernel included: QKV 98 us, O 74, gate/up 433, down 167 (1.44 PFLOP/s of bf16 MMAs, half of them for the low parts) against
-// 4 x (59, 49, 180, 120) us in passes of 256 rows on tc_gemm_kernel.
+// 4 x (108, 42, 191, 81) us in passes of 256 rows on tc_gemm_kernel.
 #pragma once
 #include "gemm_tc.cuh"
 #include "gemm_tc_w4.cuh"

@@ -62,10 +62,10 @@ bool prefill_attn_supported(const river_ctx *c) {
 
 namespace {
 template <int DH, int GQ>
-cudaError_t launch_attn_prefill_t(river_ctx *c, int n, int layer0) {
+cudaError_t launch_attn_prefill_t(river_ctx *c, int tile0, int n_tiles, int layer0) {
     const river_config &g = c->cfg;
     PrefillAttnArgs a{};
-    a.meta = c->meta(); a.tile_row0 = c->tile_row0(); a.tile_rows = c->tile_rows();
+    a.meta = c->meta(); a.tile0 = tile0; a.tile_row0 = c->tile_row0(); a.tile_rows = c->tile_rows();
     a.q = c->qbuf; a.out = c->obuf; a.kv = kv_addr(c, layer0); a.Hq = g.Hq;
     a.qscale = 1.4426950408889634f / std::sqrt((float)DH);
     a.dev_err = c->dev_err;
@@ -73,14 +73,14 @@ cudaError_t launch_attn_prefill_t(river_ctx *c, int n, int layer0) {
     const size_t smem = attn_prefill_smem_bytes(DH);
     const cudaError_t e = ensure_smem(c, attn_prefill_kernel<DH, GQ>, smem);
     if (e != cudaSuccess) return e;
-    // at most one tile per row; the kernel reads the tile count of the chunk from the step metadata
-    return launch_k(attn_prefill_kernel<DH, GQ>, dim3(n, g.Hkv), dim3(32 * GQ), smem, c->stream, true, a);
+    // (n_tiles may be an upper bound: the kernel reads the tile count of the chunk from the step metadata)
+    return launch_k(attn_prefill_kernel<DH, GQ>, dim3(n_tiles, g.Hkv), dim3(32 * GQ), smem, c->stream, true, a);
 }
 }  // namespace
 
-cudaError_t launch_attention_prefill(river_ctx *c, int n, int layer0) {
+cudaError_t launch_attention_prefill(river_ctx *c, int tile0, int n_tiles, int layer0) {
     const int gq = c->cfg.Hq / c->cfg.Hkv;
-#define ATTP(DH_, GQ_) if (c->cfg.dh == DH_ && gq == GQ_) return launch_attn_prefill_t<DH_, GQ_>(c, n, layer0);
+#define ATTP(DH_, GQ_) if (c->cfg.dh == DH_ && gq == GQ_) return launch_attn_prefill_t<DH_, GQ_>(c, tile0, n_tiles, layer0);
     ATTP(64, 1) ATTP(64, 2) ATTP(64, 4) ATTP(64, 8) ATTP(128, 1) ATTP(128, 2) ATTP(128, 4) ATTP(128, 8)
 #undef ATTP
     return cudaErrorInvalidValue;

@@ -643,7 +643,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         // ---- a3: paged GQA decode attention
         if (c->prefill_attn_now) {
             LaunchScope ls(c, K_PREFILL_ATTN, kv_read, 0, -1);
-            note(launch_attention_prefill(c, n, l - 1));
+            note(launch_attention_prefill(c, 0, n, l - 1));
         } else {
             LaunchScope ls(c, K_ATTN, kv_read, 0, -1);
             note(launch_attention(c, n, l - 1));
@@ -756,7 +756,13 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
 // host.  depth[i]: backbone blocks row i runs; so every block's row counts are known here, an empty list launches nothing,
 // and the score / compaction kernel runs only after a block some row leaves at (or, record_fail, after every block: the
 // pass that looks for the unified depth).  Both weight sets go through tc_gemm_wide_kernel, one after the other.
-int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *row_pos_host, const int32_t *depth, bool record_fail) {
+//
+// The last block owes the cache the K and V of every position, but its output is read at the n_head prompt ends only: what
+// follows QKV there runs on those rows (head[]: their row ids; head_tiles: their one-row query tiles follow the chunk's
+// n_tiles in the metadata) and on none in a pass without a prompt end.  (8B-class shape, 1024 rows: the rest of a block takes
+// 0.7-1.0 ms for all of them, 0.2 ms for one: the projections' weight streams.)
+int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *head, bool head_tiles, const int32_t *row_pos_host,
+                  const int32_t *depth, bool record_fail) {
     const river_config &g = c->cfg;
     const int L = g.L, d = g.d, F = g.F, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
     c->st.launches_last_step = 0;
@@ -781,7 +787,7 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *r
         const river_layer_weights &w = c->layers[l - 1];
         const river_ctx::LayerMaps &bm = c->wide_bmaps[l - 1], &rm = c->wide_wmaps[0];
         float *h_in = c->h[hi], *h_mid = c->h[(hi + 1) % 3], *h_out = c->h[(hi + 2) % 3];
-        const int n_of[2] = {n - n_riv, n_riv};
+        int n_of[2] = {n - n_riv, n_riv};
         const int32_t *rows_of[2] = {c->act_idx + (size_t)at * c->list_rows, c->riv_idx + (size_t)at * c->list_rows};
         const int32_t *cnt_of[2] = {c->n_act + at, c->n_riv + at};
         auto ceil_rows = [&](int set) { return 2.0 * (set ? 0.25 + 2.0 / g.group : 1.0) * (n_of[set] ? 1.0 : 0.0); };
@@ -807,9 +813,23 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *r
                             {qdim, kvdim, kvdim}, e);
                 }
         }
+        bool heads_only = l == L && head_tiles;
+        if (heads_only) {
+            int on_backbone = 0;
+            for (int i = 0; i < n_head; ++i) on_backbone += depth[head[i]] >= L ? 1 : 0;
+            heads_only = on_backbone == 0 || on_backbone == n_head;  // (one list serves them: all on one weight set)
+            if (heads_only) {
+                const int set = on_backbone == n_head ? 0 : 1;
+                n_of[set] = n_head;
+                n_of[1 - set] = 0;
+                rows_of[set] = c->head_rows();
+                cnt_of[set] = c->meta_dev + 2;  // StepMeta::n_head_rows
+            }
+            if (heads_only && n_head == 0) break;
+        }
         {
             LaunchScope ls(c, K_PREFILL_ATTN, kv_read, 0, -1);
-            note(launch_attention_prefill(c, n_tiles, l - 1));
+            note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
         }
         {
             LaunchScope ls(c, K_OPROJ, wsum * qdim * d, 0, -1);
@@ -837,14 +857,14 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *r
                 project(nullptr, F, d / kTcBM, 0, 0, 0, 0, set, m.d, m.d, m.d, {&w.rd, &w.rd, &w.rd}, {d, 0, 0}, down_e);
             }
         }
-        if (record_fail || (l < L && leave[l])) {
+        if (l < L && (record_fail || leave[l])) {
             LaunchScope ls(c, K_SCORE, (double)n * d * 8.0, 0, -1);
             note(launch_k(score_compact_kernel, dim3(n), dim3(256), 0, c->stream, true, c->meta(), l, L, g.entry_layer, g.exit_mode,
                           (const float *)h_in, (const float *)h_out, d, c->pass, (const uint8_t *)c->state_at(at), c->state_at(l),
                           lists, c->hint_act, c->tickets + 1, record_fail ? c->prefill_fail : (int32_t *)nullptr,
                           (const int32_t *)c->row_slot(), (int32_t *)nullptr));
             at = l;
-            n_riv += l < L ? leave[l] : 0;
+            n_riv += leave[l];
         }
         hi = (hi + 2) % 3;
     }
@@ -970,7 +990,13 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
             ++n_tiles;
             i = j;
         }
-        reinterpret_cast<StepMeta *>(mh)->pad2[0] = n_tiles;
+        const bool long_pass = wide && n > kWideMin, head_tiles = long_pass && n_tiles + n_head <= max_rows;
+        if (head_tiles)  // the last block attends at the prompt ends only: a one-row tile each, behind the others
+            for (int i = 0; i < n_head; ++i) {
+                mh[kMetaHdr + 8 * max_rows + n_tiles + i] = mh[kMetaHdr + 5 * max_rows + i];
+                mh[kMetaHdr + 9 * max_rows + n_tiles + i] = 1;
+            }
+        reinterpret_cast<StepMeta *>(mh)->pad2[0] = n_tiles + (head_tiles ? n_head : 0);
         c->prefill_attn_now = n >= 5 && prefill_attn_supported(c);
         const bool want_logits = logits_last && n_head > 0;
         set_io_meta(mh, tok + tok0, c->tau_i, c->row_forced(), want_logits ? c->logits_i : nullptr, c->next_i, c->exit_i,
@@ -979,8 +1005,9 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         c->rows_distinct = false;  // consecutive positions of one sequence share a chunk
         // (a short rest of at most kWideMin rows takes the batch kernels: they split K where tiles are few)
         const int32_t *pos = mh + kMetaHdr + max_rows;
-        const int rc_rows = wide && n > kWideMin ? run_rows_wide(c, n, n_tiles, n_head, pos, mh + kMetaHdr + 7 * max_rows, record_fail)
-                                                 : run_rows(c, n, n_head, pos, record_fail);
+        const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, n_head, mh + kMetaHdr + 5 * max_rows, head_tiles, pos,
+                                                      mh + kMetaHdr + 7 * max_rows, record_fail)
+                                      : run_rows(c, n, n_head, pos, record_fail);
         c->rows_distinct = true;
         c->prefill_attn_now = false;
         if (rc_rows) return rc_rows;
