@@ -324,6 +324,23 @@ __device__ __forceinline__ void stream_load_rows(const ProjIn &in, const int32_t
 // ---------------------------------------------------------------- one task = R weight rows against N activation rows
 constexpr int kStreamPF = 4;  // 16-byte loads per weight row issued together (R * kStreamPF in flight per lane)
 
+// Eight bf16 weights against eight activations: the even and the odd products in the two halves of packed fp32 operations
+// (one fma.rn.f32x2 is two FMAs for the price of one issue slot; each half rounds as the single operation does).
+__device__ __forceinline__ float dot8_bf16(const uint4 &v, const float4 &x0, const float4 &x1) {
+    float a0, a1;
+    asm("{\n\t.reg .b64 w, x, a;\n\t"
+        "mov.b64 w, {%2, %3};\n\tmov.b64 x, {%10, %11};\n\tmul.rn.f32x2 a, w, x;\n\t"
+        "mov.b64 w, {%4, %5};\n\tmov.b64 x, {%12, %13};\n\tfma.rn.f32x2 a, w, x, a;\n\t"
+        "mov.b64 w, {%6, %7};\n\tmov.b64 x, {%14, %15};\n\tfma.rn.f32x2 a, w, x, a;\n\t"
+        "mov.b64 w, {%8, %9};\n\tmov.b64 x, {%16, %17};\n\tfma.rn.f32x2 a, w, x, a;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "=f"(a0), "=f"(a1)
+        : "f"(bf16lo(v.x)), "f"(bf16hi(v.x)), "f"(bf16lo(v.y)), "f"(bf16hi(v.y)), "f"(bf16lo(v.z)), "f"(bf16hi(v.z)),
+          "f"(bf16lo(v.w)), "f"(bf16hi(v.w)), "f"(x0.x), "f"(x0.y), "f"(x0.z), "f"(x0.w), "f"(x1.x), "f"(x1.y), "f"(x1.z),
+          "f"(x1.w));
+    return a0 + a1;
+}
+
 template <int R>
 __device__ __forceinline__ void stream_issue_bf16(const uint16_t *const (&wrow)[R], int nch, int it0, int lane,
                                                   uint4 (&w)[R][kStreamPF]) {
@@ -367,14 +384,7 @@ __device__ __forceinline__ void stream_dots_bf16(const uint16_t *const (&wrow)[R
                     const float4 x0 = *reinterpret_cast<const float4 *>(xb + n * xstride);
                     const float4 x1 = *reinterpret_cast<const float4 *>(xb + n * xstride + 128);
 #pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        const uint4 v = w[r][u];
-                        float a0 = bf16lo(v.x) * x0.x, a1 = bf16hi(v.x) * x0.y;
-                        a0 = fmaf(bf16lo(v.y), x0.z, a0); a1 = fmaf(bf16hi(v.y), x0.w, a1);
-                        a0 = fmaf(bf16lo(v.z), x1.x, a0); a1 = fmaf(bf16hi(v.z), x1.y, a1);
-                        a0 = fmaf(bf16lo(v.w), x1.z, a0); a1 = fmaf(bf16hi(v.w), x1.w, a1);
-                        acc[r][n] += a0 + a1;
-                    }
+                    for (int r = 0; r < R; ++r) acc[r][n] += dot8_bf16(w[r][u], x0, x1);
                 }
             }
         }
@@ -426,14 +436,7 @@ __device__ __forceinline__ void stream_fma_bf16(const uint4 (&w)[R][kStreamPF], 
                 const float4 x0 = *reinterpret_cast<const float4 *>(xb + n * xstride);
                 const float4 x1 = *reinterpret_cast<const float4 *>(xb + n * xstride + 128);
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const uint4 v = w[r][u];
-                    float a0 = bf16lo(v.x) * x0.x, a1 = bf16hi(v.x) * x0.y;
-                    a0 = fmaf(bf16lo(v.y), x0.z, a0); a1 = fmaf(bf16hi(v.y), x0.w, a1);
-                    a0 = fmaf(bf16lo(v.z), x1.x, a0); a1 = fmaf(bf16hi(v.z), x1.y, a1);
-                    a0 = fmaf(bf16lo(v.w), x1.z, a0); a1 = fmaf(bf16hi(v.w), x1.w, a1);
-                    acc[r][n] += a0 + a1;
-                }
+                for (int r = 0; r < R; ++r) acc[r][n] += dot8_bf16(w[r][u], x0, x1);
             }
         }
     }
