@@ -100,6 +100,14 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
         const int s3 = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms * 3);
         if (tiles * s3 > tiles * a.splits && tiles * s3 <= c->num_sms * 3) { occ = 3; a.splits = s3; }
     }
+    // One CTA per SM, in the shared memory of half an SM, where it still has a long enough run of k-blocks: the other half
+    // takes the CTAs of the projection behind this one (and of the dequantising kernel beside it), which set up and request
+    // their first weights while this grid drains.  8B-class shape, 64 rows: two or three CTAs per SM 2083 us a step (8 blocks),
+    // so 2005; with fewer than a dozen k-blocks per CTA (1B-class shape, 8 rows) more CTAs win (1118 against 1224-1337).
+    if (occ >= 2 && allow_split && tiles < c->num_sms) {
+        const int s1 = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms);
+        if (s1 >= 2 && K / kTcBK / s1 >= 12) { a.splits = s1; occ = 2; }
+    }
     a.n_stages = tc_stages_at(np, occ);
     tc_cols(np, occ, &a.wide);
     // the finished tile lives in the pipeline memory
