@@ -9,15 +9,15 @@ namespace river {
 
 namespace {
 
-// Rows per tile: the tiles go to `pairs` CTA pairs in whole rounds, so a size that leaves the last round nearly full wins
-// over a larger one that does not (8B-class QKV, 1024 rows: 96 tiles of 256 rows are 2 rounds of 74 pairs, 144 tiles of 192 are
-// 2 shorter ones).  Below 96 rows an MMA takes as long as at 96.
+// Rows per tile: the tiles go to `pairs` CTA pairs in whole rounds, so a size that leaves the last round nearly full can win
+// over a larger one that does not; a round takes about as long as its rows and 128 more (8B-class gate/up, 1024 rows: 7 rounds
+// of 256 rows 297 us, 10 of 192 338, 13 of 128 388; QKV: 2 of 256 112, 2 of 192 102, 3 of 128 122).
 int wide_bn(int feature_pairs, int n, int pairs) {
     int best = 256;
     double best_t = 1e30;
     for (int bn = 256; bn >= 64; bn -= 32) {
         const int total = feature_pairs * ((n + bn - 1) / bn), rounds = (total + pairs - 1) / pairs;
-        const double t = rounds * (std::max(bn, 96) + 8.0);
+        const double t = rounds * (bn + 128.0);
         if (t < best_t * 0.995) { best_t = t; best = bn; }
     }
     return best;
