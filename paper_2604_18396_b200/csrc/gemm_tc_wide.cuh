@@ -16,7 +16,7 @@
 // working at one time share weight tiles in L2.
 //
 // What bounds it: the tensor pipe and, when passes follow each other, the power cap.  8B-class shape, 1024 rows, operand
-// kernel included: QKV 98 us, O 74, gate/up 433, down 167 (1.44 PFLOP/s of bf16 MMAs, half of them for the low parts) against
+// kernel included: QKV 96 us, O 56, gate/up 305, down 148 (1.7 PFLOP/s of bf16 MMAs, half of them for the low parts) against
 // 4 x (108, 42, 191, 81) us in passes of 256 rows on tc_gemm_kernel.
 #pragma once
 #include "gemm_tc.cuh"
@@ -31,8 +31,10 @@ constexpr int kWdOwn = 256 / (kWdChunk * kWdGroups);               // chunks of 
 constexpr uint32_t kWdABytes = kTcBM * kTcBK * 2;
 
 // ---------------------------------------------------------------- epilogues, straight from registers
-// run(): this thread holds tile row r = 32 quarter + lane of a 32-row chunk, v[e] = the value for list row n0 + e (e < live);
-// `row` is the step row id of list row n0 + lane.  Nothing is staged: the copies lay a tile's weight rows down so that
+// A thread holds tile row r = 32 quarter + lane of a 32-row chunk, v[e] = the value for list row n0 + e (e < live); `row` is the
+// step row id of list row n0 + lane.  begin() runs before the tile's first segment is there: it sets the sums' start and
+// requests what run() will need (run() gets its return value back), so that no load waits behind the last MMA (residual
+// and cache slots read in run() instead: 8B-class O 68 us against 56, down 157 against 148, 1024 rows).  Nothing is staged: the copies lay a tile's weight rows down so that
 // what belongs together (gate and up feature, the two halves of a rotary pair) sits 16 lanes apart in one warp - ONE copy
 // per tile and k-block does that, through a five-dimensional map (make_map_paired); eight copies of 16 rows each kept the
 // issuing lane from keeping up (8B-class gate/up, 1024 rows: 490 us against 433) - and lanes 0-15 finish the even
@@ -42,20 +44,21 @@ struct WdResidEpi {  // out[row][f] = resid[row][f] + value; tile rows in the ma
     float *out;
     int out_dim;
     static constexpr bool kPaired = false;
-    __device__ void run(float (&v)[32], int ft, int quarter, int lane, int live, int row, int) const {
+    __device__ int begin(float (&v)[32], int ft, int quarter, int lane, int live, int row) const {  // the sums start from the residual
         const int f = ft * kTcBM + 32 * quarter + lane;
 #pragma unroll
-        for (int e0 = 0; e0 < 32; e0 += 4) {  // four residual values requested before the first sum is stored
-            float r[4];
-            int o[4];  // (a pass holds at most 1024 rows: 32-bit offsets)
+        for (int e = 0; e < 32; ++e) {
+            const int o = __shfl_sync(0xffffffffu, row, e) * out_dim + f;  // (a pass holds at most 1024 rows: 32-bit offsets)
+            v[e] = e < live ? __ldcg(resid + o) : 0.f;
+        }
+        return 0;
+    }
+    __device__ void run(float (&v)[32], int ft, int quarter, int lane, int live, int row, int, int) const {
+        const int f = ft * kTcBM + 32 * quarter + lane;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                o[e] = __shfl_sync(0xffffffffu, row, e0 + e) * out_dim + f;
-                r[e] = e0 + e < live ? __ldcg(resid + o[e]) : 0.f;
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (e0 + e < live) out[o[e]] = r[e] + v[e0 + e];
+        for (int e = 0; e < 32; ++e) {
+            const int o = __shfl_sync(0xffffffffu, row, e) * out_dim + f;
+            if (e < live) out[o] = v[e];
         }
     }
 };
@@ -66,12 +69,18 @@ __device__ __forceinline__ void wd_trade(float v0, float v1, int lane, float &a,
     a = lane < 16 ? v0 : got;
     b = lane < 16 ? got : v1;
 }
+__device__ __forceinline__ int wd_zero(float (&v)[32]) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e) v[e] = 0.f;
+    return 0;
+}
 struct WdGateUpEpi {  // 64 features per tile -> the down projection's operand rows, as TcGateUpEpi writes them
     int F;
     uint16_t *ohi, *olo;
     int f16, up_first;  // up_first: the lower row of a pair is the up feature
     static constexpr bool kPaired = true;
-    __device__ void run(float (&v)[32], int ft, int quarter, int lane, int live, int, int n0) const {
+    __device__ int begin(float (&v)[32], int, int, int, int, int) const { return wd_zero(v); }
+    __device__ void run(float (&v)[32], int ft, int quarter, int lane, int live, int, int, int n0) const {
         const int f = ft * 64 + 16 * quarter + (lane & 15), j = f & 7;
         const int at = f16 ? (f & ~7) + (j < 4 ? 2 * j : 2 * (j - 4) + 1) : f;
         const int odd = lane >> 4;
@@ -102,29 +111,41 @@ struct WdQkvEpi {  // tiles walk the concatenated [q heads | k heads | v heads] 
     KvAddr kv;
     int *dev_err;
     static constexpr bool kPaired = true;
-    __device__ void run(float (&v)[32], int ft, int quarter, int lane, int live, int row, int) const {
-        const int half = dh >> 1, per = half >> 4, feat0 = ft * kTcBM, qdim = Hq * dh, kvdim = Hkv * dh;
-        const int which = feat0 < qdim ? 0 : (feat0 < qdim + kvdim ? 1 : 2);
+    __device__ void locate(int ft, int quarter, int &which, int &head, int &i0) const {
+        const int per = dh >> 5, feat0 = ft * kTcBM, qdim = Hq * dh, kvdim = Hkv * dh;
+        which = feat0 < qdim ? 0 : (feat0 < qdim + kvdim ? 1 : 2);
         const int base = which == 0 ? feat0 : (which == 1 ? feat0 - qdim : feat0 - qdim - kvdim);
-        const int head = base / dh + quarter / per, i = 16 * (quarter % per) + (lane & 15), odd = lane >> 4;
-        int slot = 0;  // cache row (of dh values) of list row n0 + lane, -1: none
+        head = base / dh + quarter / per;
+        i0 = 16 * (quarter % per);
+    }
+    // the cache row (of dh values) of list row n0 + lane, -1: none
+    __device__ int begin(float (&v)[32], int ft, int quarter, int lane, int live, int row) const {
+        int which, head, i0, slot = -1;
+        locate(ft, quarter, which, head, i0);
         if (which != 0 && lane < live) {
             const int page = kv.row_page[row];
-            if (page < 0 || page >= kv.n_pages) { atomicExch(dev_err, DEV_BAD_PAGE); slot = -1; }
+            if (page < 0 || page >= kv.n_pages) atomicExch(dev_err, DEV_BAD_PAGE);
             else slot = (int)(kv.base(page, which - 1, head, kv.row_pos[row] % kPage) / dh);
         }
+        wd_zero(v);
+        return slot;
+    }
+    __device__ void run(float (&v)[32], int ft, int quarter, int lane, int live, int row, int slot, int) const {
+        int which, head, i0;
+        locate(ft, quarter, which, head, i0);
+        const int half = dh >> 1, qdim = Hq * dh, i = i0 + (lane & 15), odd = lane >> 4;
 #pragma unroll
-        for (int e0 = 0; e0 < 32; e0 += 4) {
-            float2 cs[2];
-            int rw[2];
+        for (int e0 = 0; e0 < 32; e0 += 8) {
+            float2 cs[4];
+            int rw[4];
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {  // the rotations of four rows requested together
+            for (int e = 0; e < 4; ++e) {  // the rotations of eight rows requested together
                 rw[e] = __shfl_sync(0xffffffffu, row, e0 + 2 * e + odd);
                 cs[e] = make_float2(1.f, 0.f);
                 if (which != 2 && e0 + 2 * e + odd < live) cs[e] = rope_cs[rw[e] * half + i];
             }
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
+            for (int e = 0; e < 4; ++e) {
                 float lo, hi;
                 wd_trade(v[e0 + 2 * e], v[e0 + 2 * e + 1], lane, lo, hi);
                 const int at = __shfl_sync(0xffffffffu, slot, e0 + 2 * e + odd);
@@ -326,10 +347,13 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
         for (int t = pair0; t < total && !quit; t += pairs) {
             const int ft = 2 * (t / n_tiles) + (int)rank, n0 = (t % n_tiles) * bn, live = ft < a.tiles ? min(bn, n_live - n0) : 0;
             float acc[kWdOwn][kWdChunk];  // this warp's chunks: columns 32 (group + 4 i)
+            int row[kWdOwn], note[kWdOwn];  // what the epilogue reads elsewhere is requested now, under the MMAs
 #pragma unroll
-            for (int i = 0; i < kWdOwn; ++i)
-#pragma unroll
-                for (int e = 0; e < kWdChunk; ++e) acc[i][e] = 0.f;
+            for (int i = 0; i < kWdOwn; ++i) {
+                const int c = kWdChunk * (group + kWdGroups * i);
+                row[i] = c + lane < live ? a.rows[n0 + c + lane] : 0;
+                note[i] = epi.begin(acc[i], ft, q, lane, min(kWdChunk, live - c), row[i]);
+            }
 #pragma unroll 1
             for (int kb0 = 0; kb0 < nkb; kb0 += a.seg, ++j) {
                 const uint32_t buf = j & 1;
@@ -358,7 +382,7 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
 #pragma unroll
             for (int i = 0; i < kWdOwn; ++i) {
                 const int c = kWdChunk * (group + kWdGroups * i);
-                if (c < live) epi.run(acc[i], ft, q, lane, min(kWdChunk, live - c), c + lane < live ? a.rows[n0 + c + lane] : 0, n0 + c);
+                if (c < live) epi.run(acc[i], ft, q, lane, min(kWdChunk, live - c), row[i], note[i], n0 + c);
             }
         }
     }
