@@ -51,8 +51,9 @@ cudaError_t launch_tc_w4(river_ctx *c, const ProjIn &in, const CUtensorMap *cons
     // splits (measured on the 1B shape, K = 2048: 2 -> 4 splits 35 -> 31 us per layer for QKV, 33 -> 27 us for O)
     const int raw_tiles = K / (kTcBK * kW4Super);
     // (splits for one CTA per SM: the rest of the SM belongs to tc_gemm_kernel's CTAs beside this grid and to the next
-    // projection's; 8B-class shape, 61 rows on both weight sets 2069 -> 2050 us a step, 1B-class, 8 rows 1120 -> 1097)
-    a.splits = tc_pick_splits(c, tiles, raw_tiles, c->num_sms, raw_tiles <= 8 ? 2 : 4);
+    // projection's; 8B-class shape, 61 rows on both weight sets 2069 -> 2050 us a step, 1B-class, 8 rows 1120 -> 1097; with
+    // fewer than eight raw tiles the clusters this asks for cost more than they bring: tiny shape, 77 rows 149.8 -> 152.4)
+    a.splits = tc_pick_splits(c, tiles, raw_tiles, c->num_sms * (two && raw_tiles < 8 ? 2 : 1), raw_tiles <= 8 ? 2 : 4);
     if (sizeof(float) * (size_t)np * kTcLd > (size_t)a.n_stages * stage + raw) return cudaErrorInvalidValue;
     // tensor memory: accumulator + A tiles, a power of two of columns; every CTA that can be resident on an SM must get
     // its columns at once (a CTA stuck in the allocation while its cluster waits for it could not be waited out), so
