@@ -20,5 +20,8 @@ cudaError_t launch_attention(river_ctx *c, int n, int layer0);
 bool prefill_attn_supported(const river_ctx *c);
 // tensor-core causal attention of a prefill chunk's query tiles [tile0, tile0 + n_tiles) (as the step metadata lists them)
 cudaError_t launch_attention_prefill(river_ctx *c, int tile0, int n_tiles, int layer0);
+// the same on tcgen05: the query tiles [0, n_tiles) hold up to prefill_tc_positions() positions (instead of kPfBM)
+int prefill_tc_positions(const river_ctx *c);
+cudaError_t launch_attention_prefill_tc(river_ctx *c, int n_tiles, int layer0);
 
 }  // namespace river

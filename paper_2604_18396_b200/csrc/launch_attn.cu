@@ -7,6 +7,7 @@
 #include "attn_decode.cuh"
 #include "attn_small.cuh"
 #include "attn_prefill.cuh"
+#include "attn_prefill_tc.cuh"
 
 namespace river {
 
@@ -77,6 +78,30 @@ cudaError_t launch_attn_prefill_t(river_ctx *c, int tile0, int n_tiles, int laye
     return launch_k(attn_prefill_kernel<DH, GQ>, dim3(n_tiles, g.Hkv), dim3(32 * GQ), smem, c->stream, true, a);
 }
 }  // namespace
+
+namespace {
+template <int DH, int GQ>
+cudaError_t launch_attn_prefill_tc_t(river_ctx *c, int n_tiles, int layer0) {
+    PrefillTcArgs a{};
+    a.tile_row0 = c->tile_row0(); a.tile_rows = c->tile_rows();
+    a.q = c->qbuf; a.out = c->obuf; a.kv = kv_addr(c, layer0); a.Hq = c->cfg.Hq;
+    a.qscale = 1.4426950408889634f / std::sqrt((float)DH);
+    a.dev_err = c->dev_err;
+    const size_t smem = attn_prefill_tc_smem_bytes(DH);
+    const cudaError_t e = ensure_smem(c, attn_prefill_tc_kernel<DH, GQ>, smem);
+    if (e != cudaSuccess) return e;
+    return launch_k(attn_prefill_tc_kernel<DH, GQ>, dim3(n_tiles, c->cfg.Hkv), dim3(kPtThreads), smem, c->stream, true, c->kv_tmap, a);
+}
+}  // namespace
+
+int prefill_tc_positions(const river_ctx *c) { return kPtRows / (c->cfg.Hq / c->cfg.Hkv); }
+cudaError_t launch_attention_prefill_tc(river_ctx *c, int n_tiles, int layer0) {
+    const int gq = c->cfg.Hq / c->cfg.Hkv;
+#define ATTP(DH_, GQ_) if (c->cfg.dh == DH_ && gq == GQ_) return launch_attn_prefill_tc_t<DH_, GQ_>(c, n_tiles, layer0);
+    ATTP(64, 1) ATTP(64, 2) ATTP(64, 4) ATTP(64, 8) ATTP(128, 1) ATTP(128, 2) ATTP(128, 4) ATTP(128, 8)
+#undef ATTP
+    return cudaErrorInvalidValue;
+}
 
 cudaError_t launch_attention_prefill(river_ctx *c, int tile0, int n_tiles, int layer0) {
     const int gq = c->cfg.Hq / c->cfg.Hkv;

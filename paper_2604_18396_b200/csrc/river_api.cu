@@ -761,7 +761,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
 // follows QKV there runs on those rows (head[]: their row ids; head_tiles: their one-row query tiles follow the chunk's
 // n_tiles in the metadata) and on none in a pass without a prompt end.  (8B-class shape, 1024 rows: the rest of a block takes
 // 0.7-1.0 ms for all of them, 0.2 ms for one: the projections' weight streams.)
-int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *head, bool head_tiles, const int32_t *row_pos_host,
+int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, const int32_t *head, bool head_tiles, const int32_t *row_pos_host,
                   const int32_t *depth, bool record_fail) {
     const river_config &g = c->cfg;
     const int L = g.L, d = g.d, F = g.F, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
@@ -829,7 +829,8 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, int n_head, const int32_t *h
         }
         {
             LaunchScope ls(c, K_PREFILL_ATTN, kv_read, 0, -1);
-            note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
+            note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1)
+                 : tc_attn ? launch_attention_prefill_tc(c, n_tiles, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
         }
         {
             LaunchScope ls(c, K_OPROJ, wsum * qdim * d, 0, -1);
@@ -978,11 +979,18 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         }
         mh[0] = n; mh[1] = n_upd; mh[2] = n_head;
         set_attn_meta(c, mh, n);
-        // query tiles for the tensor-core prefill attention: up to 16 consecutive positions of one sequence each
+        // query tiles of the prefill attention: consecutive positions of one sequence, up to 16 - or as many as make 128
+        // query rows, for the tcgen05 kernel, where the rows of a long pass look back at 128 positions and more on average
+        // (below, its tiles are mostly padding: mini shape, prompts of 96 positions 20 against 17 us; 1B-class, 435: 30 against 32)
+        const bool long_pass = wide && n > kWideMin;
+        long long seen = 0;
+        for (int i = 0; i < n; ++i) seen += mh[kMetaHdr + max_rows + i] + 1;
+        const bool tc_attn = long_pass && seen >= 128LL * n;
+        const int tile_max = tc_attn ? prefill_tc_positions(c) : kPfBM;
         int n_tiles = 0;
         for (int i = 0; i < n;) {
             int j = i + 1;
-            while (j < n && j - i < kPfBM && mh[kMetaHdr + j] == mh[kMetaHdr + i] &&
+            while (j < n && j - i < tile_max && mh[kMetaHdr + j] == mh[kMetaHdr + i] &&
                    mh[kMetaHdr + max_rows + j] == mh[kMetaHdr + max_rows + i] + (j - i))
                 ++j;
             mh[kMetaHdr + 8 * max_rows + n_tiles] = i;
@@ -990,7 +998,7 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
             ++n_tiles;
             i = j;
         }
-        const bool long_pass = wide && n > kWideMin, head_tiles = long_pass && n_tiles + n_head <= max_rows;
+        const bool head_tiles = long_pass && n_tiles + n_head <= max_rows;
         if (head_tiles)  // the last block attends at the prompt ends only: a one-row tile each, behind the others
             for (int i = 0; i < n_head; ++i) {
                 mh[kMetaHdr + 8 * max_rows + n_tiles + i] = mh[kMetaHdr + 5 * max_rows + i];
@@ -1005,7 +1013,7 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         c->rows_distinct = false;  // consecutive positions of one sequence share a chunk
         // (a short rest of at most kWideMin rows takes the batch kernels: they split K where tiles are few)
         const int32_t *pos = mh + kMetaHdr + max_rows;
-        const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, n_head, mh + kMetaHdr + 5 * max_rows, head_tiles, pos,
+        const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, tc_attn, n_head, mh + kMetaHdr + 5 * max_rows, head_tiles, pos,
                                                       mh + kMetaHdr + 7 * max_rows, record_fail)
                                       : run_rows(c, n, n_head, pos, record_fail);
         c->rows_distinct = true;

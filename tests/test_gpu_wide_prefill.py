@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from tests.gpu_harness import INF, Pair, draw_model
-from workloads import synth
+from workloads import rtn_w4, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -72,3 +72,24 @@ def test_mixed_depths_in_one_pass(mini8):
     assert len(seen) > 1 and any(len(set(k)) > 1 for k in seen), f"no threshold separates the prompts: {list(seen)}"
     long.close()
     short.close()
+
+
+@pytest.mark.parametrize("dh,gq", [(64, 1), (64, 2), (64, 4), (64, 8), (128, 1), (128, 2), (128, 4), (128, 8)])
+def test_long_pass_attention_geometries(dh, gq):
+    """Every head dim and group size of the attention kernel, prompts that end inside and on the edges of its query tiles
+    (128 / gq positions), key tiles (64) and pages (16): the second block's cache shows the attention of every position."""
+    hkv = max(1, 512 // dh // gq, 128 // dh)
+    shape = synth.ModelShape("a", 2, 256, hkv * gq, hkv, dh, 256, 1024, seed=7, resid_decay=1.0)
+    bb = synth.make_backbone(shape, "cpu")
+    for lay in bb["layers"]:  # scores of a few units, so that the running maximum moves from tile to tile
+        lay["wq"] *= 12.0
+    rv = rtn_w4.make_river(bb, shape.group)
+    to = lambda x: x.cuda() if isinstance(x, torch.Tensor) else (  # noqa: E731
+        {k: to(v) for k, v in x.items()} if isinstance(x, dict) else type(x)(to(v) for v in x))
+    lens = [400, 129, 1, 448, 16, 30]
+    p = Pair((shape, (bb, rv), (to(bb), to(rv))), 6, 456, 8, prefill_chunk=256, kv_store=1, storage_yardstick=True, page_shuffle_seed=5)
+    p.prefill(list(range(6)), [synth.tokens(47, b, n, shape.V).numpy() for b, n in enumerate(lens)])
+    for b, n in enumerate(lens):
+        p.compare_kv(b, n, f"dh {dh} gq {gq} prompt {n}")
+    assert p.gpu.stats().device_error == 0
+    p.close()
