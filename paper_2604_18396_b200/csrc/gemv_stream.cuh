@@ -34,6 +34,7 @@ struct QkvProblem {
     float *q_out;
     KvAddr kv;
     int *dev_err;
+    __device__ int row_len() const { return K; }
     template <int R>
     __device__ int n_tasks() const { return (Hq + 2 * Hkv) * (dh / 2) / (R / 2); }
     // task -> (matrix, head, first pair index)
@@ -141,6 +142,8 @@ struct ResidProblem {  // out[row][o] = resid[row][o] + W[o] . x[row]
     int K, out_dim, group;
     const float *resid;
     float *out;
+    int ld = 0;  // inputs of a whole weight row when this launch covers a part of them (0: K)
+    __device__ int row_len() const { return ld ? ld : K; }
     template <int R> __device__ int n_tasks() const { return out_dim / R; }
     template <int R> __device__ size_t run_row(int t, int) const { return (size_t)t * R; }
     template <int R> __device__ const uint16_t *bf16_base(int, int) const { return w; }
@@ -167,6 +170,7 @@ struct GateUpProblem {  // act[row][f] = silu(Wg[f] . y) * (Wu[f] . y)
     W4 rg, ru;
     int K, F, group;
     float *act;
+    __device__ int row_len() const { return K; }
     template <int R> __device__ int n_tasks() const { return F / (R / 2); }
     template <int R> __device__ size_t run_row(int t, int) const { return (size_t)t * (R / 2); }
     template <int R> __device__ const uint16_t *bf16_base(int, int run) const { return run == 0 ? wg : wu; }
@@ -281,7 +285,7 @@ __device__ __forceinline__ void stream_load_rows(const ProjIn &in, const int32_t
             for (int k = tid; k < xstride; k += nthr) dst[k] = 0.f;
             continue;
         }
-        const float4 *src = reinterpret_cast<const float4 *>(in.src + (size_t)idx[i0 + n] * K);
+        const float4 *src = reinterpret_cast<const float4 *>(in.src + (size_t)idx[i0 + n] * (in.ld ? in.ld : K));
         const int nv = K >> 2;
         float ss = 0.f;
         for (int v0 = 0; v0 < nv; v0 += nthr * 4) {
@@ -486,18 +490,18 @@ __device__ __forceinline__ void stream_rows_bf16(const P &p, int t, const uint16
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int run = r / (R / P::NRUN), j = r % (R / P::NRUN);
-        rows[r] = p.template bf16_base<R>(t, run) + (p.template run_row<R>(t, run) + j) * (size_t)p.K;
+        rows[r] = p.template bf16_base<R>(t, run) + (p.template run_row<R>(t, run) + j) * (size_t)p.row_len();
     }
 }
 template <class P, int R>
 __device__ __forceinline__ void stream_rows_w4(const P &p, int t, W4 (&rows)[R]) {
-    const int ng = p.K / p.group;
+    const int row_len = p.row_len(), ng = row_len / p.group;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int run = r / (R / P::NRUN), j = r % (R / P::NRUN);
         const W4 b = p.template w4_base<R>(t, run);
         const size_t row = p.template run_row<R>(t, run) + j;
-        rows[r] = W4{b.codes + row * (size_t)(p.K >> 1), b.scale + row * ng, b.zero + row * ng};
+        rows[r] = W4{b.codes + row * (size_t)(row_len >> 1), b.scale + row * ng, b.zero + row * ng};
     }
 }
 

@@ -2,6 +2,7 @@
 // the merge of its argmax partials.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "launch.h"
 
@@ -61,13 +62,31 @@ cudaError_t launch_stream_t(river_ctx *c, const P &p, const ProjIn &in, const Ro
 template <class P>
 cudaError_t launch_stream(river_ctx *c, const P &p, const ProjIn &in, const RowLists &rl, int K, int tasks_r2, int n,
                           int has_river, bool pdl, int skip_backbone, const DecideArgs &dec) {
+    if constexpr (std::is_same_v<P, ResidProblem>) {
+        // Three and more rows of a long K do not fit into shared memory together, and a pass for each pair would stream the
+        // weights twice: two launches of half the inputs instead, the second adding to the first one's output (8B-class down
+        // blocks, three rows: 1424 us a step, so 1319, the row count's own instance included).
+        if (n >= 3 && !in.gain && !p.ld && K % (2 * p.group) == 0 && K % 128 == 0 && stream_smem_bytes(3, K) > 200 * 1024) {
+            ResidProblem a = p, b = p;
+            ProjIn ia = in, ib = in;
+            const int half = K / 2;
+            a.K = b.K = half; a.ld = b.ld = ia.ld = ib.ld = K;
+            b.w += half; b.rw.codes += half / 2; b.rw.scale += half / p.group; b.rw.zero += half / p.group;
+            b.resid = p.out; ib.src += half;
+            const cudaError_t e = launch_stream(c, a, ia, rl, half, tasks_r2, n, has_river, pdl, skip_backbone, dec);
+            ++c->st.launches_last_step;
+            return e != cudaSuccess ? e : launch_stream(c, b, ib, rl, half, tasks_r2, n, has_river, pdl, skip_backbone, dec);
+        }
+    }
+    // rows per pass: as many as the step has (up to four: every row costs its shared-memory reads and FMAs for every weight,
+    // a row of padding too), if they fit
     int n_sel = 1;
-    while (n_sel < n && n_sel < 4 && stream_smem_bytes(n_sel * 2, K) <= 200 * 1024) n_sel *= 2;
+    while (n_sel < n && n_sel < 4 && stream_smem_bytes(n_sel + 1, K) <= 200 * 1024) ++n_sel;
     const int r = K >= 4096 ? 2 : 4;  // weight rows per task
     const int tasks = tasks_r2 * 2 / r;
 #define STREAM_CASE(N_, R_) if (n_sel == N_ && r == R_) return launch_stream_t<P, N_, R_>(c, p, in, rl, K, tasks, has_river, pdl, skip_backbone, dec);
-    STREAM_CASE(1, 2) STREAM_CASE(2, 2) STREAM_CASE(4, 2)
-    STREAM_CASE(1, 4) STREAM_CASE(2, 4) STREAM_CASE(4, 4)
+    STREAM_CASE(1, 2) STREAM_CASE(2, 2) STREAM_CASE(3, 2) STREAM_CASE(4, 2)
+    STREAM_CASE(1, 4) STREAM_CASE(2, 4) STREAM_CASE(3, 4) STREAM_CASE(4, 4)
 #undef STREAM_CASE
     return cudaErrorInvalidValue;
 }
@@ -76,8 +95,7 @@ template cudaError_t launch_stream<ResidProblem>(river_ctx *, const ResidProblem
 template cudaError_t launch_stream<GateUpProblem>(river_ctx *, const GateUpProblem &, const ProjIn &, const RowLists &, int, int, int, int, bool, int, const DecideArgs &);
 
 cudaError_t launch_head_stream(river_ctx *c, const HeadArgs &a, int n_head) {
-    int n_sel = 1;
-    while (n_sel < n_head && n_sel < 4) n_sel *= 2;
+    const int n_sel = std::min(n_head, 4);
     const int xstride = xs_stride(a.d, 8);
     const size_t smem = sizeof(float) * (32 + (size_t)n_sel * xstride);
 #define HEAD_CASE(N_)                                                                                              \
@@ -86,7 +104,7 @@ cudaError_t launch_head_stream(river_ctx *c, const HeadArgs &a, int n_head) {
         if (e != cudaSuccess) return e;                                                                            \
         return launch_k(lm_head_kernel<N_, 4>, dim3(c->head_grid), dim3(256), smem, c->stream, true, a, xstride); \
     }
-    HEAD_CASE(1) HEAD_CASE(2) HEAD_CASE(4)
+    HEAD_CASE(1) HEAD_CASE(2) HEAD_CASE(3) HEAD_CASE(4)
 #undef HEAD_CASE
     return cudaErrorInvalidValue;
 }

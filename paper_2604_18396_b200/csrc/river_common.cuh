@@ -146,6 +146,7 @@ struct ProjIn {
     const float *src;      // [rows][K]
     const uint16_t *gain;  // bf16 [K] or nullptr = no normalisation
     float eps;
+    int ld = 0;            // row stride of src when K inputs of longer rows are taken (streaming kernels; 0: K)
 };
 
 struct KvAddr {
