@@ -314,6 +314,8 @@ struct TcArgs {
     int late_release; // 1: dependent grids may start only once this grid's own dependency is met (see the kernel)
     int one_box;      // 1: map_bhi covers the hi rows AND the lo rows behind them: one copy of 2 n_pad rows per k-block
     int wide;         // 1: hi and lo operand rows as one operand of 2 n_pad rows (the host checks the TMEM budget)
+    int halves;       // 1 (wide only): the second half of the k-blocks goes to a second accumulator, added at the end: the error
+                      // of a sum inside the tensor cores grows with its length
     int a_rows_per_map;  // a tile's 128 rows come from map tile_idx / (rows_per_map / 128) ... see tile_map()
     int gateup;       // 1: a tile is 64 rows of map 0 + 64 rows of map 1
     int qkv_q_tiles, qkv_k_tiles;  // QKV: tiles per matrix (0 otherwise)
@@ -333,11 +335,12 @@ struct TcArgs {
 // sums replace its own partial values in place (peers only ever read the rows of THEIR slices).  A CTA may not
 // exit while a peer still reads its tile: it arrives at the second cluster barrier right after its own reads and waits
 // for it after its epilogue.  Even a CTA that gave up takes part in both barriers: a cluster barrier has no time-out.
-// `wide`: the accumulator has 2 NP columns, W hi^T in [0, NP) and W lo^T in [NP, 2 NP), to be added up here.
+// `wide`: the accumulator has 2 NP columns, W hi^T in [0, NP) and W lo^T in [NP, 2 NP), to be added up here; `sets` 2: a second
+// one of the same form behind it.
 template <class Epi>
 __device__ __forceinline__ void tc_finish(const Epi &epi, float *tile, uint32_t tmem_d, uint32_t tmem_cols, int NP,
                                           int splits, int split, int tile_idx, int n_live, const int32_t *rows, bool ok,
-                                          const int *s_abort, int nthr, bool wide = false) {
+                                          const int *s_abort, int nthr, bool wide = false, int sets = 1) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp >= 2 && warp < 6 && ok && n_live > 0) {
         const int q = warp & 3;  // TMEM lane quarter this warp may read
@@ -346,10 +349,13 @@ __device__ __forceinline__ void tc_finish(const Epi &epi, float *tile, uint32_t 
             float v[16];
             tc_ld16(tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
             if (wide) {
-                float w[16];
-                tc_ld16(tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(NP + c0), w);
+#pragma unroll 1
+                for (int g = 1; g < 2 * sets; ++g) {
+                    float w[16];
+                    tc_ld16(tmem_d + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * NP + c0), w);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] += w[j];
+                    for (int j = 0; j < 16; ++j) v[j] += w[j];
+                }
             }
 #pragma unroll
             for (int j = 0; j < 16; ++j) col[(c0 + j) * kTcLd] = v[j];
@@ -429,7 +435,8 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     const bool wide = a.wide != 0;
     const int acc_n = wide ? 2 * NP : NP;
     uint32_t tmem_cols = 32;
-    while ((int)tmem_cols < acc_n) tmem_cols <<= 1;
+    const int sets = a.halves ? 2 : 1;
+    while ((int)tmem_cols < sets * acc_n) tmem_cols <<= 1;
 
     // `late_release`: the next grid in the stream is the dequantising kernel of the same projection, which runs beside
     // this one instead of behind it: it never waits for this grid at its start, so it may only start once everything
@@ -515,17 +522,19 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
             const uint32_t idesc = tc_idesc(acc_n);
             const uint64_t dfix = tc_smem_desc(0);  // everything but the address field
             const uint32_t stage16 = stage_bytes >> 4, a16 = a_bytes >> 4, b16 = b_bytes >> 4;
-            uint32_t s = 0, par = 0, addr16 = stage0 >> 4;
+            uint32_t s = 0, par = 0, addr16 = stage0 >> 4, d = tmem_d;
+            const int turn = a.halves ? (nkb + 1) / 2 : -1;  // first k-block of the second accumulator
             for (int i = 0; i < nkb_run; ++i) {
                 if (!mbar_wait(full0 + 8 * s, par, abortp, a.dev_err)) break;
                 tc_fence_after();
                 const uint64_t da = dfix | addr16, dhi = da + a16, dlo = dhi + b16;  // (addresses below 256 KB: no carry)
-                tc_mma(tmem_d, da, dhi, idesc, i > 0 ? 1u : 0u);
-                if (!wide) tc_mma(tmem_d, da, dlo, idesc, 1u);
+                if (i == turn) d += acc_n;
+                tc_mma(d, da, dhi, idesc, i > 0 && i != turn ? 1u : 0u);
+                if (!wide) tc_mma(d, da, dlo, idesc, 1u);
 #pragma unroll
                 for (int k = 1; k < kTcBK / 16; ++k) {  // UMMA K = 16 bf16 = 32 bytes: +2 in the 16-byte address field
-                    tc_mma(tmem_d, da + 2 * k, dhi + 2 * k, idesc, 1u);
-                    if (!wide) tc_mma(tmem_d, da + 2 * k, dlo + 2 * k, idesc, 1u);
+                    tc_mma(d, da + 2 * k, dhi + 2 * k, idesc, 1u);
+                    if (!wide) tc_mma(d, da + 2 * k, dlo + 2 * k, idesc, 1u);
                 }
                 tc_commit(empty0 + 8 * s);  // frees the stage once these MMAs have read it
                 if (++s == (uint32_t)S) { s = 0; par ^= 1u; addr16 = stage0 >> 4; } else addr16 += stage16;
@@ -541,7 +550,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     bool ok = mbar_wait_sleepy(smem_u32(&bars[2 * S]), 0, abortp, a.dev_err);
     tc_fence_after();
     __syncthreads();  // all TMA writes and MMA reads of the pipeline memory are over: it now holds the tile
-    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kTcThreads, wide);
+    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kTcThreads, wide, sets);
 }
 
 inline size_t tc_smem_bytes(int n_pad, int n_stages) {

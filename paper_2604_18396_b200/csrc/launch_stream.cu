@@ -64,7 +64,7 @@ cudaError_t launch_stream(river_ctx *c, const P &p, const ProjIn &in, const RowL
                           int has_river, bool pdl, int skip_backbone, const DecideArgs &dec) {
     if constexpr (std::is_same_v<P, ResidProblem>) {
         // Three and more rows of a long K do not fit into shared memory together, and a pass for each pair would stream the
-        // weights twice: two launches of half the inputs instead, the second adding to the first one's output (8B-class down
+        // weights twice: two launches of half the inputs instead, the second adding to the first one's output (8B-class
         // blocks, three rows: 1424 us a step, so 1319, the row count's own instance included).
         if (n >= 3 && !in.gain && !p.ld && K % (2 * p.group) == 0 && K % 128 == 0 && stream_smem_bytes(3, K) > 200 * 1024) {
             ResidProblem a = p, b = p;

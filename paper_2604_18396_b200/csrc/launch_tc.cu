@@ -38,6 +38,7 @@ int tc_pick_splits(const river_ctx *c, int tiles, int kb_total, int slots, int m
 namespace {
 
 constexpr size_t kSmSmem = 228 * 1024;
+constexpr int kTcHalvesRows = 64;  // operand rows up to which two CTAs' double accumulators (4 np columns each) share an SM
 constexpr size_t kCtaFixed = 1024 + 1024 + 256;  // per CTA: system reserve, alignment slack, barriers
 
 size_t tc_stage_bytes(int np) { return (size_t)kTcBM * kTcBK * 2 + 2 * (size_t)np * kTcBK * 2; }
@@ -65,6 +66,7 @@ int tc_footprints(int np, TcFootprint (&out)[2]) {
         if (!st) break;
         int wide;
         out[n].cols = tc_cols(np, occ, &wide);
+        if (occ == 2 && np <= kTcHalvesRows) out[n].cols *= 2;  // (a.halves)
         out[n].smem = tc_smem_bytes(np, st);
         if (++n == 2 || occ == 1) break;
     }
@@ -100,13 +102,15 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
         const int s3 = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms * 3);
         if (tiles * s3 > tiles * a.splits && tiles * s3 <= c->num_sms * 3) { occ = 3; a.splits = s3; }
     }
-    // One CTA per SM, in the shared memory of half an SM, where it still has a long enough run of k-blocks: the other half
-    // takes the CTAs of the projection behind this one (and of the dequantising kernel beside it), which set up and request
-    // their first weights while this grid drains.  8B-class shape, 64 rows: two or three CTAs per SM 2083 us a step (8 blocks),
-    // so 2005; with fewer than a dozen k-blocks per CTA (1B-class shape, 8 rows) more CTAs win (1118 against 1224-1337).
-    if (occ >= 2 && allow_split && tiles < c->num_sms) {
+    // Decode steps of up to 64 operand rows: one CTA per SM, in the shared memory of half an SM, where it still has a long
+    // enough run of k-blocks: the other half takes the CTAs of the projection behind this one (and of the dequantising kernel
+    // beside it), which set up and request their first weights while this grid drains.  8B-class shape, 64 rows: two or three
+    // CTAs per SM 2083 us a step (8 blocks), so 2005; with fewer than a dozen k-blocks per CTA (1B-class shape, 8 rows) more
+    // CTAs win (1118 against 1224-1337), and so they do in prefill (58 positions, 2 blocks: 589 against 596 us).  The run of
+    // k-blocks is summed in two halves, whose accumulators fit twice into an SM's tensor memory up to 64 rows.
+    if (occ >= 2 && allow_split && tiles < c->num_sms && c->rows_distinct && np <= kTcHalvesRows) {
         const int s1 = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms);
-        if (s1 >= 2 && K / kTcBK / s1 >= 12) { a.splits = s1; occ = 2; }
+        if (s1 >= 2 && K / kTcBK / s1 >= 12) { a.splits = s1; occ = 2; a.halves = 1; }
     }
     a.n_stages = tc_stages_at(np, occ);
     tc_cols(np, occ, &a.wide);
@@ -116,7 +120,8 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
     a.gateup = gateup; a.qkv_q_tiles = q_tiles; a.qkv_k_tiles = k_tiles;
     a.rows = rows; a.cnt = cnt; a.dev_err = c->dev_err;
     a.hint = hint ? hint : cnt;
-    const size_t smem = tc_smem_bytes(np, a.n_stages);
+    // (two CTAs with double accumulators and a third one of another launch never share an SM: 256 + 256 columns are all)
+    const size_t smem = std::max<size_t>(tc_smem_bytes(np, a.n_stages), a.halves ? 90 * 1024 : 0);
     e = ensure_smem(c, tc_gemm_kernel<Epi>, smem);
     if (e != cudaSuccess) return e;
     return launch_kc(tc_gemm_kernel<Epi>, dim3(tiles * a.splits), dim3(kTcThreads), smem, c->stream, true, a.splits, a0,
