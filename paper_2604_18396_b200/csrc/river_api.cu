@@ -945,26 +945,40 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
                  const int32_t *depth, float tau, bool record_fail, float *logits_last, int32_t *next_tok) {
     const river_config &g = c->cfg;
     const bool wide = c->wide_rows > 0 && !c->off_first;
-    const int max_rows = wide ? c->wide_rows : g.max_batch;
-    struct MetaRows {  // the metadata block is laid out for a chunk of this pass while it runs
-        river_ctx *c; int keep;
-        MetaRows(river_ctx *c_, int rows) : c(c_), keep(c_->meta_rows) { c->meta_rows = rows; }
-        ~MetaRows() { c->meta_rows = keep; }
-    } meta_rows(c, max_rows);
+    struct KeepMetaRows {  // the metadata block is laid out for the chunk under way, and for decode steps behind it
+        river_ctx *c; int rows;
+        explicit KeepMetaRows(river_ctx *c_) : c(c_), rows(c_->meta_rows) {}
+        ~KeepMetaRows() { c->meta_rows = rows; }
+    } keep(c);
+    // rows of the chunk that starts at position p of sequence s, if it may hold `most`: token ids are contiguous in tok, and
+    // it has no more prompt ends than the logits staging has rows
+    auto chunk_rows = [&](int s, int p, int most) {
+        const int tok0 = offsets[s] + p;
+        int n = 0;
+        for (int ends = 0; s < n_seqs && n < most && ends < c->user_max_batch && offsets[s] + p == tok0 + n; ++s, ++ends, p = 0)
+            n += std::min(offsets[s + 1] - offsets[s] - p, most - n);
+        return n;
+    };
     {
-        std::vector<float> ta(max_rows, tau);
+        long long total = 0;
+        for (int s = 0; s < n_seqs; ++s) total += offsets[s + 1] - offsets[s];
+        const std::vector<float> ta((size_t)std::min<long long>(total, c->list_rows), tau);
         CUDA_TRY(c, cudaMemcpyAsync(c->tau_i, ta.data(), sizeof(float) * ta.size(), cudaMemcpyHostToDevice, c->stream));
         CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     }
     int s = 0, p = 0;  // next (sequence, position) to schedule
     while (s < n_seqs) {
+        // A long pass if more than kWideMin rows are there for one, else the layout and the kernels of a short pass: its metadata
+        // is 11 arrays of max_batch entries, a long pass's of wide_rows (45 KB to fill and to copy, whatever the rows).
+        const bool long_pass = wide && chunk_rows(s, p, c->wide_rows) > kWideMin;
+        const int max_rows = long_pass ? c->wide_rows : g.max_batch;
+        c->meta_rows = max_rows;
         int32_t *mh = next_meta(c);
         int n = 0, n_upd = 0, n_head = 0;
-        const int tok0 = offsets[s] + p;
+        const int tok0 = offsets[s] + p, n_want = chunk_rows(s, p, max_rows);
         int head_seq[kMaxBatch];
-        while (s < n_seqs && n < max_rows && n_head < c->user_max_batch) {
+        while (n < n_want) {
             const int len = offsets[s + 1] - offsets[s];
-            if (offsets[s] + p != tok0 + n) break;  // token ids of a chunk must be contiguous in tok
             if (int rc = ensure_page(c, slots[s], p, mh, n_upd)) { rollback_pages(c, mh, n_upd); return rc; }
             mh[kMetaHdr + n] = slots[s];
             mh[kMetaHdr + max_rows + n] = p;
@@ -982,7 +996,6 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         // query tiles of the prefill attention: consecutive positions of one sequence, up to 16 - or as many as make 128
         // query rows, for the tcgen05 kernel, where the rows of a long pass look back at 128 positions and more on average
         // (below, its tiles are mostly padding: mini shape, prompts of 96 positions 20 against 17 us; 1B-class, 435: 30 against 32)
-        const bool long_pass = wide && n > kWideMin;
         long long seen = 0;
         for (int i = 0; i < n; ++i) seen += mh[kMetaHdr + max_rows + i] + 1;
         const bool tc_attn = long_pass && seen >= 128LL * n;
