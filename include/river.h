@@ -51,8 +51,10 @@ enum {
                              tcgen05 GEMM */
     RIVER_F_TMA_ATTN = 32, /* diagnostic: steps of 1-4 rows through the TMA-fed attention kernel too (default: the
                               small-step kernel) */
-    RIVER_F_SERIAL_TC = 64 /* diagnostic: the two tcgen05 GEMMs of a projection (backbone rows, exit-layer rows) one
+    RIVER_F_SERIAL_TC = 64, /* diagnostic: the two tcgen05 GEMMs of a projection (backbone rows, exit-layer rows) one
                               after the other (default: in flight together) */
+    RIVER_F_SHORT_PASSES = 128 /* prompts go through the blocks in passes of prefill_chunk positions, never in long ones (see
+                              prefill_chunk); the workspace is without their buffers */
 };
 
 typedef struct river_config {
@@ -69,10 +71,11 @@ typedef struct river_config {
     uint32_t page_shuffle_seed;/* != 0: hand pages out in a seeded shuffled order */
     uint32_t flags;
     int32_t prefill_chunk;     /* prompt positions river_prefill runs per pass through the blocks (0 = max_batch, at most
-                                  256): every pass streams the weights once, so larger chunks make prefill cheaper; from
-                                  128 on (RIVER_KV_RIVER, shapes of the tensor-core paths) a pass takes up to four chunks,
-                                  at most 1024 positions; the workspace grows with max(max_batch, prefill_chunk) and with
-                                  the rows of a pass */
+                                  256): every pass streams the weights once, so larger chunks make prefill cheaper; the
+                                  workspace grows with max(max_batch, prefill_chunk).  Chunks of 128 and more (RIVER_KV_RIVER,
+                                  shapes of the tensor-core paths, unless RIVER_F_SHORT_PASSES) allow long passes of up to four
+                                  chunks, at most 1024 positions; these add to the workspace the buffers of a pass's rows and
+                                  one projection's exit-layer weights in f16: 2 max(2 F, Hq dh + 2 Hkv dh) d bytes */
     int32_t kv_strategy;       /* what happens in the blocks a token skips (Section 3; RIVER_KV_*): the method's KV-Shared
                                   Exit River, or one of the strategies it is compared with, on the same kernels */
 } river_config;

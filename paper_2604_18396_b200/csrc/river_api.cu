@@ -101,14 +101,15 @@ bool w4_shape_ok(const river_config &g) { return g.group == 64 && g.d % 256 == 0
 constexpr int kWideMin = 128;  // a pass of up to this many rows takes the batch kernels, which split K where tiles are few
 // Rows of a long prefill pass (0: this configuration has none).  A pass streams every weight once and its projections run
 // on CTA pairs at about the tensor-core rate only when there are tiles for all of them, so prompts go through in passes of
-// up to 1024 rows wherever the caller allows chunks of 128 and more (8B-class shape, 1024 positions, per block: four passes of
-// 256 rows through the batch kernels 1.87 ms, one pass 0.9 ms).  The workspace pays for it: about 0.2 MB per
-// row of the 8B-class shape plus one projection's exit-layer weights in f16.
+// up to 1024 rows wherever the caller asks for chunks of 128 and more (8B-class shape, 1024 positions, per block: four passes of
+// 256 rows through the batch kernels 1.87 ms, one pass 0.77 ms).  The workspace pays for it (8B-class shape, chunks of 256: 374 MB,
+// 235 of them one projection's exit-layer weights in f16), so it is prefill_chunk that asks, not max_batch: a context for wide decode
+// steps alone keeps the workspace of its steps.
 int wide_rows_for(const river_config &c) {
-    if (c.max_batch < 128 || c.kv_strategy != RIVER_KV_RIVER || (c.flags & (RIVER_F_NO_TC | RIVER_F_NO_W4TC)) || !tc_shape_ok(c) ||
+    if (c.prefill_chunk < 128 || (c.flags & RIVER_F_SHORT_PASSES) || c.kv_strategy != RIVER_KV_RIVER || (c.flags & (RIVER_F_NO_TC | RIVER_F_NO_W4TC)) || !tc_shape_ok(c) ||
         !w4_shape_ok(c))
         return 0;
-    return std::min(kMaxBatch, (4 * c.max_batch + 127) / 128 * 128);
+    return std::min(kMaxBatch, (4 * c.prefill_chunk + 127) / 128 * 128);
 }
 
 // (c: the effective configuration, whose max_batch is the rows of a decode step or a short prefill pass)

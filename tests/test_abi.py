@@ -58,3 +58,20 @@ def test_size_queries_and_config_checks_need_no_gpu(lib):
     assert lib.river_init(ctypes.byref(cfg), None, None, 0, None, 0, None, ctypes.byref(h)) == -2
     assert b"head dim" in lib.river_last_error(None)
     assert lib.river_seq_len(None, 0) == -5
+
+
+def test_long_pass_buffers_are_paid_for_by_contexts_that_ask_for_long_passes(lib):
+    from workloads import synth
+
+    def ws(max_batch, chunk, flags=0):
+        cfg = binding.make_config(synth.SHAPES["8b"], max_seqs=64, max_pages_per_seq=64, n_pages=64, max_batch=max_batch,
+                                  prefill_chunk=chunk, flags=flags)
+        return lib.river_workspace_bytes(ctypes.byref(cfg))
+
+    off = binding.RIVER_F_NO_W4TC  # (no long passes without the dequantising GEMM)
+    for rows, chunk in ((128, 0), (256, 0), (256, 64), (1024, 0), (8, 127)):  # wide steps, or chunks too small: nothing for prompts
+        assert ws(rows, chunk) == ws(rows, chunk, off), (rows, chunk)
+    w_f16 = 2 * 2 * 14336 * 4096
+    for rows in (8, 64, 300):
+        assert ws(rows, 256, binding.RIVER_F_SHORT_PASSES) == ws(rows, 256, off)
+        assert ws(rows, 256) > ws(rows, 256, off) + w_f16
