@@ -16,11 +16,10 @@
 #pragma once
 #include <cuda_fp16.h>
 #include "mbar_tma.cuh"
+#include "tc_plan.h"
 
 namespace river {
 
-constexpr int kTcBM = 128;      // output features per tile (UMMA M)
-constexpr int kTcBK = 64;       // K per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kTcThreads = 192; // warp 0: TMA, warp 1: MMA + TMEM allocation, warps 2..5: epilogue
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

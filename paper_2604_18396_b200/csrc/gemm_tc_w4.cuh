@@ -29,10 +29,6 @@ namespace river {
 
 constexpr int kW4DqWarps = 8;                         // dequantisation warps: two per TMEM lane quarter (even / odd k-blocks)
 constexpr int kW4Threads = 64 + 32 * kW4DqWarps;      // warp 0: TMA, warp 1: MMA + TMEM, warps 2..9: dequant / epilogue
-constexpr int kW4Super = 4;                           // k-blocks per raw code tile: 4 x 32 bytes of codes per row
-constexpr int kW4RawBufs = 2;
-constexpr uint32_t kW4RawBytes = kTcBM * 128;         // one raw code tile
-constexpr uint32_t kW4ACols = kTcBK / 2;              // TMEM columns of one A tile: 64 f16 per row, two per column
 
 // A from tensor memory (lane = tile row, column c = inputs 2 c and 2 c + 1 of the k-block), B from shared memory.
 __device__ __forceinline__ void tc_mma_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
@@ -138,6 +134,7 @@ struct TcW4Args {
                        // late_release): no wait at the start, the wait for that grid comes before the CTA exits
     int one_box;       // 1: map_bhi covers the hi rows AND the lo rows behind them: one copy of 2 n_pad rows per k-block
     int wide;          // 1: hi and lo activation rows as one operand of 2 n_pad rows (the host checks the TMEM budget)
+    int sets;          // 2 (wide only): the second half of the k-blocks goes to a second accumulator, added at the end
     int gateup;        // 1: a tile is 64 rows of matrix 0 + 64 rows of matrix 1
     int qkv_q_tiles, qkv_k_tiles;  // QKV: tiles per matrix (0 otherwise)
     const uint16_t *scale[3], *zero[3];  // bf16 [rows][K/64] of the up to three matrices behind the code maps
@@ -196,8 +193,9 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
     const int nsb = sb1 - sb0, kb0 = sb0 * kW4Super, nkb = nsb * kW4Super;
     const bool wide = a.wide != 0;  // as in tc_gemm_kernel: one MMA per 16 inputs, D = [W hi^T | W lo^T]
     const int acc_n = wide ? 2 * NP : NP;
-    uint32_t tmem_cols = 32;  // accumulator in columns [0, acc_n), then S A tiles of 32 columns
-    while (tmem_cols < (uint32_t)acc_n + (uint32_t)S * kW4ACols) tmem_cols <<= 1;
+    const uint32_t a_col = (uint32_t)(a.sets * acc_n);  // accumulators in columns [0, a_col), then S A tiles of 32 columns
+    uint32_t tmem_cols = 32;
+    while (tmem_cols < a_col + (uint32_t)S * kW4ACols) tmem_cols <<= 1;
 
     pdl_launch();
     if (tid == 0) {
@@ -310,18 +308,20 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
             const uint64_t dfix = tc_smem_desc(0);  // everything but the address field
             const uint32_t stage16 = stage_bytes >> 4, b16 = b_bytes >> 4;
             const uint32_t afull0 = smem_u32(b_afull), empty0 = smem_u32(b_empty);
-            const uint32_t ta0 = tmem_d + (uint32_t)acc_n;
-            uint32_t s = 0, par = 0, addr16 = smem_u32(stages) >> 4, ta = ta0;  // incremental: no division per k-block
+            const uint32_t ta0 = tmem_d + a_col;
+            uint32_t s = 0, par = 0, addr16 = smem_u32(stages) >> 4, ta = ta0, d = tmem_d;  // incremental: no division per k-block
+            const int turn = a.sets == 2 ? (nkb + 1) / 2 : -1;  // first k-block of the second accumulator
             for (int i = 0; i < nkb_run; ++i) {
                 if (!mbar_wait(afull0 + 8 * s, par, abortp, a.dev_err)) break;
                 tc_fence_after();
                 const uint64_t dhi = dfix | addr16, dlo = dhi + b16;  // (addresses below 256 KB: no carry)
-                tc_mma_ts(tmem_d, ta, dhi, idesc, i > 0 ? 1u : 0u);
-                if (!wide) tc_mma_ts(tmem_d, ta, dlo, idesc, 1u);
+                if (i == turn) d += acc_n;
+                tc_mma_ts(d, ta, dhi, idesc, i > 0 && i != turn ? 1u : 0u);
+                if (!wide) tc_mma_ts(d, ta, dlo, idesc, 1u);
 #pragma unroll
                 for (int k = 1; k < kTcBK / 16; ++k) {  // 16 inputs = 8 columns of A = 32 bytes of a B row
-                    tc_mma_ts(tmem_d, ta + 8 * k, dhi + 2 * k, idesc, 1u);
-                    if (!wide) tc_mma_ts(tmem_d, ta + 8 * k, dlo + 2 * k, idesc, 1u);
+                    tc_mma_ts(d, ta + 8 * k, dhi + 2 * k, idesc, 1u);
+                    if (!wide) tc_mma_ts(d, ta + 8 * k, dlo + 2 * k, idesc, 1u);
                 }
                 tc_commit(empty0 + 8 * s);
                 if (++s == (uint32_t)S) { s = 0; par ^= 1u; addr16 = smem_u32(stages) >> 4; ta = ta0; }
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
         // ---- dequantisation: this warp may write TMEM lanes 32 (warp % 4) .. + 31 = tile rows; the two warps of a
         // lane quarter take the even and the odd k-blocks (S is even: each keeps to its own stages)
         const int r = 32 * (warp & 3) + lane, grp = (warp - 2) >> 2;
-        const uint32_t ta_lane = tmem_d + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)acc_n;
+        const uint32_t ta_lane = tmem_d + ((uint32_t)(32 * (warp & 3)) << 16) + a_col;
         int mi = m0;
         size_t grow = (size_t)ay + r;  // row inside its matrix
         if (a.gateup && r >= 64) { mi = m1; grow = (size_t)ay1 + (r - 64); }
@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
     bool ok = n_live > 0 ? mbar_wait(smem_u32(b_acc), 0, abortp, a.dev_err) : true;
     tc_fence_after();
     __syncthreads();  // all copies into and MMA reads of the pipeline memory are over: it now holds the tile
-    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kW4Threads, wide);
+    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kW4Threads, wide, a.sets);
     if (a.overlap) pdl_wait();
 }
 

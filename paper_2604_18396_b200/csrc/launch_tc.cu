@@ -19,46 +19,6 @@ const river_ctx::BMap *tc_bmap(river_ctx *c, int K, int np, bool w4, bool alt) {
     return &c->tc_bmaps.back();
 }
 
-// K-splits per tile: fill whole waves of the CTA slots, keep at least four 64-wide k-blocks per split; no split at
-// all when there is a tile for every SM.  The kernel is memory-bound, so what matters is that all CTAs are resident
-// together and every SM slot streams.
-int tc_pick_splits(const river_ctx *c, int tiles, int kb_total, int slots, int min_kb) {
-    int best = 1;
-    double best_eff = 0.0;
-    if (tiles >= c->num_sms) return 1;  // every SM has a tile of its own: splitting only adds reductions
-    for (int s = 1; s <= 8; ++s) {  // a cluster holds at most 8 CTAs
-        if (s > 1 && kb_total / s < min_kb) break;
-        const int ctas = tiles * s, waves = (ctas + slots - 1) / slots;
-        const double eff = (double)ctas / ((double)waves * slots);
-        if (eff > best_eff + 0.02) { best_eff = eff; best = s; }
-    }
-    return best;
-}
-
-namespace {
-
-constexpr size_t kSmSmem = 228 * 1024;
-constexpr int kTcHalvesRows = 64;  // operand rows up to which two CTAs' double accumulators (4 np columns each) share an SM
-constexpr size_t kCtaFixed = 1024 + 1024 + 256;  // per CTA: system reserve, alignment slack, barriers
-
-size_t tc_stage_bytes(int np) { return (size_t)kTcBM * kTcBK * 2 + 2 * (size_t)np * kTcBK * 2; }
-// pipeline stages with `occ` CTAs per SM (0: they do not fit)
-int tc_stages_at(int np, int occ) {
-    const size_t stage = tc_stage_bytes(np), room = std::min<size_t>(kSmSmem / occ, 227 * 1024);
-    return room < kCtaFixed + 2 * stage ? 0 : (int)std::min<size_t>(occ == 1 ? 8 : occ == 2 ? 4 : 3, (room - kCtaFixed) / stage);
-}
-// hi | lo as one operand doubles the accumulator columns; all CTAs that can be resident on an SM must get their
-// tensor memory at once (a CTA stuck in the allocation while its cluster waits for it could not be waited out)
-int tc_cols(int np, int occ, int *wide) {
-    int cols = 32;
-    while (cols < 2 * np) cols <<= 1;
-    *wide = (2 * np <= 256 && occ * cols <= 512) ? 1 : 0;
-    if (!*wide) { cols = 32; while (cols < np) cols <<= 1; }
-    return cols;
-}
-
-}  // namespace
-
 int tc_footprints(int np, TcFootprint (&out)[2]) {
     int n = 0;
     for (int occ = tc_stages_at(np, 2) ? 2 : 1; occ <= 3; ++occ) {
@@ -93,30 +53,13 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
     TcArgs a{};
     a.K = K; a.n_pad = np; a.one_box = bm->one ? 1 : 0; a.late_release = late_release ? 1 : 0;
     const size_t stage = tc_stage_bytes(np);
-    // CTAs per SM: two with three stages each, or three with two when that puts more CTAs of one wave to work (while
-    // one CTA drains its accumulator and takes part in the cluster reduction the others keep the weight stream going);
-    // one with deep stages when the operand tiles are too large for that.
-    int occ = tc_stages_at(np, 2) ? 2 : 1;
-    a.splits = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms * occ);
-    if (occ == 2 && tc_stages_at(np, 3) && allow_split) {
-        const int s3 = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms * 3);
-        if (tiles * s3 > tiles * a.splits && tiles * s3 <= c->num_sms * 3) { occ = 3; a.splits = s3; }
-    }
-    // Decode steps of up to 64 operand rows: one CTA per SM, in the shared memory of half an SM, where it still has a long
-    // enough run of k-blocks: the other half takes the CTAs of the projection behind this one (and of the dequantising kernel
-    // beside it), which set up and request their first weights while this grid drains.  8B-class shape, 64 rows: two or three
-    // CTAs per SM 2083 us a step (8 blocks), so 2005; with fewer than a dozen k-blocks per CTA (1B-class shape, 8 rows) more
-    // CTAs win (1118 against 1224-1337), and so they do in prefill (58 positions, 2 blocks: 589 against 596 us).  The run of
-    // k-blocks is summed in two halves, whose accumulators fit twice into an SM's tensor memory up to 64 rows.
-    if (occ >= 2 && allow_split && tiles < c->num_sms && c->rows_distinct && np <= kTcHalvesRows) {
-        const int s1 = tc_pick_splits(c, tiles, K / kTcBK, c->num_sms);
-        if (s1 >= 2 && K / kTcBK / s1 >= 12) { a.splits = s1; occ = 2; a.halves = 1; }
-    }
+    const TcPlan plan = tc_plan(c->num_sms, np, tiles, K, allow_split, c->rows_distinct);
+    const int occ = plan.occ;
+    a.splits = plan.splits; a.halves = plan.halves;
     a.n_stages = tc_stages_at(np, occ);
     tc_cols(np, occ, &a.wide);
     // the finished tile lives in the pipeline memory
     if (sizeof(float) * (size_t)np * kTcLd > (size_t)a.n_stages * stage) return cudaErrorInvalidValue;
-    if (!allow_split) a.splits = 1;
     a.gateup = gateup; a.qkv_q_tiles = q_tiles; a.qkv_k_tiles = k_tiles;
     a.rows = rows; a.cnt = cnt; a.dev_err = c->dev_err;
     a.hint = hint ? hint : cnt;

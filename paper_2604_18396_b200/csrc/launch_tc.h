@@ -15,7 +15,6 @@ enum : int { kTcPrep = 1, kTcGemm = 2, kTcBoth = 3 };
 // rows (two or three CTAs per SM): what a kernel that shares the SMs with it must budget against.
 struct TcFootprint { size_t smem; int cols; };
 int tc_footprints(int np, TcFootprint (&out)[2]);
-int tc_pick_splits(const river_ctx *c, int tiles, int kb_total, int slots, int min_kb = 4);
 
 // launch_tc.cu: backbone rows, 5 <= rows <= 256
 template <class Epi>

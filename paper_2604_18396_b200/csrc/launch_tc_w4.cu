@@ -39,29 +39,14 @@ cudaError_t launch_tc_w4(river_ctx *c, const ProjIn &in, const CUtensorMap *cons
     if (!(phase & kTcGemm)) return e;
     TcW4Args a{};
     a.K = K; a.n_pad = np; a.one_box = bm->one ? 1 : 0;
-    const size_t stage = 2 * (size_t)np * kTcBK * 2;  // the activations' hi and lo tiles; the A tiles are in tensor memory
-    const size_t raw = (size_t)kW4RawBufs * kW4RawBytes;
-    // two CTAs per SM (16 dequantisation warps) when two stages fit in half of the shared memory; an even number of
-    // stages (the two dequantisation warps of a lane quarter alternate)
-    const bool two = 2 * stage + raw + 4096 <= 110 * 1024;
-    a.n_stages = two ? (int)std::min<size_t>(4, (110 * 1024 - raw - 4096) / stage)
-                     : (int)std::max<size_t>(2, std::min<size_t>(4, (214 * 1024 - raw) / stage));
-    a.n_stages &= ~1;
-    // in raw tiles of four k-blocks: at least four per split, two when K is so short that four would allow only two
-    // splits (measured on the 1B shape, K = 2048: 2 -> 4 splits 35 -> 31 us per layer for QKV, 33 -> 27 us for O)
-    const int raw_tiles = K / (kTcBK * kW4Super);
-    // (splits for one CTA per SM: the rest of the SM belongs to tc_gemm_kernel's CTAs beside this grid and to the next
-    // projection's; 8B-class shape, 61 rows on both weight sets 2069 -> 2050 us a step, 1B-class, 8 rows 1120 -> 1097; with
-    // fewer than eight raw tiles the clusters this asks for cost more than they bring: tiny shape, 77 rows 149.8 -> 152.4)
-    a.splits = tc_pick_splits(c, tiles, raw_tiles, c->num_sms * (two && raw_tiles < 8 ? 2 : 1), raw_tiles <= 8 ? 2 : 4);
+    const size_t stage = 2 * (size_t)np * kTcBK * 2, raw = (size_t)kW4RawBufs * kW4RawBytes;
+    const W4Plan plan = w4_plan(c->num_sms, np, tiles, K, c->rows_distinct);
+    a.n_stages = plan.n_stages; a.splits = plan.splits; a.wide = plan.wide; a.sets = plan.sets;
     if (sizeof(float) * (size_t)np * kTcLd > (size_t)a.n_stages * stage + raw) return cudaErrorInvalidValue;
-    // tensor memory: accumulator + A tiles, a power of two of columns; every CTA that can be resident on an SM must get
+    // tensor memory: accumulators + A tiles, a power of two of columns; every CTA that can be resident on an SM must get
     // its columns at once (a CTA stuck in the allocation while its cluster waits for it could not be waited out), so
     // the shared-memory request is padded until no more than `occ` CTAs fit
-    const int occ = two ? 2 : 1;
-    auto cols_for = [&](int acc) { int cols = 32; while (cols < acc + a.n_stages * (int)kW4ACols) cols <<= 1; return cols; };
-    a.wide = (2 * np <= 256 && occ * cols_for(2 * np) <= 512) ? 1 : 0;
-    const int cols = cols_for(a.wide ? 2 * np : np);
+    const int occ = plan.occ, cols = plan.cols;
     if (occ * cols > 512) return cudaErrorInvalidValue;
     const size_t sm_smem = 228 * 1024;
     size_t smem = std::max(tc_w4_smem_bytes(np, a.n_stages), sm_smem / (occ + 1) + 1024);

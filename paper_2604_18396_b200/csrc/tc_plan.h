@@ -1,0 +1,119 @@
+// How the tensor-core projections cut their work: K-splits, pipeline stages, accumulators and accumulation segments.  Host
+// arithmetic on sizes only, without CUDA types, so that the rules can be checked where there is no GPU.
+#pragma once
+#include <algorithm>
+#include <cstddef>
+#include <cstdint>
+
+namespace river {
+
+constexpr int kTcBM = 128;      // output features per tile (UMMA M)
+constexpr int kTcBK = 64;       // K per stage: 64 bf16 = one 128-byte swizzle row
+constexpr int kW4Super = 4;     // k-blocks per raw code tile: 4 x 32 bytes of codes per row
+constexpr int kW4RawBufs = 2;
+constexpr uint32_t kW4RawBytes = kTcBM * 128;  // one raw code tile
+constexpr uint32_t kW4ACols = kTcBK / 2;       // TMEM columns of one A tile: 64 f16 per row, two per column
+
+constexpr size_t kSmSmem = 228 * 1024;
+constexpr int kTcHalvesRows = 64;  // operand rows up to which two CTAs' double accumulators (4 np columns each) share an SM
+constexpr size_t kCtaFixed = 1024 + 1024 + 256;  // per CTA: system reserve, alignment slack, barriers
+
+// K-splits per tile: fill whole waves of the CTA slots, keep at least four 64-wide k-blocks per split; no split at
+// all when there is a tile for every SM.  The kernel is memory-bound, so what matters is that all CTAs are resident
+// together and every SM slot streams.
+inline int tc_pick_splits(int num_sms, int tiles, int kb_total, int slots, int min_kb = 4) {
+    int best = 1;
+    double best_eff = 0.0;
+    if (tiles >= num_sms) return 1;  // every SM has a tile of its own: splitting only adds reductions
+    for (int s = 1; s <= 8; ++s) {  // a cluster holds at most 8 CTAs
+        if (s > 1 && kb_total / s < min_kb) break;
+        const int ctas = tiles * s, waves = (ctas + slots - 1) / slots;
+        const double eff = (double)ctas / ((double)waves * slots);
+        if (eff > best_eff + 0.02) { best_eff = eff; best = s; }
+    }
+    return best;
+}
+
+inline size_t tc_stage_bytes(int np) { return (size_t)kTcBM * kTcBK * 2 + 2 * (size_t)np * kTcBK * 2; }
+// pipeline stages with `occ` CTAs per SM (0: they do not fit)
+inline int tc_stages_at(int np, int occ) {
+    const size_t stage = tc_stage_bytes(np), room = std::min<size_t>(kSmSmem / occ, 227 * 1024);
+    return room < kCtaFixed + 2 * stage ? 0 : (int)std::min<size_t>(occ == 1 ? 8 : occ == 2 ? 4 : 3, (room - kCtaFixed) / stage);
+}
+// hi | lo as one operand doubles the accumulator columns; all CTAs that can be resident on an SM must get their
+// tensor memory at once (a CTA stuck in the allocation while its cluster waits for it could not be waited out)
+inline int tc_cols(int np, int occ, int *wide) {
+    int cols = 32;
+    while (cols < 2 * np) cols <<= 1;
+    *wide = (2 * np <= 256 && occ * cols <= 512) ? 1 : 0;
+    if (!*wide) { cols = 32; while (cols < np) cols <<= 1; }
+    return cols;
+}
+
+// tc_gemm_kernel: CTAs per SM and K-splits.  `decode`: the rows are a decode step's (not a prefill pass's).
+struct TcPlan { int occ, splits, halves; };
+inline TcPlan tc_plan(int num_sms, int np, int tiles, int K, bool allow_split, bool decode) {
+    TcPlan p{};
+    // CTAs per SM: two with three stages each, or three with two when that puts more CTAs of one wave to work (while
+    // one CTA drains its accumulator and takes part in the cluster reduction the others keep the weight stream going);
+    // one with deep stages when the operand tiles are too large for that.
+    p.occ = tc_stages_at(np, 2) ? 2 : 1;
+    p.splits = tc_pick_splits(num_sms, tiles, K / kTcBK, num_sms * p.occ);
+    if (p.occ == 2 && tc_stages_at(np, 3) && allow_split) {
+        const int s3 = tc_pick_splits(num_sms, tiles, K / kTcBK, num_sms * 3);
+        if (tiles * s3 > tiles * p.splits && tiles * s3 <= num_sms * 3) { p.occ = 3; p.splits = s3; }
+    }
+    // Decode steps of up to 64 operand rows: one CTA per SM, in the shared memory of half an SM, where it still has a long
+    // enough run of k-blocks: the other half takes the CTAs of the projection behind this one (and of the dequantising kernel
+    // beside it), which set up and request their first weights while this grid drains.  8B-class shape, 64 rows: two or three
+    // CTAs per SM 2083 us a step (8 blocks), so 2005; with fewer than a dozen k-blocks per CTA (1B-class shape, 8 rows) more
+    // CTAs win (1118 against 1224-1337), and so they do in prefill (58 positions, 2 blocks: 589 against 596 us).  The run of
+    // k-blocks is summed in two halves, whose accumulators fit twice into an SM's tensor memory up to 64 rows.
+    if (p.occ >= 2 && allow_split && tiles < num_sms && decode && np <= kTcHalvesRows) {
+        const int s1 = tc_pick_splits(num_sms, tiles, K / kTcBK, num_sms);
+        if (s1 >= 2 && K / kTcBK / s1 >= 12) { p.splits = s1; p.occ = 2; p.halves = 1; }
+    }
+    if (!allow_split) p.splits = 1;
+    return p;
+}
+
+// tc_gemm_w4_kernel: stages (an even number: the two dequantisation warps of a lane quarter alternate), CTAs per SM, K-splits
+// in whole raw tiles, accumulators.  hi | lo as one operand (`wide`) as above.
+struct W4Plan { int occ, n_stages, splits, wide, sets, cols; };  // cols: tensor-memory columns per CTA (occ * cols > 512: does not fit)
+inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode) {
+    W4Plan p{};
+    const size_t stage = 2 * (size_t)np * kTcBK * 2;  // the activations' hi and lo tiles; the A tiles are in tensor memory
+    const size_t raw = (size_t)kW4RawBufs * kW4RawBytes;
+    // two CTAs per SM (16 dequantisation warps) when two stages fit in half of the shared memory
+    const bool two = 2 * stage + raw + 4096 <= 110 * 1024;
+    p.occ = two ? 2 : 1;
+    p.n_stages = two ? (int)std::min<size_t>(4, (110 * 1024 - raw - 4096) / stage)
+                     : (int)std::max<size_t>(2, std::min<size_t>(4, (214 * 1024 - raw) / stage));
+    p.n_stages &= ~1;
+    auto cols_for = [&](int acc) { int cols = 32; while (cols < acc + p.n_stages * (int)kW4ACols) cols <<= 1; return cols; };
+    p.wide = (2 * np <= 256 && p.occ * cols_for(2 * np) <= 512) ? 1 : 0;
+    p.sets = 1;
+    // in raw tiles of four k-blocks: at least four per split, two when K is so short that four would allow only two
+    // splits (measured on the 1B shape, K = 2048: 2 -> 4 splits 35 -> 31 us per layer for QKV, 33 -> 27 us for O)
+    const int raw_tiles = K / (kTcBK * kW4Super), min_raw = raw_tiles <= 8 ? 2 : 4;
+    p.splits = tc_pick_splits(num_sms, tiles, raw_tiles, num_sms * p.occ, min_raw);
+    // Decode steps: splits for one CTA per SM, the rest of the SM belongs to tc_gemm_kernel's CTAs beside this grid and to the
+    // next projection's (1B-class, 8 rows 1120 -> 1097 us a step) - where the longer run can be summed in two accumulators of
+    // half of it each, so that no sum inside the tensor cores takes more inputs: its error grows with their number (8B-class QKV on
+    // exact weights against 64-bit arithmetic: 1.5e-7 split over every slot, 2.0e-7 with one accumulator and half the splits, 1.1e-7
+    // with two).  That is up to 32 operand rows: 2 x 2 np columns beside four A tiles are the 256 that one accumulator takes as well.
+    // With fewer than eight raw tiles the clusters this asks for cost more than they bring (tiny shape, 77 rows 149.8 -> 152.4),
+    // and in prefill passes they do whatever K is (8B-class, 20 positions on the exit layers 524 -> 541).
+    if (two && decode && raw_tiles >= 8) {
+        const int s1 = tc_pick_splits(num_sms, tiles, raw_tiles, num_sms, min_raw);
+        if (s1 >= p.splits) p.splits = s1;
+        else if (p.wide && p.occ * cols_for(4 * np) <= 512 && (raw_tiles + s1 - 1) / s1 <= 2 * ((raw_tiles + p.splits - 1) / p.splits)) {
+            p.splits = s1;
+            p.sets = 2;
+        }
+    }
+    p.cols = cols_for(p.sets * (p.wide ? 2 * np : np));
+    return p;
+}
+
+}  // namespace river

@@ -1,0 +1,58 @@
+"""The rules that cut the tensor-core projections' work (csrc/tc_plan.h), compiled for the host: how many inputs one sum inside
+the tensor cores takes, at most."""
+import ctypes
+import itertools
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SHIM = r"""
+#include "tc_plan.h"
+extern "C" {
+int pick(int sms, int tiles, int kb, int slots, int min_kb) { return river::tc_pick_splits(sms, tiles, kb, slots, min_kb); }
+void w4(int sms, int np, int tiles, int K, int decode, int *o) {
+    const river::W4Plan p = river::w4_plan(sms, np, tiles, K, decode != 0);
+    o[0] = p.occ; o[1] = p.n_stages; o[2] = p.splits; o[3] = p.wide; o[4] = p.sets; o[5] = p.cols;
+}
+}
+"""
+SMS = 148
+
+
+@pytest.fixture(scope="module")
+def plan(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    (d / "shim.cpp").write_text(SHIM)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2604_18396_b200", "csrc"),
+                           str(d / "shim.cpp"), "-o", str(d / "shim.so")])
+    return ctypes.CDLL(str(d / "shim.so"))
+
+
+def ceil_div(a, b):
+    return -(-a // b)
+
+
+# (128-feature tiles, K) of the repository's shapes - QKV, O, gate/up, down - and others of the same range
+SHAPES = sorted({(4, 256), (2, 256), (16, 256), (2, 1024), (12, 512), (4, 1024), (24, 512), (4, 1536), (24, 2048), (16, 2048), (128, 2048),
+                 (16, 8192), (48, 4096), (32, 4096), (224, 4096), (32, 14336)} | set(itertools.product((1, 3, 8, 20, 56, 100, 147), (2048, 2304, 5120, 16384))))
+
+
+@pytest.mark.parametrize("np", range(16, 257, 16))
+def test_exit_layer_sums_take_no_more_inputs_than_a_split_over_every_slot(plan, np):
+    o = (ctypes.c_int * 6)()
+    for tiles, K in SHAPES:
+        raw = K // 256
+        for decode in (0, 1):
+            plan.w4(SMS, np, tiles, K, decode, o)
+            occ, stages, splits, wide, sets, cols = o
+            every_slot = plan.pick(SMS, tiles, raw, SMS * occ, 2 if raw <= 8 else 4)
+            assert 1 <= splits <= 8 and splits <= raw and stages >= 2 and stages % 2 == 0 and occ * cols <= 512
+            assert cols >= sets * (2 * np if wide else np) + 32 * stages and (sets == 1 or wide)
+            # k-blocks that one accumulator takes, at most: a CTA's raw tiles hold four each, two halves of them with two accumulators
+            assert ceil_div(4 * ceil_div(raw, splits), sets) <= 4 * ceil_div(raw, every_slot), (tiles, K, decode)
+    # 64 rows of the 8B shape's down projection, of its QKV, and the 1B shape's gate/up
+    for tiles, K, longest in ((32, 14336, 1792), (48, 4096, 1024), (128, 2048, 1024)):
+        plan.w4(SMS, np, tiles, K, 1, o)
+        assert np > 128 or 256 * ceil_div(ceil_div(K // 256, o[2]), o[4]) <= longest, (tiles, K)
