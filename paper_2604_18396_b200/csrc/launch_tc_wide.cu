@@ -66,9 +66,7 @@ cudaError_t launch_tc_wide(river_ctx *c, const CUtensorMap &a0, const CUtensorMa
     a.K = K; a.tiles = tiles; a.f16 = f16 ? 1 : 0; a.q_tiles = q_tiles; a.k_tiles = k_tiles;
     a.run_step = run_step; a.head_step = head_step;
     a.rows = rows; a.cnt = cnt; a.dev_err = c->dev_err;
-    // accumulation segments (see the kernel): 1024 inputs, 512 where K is short - never longer sums than the K-split batch
-    // kernels of the same shapes take
-    a.seg = K >= 4096 ? 16 : 8;
+    a.seg = tc_wide_segment(c->num_sms, c->cfg.max_batch, tiles, K, f16);
     a.bn = wide_bn(feature_pairs, n_list, pairs);
     const river_ctx::WMap *bm = wide_map(c, K, a.bn, alt_operand);
     if (!bm) return cudaErrorInvalidValue;

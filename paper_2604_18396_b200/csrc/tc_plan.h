@@ -116,4 +116,22 @@ inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode) {
     return p;
 }
 
+// tc_gemm_wide_kernel: k-blocks per accumulation segment.  1024 inputs, 512 where K is short, and never more than the longest
+// sum that the batch kernels' K-splits make of the same projection in passes of `pass_rows` rows (1B-class shape: 256 inputs for
+// O and gate/up, 384 for QKV; 8B-class: 1024 for all), since the error of a sum inside the tensor cores grows with its length:
+// cache of 300 positions, mini shape, against 64-bit arithmetic 5.5e-4 with 512 inputs everywhere, 5.06e-4 so, as in short
+// passes; logits of 1000 positions, 1B-class blocks, 1.78e-4 and 1.72e-4.  It costs 1-2 % of a prompt on those shapes.
+inline int tc_wide_segment(int num_sms, int pass_rows, int tiles, int K, bool f16) {
+    const int np = std::min(256, (pass_rows + 15) / 16 * 16), kb = K / kTcBK;
+    int run;
+    if (f16) {
+        const int splits = w4_plan(num_sms, np, tiles, K, false).splits, raw = kb / kW4Super;
+        run = (raw + splits - 1) / splits * kW4Super;
+    } else {
+        const int splits = tc_plan(num_sms, np, tiles, K, true, false).splits;
+        run = (kb + splits - 1) / splits;
+    }
+    return std::min(K >= 4096 ? 16 : 8, run);
+}
+
 }  // namespace river

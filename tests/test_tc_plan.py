@@ -16,6 +16,8 @@ void w4(int sms, int np, int tiles, int K, int decode, int *o) {
     const river::W4Plan p = river::w4_plan(sms, np, tiles, K, decode != 0);
     o[0] = p.occ; o[1] = p.n_stages; o[2] = p.splits; o[3] = p.wide; o[4] = p.sets; o[5] = p.cols;
 }
+int tc_splits(int sms, int np, int tiles, int K) { return river::tc_plan(sms, np, tiles, K, true, false).splits; }
+int wide_segment(int sms, int rows, int tiles, int K, int f16) { return river::tc_wide_segment(sms, rows, tiles, K, f16 != 0); }
 }
 """
 SMS = 148
@@ -56,3 +58,18 @@ def test_exit_layer_sums_take_no_more_inputs_than_a_split_over_every_slot(plan, 
     for tiles, K, longest in ((32, 14336, 1792), (48, 4096, 1024), (128, 2048, 1024)):
         plan.w4(SMS, np, tiles, K, 1, o)
         assert np > 128 or 256 * ceil_div(ceil_div(K // 256, o[2]), o[4]) <= longest, (tiles, K)
+
+
+@pytest.mark.parametrize("chunk", [128, 160, 200, 256])
+def test_long_pass_sums_are_no_longer_than_short_passes(plan, chunk):
+    o = (ctypes.c_int * 6)()
+    np = ceil_div(chunk, 16) * 16
+    for tiles, K in SHAPES:
+        kb = K // 64
+        for f16 in (0, 1):
+            if f16:
+                plan.w4(SMS, np, tiles, K, 0, o)
+                longest = 4 * ceil_div(kb // 4, o[2])
+            else:
+                longest = ceil_div(kb, plan.tc_splits(SMS, np, tiles, K))
+            assert 1 <= plan.wide_segment(SMS, chunk, tiles, K, f16) <= min(16, longest), (tiles, K, f16)
