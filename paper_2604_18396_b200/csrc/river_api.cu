@@ -98,7 +98,6 @@ bool tc_shape_ok(const river_config &g) {
 }
 bool w4_shape_ok(const river_config &g) { return g.group == 64 && g.d % 256 == 0 && g.F % 256 == 0 && (g.Hq * g.dh) % 256 == 0; }
 
-constexpr int kWideMin = 128;  // a pass of up to this many rows takes the batch kernels, which split K where tiles are few
 // Rows of a long prefill pass (0: this configuration has none).  A pass streams every weight once and its projections run
 // on CTA pairs at about the tensor-core rate only when there are tiles for all of them, so prompts go through in passes of
 // up to 1024 rows wherever the caller asks for chunks of 128 and more (8B-class shape, 1024 positions, per block: four passes of
@@ -951,14 +950,17 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         explicit KeepMetaRows(river_ctx *c_) : c(c_), rows(c_->meta_rows) {}
         ~KeepMetaRows() { c->meta_rows = rows; }
     } keep(c);
-    // rows of the chunk that starts at position p of sequence s, if it may hold `most`: token ids are contiguous in tok, and
-    // it has no more prompt ends than the logits staging has rows
-    auto chunk_rows = [&](int s, int p, int most) {
+    // rows of the chunk that starts at position p of sequence s, if it may hold `most` (token ids are contiguous in tok, and it
+    // has no more prompt ends than the logits staging has rows), and the least depth among them
+    struct Chunk { int rows, least; };
+    auto chunk_at = [&](int s, int p, int most) {
         const int tok0 = offsets[s] + p;
-        int n = 0;
-        for (int ends = 0; s < n_seqs && n < most && ends < c->user_max_batch && offsets[s] + p == tok0 + n; ++s, ++ends, p = 0)
-            n += std::min(offsets[s + 1] - offsets[s] - p, most - n);
-        return n;
+        Chunk k{0, g.L};
+        for (int ends = 0; s < n_seqs && k.rows < most && ends < c->user_max_batch && offsets[s] + p == tok0 + k.rows; ++s, ++ends, p = 0) {
+            k.rows += std::min(offsets[s + 1] - offsets[s] - p, most - k.rows);
+            k.least = std::min(k.least, depth[s]);
+        }
+        return k;
     };
     {
         long long total = 0;
@@ -969,14 +971,15 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
     }
     int s = 0, p = 0;  // next (sequence, position) to schedule
     while (s < n_seqs) {
-        // A long pass if more than kWideMin rows are there for one, else the layout and the kernels of a short pass: its metadata
-        // is 11 arrays of max_batch entries, a long pass's of wide_rows (45 KB to fill and to copy, whatever the rows).
-        const bool long_pass = wide && chunk_rows(s, p, c->wide_rows) > kWideMin;
+        // A long pass if there are rows enough for one, else the layout and the kernels of a short pass: its metadata is 11 arrays
+        // of max_batch entries, a long pass's of wide_rows (45 KB to fill and to copy, whatever the rows).
+        const Chunk most = chunk_at(s, p, wide ? c->wide_rows : g.max_batch);
+        const bool long_pass = wide && most.rows >= tc_long_pass_rows(g.d, g.L, g.L - most.least, g.max_batch);
         const int max_rows = long_pass ? c->wide_rows : g.max_batch;
         c->meta_rows = max_rows;
         int32_t *mh = next_meta(c);
         int n = 0, n_upd = 0, n_head = 0;
-        const int tok0 = offsets[s] + p, n_want = chunk_rows(s, p, max_rows);
+        const int tok0 = offsets[s] + p, n_want = chunk_at(s, p, max_rows).rows;
         int head_seq[kMaxBatch];
         while (n < n_want) {
             const int len = offsets[s + 1] - offsets[s];
@@ -1025,7 +1028,6 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
                     nullptr);
         if (int rc = push_meta(c, mh)) return rc;
         c->rows_distinct = false;  // consecutive positions of one sequence share a chunk
-        // (a short rest of at most kWideMin rows takes the batch kernels: they split K where tiles are few)
         const int32_t *pos = mh + kMetaHdr + max_rows;
         const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, tc_attn, n_head, mh + kMetaHdr + 5 * max_rows, head_tiles, pos,
                                                       mh + kMetaHdr + 7 * max_rows, record_fail)

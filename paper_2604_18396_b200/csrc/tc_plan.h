@@ -134,4 +134,18 @@ inline int tc_wide_segment(int num_sms, int pass_rows, int tiles, int K, bool f1
     return std::min(K >= 4096 ? 16 : 8, run);
 }
 
+// Rows from which a prefill pass that the batch kernels could take as well (up to `max_rows` rows, 256 at most) is a long one.
+// `exit_blocks` of its L blocks have rows on the exit layers.  The pair kernel's time hardly depends on the rows up to 256 - its
+// tiles fill the chip late, and every exit-layer matrix is expanded first - the batch kernels' grows with them, the later the wider
+// the blocks.  Measured, batch / pair kernels, us (blocks on the exit layers / all, 1 prompt):
+//   mini 0/6      129 rows 642 / 490
+//   d 1024 0/4    160: 460 / 462   176: 481 / 467      3/4  176: 513 / 535   192: 540 / 534
+//   1B 0/3        144: 553 / 647   145: 933 / 645      2/3  176: 771 / 779   192: 785 / 778
+//   d 3072 0/3    144: 636 / 707   145: 1018 / 708     2/3  176: 890 / 904   192: 919 / 907
+//   8B 0/2        160: 783 / 820   176: 851 / 838      1/2  208: 879 / 1036  256: 1019 / 1056   257 (two passes): 1206 / 1132
+inline int tc_long_pass_rows(int d, int L, int exit_blocks, int max_rows) {
+    const int base = d >= 4096 ? 160 : d >= 1024 ? 144 : 128, more = d >= 4096 ? 220 : d >= 1024 ? 60 : 0;
+    return std::min(base + more * exit_blocks / L, std::min(max_rows, 256)) + 1;
+}
+
 }  // namespace river

@@ -17,6 +17,7 @@ void w4(int sms, int np, int tiles, int K, int decode, int *o) {
     o[0] = p.occ; o[1] = p.n_stages; o[2] = p.splits; o[3] = p.wide; o[4] = p.sets; o[5] = p.cols;
 }
 int tc_splits(int sms, int np, int tiles, int K) { return river::tc_plan(sms, np, tiles, K, true, false).splits; }
+int long_pass_rows(int d, int L, int exit_blocks, int max_rows) { return river::tc_long_pass_rows(d, L, exit_blocks, max_rows); }
 int wide_segment(int sms, int rows, int tiles, int K, int f16) { return river::tc_wide_segment(sms, rows, tiles, K, f16 != 0); }
 }
 """
@@ -73,3 +74,10 @@ def test_long_pass_sums_are_no_longer_than_short_passes(plan, chunk):
             else:
                 longest = ceil_div(kb, plan.tc_splits(SMS, np, tiles, K))
             assert 1 <= plan.wide_segment(SMS, chunk, tiles, K, f16) <= min(16, longest), (tiles, K, f16)
+
+
+def test_rows_of_a_long_pass(plan):
+    assert [plan.long_pass_rows(d, 2, x, 256) for d, x in ((256, 0), (512, 2), (1024, 0), (2048, 2), (3072, 0), (4096, 0), (4096, 1), (8192, 2))] == [
+        129, 129, 145, 205, 145, 161, 257, 257]
+    assert plan.long_pass_rows(4096, 32, 32, 128) == 129  # never more than one short pass can hold, nor than the batch kernels take
+    assert plan.long_pass_rows(4096, 32, 32, 1024) == 257
