@@ -10,6 +10,8 @@
 // the rows still in the backbone (bf16 weights) and the rows in the exit layers (4-bit codes + bf16 scale / zero
 // per group, dequantised on the fly as (q - z) * s); which set is non-empty is read on the device.
 #pragma once
+#include <type_traits>
+
 #include "river_common.cuh"
 
 namespace river {
@@ -941,8 +943,25 @@ __global__ void __launch_bounds__(512) stream_proj_kernel(const P p, const ProjI
         if (na == 0)
             stream_pass_w4<P, N, R, true>(p, in, riv_idx, nr, xstride, xs, xq, xsc, xsum, red, t0, t1, prestaged, fast, pre4);
     } else {
-        stream_pass_bf16<P, N, R>(p, in, act_idx, na, xstride, xs, red, t0, t1, prestaged, fast, pre_kind == 1, pre4.q);
-        stream_pass_w4<P, N, R, false>(p, in, riv_idx, nr, xstride, xs, xq, xsc, xsum, red, t0, t1, prestaged, fast, pre4);
+        // A step of three or four rows is a list of each weight set, and every row of padding costs its shared-memory reads and
+        // FMAs for every weight: a list of one or two rows takes the two-row pass (8B-class blocks, two rows on each set: 651 us a
+        // step with four-row passes, 598 so).  With two weight rows per task only: four of them spill as it is, and the second form
+        // would make them spill more (1B class, three rows on the backbone 338 -> 343).
+        auto bf16_pass = [&](auto rows) {
+            stream_pass_bf16<P, decltype(rows)::value, R>(p, in, act_idx, na, xstride, xs, red, t0, t1, prestaged, fast, pre_kind == 1, pre4.q);
+        };
+        auto w4_pass = [&](auto rows) {
+            stream_pass_w4<P, decltype(rows)::value, R, false>(p, in, riv_idx, nr, xstride, xs, xq, xsc, xsum, red, t0, t1, prestaged, fast, pre4);
+        };
+        using All = std::integral_constant<int, N>;
+        using Two = std::integral_constant<int, 2>;
+        if constexpr (N > 2 && R == 2) {
+            if (na <= 2) bf16_pass(Two{}); else bf16_pass(All{});
+            if (nr <= 2) w4_pass(Two{}); else w4_pass(All{});
+        } else {
+            bf16_pass(All{});
+            w4_pass(All{});
+        }
     }
 }
 
