@@ -74,7 +74,6 @@ cudaError_t launch_stream(river_ctx *c, const P &p, const ProjIn &in, const RowL
             b.w += half; b.rw.codes += half / 2; b.rw.scale += half / p.group; b.rw.zero += half / p.group;
             b.resid = p.out; ib.src += half;
             const cudaError_t e = launch_stream(c, a, ia, rl, half, tasks_r2, n, has_river, pdl, skip_backbone, dec);
-            ++c->st.launches_last_step;
             return e != cudaSuccess ? e : launch_stream(c, b, ib, rl, half, tasks_r2, n, has_river, pdl, skip_backbone, dec);
         }
     }

@@ -47,7 +47,6 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
         e = launch_k(tc_prep_kernel, dim3(np, (K + kPrepChunk - 1) / kPrepChunk), dim3(256), 0, c->stream, true, in, rows, cnt, K,
                      c->tc_xhi, bm->lo_ptr);
         if (e != cudaSuccess) return e;
-        ++c->st.launches_last_step;
     }
     if (!(phase & kTcGemm)) return e;
     TcArgs a{};

@@ -17,7 +17,6 @@ cudaError_t launch_tc_prep_pair(river_ctx *c, const ProjIn &in, int K, int n, co
     PrepPair p{rows_a, cnt_a, rows_r, cnt_r, c->tc_xhi, alo, reinterpret_cast<__half *>(c->tc_x4),
                reinterpret_cast<__half *>(br->lo_ptr), (K + kPrepChunk - 1) / kPrepChunk};
     const int yr = (K + 2 * kPrepChunk - 1) / (2 * kPrepChunk);
-    ++c->st.launches_last_step;
     return launch_k(tc_prep_pair_kernel, dim3(np, p.ya + yr), dim3(256), 0, c->stream, true, in, p, K);
 }
 
@@ -34,7 +33,6 @@ cudaError_t launch_tc_w4(river_ctx *c, const ProjIn &in, const CUtensorMap *cons
         e = launch_k(tc_prep_w4_kernel, dim3(np, (K + 2 * kPrepChunk - 1) / (2 * kPrepChunk)), dim3(256), 0, c->stream, true, in,
                      rows, cnt, K, reinterpret_cast<__half *>(c->tc_x4), reinterpret_cast<__half *>(bm->lo_ptr));
         if (e != cudaSuccess) return e;
-        ++c->st.launches_last_step;
     }
     if (!(phase & kTcGemm)) return e;
     TcW4Args a{};

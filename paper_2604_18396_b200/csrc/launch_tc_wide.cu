@@ -37,7 +37,6 @@ const river_ctx::WMap *wide_map(river_ctx *c, int K, int bn, bool alt) {
 
 cudaError_t launch_wide_operand(river_ctx *c, const ProjIn &in, int K, int n_list, const int32_t *rows, const int32_t *cnt, bool f16) {
     uint16_t *hi = wide_operand(c, false), *lo = hi + (size_t)c->wide_rows * K;
-    ++c->st.launches_last_step;
     if (f16)
         return launch_k(tc_prep_w4_kernel, dim3(n_list, (K + 2 * kPrepChunk - 1) / (2 * kPrepChunk)), dim3(256), 0, c->stream, true,
                         in, rows, cnt, K, reinterpret_cast<__half *>(hi), reinterpret_cast<__half *>(lo));
@@ -53,7 +52,6 @@ cudaError_t launch_w4_expand(river_ctx *c, const river_w4 *const (&w)[3], const 
         if (rows[i]) e.m[i] = w4_of(*w[i]);
         threads += (long long)rows[i] * (K / 32);
     }
-    ++c->st.launches_last_step;
     return launch_k(w4_expand_kernel, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, c->stream, true, e, K, c->wide_w);
 }
 

@@ -372,7 +372,6 @@ struct LaunchScope {
     river_ctx *c;
     int idx = -1;
     LaunchScope(river_ctx *c_, int cls, double bytes_act, double bytes_riv, int list_idx) : c(c_) {
-        ++c->st.launches_last_step;
         if (!c->profiling) return;
         idx = (int)c->prof_rec.size();
         if ((size_t)(2 * idx + 1) >= c->prof_ev.size()) { idx = -1; return; }
@@ -521,12 +520,10 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
             // hint is the step's row count: the kernel always waits for the real count)
             note(launch_tc(c, in, tm->k, tm->v, tm->v, d, 2 * kvdim / kTcBM, n, 0, kvdim / kTcBM, kvdim / kTcBM, ri, nr, e,
                            true, c->meta_dev /* StepMeta::n_rows */));
-            ++c->st.launches_last_step;
         } else {
             QkvProblem pk = p;
             pk.Hq = 0;
             note(launch_stream(c, pk, in, rl, d, 2 * g.Hkv * (g.dh / 2), n, 2, true, 0, DecideArgs{}));
-            ++c->st.launches_last_step;
         }
     }
     return err;
@@ -572,7 +569,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     const river_config &g = c->cfg;
     const int L = g.L, d = g.d, B = c->list_rows;
     int32_t *fail_buf = record_fail ? c->prefill_fail : nullptr;
-    c->st.launches_last_step = 0;
+    const int64_t launched = t_launches;
     Lists lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, B};
     const int qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
     const double w4f = 0.25 + 2.0 / g.group;  // bytes of a 4-bit copy relative to bf16: (1/2 + 4/G) / 2
@@ -747,6 +744,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     }
     if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(err));
+    c->st.launches_last_step = (int32_t)(t_launches - launched);
     c->st.launches_total += c->st.launches_last_step;
     if (c->profiling) return profile_collect(c);
     return 0;
@@ -765,7 +763,7 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
                   const int32_t *depth, bool record_fail) {
     const river_config &g = c->cfg;
     const int L = g.L, d = g.d, F = g.F, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
-    c->st.launches_last_step = 0;
+    const int64_t launched = t_launches;
     cudaError_t err = cudaSuccess;
     auto note = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
     std::vector<int> leave(L + 1, 0);  // rows that leave after block l
@@ -872,6 +870,7 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
     if (n_head > 0) note(launch_head(c, c->h[hi], n_head));
     if (err == cudaSuccess) err = cudaGetLastError();
     if (err != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(err));
+    c->st.launches_last_step = (int32_t)(t_launches - launched);
     c->st.launches_total += c->st.launches_last_step;
     if (c->profiling) return profile_collect(c);
     return 0;
@@ -1329,7 +1328,7 @@ int river_attention(river_ctx *c, int layer, int n_rows, const int32_t *slots, c
     c->obuf = out;
     c->attn_skip = nullptr;  // every listed row attends
     c->attn_layer1 = 0;      // ... to every cached position
-    c->st.launches_last_step = 0;
+    const int64_t launched = t_launches;
     cudaError_t e;
     {
         double kv_read = 0.0;
@@ -1340,6 +1339,7 @@ int river_attention(river_ctx *c, int layer, int n_rows, const int32_t *slots, c
     c->qbuf = q_keep;
     c->obuf = o_keep;
     if (e != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(e));
+    c->st.launches_last_step = (int32_t)(t_launches - launched);
     c->st.launches_total += c->st.launches_last_step;
     if (c->profiling) return profile_collect(c);
     return RIVER_OK;
@@ -1356,12 +1356,13 @@ int river_project_kv(river_ctx *c, int layer, int use_exit_layer, int n_rows, co
     }
     float *q_keep = c->qbuf;
     if (q_out) c->qbuf = q_out;
-    c->st.launches_last_step = 0;
+    const int64_t launched = t_launches;
     const cudaError_t e = launch_qkv(c, layer, n_rows, h, DecideArgs{}, (double)n_rows * 4.0 * c->cfg.Hkv * c->cfg.dh);
     c->qbuf = q_keep;
     if (e != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(e));
     if (!use_exit_layer && c->off_first && layer >= c->off_first)
         CUDA_TRY(c, cudaEventRecord(c->off_freed[(layer - c->off_first) & 1], c->stream));
+    c->st.launches_last_step = (int32_t)(t_launches - launched);
     c->st.launches_total += c->st.launches_last_step;
     if (c->profiling) return profile_collect(c);
     return RIVER_OK;

@@ -139,6 +139,7 @@ namespace river {
 // Launch with the programmatic-dependent-launch attribute: the kernel may start while its predecessor in the
 // stream is still running and orders itself with griddepcontrol.wait.  Every kernel launched this way calls
 // griddepcontrol.wait before it touches anything a predecessor writes.
+inline thread_local int64_t t_launches = 0;  // kernels this thread has launched: a step's count is what it adds
 template <class... KArgs, class... Args>
 cudaError_t launch_kc(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool pdl,
                       int cluster_x, Args &&...args) {
@@ -163,6 +164,7 @@ cudaError_t launch_kc(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem
     }
     cfg.attrs = at;
     cfg.numAttrs = na;
+    ++t_launches;
     return cudaLaunchKernelEx(&cfg, kern, KArgs(std::forward<Args>(args))...);
 }
 template <class... KArgs, class... Args>
