@@ -789,7 +789,7 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
         const int32_t *rows_of[2] = {c->act_idx + (size_t)at * c->list_rows, c->riv_idx + (size_t)at * c->list_rows};
         const int32_t *cnt_of[2] = {c->n_act + at, c->n_riv + at};
         auto ceil_rows = [&](int set) { return 2.0 * (set ? 0.25 + 2.0 / g.group : 1.0) * (n_of[set] ? 1.0 : 0.0); };
-        const double wsum = ceil_rows(0) + ceil_rows(1);  // bytes per weight this block streams
+        auto wsum = [&] { return ceil_rows(0) + ceil_rows(1); };  // bytes per weight that the rows of n_of stream
         // one projection on the weight set(s) that have rows: the operand rows (unless the projection before wrote them),
         // the f16 weights of the exit layer, the GEMM
         auto project = [&](const ProjIn *in, int K, int tiles, int q_tiles, int k_tiles, int run_step, int head_step, int set, const CUtensorMap &m0,
@@ -801,7 +801,7 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
                                 set == 1, in == nullptr));
         };
         {
-            LaunchScope ls(c, K_QKV, wsum * (qdim + 2.0 * kvdim) * d + (double)n * 4.0 * kvdim, 0, -1);
+            LaunchScope ls(c, K_QKV, wsum() * (qdim + 2.0 * kvdim) * d + (double)n * 4.0 * kvdim, 0, -1);
             const WdQkvEpi e{g.Hq, g.Hkv, g.dh, c->rope_cs, c->qbuf, kv_addr(c, l - 1), c->dev_err};
             const ProjIn in{h_in, (const uint16_t *)w.attn_norm, g.rms_eps};
             for (int set = 0; set < 2; ++set)
@@ -826,12 +826,17 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
             if (heads_only && n_head == 0) break;
         }
         {
-            LaunchScope ls(c, K_PREFILL_ATTN, kv_read, 0, -1);
+            double kv_bytes = kv_read;
+            if (heads_only) {
+                kv_bytes = 0.0;
+                for (int i = 0; i < n_head; ++i) kv_bytes += (double)(row_pos_host[head[i]] + 1) * 4.0 * kvdim;
+            }
+            LaunchScope ls(c, K_PREFILL_ATTN, kv_bytes, 0, -1);
             note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1)
                  : tc_attn ? launch_attention_prefill_tc(c, n_tiles, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
         }
         {
-            LaunchScope ls(c, K_OPROJ, wsum * qdim * d, 0, -1);
+            LaunchScope ls(c, K_OPROJ, wsum() * qdim * d, 0, -1);
             const WdResidEpi e{h_in, h_mid, d};
             const ProjIn in{c->obuf, nullptr, 0.f};
             for (int set = 0; set < 2; ++set)
