@@ -83,15 +83,21 @@ class Pair:
         self.V = self.shape.V
 
     # ---- both sides
-    def prefill(self, slots: List[int], prompts: List[np.ndarray], exit_layer: Optional[int] = None):
+    def prefill(self, slots: List[int], prompts: List[np.ndarray], exit_layer: Optional[int] = None, logits: bool = False):
+        """logits: also compare the logits of every prompt's last position."""
+        want = []
         for s, p in zip(slots, prompts):
-            self.oracle.prefill(s, p, exit_layer)
+            want.append(self.oracle.prefill(s, p, exit_layer)[0])
             self.depth.setdefault(s, []).extend([self.L if exit_layer is None else exit_layer] * len(p))
             if self.twin:
                 self.twin.prefill(s, p, exit_layer)
         tok = torch.from_numpy(np.concatenate(prompts).astype(np.int32)).cuda()
         offs = np.concatenate([[0], np.cumsum([len(p) for p in prompts])]).tolist()
-        self.gpu.prefill(slots, tok, offs, exit_layer)
+        lg = torch.empty((len(slots), self.V), dtype=torch.float32, device="cuda") if logits else None
+        self.gpu.prefill(slots, tok, offs, exit_layer, lg)
+        if logits:
+            torch.cuda.synchronize()
+            self.compare_logits(lg.cpu().numpy(), np.stack(want), f"prompts of {[len(p) for p in prompts]}, depth {exit_layer}")
 
     def fill_history(self, lens: List[int], seed: int = 31):
         """The same N(0,1) bf16 K/V history of lens[b] positions in slot b of both caches (an oracle prefill of long

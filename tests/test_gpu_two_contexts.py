@@ -10,16 +10,17 @@ pytestmark = pytest.mark.gpu
 
 
 def test_contexts_with_other_prompt_lengths_do_not_disturb_each_other():
-    # the shared memory a projection launch asks for does not grow with the rows of the chunk: 200 rows ask for more than 256
+    # a projection of 60 rows asks for more shared memory (three stages of 32 KB per CTA) than one of 12 (at most four of 20 KB), so a
+    # limit that the second context set for its own launches alone would be too low for the first one's next prompt
     shape, _, (bb, rv) = draw_model("mini8")
-    cfg = make_config(shape, max_seqs=1, max_pages_per_seq=32, n_pages=32, max_batch=8, prefill_chunk=256)
+    cfg = make_config(shape, max_seqs=1, max_pages_per_seq=8, n_pages=8, max_batch=8, prefill_chunk=64)
     a, b = River(cfg, bb, rv), River(cfg, bb, rv)
-    tok = synth.tokens(3, 0, 256, shape.V).cuda()
+    tok = synth.tokens(3, 0, 60, shape.V).cuda()
     out = [torch.empty((1, shape.V), device="cuda") for _ in range(2)]
-    a.prefill([0], tok[:200].contiguous(), [0, 200], None, out[0])
-    b.prefill([0], tok, [0, 256])
+    a.prefill([0], tok, [0, 60], None, out[0])
+    b.prefill([0], tok[:12].contiguous(), [0, 12])
     a.release(0)
-    a.prefill([0], tok[:200].contiguous(), [0, 200], None, out[1])
+    a.prefill([0], tok, [0, 60], None, out[1])
     torch.cuda.synchronize()
     assert torch.equal(out[0], out[1])
     a.close()
