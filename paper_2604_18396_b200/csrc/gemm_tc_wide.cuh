@@ -15,9 +15,10 @@
 // epilogue under the next tile's MMAs.  Tiles go to the pairs in the order (features outer, rows inner), so that the pairs
 // working at one time share weight tiles in L2.
 //
-// What bounds it: the tensor pipe and, when passes follow each other, the power cap.  8B-class shape, 1024 rows, operand
-// kernel included: QKV 96 us, O 56, gate/up 305, down 148 (1.7 PFLOP/s of bf16 MMAs, half of them for the low parts) against
-// 4 x (108, 42, 191, 81) us in passes of 256 rows on tc_gemm_kernel.
+// What bounds it: the tensor pipe for gate/up and down (81 and 76 % of the kernel's time busy under ncu), and the power cap
+// when passes follow each other; QKV and O (65 and 63 %) have too few tiles for whole rounds.  8B-class shape, 1024 rows, inside
+// passes that follow each other, operand kernel included: QKV 100 us, O 63, gate/up 331, down 158 - 1.03, 1.09, 1.45 and 1.52 PFLOP/s of
+// bf16 MMAs, half of them for the low parts - against 4 x (108, 42, 191, 81) us in passes of 256 rows on tc_gemm_kernel.
 #pragma once
 #include "gemm_tc.cuh"
 #include "gemm_tc_w4.cuh"
@@ -39,7 +40,10 @@ constexpr uint32_t kWdABytes = kTcBM * kTcBK * 2;
 // per tile and k-block does that, through a five-dimensional map (make_map_paired); eight copies of 16 rows each kept the
 // issuing lane from keeping up (8B-class gate/up, 1024 rows: 490 us against 433) - and lanes 0-15 finish the even
 // rows of the chunk, lanes 16-31 the odd ones.
-struct WdResidEpi {  // out[row][f] = resid[row][f] + value; tile rows in the matrix's own order
+// out[row][f] = resid[row][f] + value; tile rows in the matrix's own order.  The sums start from the residual: every segment is
+// rounded at its magnitude (14 times for K = 14336).  Added once, before the last segment, it moved no distance from 64-bit
+// arithmetic (mini, 1B-class and 8B-class blocks, 300 and 1000 positions: the third digit) and cost 2-7 % of a prompt.
+struct WdResidEpi {
     const float *resid;
     float *out;
     int out_dim;
@@ -171,7 +175,7 @@ struct WdQkvEpi {  // tiles walk the concatenated [q heads | k heads | v heads] 
 struct TcWideArgs {
     int K;              // inner dimension (multiple of 64)
     int bn;             // rows per tile (multiple of 32, <= 256)
-    int tiles;          // 128-feature tiles
+    int tiles;          // 128-feature tiles (an even number)
     int n_stages;
     int seg;            // k-blocks per accumulation segment
     int f16;            // operands are f16 (dequantised exit-layer weights), else bf16
@@ -270,7 +274,7 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
     volatile int *abortp = &s_abort;
     pdl_wait();
     const int n_live = *a.cnt;
-    const int n_tiles = (n_live + bn - 1) / bn, total = n_live > 0 ? ((a.tiles + 1) / 2) * n_tiles : 0;
+    const int n_tiles = (n_live + bn - 1) / bn, total = n_live > 0 ? (a.tiles / 2) * n_tiles : 0;
     const int pair0 = blockIdx.x >> 1, pairs = gridDim.x >> 1, nkb = a.K / kTcBK;
 
     if (warp == 0) {
@@ -281,7 +285,7 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
             bool ok = true;
             for (int t = pair0; t < total && ok; t += pairs) {
                 const int ft = 2 * (t / n_tiles) + (int)rank, by = (t % n_tiles) * bn + (int)rank * (bn / 2);
-                // where this CTA's weight rows live (a tile beyond the last reads rows beyond its matrix: zeros)
+                // where this CTA's weight rows live
                 const CUtensorMap *ma = &map_a0;
                 int at = ft;  // tile inside its matrix
                 if (a.q_tiles) {
@@ -345,7 +349,7 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
         int j = 0;
         bool quit = false;
         for (int t = pair0; t < total && !quit; t += pairs) {
-            const int ft = 2 * (t / n_tiles) + (int)rank, n0 = (t % n_tiles) * bn, live = ft < a.tiles ? min(bn, n_live - n0) : 0;
+            const int ft = 2 * (t / n_tiles) + (int)rank, n0 = (t % n_tiles) * bn, live = min(bn, n_live - n0);
             float acc[kWdOwn][kWdChunk];  // this warp's chunks: columns 32 (group + 4 i)
             int row[kWdOwn], note[kWdOwn];  // what the epilogue reads elsewhere is requested now, under the MMAs
 #pragma unroll
@@ -401,32 +405,6 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
 
 inline size_t tc_wide_smem_bytes(int bn, int n_stages) {
     return 1024 + (size_t)n_stages * (kWdABytes + (size_t)bn * kTcBK * 2) + sizeof(uint64_t) * (2 * n_stages + 4);
-}
-
-// ---------------------------------------------------------------- exit-layer weights in f16, for the same kernel
-// With hundreds of rows a 4-bit matrix is worth expanding once per pass: row r of the (up to three) matrices laid one after
-// the other becomes K f16 values (q - z) * s - one rounding, as in tc_gemm_w4_kernel - with the inputs of every group of
-// eight in the order (0,4,1,5,2,6,3,7) that the f16 operand rows have too.  A thread expands 32 codes.  Bound by HBM:
-// 0.56 bytes read and 2 written per weight.
-struct W4Expand { W4 m[3]; int rows[3]; };
-static __global__ void __launch_bounds__(256) w4_expand_kernel(const W4Expand e, int K, __half *out) {
-    pdl_launch();
-    pdl_wait();  // the GEMM before may still read the previous projection's expansion
-    const int per_row = K >> 5;
-    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    int r = (int)(i / per_row), m = 0;
-    const int c = (int)(i % per_row);  // 32-input run of the row
-    if (r >= e.rows[0] + e.rows[1] + e.rows[2]) return;
-    uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)r * K + 32 * c);
-    while (r >= e.rows[m]) { r -= e.rows[m]; ++m; }
-    const W4 w = e.m[m];
-    const size_t g = (size_t)r * (K >> 6) + (c >> 1);
-    const __half2 s2 = __float2half2_rn(bf16f(w.scale[g])), z2 = __float2half2_rn(bf16f(w.zero[g]));
-    const uint4 v = ldg_stream16(w.codes + (size_t)r * (K >> 1) + 16 * c);
-    dst[0] = w4_word_to_f16(v.x, z2, s2);
-    dst[1] = w4_word_to_f16(v.y, z2, s2);
-    dst[2] = w4_word_to_f16(v.z, z2, s2);
-    dst[3] = w4_word_to_f16(v.w, z2, s2);
 }
 
 }  // namespace river

@@ -9,9 +9,35 @@ namespace river {
 
 namespace {
 
+// ---------------------------------------------------------------- exit-layer weights in f16, for the same kernel
+// With hundreds of rows a 4-bit matrix is worth expanding once per pass: row r of the (up to three) matrices laid one after
+// the other becomes K f16 values (q - z) * s - one rounding, as in tc_gemm_w4_kernel - with the inputs of every group of
+// eight in the order (0,4,1,5,2,6,3,7) that the f16 operand rows have too.  A thread expands 32 codes.  Bound by HBM:
+// 0.56 bytes read and 2 written per weight.
+struct W4Expand { W4 m[3]; int rows[3]; };
+__global__ void __launch_bounds__(256) w4_expand_kernel(const W4Expand e, int K, __half *out) {
+    pdl_launch();
+    pdl_wait();  // the GEMM before may still read the previous projection's expansion
+    const int per_row = K >> 5;
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    int r = (int)(i / per_row), m = 0;
+    const int c = (int)(i % per_row);  // 32-input run of the row
+    if (r >= e.rows[0] + e.rows[1] + e.rows[2]) return;
+    uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)r * K + 32 * c);
+    while (r >= e.rows[m]) { r -= e.rows[m]; ++m; }
+    const W4 w = e.m[m];
+    const size_t g = (size_t)r * (K >> 6) + (c >> 1);
+    const __half2 s2 = __float2half2_rn(bf16f(w.scale[g])), z2 = __float2half2_rn(bf16f(w.zero[g]));
+    const uint4 v = ldg_stream16(w.codes + (size_t)r * (K >> 1) + 16 * c);
+    dst[0] = w4_word_to_f16(v.x, z2, s2);
+    dst[1] = w4_word_to_f16(v.y, z2, s2);
+    dst[2] = w4_word_to_f16(v.z, z2, s2);
+    dst[3] = w4_word_to_f16(v.w, z2, s2);
+}
+
 // Rows per tile: the tiles go to `pairs` CTA pairs in whole rounds, so a size that leaves the last round nearly full can win
-// over a larger one that does not; a round takes about as long as its rows and 128 more (8B-class gate/up, 1024 rows: 7 rounds
-// of 256 rows 297 us, 10 of 192 338, 13 of 128 388; QKV: 2 of 256 112, 2 of 192 102, 3 of 128 122).
+// over a larger one that does not; a round takes about as long as its rows and 128 more (with the operand kernel, by itself: 8B-class gate/up, 1024 rows, 7 rounds of 256 rows 297 us, 10 of 192 338, 13 of 128 388; QKV: 2 of 256 112, 2 of
+// 192 102, 3 of 128 122).
 int wide_bn(int feature_pairs, int n, int pairs) {
     int best = 256;
     double best_t = 1e30;
@@ -60,7 +86,8 @@ cudaError_t launch_tc_wide(river_ctx *c, const CUtensorMap &a0, const CUtensorMa
                            int n_list, int q_tiles, int k_tiles, int run_step, int head_step, const int32_t *rows, const int32_t *cnt,
                            const Epi &epi, bool f16, bool alt_operand) {
     TcWideArgs a{};
-    const int feature_pairs = (tiles + 1) / 2, pairs = c->num_sms / 2;
+    const int feature_pairs = tiles / 2, pairs = c->num_sms / 2;
+    if (tiles & 1) return cudaErrorInvalidValue;  // (every shape of the exit layers' tensor-core kernels has whole pairs of tiles)
     a.K = K; a.tiles = tiles; a.f16 = f16 ? 1 : 0; a.q_tiles = q_tiles; a.k_tiles = k_tiles;
     a.run_step = run_step; a.head_step = head_step;
     a.rows = rows; a.cnt = cnt; a.dev_err = c->dev_err;

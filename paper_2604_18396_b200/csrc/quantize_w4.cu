@@ -163,7 +163,7 @@ extern "C" int river_quantize_w4(const void *w, int out, int in, int group, int 
                                  void *zero, void *cuda_stream) {
     if (!w || !codes || !scale || !zero || out <= 0 || in <= 0 || refine_iters < 0 || refine_iters > 1000) return RIVER_E_BADARG;
     if (!(group == 32 || group == 64 || group == kMaxGroup) || in % group) return RIVER_E_SHAPE;
-    if (((uintptr_t)w | (uintptr_t)codes) & 15) return RIVER_E_BADARG;  // 16-byte loads / 4-byte stores of whole groups
+    if (((uintptr_t)w | (uintptr_t)codes) & 15) return RIVER_E_BADARG;  // whole groups in 16-byte loads and stores
     const long long n_groups = (long long)out * (in / group);
     const unsigned grid = (unsigned)((n_groups + 127) / 128);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
