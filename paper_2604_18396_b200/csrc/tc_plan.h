@@ -98,7 +98,7 @@ inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode) {
     const int raw_tiles = K / (kTcBK * kW4Super), min_raw = raw_tiles <= 8 ? 2 : 4;
     p.splits = tc_pick_splits(num_sms, tiles, raw_tiles, num_sms * p.occ, min_raw);
     // Decode steps: splits for one CTA per SM, the rest of the SM belongs to tc_gemm_kernel's CTAs beside this grid and to the
-    // next projection's (1B-class, 8 rows 1120 -> 1097 us a step) - where the longer run can be summed in two accumulators of
+    // next projection's (1B-class, 8 rows 1120 -> 1109 us a step) - where the longer run can be summed in two accumulators of
     // half of it each, so that no sum inside the tensor cores takes more inputs: its error grows with their number (8B-class QKV on
     // exact weights against 64-bit arithmetic: 1.5e-7 split over every slot, 2.0e-7 with one accumulator and half the splits, 1.1e-7
     // with two).  That is up to 32 operand rows: 2 x 2 np columns beside four A tiles are the 256 that one accumulator takes as well.
