@@ -95,10 +95,14 @@ __device__ __forceinline__ float refine_sum_plain(const unsigned long long (&d)[
 //     the roundings of the 32-bit operations (each is below 2^-23 of them) and keeps 1 % from the threshold.
 //   * with w_e = 0 the second division is x / s, the same in every round: taken once.
 //   * when the group's own range needs no clamp, neither does any of its weights (adding z is monotonic).
+//   * a round that gives back the zero-point it started from, bit for bit, is what every round behind it would do too - as
+//     long as the threshold, which only falls with the rounds, is zero for this group in the last one as well: done.  Of the
+//     20 rounds on normally distributed weights a group of 64 takes 4.2 so, the slowest of a warp's 32 groups 11.2.
 // What is left are four packed additions per pair and the sum, whose order the bits depend on.
-// Measured on 4096 x 14336, 64 inputs per group, 20 rounds: 5488 us with the general round everywhere, 295 us so.
+// Measured on 4096 x 14336, 64 inputs per group, 20 rounds: 5488 us with the general round everywhere, 295 us
+// with every round taken, 222 us so.
 template <int G>
-__global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w, long long n_groups, int refine_iters,
+__global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w, long long n_groups, int refine_iters, float last_inv_beta,
                                                           uint8_t *codes, __nv_bfloat16 *scale, __nv_bfloat16 *zero) {
     const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= n_groups) return;
@@ -123,6 +127,7 @@ __global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w
     const float dmin = __fdiv_rn(mn, s), dmax = __fdiv_rn(mx, s);  // rounding is monotonic: every d lies between them
     const float xabs = fmaxf(fabsf(mn), fabsf(mx));
     float beta = 10.0f;
+    const float last_threshold = 0.99f * powf(last_inv_beta, 1.0f / 1.3f);
     for (int it = 0; it < refine_iters; ++it) {
         const float inv_beta = __fdiv_rn(1.0f, beta);
         const float lo = dmin + z, hi = dmax + z;  // the group's range on the code grid
@@ -132,7 +137,9 @@ __global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w
         if (!(bound < 0.99f * powf(inv_beta, 1.0f / 1.3f))) sum = refine_sum_general<G>(xp, d, s, z, inv_beta);  // (NaN too)
         else if (lo >= -0.5f && hi < 15.5f) sum = refine_sum_plain<G, false>(d, z);
         else sum = refine_sum_plain<G, true>(d, z);
+        const float before = z;
         z = __fdiv_rn(sum, (float)G);
+        if (__float_as_uint(z) == __float_as_uint(before) && bound < last_threshold) break;
         beta = __fmul_rn(beta, 1.01f);
     }
     float zb = bf16_round(z);
@@ -167,11 +174,14 @@ extern "C" int river_quantize_w4(const void *w, int out, int in, int group, int 
     const long long n_groups = (long long)out * (in / group);
     const unsigned grid = (unsigned)((n_groups + 127) / 128);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    volatile float last_beta = 10.0f;  // of the last round: as the kernel's own chain of single products gives it
+    for (int i = 1; i < refine_iters; ++i) last_beta = last_beta * 1.01f;
+    const float last_inv_beta = 1.0f / last_beta;
     const __nv_bfloat16 *wp = static_cast<const __nv_bfloat16 *>(w);
     uint8_t *cp = static_cast<uint8_t *>(codes);
     __nv_bfloat16 *sp = static_cast<__nv_bfloat16 *>(scale), *zp = static_cast<__nv_bfloat16 *>(zero);
-    if (group == 32) quantize_w4_kernel<32><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, cp, sp, zp);
-    else if (group == 64) quantize_w4_kernel<64><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, cp, sp, zp);
-    else quantize_w4_kernel<128><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, cp, sp, zp);
+    if (group == 32) quantize_w4_kernel<32><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_inv_beta, cp, sp, zp);
+    else if (group == 64) quantize_w4_kernel<64><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_inv_beta, cp, sp, zp);
+    else quantize_w4_kernel<128><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_inv_beta, cp, sp, zp);
     return cudaGetLastError() == cudaSuccess ? RIVER_OK : RIVER_E_DEVICE;
 }
