@@ -39,21 +39,32 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
     return v;
 }
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long v;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
 __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
     unsigned long long v;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
     return v;
 }
 
+// The residual below which the soft threshold leaves nothing, (1 / beta)^(1 / 1.3), less 1 %: beta is 10 in the first round and
+// grows by 1.01.  (A thousand single products are off by less than 1e-4 of it.)
+constexpr float kThreshold0 = 0.99f * 0.170125f, kThresholdStep = 0.9923751f;
+
 // One refinement round over a thread's group: the sum of q - (x - w_e) / s in the group's order, d = x / s.
-// The general form, with the soft threshold.
+// The general form, with the soft threshold (which wants the weights themselves: read again, so that a group's registers need
+// not hold them beside d through the rounds that do without).
 template <int G>
-__device__ __forceinline__ float refine_sum_general(const uint32_t (&xp)[G / 2], const unsigned long long (&d)[G / 2], float s, float z, float inv_beta) {
+__device__ __forceinline__ float refine_sum_general(const uint32_t *x2, const unsigned long long (&d)[G / 2], float s, float z, float inv_beta) {
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < G; ++i) {
         const F2 dd = unpack2(d[i / 2]);
-        const float x = __uint_as_float((i & 1) ? (xp[i / 2] & 0xffff0000u) : (xp[i / 2] << 16));
+        const uint32_t xw = x2[i / 2];
+        const float x = __uint_as_float((i & 1) ? (xw & 0xffff0000u) : (xw << 16));
         const float q = fminf(fmaxf(rintf(__fadd_rn((i & 1) ? dd.y : dd.x, z)), 0.f), 15.f);
         const float e = __fsub_rn(x, __fmul_rn(__fsub_rn(q, z), s));
         const float ae = fabsf(e);
@@ -100,9 +111,11 @@ __device__ __forceinline__ float refine_sum_plain(const unsigned long long (&d)[
 //     20 rounds on normally distributed weights a group of 64 takes 4.2 so, the slowest of a warp's 32 groups 11.2.
 // What is left are four packed additions per pair and the sum, whose order the bits depend on.
 // Measured on 4096 x 14336, 64 inputs per group, 20 rounds: 5488 us with the general round everywhere, 295 us
-// with every round taken, 222 us so.
+// with every round taken, 222 us with the rounds that change something - 8 us a round and 130 us around them, spent on the quotients
+// x / s, a power per round for the threshold, and the codes' rounding and conversion (16 a clock each): 142 us with the quotients
+// from the reciprocal, the threshold carried along and the codes rounded by an addition.
 template <int G>
-__global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w, long long n_groups, int refine_iters, float last_inv_beta,
+__global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w, long long n_groups, int refine_iters, float last_threshold,
                                                           uint8_t *codes, __nv_bfloat16 *scale, __nv_bfloat16 *zero) {
     const long long gi = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= n_groups) return;
@@ -122,40 +135,59 @@ __global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w
     if (constant || s == 0.f) s = 1.f;
     float z = __fdiv_rn(-mn, s);
     unsigned long long d[G / 2];
+    // x / s, correctly rounded: with the reciprocal r = 1 / s correctly rounded, q = x r and the exact remainder x - q s, the sum
+    // q + (x - q s) r is (Markstein, IBM J. Res. Dev. 34, 1990; true of every pair of 8-bit mantissas) - as long as the remainder
+    // does not underflow: every weight of the group zero or at least 2^-60 in magnitude, s and the weights at most 2^60.
+    uint32_t tiny = 0u;  // bit 15 of a half: a weight that is neither
 #pragma unroll
-    for (int i = 0; i < G / 2; ++i) d[i] = pack2(__fdiv_rn(x_at(2 * i), s), __fdiv_rn(x_at(2 * i + 1), s));
+    for (int i = 0; i < G / 2; ++i) {
+        const uint32_t u = xp[i] & 0x7fff7fffu;
+        tiny |= (u + 0x7fff7fffu) & ~(u + 0x5e805e80u);  // (0x8000 - 0x2180, the exponent of 2^-60)
+    }
+    if ((tiny & 0x80008000u) == 0u && s >= 0x1p-60f && s <= 0x1p60f && fmaxf(fabsf(mn), fabsf(mx)) <= 0x1p60f) {
+        const float r = __frcp_rn(s);
+        const unsigned long long r2 = pack2(r, r), s2 = pack2(-s, -s);
+#pragma unroll
+        for (int i = 0; i < G / 2; ++i) {
+            const unsigned long long x = pack2(x_at(2 * i), x_at(2 * i + 1)), q = mul2(x, r2);
+            d[i] = fma2(fma2(q, s2, x), r2, q);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < G / 2; ++i) d[i] = pack2(__fdiv_rn(x_at(2 * i), s), __fdiv_rn(x_at(2 * i + 1), s));
+    }
     const float dmin = __fdiv_rn(mn, s), dmax = __fdiv_rn(mx, s);  // rounding is monotonic: every d lies between them
     const float xabs = fmaxf(fabsf(mn), fabsf(mx));
-    float beta = 10.0f;
-    const float last_threshold = 0.99f * powf(last_inv_beta, 1.0f / 1.3f);
+    float beta = 10.0f, threshold = kThreshold0;
     for (int it = 0; it < refine_iters; ++it) {
-        const float inv_beta = __fdiv_rn(1.0f, beta);
         const float lo = dmin + z, hi = dmax + z;  // the group's range on the code grid
         const float off = fmaxf(0.5f, fmaxf(-lo, hi - 15.f));
         const float bound = s * off + 1e-6f * (xabs + (15.f + fabsf(z)) * s);
         float sum;
-        if (!(bound < 0.99f * powf(inv_beta, 1.0f / 1.3f))) sum = refine_sum_general<G>(xp, d, s, z, inv_beta);  // (NaN too)
+        if (!(bound < threshold)) sum = refine_sum_general<G>(reinterpret_cast<const uint32_t *>(src), d, s, z, __fdiv_rn(1.0f, beta));  // (NaN too)
         else if (lo >= -0.5f && hi < 15.5f) sum = refine_sum_plain<G, false>(d, z);
         else sum = refine_sum_plain<G, true>(d, z);
         const float before = z;
-        z = __fdiv_rn(sum, (float)G);
+        z = __fmul_rn(sum, 1.0f / (float)G);  // (a power of two)
         if (__float_as_uint(z) == __float_as_uint(before) && bound < last_threshold) break;
         beta = __fmul_rn(beta, 1.01f);
+        threshold *= kThresholdStep;
     }
     float zb = bf16_round(z);
     if (constant) zb = bf16_round(-mn);
+    const unsigned long long zb2 = pack2(zb, zb), up = pack2(12582912.f, 12582912.f);
     uint32_t packed[G / 8];
 #pragma unroll
     for (int i = 0; i < G / 8; ++i) {
         uint32_t p = 0u;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const F2 dd = unpack2(d[4 * i + j / 2]);
-            float q = fminf(fmaxf(rintf(__fadd_rn((j & 1) ? dd.y : dd.x, zb)), 0.f), 15.f);
-            if (constant) q = 0.f;
-            p |= (uint32_t)q << (4 * j);  // low nibble = even input
+        for (int j = 0; j < 4; ++j) {
+            // clamped, then rounded to the nearest even integer by adding 1.5 * 2^23, whose last bits are the code then
+            const F2 v = unpack2(add2(d[4 * i + j], zb2));
+            const F2 q = unpack2(add2(pack2(fminf(fmaxf(v.x, 0.f), 15.f), fminf(fmaxf(v.y, 0.f), 15.f)), up));
+            p |= (__float_as_uint(q.x) & 15u) << (8 * j) | (__float_as_uint(q.y) & 15u) << (8 * j + 4);  // low nibble = even input
         }
-        packed[i] = p;
+        packed[i] = constant ? 0u : p;
     }
     uint4 *dst = reinterpret_cast<uint4 *>(codes + gi * (G / 2));
 #pragma unroll
@@ -174,14 +206,13 @@ extern "C" int river_quantize_w4(const void *w, int out, int in, int group, int 
     const long long n_groups = (long long)out * (in / group);
     const unsigned grid = (unsigned)((n_groups + 127) / 128);
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    volatile float last_beta = 10.0f;  // of the last round: as the kernel's own chain of single products gives it
-    for (int i = 1; i < refine_iters; ++i) last_beta = last_beta * 1.01f;
-    const float last_inv_beta = 1.0f / last_beta;
+    float last_threshold = kThreshold0;  // of the last round
+    for (int i = 1; i < refine_iters; ++i) last_threshold *= kThresholdStep;
     const __nv_bfloat16 *wp = static_cast<const __nv_bfloat16 *>(w);
     uint8_t *cp = static_cast<uint8_t *>(codes);
     __nv_bfloat16 *sp = static_cast<__nv_bfloat16 *>(scale), *zp = static_cast<__nv_bfloat16 *>(zero);
-    if (group == 32) quantize_w4_kernel<32><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_inv_beta, cp, sp, zp);
-    else if (group == 64) quantize_w4_kernel<64><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_inv_beta, cp, sp, zp);
-    else quantize_w4_kernel<128><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_inv_beta, cp, sp, zp);
+    if (group == 32) quantize_w4_kernel<32><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_threshold, cp, sp, zp);
+    else if (group == 64) quantize_w4_kernel<64><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_threshold, cp, sp, zp);
+    else quantize_w4_kernel<128><<<grid, 128, 0, st>>>(wp, n_groups, refine_iters, last_threshold, cp, sp, zp);
     return cudaGetLastError() == cudaSuccess ? RIVER_OK : RIVER_E_DEVICE;
 }
