@@ -968,7 +968,19 @@ __global__ void __launch_bounds__(512) stream_proj_kernel(const P p, const ProjI
 // ---------------------------------------------------------------- a8: final norm + LM head + argmax partials
 // logits = W_lm . RMSNorm(h) for the rows that need them (all rows of a decode step; the last prompt position in
 // prefill), written as fp32 if the caller gave a buffer, and the greedy next token: every CTA keeps the best
-// (value, id) of its share of the vocabulary (ties -> lowest id), a second small kernel merges the CTAs.
+// (value, id) of its share of the vocabulary (ties -> lowest id), and the CTA that finishes last (atomic ticket, no spinning)
+// merges them.  In decode steps it also notes the last block's score - a diagnostic: no exit is taken there - and the final row
+// lists.  (Two launches fewer a step than with small kernels behind this one.)
+struct HeadEnd {
+    unsigned *ticket;                // zero between launches
+    unsigned long long *exit_hist;   // decode steps (else null): [L + 1] counters of the exit layers taken so far
+    const float *h_prev;             // decode steps (else null): input of block L, fp32 [rows][d]
+    const uint8_t *state_in;         // exit flags entering block L, and behind it
+    uint8_t *state_out;
+    int L;
+    Lists lists;
+    int32_t *hint_act;
+};
 struct HeadArgs {
     const uint16_t *w;  // [V][d]
     ProjIn in;
@@ -977,15 +989,40 @@ struct HeadArgs {
     const StepMeta *meta; // n_head_rows, logits [n_head_rows][V] or nullptr (indexed by position in `rows`)
     float *part_val;      // [max_batch][gridDim.x]
     int32_t *part_idx;
+    HeadEnd end;
 };
 
+// The better of two candidates for the greedy token: the larger value, the lower id where they are equal.
+__device__ __forceinline__ void head_better(float &bv, int &bi, float v, int id) {
+    if (v > bv || (v == bv && id < bi)) { bv = v; bi = id; }
+}
+// The CTA's best candidate, in thread 0 (all threads call it; s_val / s_idx: a word per warp).
+__device__ __forceinline__ void head_block_best(float &bv, int &bi, float *s_val, int *s_idx) {
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        head_better(bv, bi, ov, oi);
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) { s_val[warp] = bv; s_idx[warp] = bi; }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) head_better(bv, bi, s_val[w], s_idx[w]);
+}
+
+// One row: two weight rows a task on sixteen warps, the next batch of loads under the current one's arithmetic, as in
+// stream_pass_bf16; more rows: four weight rows on eight warps, whose registers hold no second batch.  One CTA fits an SM, and the
+// grid is one CTA per SM (two, of which the second half of the CTAs waited for the first and staged the row again, and loads not
+// pipelined: 8B-class, one row 2343 us a step, so 2287; three rows, 8 blocks 1326 -> 1309).
+__host__ __device__ constexpr int head_threads(int n) { return n == 1 ? 512 : 256; }
 template <int N, int R>
-__global__ void __launch_bounds__(256) lm_head_kernel(const HeadArgs a, int xstride) {
+__global__ void __launch_bounds__(head_threads(N)) lm_head_kernel(const HeadArgs a, int xstride) {
     extern __shared__ __align__(16) float stream_smem[];
-    float *red = stream_smem;
-    float *xs = stream_smem + 32;
-    __shared__ float s_val[8][N];
-    __shared__ int s_idx[8][N];
+    float *red = stream_smem;  // 64
+    float *xs = stream_smem + 64;
+    __shared__ float s_val[head_threads(N) / 32][N];
+    __shared__ int s_idx[head_threads(N) / 32][N];
+    constexpr bool PIPE = N * R <= 2;
     const int K = a.d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     pdl_launch();
@@ -1011,13 +1048,43 @@ __global__ void __launch_bounds__(256) lm_head_kernel(const HeadArgs a, int xstr
         int besti[N];
 #pragma unroll
         for (int n = 0; n < N; ++n) { best[n] = -CUDART_INF_F; besti[n] = 0x7fffffff; }
+        const int nch = K >> 3, nit = (nch + 31) >> 5;
+        if (PIPE && i0 > 0 && t0 + warp < t1) {
+            const uint16_t *rows[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) rows[r] = a.w + ((size_t)(t0 + warp) * R + r) * K;
+            stream_issue_bf16<R>(rows, nch, 0, lane, pre);
+        }
         for (int t = t0 + warp; t < t1; t += nwarps) {
             const size_t o0 = (size_t)t * R;
             const uint16_t *rows[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) rows[r] = a.w + (o0 + r) * K;
             float acc[R][N];
-            stream_dots_bf16<N, R>(rows, xs, K, xstride, have_pre && i0 == 0 && t == t0 + warp, pre, acc);
+            if constexpr (PIPE) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int n = 0; n < N; ++n) acc[r][n] = 0.f;
+                for (int it0 = 0; it0 < nit; it0 += kStreamPF) {
+                    uint4 w[R][kStreamPF];
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int u = 0; u < kStreamPF; ++u) w[r][u] = pre[r][u];
+                    if (it0 + kStreamPF < nit) {
+                        stream_issue_bf16<R>(rows, nch, it0 + kStreamPF, lane, pre);
+                    } else if (t + nwarps < t1) {
+                        const uint16_t *nrows[R];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) nrows[r] = rows[r] + (size_t)nwarps * R * K;
+                        stream_issue_bf16<R>(nrows, nch, 0, lane, pre);
+                    }
+                    stream_fma_bf16<N, R>(w, xs, xstride, it0, nch, lane, acc);
+                }
+            } else {
+                stream_dots_bf16<N, R>(rows, xs, K, xstride, have_pre && i0 == 0 && t == t0 + warp, pre, acc);
+            }
 #pragma unroll
             for (int n = 0; n < N; ++n)
 #pragma unroll
@@ -1044,9 +1111,67 @@ __global__ void __launch_bounds__(256) lm_head_kernel(const HeadArgs a, int xstr
             a.part_idx[(size_t)(i0 + n) * gridDim.x + blockIdx.x] = bi;
         }
     }
+    // ---- the last CTA: the greedy tokens of all rows, the last block's scores, the final lists
+    const HeadEnd &f = a.end;
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(f.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (threadIdx.x == 0) *f.ticket = 0u;
+    for (int i = 0; i < cnt; ++i) {
+        float bv = -CUDART_INF_F;
+        int bi = 0x7fffffff;
+        for (int p = threadIdx.x; p < (int)gridDim.x; p += blockDim.x)
+            head_better(bv, bi, __ldcg(a.part_val + (size_t)i * gridDim.x + p), __ldcg(a.part_idx + (size_t)i * gridDim.x + p));
+        __syncthreads();
+        head_block_best(bv, bi, &s_val[0][0], &s_idx[0][0]);
+        if (threadIdx.x == 0) {
+            a.meta->next_tok[i] = bi == 0x7fffffff ? 0 : bi;  // a row without any comparable logit (all NaN) yields token 0
+            if (f.exit_hist) atomicAdd(f.exit_hist + a.meta->exit_layer[i], 1ull);
+        }
+    }
+    if (!f.h_prev) return;
+    const int n = a.meta->n_rows, nv = K >> 2;
+    float *scores = a.meta->scores;
+    for (int b = 0; b < n && scores; ++b) {  // Eq. 1 on the last block's input and output
+        if (f.state_in[b]) continue;
+        const float4 *x4 = reinterpret_cast<const float4 *>(f.h_prev + (size_t)b * K), *y4 = reinterpret_cast<const float4 *>(a.in.src + (size_t)b * K);
+        float ab = 0.f, aa = 0.f, bb = 0.f;
+        for (int v = threadIdx.x; v < nv; v += blockDim.x) {
+            const float4 x = __ldcg(x4 + v), y = __ldcg(y4 + v);
+            ab += x.x * y.x + x.y * y.y + x.z * y.z + x.w * y.w;
+            aa += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+            bb += y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w;
+        }
+        ab = warp_sum(ab); aa = warp_sum(aa); bb = warp_sum(bb);
+        __syncthreads();
+        if (lane == 0) { red[warp] = ab; red[16 + warp] = aa; red[32 + warp] = bb; }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            ab = aa = bb = 0.f;
+            for (int w = 0; w < nwarps; ++w) { ab += red[w]; aa += red[16 + w]; bb += red[32 + w]; }
+            scores[(size_t)b * f.L + (f.L - 1)] = transition_score(ab, aa, bb);
+        }
+    }
+    if (threadIdx.x == 0) {
+        int32_t *A = f.lists.act_idx + (size_t)f.L * f.lists.max_batch, *Rv = f.lists.riv_idx + (size_t)f.L * f.lists.max_batch;
+        int na = 0, nr = 0;
+        for (int b = 0; b < n; ++b) {
+            const uint8_t gone = f.state_in[b] ? 1 : 0;
+            f.state_out[b] = gone;
+            if (gone) Rv[nr++] = b;
+            else A[na++] = b;
+        }
+        f.lists.n_act[f.L] = na;
+        f.lists.n_riv[f.L] = nr;
+        *f.hint_act = na;
+    }
 }
 
-// exit_hist (decode steps only, else null): [L + 1] counters of the exit layers taken so far - the head rows of a decode
+// The merge behind the tensor-core LM head.  exit_hist (decode steps only, else null): [L + 1] counters of the exit layers taken so far - the head rows of a decode
 // step are its rows, and their exit layers are final by now.
 static __global__ void argmax_final_kernel(const StepMeta *meta, const float *part_val, const int32_t *part_idx, int nparts,
                                            unsigned long long *exit_hist) {
@@ -1059,25 +1184,12 @@ static __global__ void argmax_final_kernel(const StepMeta *meta, const float *pa
     float bv = -CUDART_INF_F;
     int bi = 0x7fffffff;
     for (int p = threadIdx.x; p < nparts; p += blockDim.x) {
-        const float v = part_val[(size_t)i * nparts + p];
-        const int id = part_idx[(size_t)i * nparts + p];
-        if (v > bv || (v == bv && id < bi)) { bv = v; bi = id; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+        head_better(bv, bi, part_val[(size_t)i * nparts + p], part_idx[(size_t)i * nparts + p]);
     }
     __shared__ float sv[32];
     __shared__ int si[32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { sv[warp] = bv; si[warp] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-            if (sv[w] > bv || (sv[w] == bv && si[w] < bi)) { bv = sv[w]; bi = si[w]; }
-        next_tok[i] = bi == 0x7fffffff ? 0 : bi;  // a row without any comparable logit (all NaN) yields token 0
-    }
+    head_block_best(bv, bi, sv, si);
+    if (threadIdx.x == 0) next_tok[i] = bi == 0x7fffffff ? 0 : bi;  // (as above)
 }
 
 inline size_t stream_smem_bytes(int N, int K) {

@@ -96,14 +96,14 @@ template cudaError_t launch_stream<GateUpProblem>(river_ctx *, const GateUpProbl
 cudaError_t launch_head_stream(river_ctx *c, const HeadArgs &a, int n_head) {
     const int n_sel = std::min(n_head, 4);
     const int xstride = xs_stride(a.d, 8);
-    const size_t smem = sizeof(float) * (32 + (size_t)n_sel * xstride);
-#define HEAD_CASE(N_)                                                                                              \
+    const size_t smem = sizeof(float) * (64 + (size_t)n_sel * xstride);
+#define HEAD_CASE(N_, R_)                                                                                          \
     if (n_sel == N_) {                                                                                             \
-        const cudaError_t e = ensure_smem(c, lm_head_kernel<N_, 4>, smem);                                         \
+        const cudaError_t e = ensure_smem(c, lm_head_kernel<N_, R_>, smem);                                        \
         if (e != cudaSuccess) return e;                                                                            \
-        return launch_k(lm_head_kernel<N_, 4>, dim3(c->head_grid), dim3(256), smem, c->stream, true, a, xstride); \
+        return launch_k(lm_head_kernel<N_, R_>, dim3(c->head_grid), dim3(head_threads(N_)), smem, c->stream, true, a, xstride); \
     }
-    HEAD_CASE(1) HEAD_CASE(2) HEAD_CASE(3) HEAD_CASE(4)
+    HEAD_CASE(1, 2) HEAD_CASE(2, 4) HEAD_CASE(3, 4) HEAD_CASE(4, 4)
 #undef HEAD_CASE
     return cudaErrorInvalidValue;
 }

@@ -530,7 +530,8 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
 }
 
 // a8: final norm + LM head + greedy token for the n_head rows that need logits.
-cudaError_t launch_head(river_ctx *c, const float *h, int n_head) {
+// prev_in (steps of up to four rows): the last block's input, whose score and row lists the head's last CTA then notes as well.
+cudaError_t launch_head(river_ctx *c, const float *h, int n_head, const float *prev_in = nullptr) {
     const river_config &g = c->cfg;
     const int d = g.d;
     cudaError_t err = cudaSuccess;
@@ -549,7 +550,15 @@ cudaError_t launch_head(river_ctx *c, const float *h, int n_head) {
                        c->head_rows(), c->meta_dev + 2 /* StepMeta::n_head_rows */, e, false, nullptr));
     } else {
         LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
+        a.end.ticket = c->tickets + 2;
+        a.end.exit_hist = c->rows_distinct ? c->exit_hist : nullptr;  // (not for prefill chunks)
+        a.end.h_prev = prev_in;
+        a.end.L = g.L;
+        a.end.state_in = c->state_at(g.L - 1); a.end.state_out = c->state_at(g.L);
+        a.end.lists = Lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, c->list_rows};
+        a.end.hint_act = c->hint_act;
         note(launch_head_stream(c, a, n_head));
+        return err;
     }
     {
         LaunchScope ls(c, K_ARGMAX, 0, 0, -1);
@@ -734,9 +743,11 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         prev_in = h_in;
         hi = (hi + 2) % 3;
     }
-    if (n_head > 0) note(launch_head(c, c->h[hi], n_head));
-    // small steps: the last block's score (a diagnostic: no exit is taken after block L) and the final row lists
-    if (fold) launch_score(L, prev_in, c->h[hi]);
+    // small steps: the last block's score (a diagnostic: no exit is taken after block L) and the final row lists, noted by the
+    // LM head of a decode step (prefill chunks may have none)
+    const bool head_notes = fold && c->rows_distinct && n_head == n;
+    if (n_head > 0) note(launch_head(c, c->h[hi], n_head, head_notes ? prev_in : nullptr));
+    if (fold && !head_notes) launch_score(L, prev_in, c->h[hi]);
     if (strat == RIVER_KV_MASK) {  // what the later tokens' attention may see of this step's positions
         LaunchScope ls(c, K_SCORE, 0, 0, -1);
         note(launch_k(depth_note_kernel, dim3((n + 127) / 128), dim3(128), 0, c->stream, true, c->meta(),
@@ -1116,6 +1127,7 @@ int river_init(const river_config *cfg, const river_weights *w, void *kv_pool, s
         return bail("cudaDeviceGetAttribute failed");
     if (cc_major != 10) return bail("this library is built for sm_100a (B200) only");
     c->device = dev;
+    c->head_grid = std::min(c->head_grid, c->num_sms);  // (one CTA fits an SM)
     if (make_kv_tensor_map(c)) { river_destroy(c); return RIVER_E_DEVICE; }
     c->tc_ok = !(cfg->flags & RIVER_F_NO_TC) && tc_shape_ok(*cfg) && make_tc_maps(c);
     c->w4tc_ok = c->tc_ok && !(cfg->flags & RIVER_F_NO_W4TC) && make_w4_maps(c);
