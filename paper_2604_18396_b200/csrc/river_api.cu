@@ -567,6 +567,116 @@ cudaError_t launch_head(river_ctx *c, const float *h, int n_head, const float *p
     return err;
 }
 
+// What follows attention in block l (a4, a5: O, gate/up and down projections, with their residuals) for the rows of `rl`, n at most,
+// on the kernels of decode steps.  sets: 1 = the backbone's rows, 2 = the exit layers', 3 = both.  list_idx: the list whose counts
+// say which weights were read (timing), -1: all of `sets`.  hint_riv: a count that is never below the exit layers' rows.
+cudaError_t block_tail(river_ctx *c, int l, int n, const RowLists &rl, int sets, int list_idx, const int32_t *hint_riv, const float *h_in, float *h_mid,
+                       float *h_out, float *act) {
+    const river_config &g = c->cfg;
+    const int d = g.d, qdim = g.Hq * g.dh;
+    const double w4f = 0.25 + 2.0 / g.group;  // bytes of a 4-bit copy relative to bf16: (1/2 + 4/G) / 2
+    const river_layer_weights &w = c->layers[l - 1];
+    cudaError_t err = cudaSuccess;
+    auto note = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
+    auto bytes_act = [&](double wb) { return list_idx >= 0 ? wb : (sets & 1 ? wb : 0.0) + (sets & 2 ? wb * w4f : 0.0); };
+    const int has_river = sets & 2 ? 1 : 0;
+    // With more rows than one CUDA-core pass takes, the rows go to the tensor-core GEMMs; the stream kernel serves what they do not.
+    // (Exit layers alone, the end of a long prefill pass: on the GEMM however few the rows are, since its activations keep 22 bits
+    // as those of the pass do, the stream kernel's 15.)
+    const bool tc = c->tc_ok && n <= c->tc_max_pad && (n >= 5 || sets == 2);
+    const river_ctx::LayerMaps *tm = tc ? &c->tc_maps[l - 1] : nullptr;
+    const river_ctx::LayerMaps *wm = (tc && c->w4tc_ok && has_river) ? &c->w4_maps[l - 1] : nullptr;
+    const int skip_bb = tc || !(sets & 1) ? 1 : 0;
+    auto pair = [&](const ProjIn &in, int K, int rows, const RowLists &lists, auto &&backbone, auto &&river, bool operand_ready = false) {
+        if (!(sets & 1)) return wm ? river(operand_ready ? kTcGemm : kTcBoth, false) : cudaSuccess;
+        return tc_pair(c, wm != nullptr, in, K, rows, lists, backbone, river, operand_ready);
+    };
+    // ---- a4: O projection + residual
+    {
+        const double wb = 2.0 * qdim * d;
+        LaunchScope ls(c, K_OPROJ, bytes_act(wb), wb * w4f, list_idx);
+        ResidProblem p{};
+        p.w = (const uint16_t *)w.wo; p.rw = w4_of(w.ro); p.K = qdim; p.out_dim = d; p.group = g.group;
+        p.resid = h_in; p.out = h_mid;
+        const ProjIn in{c->obuf, nullptr, 0.f};
+        if (tc) {
+            const TcResidEpi e{h_in, h_mid, d};
+            const CUtensorMap *const cm[3] = {wm ? &wm->o : nullptr, wm ? &wm->o : nullptr, wm ? &wm->o : nullptr};
+            const river_w4 *const cw[3] = {&w.ro, &w.ro, &w.ro};
+            note(pair(in, qdim, n, rl,
+                      [&](int phase, bool late) {
+                          return launch_tc(c, in, tm->o, tm->o, tm->o, qdim, d / kTcBM, n, 0, 0, 0, rl.act_idx, rl.n_act, e, true,
+                                              rl.hint_act, phase, late);
+                         },
+                      [&](int phase, bool beside) {
+                          return launch_tc_w4(c, in, cm, cw, qdim, d / kTcBM, n, 0, 0, 0, rl.riv_idx, rl.n_riv, hint_riv, e, phase, beside);
+                         }));
+        }
+        if (!wm && (!tc || has_river))
+            note(launch_stream(c, p, in, rl, qdim, d / 2, n, has_river, true, skip_bb, DecideArgs{}));
+    }
+    // ---- a5: FFN norm + gate/up + SwiGLU
+    {
+        const double wb = 2.0 * 2.0 * g.F * d;
+        LaunchScope ls(c, K_GATEUP, bytes_act(wb), wb * w4f, list_idx);
+        GateUpProblem p{};
+        p.wg = (const uint16_t *)w.wg; p.wu = (const uint16_t *)w.wu; p.rg = w4_of(w.rg); p.ru = w4_of(w.ru);
+        p.K = d; p.F = g.F; p.group = g.group; p.act = act;
+        const ProjIn in{h_mid, (const uint16_t *)w.ffn_norm, g.rms_eps};
+        if (tc) {
+            // the epilogues also write the down projection's operand rows (second operand buffers: this
+            // projection's own operand is still being read while they do)
+            const int npad = (n + 15) / 16 * 16;
+            TcGateUpEpi e{act, g.F}, e4{act, g.F};
+            if (const river_ctx::BMap *bd = tc_bmap(c, g.F, npad, false, true)) {
+                e.ohi = reinterpret_cast<uint16_t *>(bd->base); e.olo = reinterpret_cast<uint16_t *>(bd->lo_ptr); e.omode = 1;
+            } else note(cudaErrorInvalidValue);
+            if (wm) {
+                if (const river_ctx::BMap *bd = tc_bmap(c, g.F, npad, true, true)) {
+                    e4.ohi = reinterpret_cast<uint16_t *>(bd->base); e4.olo = reinterpret_cast<uint16_t *>(bd->lo_ptr); e4.omode = 2;
+                } else note(cudaErrorInvalidValue);
+            }
+            const CUtensorMap *const cm[3] = {wm ? &wm->g : nullptr, wm ? &wm->u : nullptr, wm ? &wm->u : nullptr};
+            const river_w4 *const cw[3] = {&w.rg, &w.ru, &w.ru};
+            note(pair(in, d, n, rl,
+                      [&](int phase, bool late) {
+                          return launch_tc(c, in, tm->g, tm->u, tm->u, d, g.F / 64, n, 1, 0, 0, rl.act_idx, rl.n_act, e, true,
+                                              rl.hint_act, phase, late);
+                         },
+                      [&](int phase, bool beside) {
+                          return launch_tc_w4(c, in, cm, cw, d, g.F / 64, n, 1, 0, 0, rl.riv_idx, rl.n_riv, hint_riv, e4, phase, beside);
+                         }));
+        }
+        if (!wm && (!tc || has_river)) note(launch_stream(c, p, in, rl, d, g.F, n, has_river, true, skip_bb, DecideArgs{}));
+    }
+    // ---- a5: down projection + residual
+    {
+        const double wb = 2.0 * g.F * d;
+        LaunchScope ls(c, K_DOWN, bytes_act(wb), wb * w4f, list_idx);
+        ResidProblem p{};
+        p.w = (const uint16_t *)w.wd; p.rw = w4_of(w.rd); p.K = g.F; p.out_dim = d; p.group = g.group;
+        p.resid = h_mid; p.out = h_out;
+        const ProjIn in{act, nullptr, 0.f};
+        if (tc) {
+            const TcResidEpi e{h_mid, h_out, d};
+            const CUtensorMap *const cm[3] = {wm ? &wm->d : nullptr, wm ? &wm->d : nullptr, wm ? &wm->d : nullptr};
+            const river_w4 *const cw[3] = {&w.rd, &w.rd, &w.rd};
+            note(pair(in, g.F, n, rl,
+                      [&](int phase, bool late) {
+                          return launch_tc(c, in, tm->d, tm->d, tm->d, g.F, d / kTcBM, n, 0, 0, 0, rl.act_idx, rl.n_act, e, true,
+                                              rl.hint_act, phase, late, true);
+                         },
+                      [&](int phase, bool beside) {
+                          return launch_tc_w4(c, in, cm, cw, g.F, d / kTcBM, n, 0, 0, 0, rl.riv_idx, rl.n_riv, hint_riv, e, phase, beside, true);
+                         },
+                         true));  // operand rows: written by the gate/up epilogues
+        }
+        if (!wm && (!tc || has_river))
+            note(launch_stream(c, p, in, rl, g.F, d / 2, n, has_river, true, skip_bb, DecideArgs{}));
+    }
+    return err;
+}
+
 // The launch sequence of one step over the rows described in the device metadata (rows, positions, caller buffers).
 //
 // Steps of up to four rows: per block QKV, attention, O, gate/up, down - the exit decision of block l is taken by the
@@ -580,8 +690,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     int32_t *fail_buf = record_fail ? c->prefill_fail : nullptr;
     const int64_t launched = t_launches;
     Lists lists{c->act_idx, c->riv_idx, c->n_act, c->n_riv, B};
-    const int qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
-    const double w4f = 0.25 + 2.0 / g.group;  // bytes of a 4-bit copy relative to bf16: (1/2 + 4/G) / 2
+    const int kvdim = g.Hkv * g.dh;
     double kv_read = 0.0;
     for (int i = 0; i < n; ++i) kv_read += (double)(row_pos_host[i] + 1) * 2.0 * kvdim * 2.0;
     const double kv_write = (double)n * 2.0 * kvdim * 2.0;
@@ -591,7 +700,6 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     // the decisions ride in the QKV kernels - unless the host has to see every decision before it stages a block
     // (offloading) or the rows that left take another route than the 4-bit copies (then: score kernel per block)
     const bool fold = n <= 4 && !c->off_first && strat == RIVER_KV_RIVER;
-    const DecideArgs no_dec{};
 
     {
         LaunchScope ls(c, K_BEGIN, (double)n * d * 2.0, 0, -1);
@@ -621,7 +729,6 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         const river_ctx::LayerMaps *tm = tc ? &c->tc_maps[l - 1] : nullptr;
         const river_ctx::LayerMaps *wm = (tc && c->w4tc_ok && has_river) ? &c->w4_maps[l - 1] : nullptr;
         const int32_t *nrh = c->n_riv + std::max(0, l - 2);  // never above the count entering this block
-        const int skip_bb = tc ? 1 : 0;
         bool staged = false;
         if (c->off_first && l >= c->off_first)
             if (int rc = offload_before_layer(c, l, &staged)) return rc;
@@ -654,89 +761,8 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
             LaunchScope ls(c, K_ATTN, kv_read, 0, -1);
             note(launch_attention(c, n, l - 1));
         }
-        // ---- a4: O projection + residual
-        {
-            const double wb = 2.0 * qdim * d;
-            LaunchScope ls(c, K_OPROJ, wb, wb * w4f, l - 1);
-            ResidProblem p{};
-            p.w = (const uint16_t *)w.wo; p.rw = w4_of(w.ro); p.K = qdim; p.out_dim = d; p.group = g.group;
-            p.resid = h_in; p.out = h_mid;
-            const ProjIn in{c->obuf, nullptr, 0.f};
-            if (tc) {
-                const TcResidEpi e{h_in, h_mid, d};
-                const CUtensorMap *const cm[3] = {wm ? &wm->o : nullptr, wm ? &wm->o : nullptr, wm ? &wm->o : nullptr};
-                const river_w4 *const cw[3] = {&w.ro, &w.ro, &w.ro};
-                note(tc_pair(c, wm != nullptr, in, qdim, n, rl,
-                             [&](int phase, bool late) {
-                                 return launch_tc(c, in, tm->o, tm->o, tm->o, qdim, d / kTcBM, n, 0, 0, 0, ai, na, e, true,
-                                                  c->hint_act, phase, late);
-                             },
-                             [&](int phase, bool beside) {
-                                 return launch_tc_w4(c, in, cm, cw, qdim, d / kTcBM, n, 0, 0, 0, ri, nr, nrh, e, phase, beside);
-                             }));
-            }
-            if (!wm && (!tc || has_river))
-                note(launch_stream(c, p, in, rl, qdim, d / 2, n, has_river, true, skip_bb, no_dec));
-        }
-        // ---- a5: FFN norm + gate/up + SwiGLU
-        {
-            const double wb = 2.0 * 2.0 * g.F * d;
-            LaunchScope ls(c, K_GATEUP, wb, wb * w4f, l - 1);
-            GateUpProblem p{};
-            p.wg = (const uint16_t *)w.wg; p.wu = (const uint16_t *)w.wu; p.rg = w4_of(w.rg); p.ru = w4_of(w.ru);
-            p.K = d; p.F = g.F; p.group = g.group; p.act = c->act;
-            const ProjIn in{h_mid, (const uint16_t *)w.ffn_norm, g.rms_eps};
-            if (tc) {
-                // the epilogues also write the down projection's operand rows (second operand buffers: this
-                // projection's own operand is still being read while they do)
-                const int npad = (n + 15) / 16 * 16;
-                TcGateUpEpi e{c->act, g.F}, e4{c->act, g.F};
-                if (const river_ctx::BMap *bd = tc_bmap(c, g.F, npad, false, true)) {
-                    e.ohi = reinterpret_cast<uint16_t *>(bd->base); e.olo = reinterpret_cast<uint16_t *>(bd->lo_ptr); e.omode = 1;
-                } else note(cudaErrorInvalidValue);
-                if (wm) {
-                    if (const river_ctx::BMap *bd = tc_bmap(c, g.F, npad, true, true)) {
-                        e4.ohi = reinterpret_cast<uint16_t *>(bd->base); e4.olo = reinterpret_cast<uint16_t *>(bd->lo_ptr); e4.omode = 2;
-                    } else note(cudaErrorInvalidValue);
-                }
-                const CUtensorMap *const cm[3] = {wm ? &wm->g : nullptr, wm ? &wm->u : nullptr, wm ? &wm->u : nullptr};
-                const river_w4 *const cw[3] = {&w.rg, &w.ru, &w.ru};
-                note(tc_pair(c, wm != nullptr, in, d, n, rl,
-                             [&](int phase, bool late) {
-                                 return launch_tc(c, in, tm->g, tm->u, tm->u, d, g.F / 64, n, 1, 0, 0, ai, na, e, true,
-                                                  c->hint_act, phase, late);
-                             },
-                             [&](int phase, bool beside) {
-                                 return launch_tc_w4(c, in, cm, cw, d, g.F / 64, n, 1, 0, 0, ri, nr, nrh, e4, phase, beside);
-                             }));
-            }
-            if (!wm && (!tc || has_river)) note(launch_stream(c, p, in, rl, d, g.F, n, has_river, true, skip_bb, no_dec));
-        }
-        // ---- a5: down projection + residual
-        {
-            const double wb = 2.0 * g.F * d;
-            LaunchScope ls(c, K_DOWN, wb, wb * w4f, l - 1);
-            ResidProblem p{};
-            p.w = (const uint16_t *)w.wd; p.rw = w4_of(w.rd); p.K = g.F; p.out_dim = d; p.group = g.group;
-            p.resid = h_mid; p.out = h_out;
-            const ProjIn in{c->act, nullptr, 0.f};
-            if (tc) {
-                const TcResidEpi e{h_mid, h_out, d};
-                const CUtensorMap *const cm[3] = {wm ? &wm->d : nullptr, wm ? &wm->d : nullptr, wm ? &wm->d : nullptr};
-                const river_w4 *const cw[3] = {&w.rd, &w.rd, &w.rd};
-                note(tc_pair(c, wm != nullptr, in, g.F, n, rl,
-                             [&](int phase, bool late) {
-                                 return launch_tc(c, in, tm->d, tm->d, tm->d, g.F, d / kTcBM, n, 0, 0, 0, ai, na, e, true,
-                                                  c->hint_act, phase, late, true);
-                             },
-                             [&](int phase, bool beside) {
-                                 return launch_tc_w4(c, in, cm, cw, g.F, d / kTcBM, n, 0, 0, 0, ri, nr, nrh, e, phase, beside, true);
-                             },
-                             true));  // operand rows: written by the gate/up epilogues
-            }
-            if (!wm && (!tc || has_river))
-                note(launch_stream(c, p, in, rl, g.F, d / 2, n, has_river, true, skip_bb, no_dec));
-        }
+        // ---- a4, a5
+        note(block_tail(c, l, n, rl, 1 | (has_river ? 2 : 0), l - 1, nrh, h_in, h_mid, h_out, c->act));
         // ---- a6 + a7: exit score, decision, compaction -> row lists entering block l+1
         if (!fold) launch_score(l, h_in, h_out);
         if (staged) note(cudaEventRecord(c->off_freed[(l - c->off_first) & 1], c->stream));  // the slot may be refilled
@@ -760,6 +786,12 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     if (c->profiling) return profile_collect(c);
     return 0;
 }
+
+// Prompt ends up to which the last block of a long pass runs behind QKV on the kernels of decode steps, whose K-splits put every SM to
+// work on a few rows: the pair kernel has a pair per 256 features, and every exit-layer matrix is expanded for it first (1B-class,
+// two prompts on the exit layers 2492 us, so 2396; 8B-class, 1024 positions, 8 blocks 6051 -> 5967; mini shape, 5 prompts 592 -> 569).
+// As many as those kernels take in less time than the pair kernel on every shape (tc_long_pass_rows).
+constexpr int kHeadRowsMost = 128;
 
 // The launch sequence of a long prefill pass: more rows than one launch of the batch kernels takes, depths known on the
 // host.  depth[i]: backbone blocks row i runs; so every block's row counts are known here, an empty list launches nothing,
@@ -845,6 +877,12 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
             LaunchScope ls(c, K_PREFILL_ATTN, kv_bytes, 0, -1);
             note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1)
                  : tc_attn ? launch_attention_prefill_tc(c, n_tiles, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
+        }
+        if (heads_only && n_head <= kHeadRowsMost) {  // one list: head[]
+            const RowLists rl{c->head_rows(), c->meta_dev + 2, c->head_rows(), c->meta_dev + 2, c->meta_dev + 2, c->meta_dev, c->state_at(at)};
+            note(block_tail(c, l, n_head, rl, n_of[0] ? 1 : 2, -1, c->meta_dev + 2, h_in, h_mid, h_out, reinterpret_cast<float *>(wide_operand(c, true))));
+            hi = (hi + 2) % 3;
+            break;
         }
         {
             LaunchScope ls(c, K_OPROJ, wsum() * qdim * d, 0, -1);
