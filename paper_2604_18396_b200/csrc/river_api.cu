@@ -226,11 +226,15 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
         return mh[kMetaHdr + c->meta_rows + x] > mh[kMetaHdr + c->meta_rows + y];
     });
     // the small-step kernel: one CTA per (row, kv head, split), chunks in whole pages
+    // of at least 64 positions - its sixteen warps take four each at a time, so shorter ones end no sooner - and no more splits than
+    // that makes: each costs a ticket and a partial, and a context of one split needs no merge.  (The grid is small_attn_splits
+    // whatever the context is: a captured launch keeps it.  Tiny shape, one row, 32 positions, three contexts in flight: 64 splits
+    // of 16 positions 75 us a step, one of 64 61.)
     const int Sc = small_attn_splits(c->num_sms, n, g.Hkv);
     int cchunk = (max_pos + 1 + Sc - 1) / Sc;
-    cchunk = std::max(kPage, (cchunk + kPage - 1) / kPage * kPage);
-    mh[6] = cchunk;  // StepMeta::pad[0]
-    mh[7] = Sc;      // StepMeta::pad[1]
+    cchunk = std::max(4 * kSmallAttnWarps, (cchunk + kPage - 1) / kPage * kPage);
+    mh[6] = cchunk;                               // StepMeta::pad[0]
+    mh[7] = (max_pos + cchunk) / cchunk;          // StepMeta::pad[1]
     // the small-step kernel walks a split in batches of 4 positions per warp without a load pipeline, but requests the
     // cache before the grid dependency resolves: in the replayed step it wins up to four batches per warp (contexts up
     // to ~4.6 K at one row: 3.84 -> 3.49 ms per step at 4 K), beyond that the TMA-fed kernel's staging pays
