@@ -13,9 +13,16 @@ namespace {
 // Launch geometry: warps per CTA and CTAs per SM such that every warp gets the same number of tasks (a task is R
 // weight rows) and at least 16 warps per SM have loads in flight; searched once per (kernel, task count, K).
 struct StreamGeom { int threads, grid; };
+constexpr size_t kLatencyBytes = 16 * 1024;
 
 template <class Kern>
-StreamGeom pick_geometry(river_ctx *c, Kern kern, int tasks, size_t smem) {
+StreamGeom pick_geometry(river_ctx *c, Kern kern, int tasks, size_t smem, int R, int K) {
+    // A projection whose share of an SM is a few KB is latency, not a stream: as many warps as the share has tasks (at least four, and as
+    // many as hold one row in registers, XF pieces a thread), and no CTA without one.  Sixteen
+    // warps on every SM for one task each cost a step of the tiny shape (one row) 61 us with three contexts in flight, these 40.
+    const int share = (tasks + c->num_sms - 1) / c->num_sms, hold = (K + 255) / 256;
+    if (share <= 16 && hold <= 16 && share * 2 * (size_t)R * K <= kLatencyBytes)
+        return StreamGeom{32 * std::max(std::max(4, hold), share), std::min(tasks, c->num_sms)};
     StreamGeom best{256, c->num_sms};
     double best_cost = 1e30;
     int best_w = 0;
@@ -49,7 +56,7 @@ cudaError_t launch_stream_t(river_ctx *c, const P &p, const ProjIn &in, const Ro
     if (!geom) {
         const cudaError_t e = ensure_smem(c, kern, smem);
         if (e != cudaSuccess) return e;
-        const StreamGeom g = pick_geometry(c, kern, tasks, smem);
+        const StreamGeom g = pick_geometry(c, kern, tasks, smem, R, K);
         c->geoms.push_back({fn, tasks, K, g.threads, g.grid});
         geom = &c->geoms.back();
     }
