@@ -13,16 +13,16 @@ namespace {
 // Launch geometry: warps per CTA and CTAs per SM such that every warp gets the same number of tasks (a task is R
 // weight rows) and at least 16 warps per SM have loads in flight; searched once per (kernel, task count, K).
 struct StreamGeom { int threads, grid; };
-constexpr size_t kLatencyBytes = 16 * 1024;
 
 template <class Kern>
 StreamGeom pick_geometry(river_ctx *c, Kern kern, int tasks, size_t smem, int R, int K) {
-    // A projection whose share of an SM is a few KB is latency, not a stream: as many warps as the share has tasks (at least four, and as
-    // many as hold one row in registers, XF pieces a thread), and no CTA without one.  Sixteen
-    // warps on every SM for one task each cost a step of the tiny shape (one row) 61 us with three contexts in flight, these 40.
-    const int share = (tasks + c->num_sms - 1) / c->num_sms, hold = (K + 255) / 256;
-    if (share <= 16 && hold <= 16 && share * 2 * (size_t)R * K <= kLatencyBytes)
-        return StreamGeom{32 * std::max(std::max(4, hold), share), std::min(tasks, c->num_sms)};
+    // Where an SM's share is a task for each of its warps at most: as many warps as tasks (at least four, and as many as hold one row
+    // in registers, XF pieces a thread), and no CTA without a task.  The other warps, of sixteen, would have nothing to stream, but
+    // stage the row and wait for each other with the rest, and keep the registers from whatever runs beside this grid.  Three
+    // contexts in flight, us a step, sixteen warps everywhere against this: tiny shape, one row 61 / 40; mini 133 / 67; 1B-class, 4
+    // blocks, three rows 280 / 238; one context by itself 2-10 % less or the same.
+    const int share = (tasks + c->num_sms - 1) / c->num_sms, hold = (K + 127) / 128 / (R == 2 ? 4 : 2);
+    if (share <= 16 && hold <= 16) return StreamGeom{32 * std::max(std::max(4, hold), share), std::min(tasks, c->num_sms)};
     StreamGeom best{256, c->num_sms};
     double best_cost = 1e30;
     int best_w = 0;
@@ -104,11 +104,13 @@ cudaError_t launch_head_stream(river_ctx *c, const HeadArgs &a, int n_head) {
     const int n_sel = std::min(n_head, 4);
     const int xstride = xs_stride(a.d, 8);
     const size_t smem = sizeof(float) * (64 + (size_t)n_sel * xstride);
+    const int share = (a.V / (n_sel == 1 ? 2 : 4) + c->head_grid - 1) / c->head_grid;  // (as pick_geometry)
+    const int threads = std::min(head_threads(n_sel), 32 * std::max(4, share));
 #define HEAD_CASE(N_, R_)                                                                                          \
     if (n_sel == N_) {                                                                                             \
         const cudaError_t e = ensure_smem(c, lm_head_kernel<N_, R_>, smem);                                        \
         if (e != cudaSuccess) return e;                                                                            \
-        return launch_k(lm_head_kernel<N_, R_>, dim3(c->head_grid), dim3(head_threads(N_)), smem, c->stream, true, a, xstride); \
+        return launch_k(lm_head_kernel<N_, R_>, dim3(c->head_grid), dim3(threads), smem, c->stream, true, a, xstride); \
     }
     HEAD_CASE(1, 2) HEAD_CASE(2, 4) HEAD_CASE(3, 4) HEAD_CASE(4, 4)
 #undef HEAD_CASE
