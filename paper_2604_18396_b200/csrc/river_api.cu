@@ -573,7 +573,7 @@ cudaError_t launch_head(river_ctx *c, const float *h, int n_head, const float *p
 
 // What follows attention in block l (a4, a5: O, gate/up and down projections, with their residuals) for the rows of `rl`, n at most,
 // on the kernels of decode steps.  sets: 1 = the backbone's rows, 2 = the exit layers', 3 = both.  list_idx: the list whose counts
-// say which weights were read (timing), -1: all of `sets`.  hint_riv: a count that is never below the exit layers' rows.
+// say which weights were read (timing), -1: all of `sets`.  hint_riv: a count that is never above the exit layers' rows.
 cudaError_t block_tail(river_ctx *c, int l, int n, const RowLists &rl, int sets, int list_idx, const int32_t *hint_riv, const float *h_in, float *h_mid,
                        float *h_out, float *act) {
     const river_config &g = c->cfg;
