@@ -52,7 +52,9 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
     TcArgs a{};
     a.K = K; a.n_pad = np; a.one_box = bm->one ? 1 : 0; a.late_release = late_release ? 1 : 0;
     const size_t stage = tc_stage_bytes(np);
-    const TcPlan plan = tc_plan(c->num_sms, np, tiles, K, allow_split, c->rows_distinct);
+    const int most = c->short_sums ? tc_wide_segment(c->num_sms, c->cfg.max_batch, tiles, K, false) : 0;
+    const TcPlan plan = tc_plan(c->num_sms, np, tiles, K, allow_split, c->rows_distinct, most);
+    if (!plan.splits) return cudaErrorInvalidValue;
     const int occ = plan.occ;
     a.splits = plan.splits; a.halves = plan.halves;
     a.n_stages = tc_stages_at(np, occ);

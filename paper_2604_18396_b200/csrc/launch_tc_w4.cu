@@ -38,7 +38,9 @@ cudaError_t launch_tc_w4(river_ctx *c, const ProjIn &in, const CUtensorMap *cons
     TcW4Args a{};
     a.K = K; a.n_pad = np; a.one_box = bm->one ? 1 : 0;
     const size_t stage = 2 * (size_t)np * kTcBK * 2, raw = (size_t)kW4RawBufs * kW4RawBytes;
-    const W4Plan plan = w4_plan(c->num_sms, np, tiles, K, c->rows_distinct);
+    const int most = c->short_sums ? tc_wide_segment(c->num_sms, c->cfg.max_batch, tiles, K, true) : 0;
+    const W4Plan plan = w4_plan(c->num_sms, np, tiles, K, c->rows_distinct, most);
+    if (!plan.splits) return cudaErrorInvalidValue;
     a.n_stages = plan.n_stages; a.splits = plan.splits; a.wide = plan.wide; a.sets = plan.sets;
     if (sizeof(float) * (size_t)np * kTcLd > (size_t)a.n_stages * stage + raw) return cudaErrorInvalidValue;
     // tensor memory: accumulators + A tiles, a power of two of columns; every CTA that can be resident on an SM must get

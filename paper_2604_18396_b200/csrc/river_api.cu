@@ -791,12 +791,6 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     return 0;
 }
 
-// Prompt ends up to which the last block of a long pass runs behind QKV on the kernels of decode steps, whose K-splits put every SM to
-// work on a few rows: the pair kernel has a pair per 256 features, and every exit-layer matrix is expanded for it first (1B-class,
-// two prompts on the exit layers 2492 us, so 2396; 8B-class, 1024 positions, 8 blocks 6051 -> 5967; mini shape, 5 prompts 592 -> 569).
-// As many as those kernels take in less time than the pair kernel on every shape (tc_long_pass_rows).
-constexpr int kHeadRowsMost = 128;
-
 // The launch sequence of a long prefill pass: more rows than one launch of the batch kernels takes, depths known on the
 // host.  depth[i]: backbone blocks row i runs; so every block's row counts are known here, an empty list launches nothing,
 // and the score / compaction kernel runs only after a block some row leaves at (or, record_fail, after every block: the
@@ -882,9 +876,11 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
             note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1)
                  : tc_attn ? launch_attention_prefill_tc(c, n_tiles, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
         }
-        if (heads_only && n_head <= kHeadRowsMost) {  // one list: head[]
+        if (heads_only && tc_ends_fit(c->num_sms, g.max_batch, n_head, d, qdim, F, !n_of[0])) {  // one list: head[]
+            c->short_sums = true;
             const RowLists rl{c->head_rows(), c->meta_dev + 2, c->head_rows(), c->meta_dev + 2, c->meta_dev + 2, c->meta_dev, c->state_at(at)};
             note(block_tail(c, l, n_head, rl, n_of[0] ? 1 : 2, -1, c->meta_dev + 2, h_in, h_mid, h_out, reinterpret_cast<float *>(wide_operand(c, true))));
+            c->short_sums = false;
             hi = (hi + 2) % 3;
             break;
         }

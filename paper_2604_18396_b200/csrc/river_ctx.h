@@ -66,6 +66,7 @@ struct river_ctx {
     int32_t *slot_cap = nullptr;  // [max_seqs] Mono-Decreasing Exit: the depth the sequence's last token reached
     bool prefill_attn_now = false;  // this chunk's attention runs on the tensor-core prefill kernel
     bool rows_distinct = true;  // every row of the current step is a different sequence (decode), not a prefill chunk
+    bool short_sums = false;    // the batch kernels' projections under way sum no more inputs at a time than a long pass's (tc_wide_segment)
     struct GraphEntry { int n; bool small_attn; int attn_splits; cudaGraphExec_t exec; int launches; };
     std::vector<GraphEntry> graphs;
     double *inv_freq;

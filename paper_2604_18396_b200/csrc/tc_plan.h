@@ -15,6 +15,7 @@ constexpr uint32_t kW4RawBytes = kTcBM * 128;  // one raw code tile
 constexpr uint32_t kW4ACols = kTcBK / 2;       // TMEM columns of one A tile: 64 f16 per row, two per column
 
 constexpr size_t kSmSmem = 228 * 1024;
+constexpr int kTcMostSplits = 8;   // CTAs of a cluster
 constexpr int kTcHalvesRows = 64;  // operand rows up to which two CTAs' double accumulators (4 np columns each) share an SM
 constexpr size_t kCtaFixed = 1024 + 1024 + 256;  // per CTA: system reserve, alignment slack, barriers
 
@@ -25,7 +26,7 @@ inline int tc_pick_splits(int num_sms, int tiles, int kb_total, int slots, int m
     int best = 1;
     double best_eff = 0.0;
     if (tiles >= num_sms) return 1;  // every SM has a tile of its own: splitting only adds reductions
-    for (int s = 1; s <= 8; ++s) {  // a cluster holds at most 8 CTAs
+    for (int s = 1; s <= kTcMostSplits; ++s) {
         if (s > 1 && kb_total / s < min_kb) break;
         const int ctas = tiles * s, waves = (ctas + slots - 1) / slots;
         const double eff = (double)ctas / ((double)waves * slots);
@@ -50,9 +51,10 @@ inline int tc_cols(int np, int occ, int *wide) {
     return cols;
 }
 
-// tc_gemm_kernel: CTAs per SM and K-splits.  `decode`: the rows are a decode step's (not a prefill pass's).
+// tc_gemm_kernel: CTAs per SM and K-splits.  `decode`: the rows are a decode step's (not a prefill pass's).  `most_kb`: the most
+// k-blocks that one accumulator may sum (0: as many as it comes to); 0 splits: no plan keeps to it.
 struct TcPlan { int occ, splits, halves; };
-inline TcPlan tc_plan(int num_sms, int np, int tiles, int K, bool allow_split, bool decode) {
+inline TcPlan tc_plan(int num_sms, int np, int tiles, int K, bool allow_split, bool decode, int most_kb = 0) {
     TcPlan p{};
     // CTAs per SM: two with three stages each, or three with two when that puts more CTAs of one wave to work (while
     // one CTA drains its accumulator and takes part in the cluster reduction the others keep the weight stream going);
@@ -74,13 +76,22 @@ inline TcPlan tc_plan(int num_sms, int np, int tiles, int K, bool allow_split, b
         if (s1 >= 2 && K / kTcBK / s1 >= 12) { p.splits = s1; p.occ = 2; p.halves = 1; }
     }
     if (!allow_split) p.splits = 1;
+    // A bound on the sums: two accumulators where they fit, and then as few splits as keep to it - more of them, in whole waves of
+    // CTAs, only add reductions (one 8B-class block's pass that ends on 5 rows: gate/up in 2 splits 268 us, in 5 278).
+    const int kb = K / kTcBK;
+    if (most_kb && ((kb + p.splits - 1) / p.splits + p.halves) / (1 + p.halves) > most_kb) {
+        p.occ = tc_stages_at(np, 2) ? 2 : 1;
+        p.halves = p.occ == 2 && np <= kTcHalvesRows ? 1 : 0;
+        p.splits = std::max(p.splits, (kb - 1) / (most_kb << p.halves) + 1);
+        if (p.splits > kTcMostSplits) p.splits = 0;
+    }
     return p;
 }
 
 // tc_gemm_w4_kernel: stages (an even number: the two dequantisation warps of a lane quarter alternate), CTAs per SM, K-splits
-// in whole raw tiles, accumulators.  hi | lo as one operand (`wide`) as above.
+// in whole raw tiles, accumulators.  hi | lo as one operand (`wide`) and `most_kb` as above.
 struct W4Plan { int occ, n_stages, splits, wide, sets, cols; };  // cols: tensor-memory columns per CTA (occ * cols > 512: does not fit)
-inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode) {
+inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode, int most_kb = 0) {
     W4Plan p{};
     const size_t stage = 2 * (size_t)np * kTcBK * 2;  // the activations' hi and lo tiles; the A tiles are in tensor memory
     const size_t raw = (size_t)kW4RawBufs * kW4RawBytes;
@@ -112,6 +123,12 @@ inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode) {
             p.sets = 2;
         }
     }
+    if (most_kb && (raw_tiles + p.splits - 1) / p.splits * kW4Super > most_kb * p.sets) {  // (as in tc_plan)
+        p.sets = p.wide && p.occ * cols_for(4 * np) <= 512 ? 2 : 1;
+        const int most_raw = most_kb * p.sets / kW4Super;
+        p.splits = most_raw ? std::max(p.splits, (raw_tiles - 1) / most_raw + 1) : 0;
+        if (p.splits > kTcMostSplits) p.splits = 0;
+    }
     p.cols = cols_for(p.sets * (p.wide ? 2 * np : np));
     return p;
 }
@@ -132,6 +149,32 @@ inline int tc_wide_segment(int num_sms, int pass_rows, int tiles, int K, bool f1
         run = (kb + splits - 1) / splits;
     }
     return std::min(K >= 4096 ? 16 : 8, run);
+}
+
+// Whether the last block of a long pass runs behind QKV (O, gate / up, down; f16: on the exit layers) on the kernels of decode steps,
+// for `ends` prompt ends.  Those put every SM to work on a few rows, by K-splits, where the pair kernel has a pair per 256 features
+// and every exit-layer matrix is expanded for it first; their time grows with the rows sooner.  And only where every sum inside the
+// tensor cores stays as short as the pair kernel's (up to four rows on the backbone never enter them): with the batch kernels' own
+// plans the logits of 20 ends behind one 8B-class block are 1.04e-5 from 64-bit arithmetic (8.4e-6 on the exit layers), on the pair
+// kernel 9.9e-6 (7.6e-6), with this bound 9.6e-6 (7.2e-6).  Passes of 512 positions through one block, us, pair kernel / so:
+//   ends             5         16        32        48        64        96
+//   8B   backbone  383/268   384/268   387/276   394/296   407/316   (down: 224 k-blocks, 8 splits x 2 accumulators x 16 up to 64 rows)
+//        exit      566/298   565/299   573/309   (two accumulators up to 32 rows)
+//   3072 backbone  271/198   271/198   275/207   284/223   293/237   317/316
+//        exit      357/224   357/224   362/237   370/258   380/274   406/314
+//   1B   backbone  242/168   241/167   244/176   250/193   258/203   277/272   (128: 293/309)
+//        exit      288/179   286/177   292/184   299/204   309/218   328/242
+//   mini backbone  133/108   132/110   139/116   150/126   149/134   159/153   (128: 170/172)
+//        exit      144/122   147/124   151/132   164/137   162/145   172/162
+constexpr int kTcEndsMost = 96;
+inline bool tc_ends_fit(int num_sms, int pass_rows, int ends, int d, int qdim, int F, bool f16) {
+    if (ends <= 4 && !f16) return true;
+    const int np = (ends + 15) / 16 * 16, shapes[3][2] = {{d / kTcBM, qdim}, {F / 64, d}, {d / kTcBM, F}};
+    for (const auto &[tiles, K] : shapes) {
+        const int most = tc_wide_segment(num_sms, pass_rows, tiles, K, f16);
+        if (!(f16 ? w4_plan(num_sms, np, tiles, K, false, most).splits : tc_plan(num_sms, np, tiles, K, true, false, most).splits)) return false;
+    }
+    return ends <= kTcEndsMost;
 }
 
 // Rows from which a prefill pass that the batch kernels could take as well (up to `max_rows` rows, 256 at most) is a long one.
