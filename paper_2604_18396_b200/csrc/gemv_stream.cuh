@@ -13,6 +13,7 @@
 #include <type_traits>
 
 #include "river_common.cuh"
+#include "stream_plan.h"
 
 namespace river {
 
@@ -818,7 +819,7 @@ __global__ void __launch_bounds__(512) stream_proj_kernel(const P p, const ProjI
         }
     }
     // Per-step constants of the decision and the norm gain, fetched before the wait.
-    constexpr int XF = R == 2 ? 4 : 2;  // 128-bit pieces of a row a thread keeps in registers (one-row steps)
+    constexpr int XF = kStreamPieces<R>;  // 128-bit pieces of a row a thread keeps in registers (one-row steps)
     const int nv = K >> 2, tid = threadIdx.x, nthr = blockDim.x;
     const int n = *rl.n_rows;
     const bool small = n <= N;       // the whole step in one pass: lists come from the exit flags

@@ -5,24 +5,18 @@
 #include <type_traits>
 
 #include "launch.h"
+#include "stream_plan.h"
 
 namespace river {
 
 namespace {
 
-// Launch geometry: warps per CTA and CTAs per SM such that every warp gets the same number of tasks (a task is R
-// weight rows) and at least 16 warps per SM have loads in flight; searched once per (kernel, task count, K).
-struct StreamGeom { int threads, grid; };
-
+// Launch geometry: stream_small_share's where it applies; else warps per CTA and CTAs per SM such that every warp gets the same
+// number of tasks (a task is R weight rows) and at least 16 warps per SM have loads in flight.  Chosen once per (kernel, task count, K).
 template <class Kern>
 StreamGeom pick_geometry(river_ctx *c, Kern kern, int tasks, size_t smem, int R, int K) {
-    // Where an SM's share is a task for each of its warps at most: as many warps as tasks (at least four, and as many as hold one row
-    // in registers, XF pieces a thread), and no CTA without a task.  The other warps, of sixteen, would have nothing to stream, but
-    // stage the row and wait for each other with the rest, and keep the registers from whatever runs beside this grid.  Three
-    // contexts in flight, us a step, sixteen warps everywhere against this: tiny shape, one row 61 / 40; mini 133 / 67; 1B-class, 4
-    // blocks, three rows 280 / 238; one context by itself 2-10 % less or the same.
-    const int share = (tasks + c->num_sms - 1) / c->num_sms, hold = (K + 127) / 128 / (R == 2 ? 4 : 2);
-    if (share <= 16 && hold <= 16) return StreamGeom{32 * std::max(std::max(4, hold), share), std::min(tasks, c->num_sms)};
+    StreamGeom small;
+    if (stream_small_share(c->num_sms, tasks, K, R, small)) return small;
     StreamGeom best{256, c->num_sms};
     double best_cost = 1e30;
     int best_w = 0;
