@@ -12,11 +12,12 @@ namespace river {
 namespace {
 
 // Launch geometry: stream_small_share's where it applies; else warps per CTA and CTAs per SM such that every warp gets the same
-// number of tasks (a task is R weight rows) and at least 16 warps per SM have loads in flight.  Chosen once per (kernel, task count, K).
+// number of tasks (a task is R weight rows) and at least 16 warps per SM have loads in flight.  Chosen once per (kernel, task count, K, whether
+// the rows are few).
 template <class Kern>
-StreamGeom pick_geometry(river_ctx *c, Kern kern, int tasks, size_t smem, int R, int K) {
+StreamGeom pick_geometry(river_ctx *c, Kern kern, int rows, int tasks, size_t smem, int R, int K) {
     StreamGeom small;
-    if (stream_small_share(c->num_sms, tasks, K, R, small)) return small;
+    if (stream_small_share(c->num_sms, rows, tasks, K, R, small)) return small;
     StreamGeom best{256, c->num_sms};
     double best_cost = 1e30;
     int best_w = 0;
@@ -39,19 +40,20 @@ StreamGeom pick_geometry(river_ctx *c, Kern kern, int tasks, size_t smem, int R,
 }
 
 template <class P, int N, int R>
-cudaError_t launch_stream_t(river_ctx *c, const P &p, const ProjIn &in, const RowLists &rl, int K, int tasks,
+cudaError_t launch_stream_t(river_ctx *c, const P &p, const ProjIn &in, const RowLists &rl, int K, int tasks, int n,
                             int has_river, bool pdl, int skip_backbone, const DecideArgs &dec) {
     const size_t smem = stream_smem_bytes(N, K);
     auto kern = stream_proj_kernel<P, N, R>;
     const void *fn = reinterpret_cast<const void *>(kern);
     const river_ctx::Geom *geom = nullptr;
+    const bool few = n <= kStreamFewRows;
     for (auto &e : c->geoms)
-        if (e.fn == fn && e.tasks == tasks && e.K == K) geom = &e;
+        if (e.fn == fn && e.tasks == tasks && e.K == K && e.few == few) geom = &e;
     if (!geom) {
         const cudaError_t e = ensure_smem(c, kern, smem);
         if (e != cudaSuccess) return e;
-        const StreamGeom g = pick_geometry(c, kern, tasks, smem, R, K);
-        c->geoms.push_back({fn, tasks, K, g.threads, g.grid});
+        const StreamGeom g = pick_geometry(c, kern, n, tasks, smem, R, K);
+        c->geoms.push_back({fn, tasks, K, few, g.threads, g.grid});
         geom = &c->geoms.back();
     }
     return launch_k(kern, dim3(geom->grid), dim3(geom->threads), smem, c->stream, pdl, p, in, rl, has_river,
@@ -84,7 +86,7 @@ cudaError_t launch_stream(river_ctx *c, const P &p, const ProjIn &in, const RowL
     while (n_sel < n && n_sel < 4 && stream_smem_bytes(n_sel + 1, K) <= 200 * 1024) ++n_sel;
     const int r = K >= 4096 ? 2 : 4;  // weight rows per task
     const int tasks = tasks_r2 * 2 / r;
-#define STREAM_CASE(N_, R_) if (n_sel == N_ && r == R_) return launch_stream_t<P, N_, R_>(c, p, in, rl, K, tasks, has_river, pdl, skip_backbone, dec);
+#define STREAM_CASE(N_, R_) if (n_sel == N_ && r == R_) return launch_stream_t<P, N_, R_>(c, p, in, rl, K, tasks, n, has_river, pdl, skip_backbone, dec);
     STREAM_CASE(1, 2) STREAM_CASE(2, 2) STREAM_CASE(3, 2) STREAM_CASE(4, 2)
     STREAM_CASE(1, 4) STREAM_CASE(2, 4) STREAM_CASE(3, 4) STREAM_CASE(4, 4)
 #undef STREAM_CASE

@@ -103,10 +103,10 @@ struct river_ctx {
     int off_slot_layer[2] = {-1, -1};
 
     // per-context launch bookkeeping: the dynamic shared memory limit of every kernel that was set up, and the launch geometry
-    // of the streaming kernels per (kernel, task count, K)
+    // of the streaming kernels per (kernel, task count, K, up to four rows or more)
     struct SmemAttr { const void *fn; size_t bytes; };
     std::vector<SmemAttr> smem_attr;
-    struct Geom { const void *fn; int tasks, K, threads, grid; };
+    struct Geom { const void *fn; int tasks, K; bool few; int threads, grid; };
     std::vector<Geom> geoms;
 
     // optional per-kernel timing (river_profile): events around every launch of a step

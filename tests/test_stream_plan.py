@@ -8,9 +8,9 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SHIM = r"""
 #include "stream_plan.h"
-extern "C" int small(int sms, int tasks, int K, int R, int *o) {
+extern "C" int small(int sms, int rows, int tasks, int K, int R, int *o) {
     river::StreamGeom g{0, 0};
-    const bool is = river::stream_small_share(sms, tasks, K, R, g);
+    const bool is = river::stream_small_share(sms, rows, tasks, K, R, g);
     o[0] = g.threads; o[1] = g.grid; o[2] = R == 2 ? river::kStreamPieces<2> : river::kStreamPieces<4>;
     return is ? 1 : 0;
 }
@@ -34,10 +34,16 @@ def test_the_warps_hold_a_row(plan, tasks, R, K_from, K_to):
     o = (ctypes.c_int * 3)()
     share = -(-tasks // SMS)
     for K in range(K_from, K_to, 32):
-        is_small = plan.small(SMS, tasks, K, R, o)
+        is_small = plan.small(SMS, 1, tasks, K, R, o)
         assert bool(is_small) == (share <= 16)
         if is_small:
             threads, grid, pieces = o
             assert threads * pieces * 4 >= K, K
             assert grid == min(tasks, SMS) and threads % 32 == 0 and max(128, 32 * share) <= threads <= 512
             assert threads <= 32 * max(4, share) or (threads - 32) * pieces * 4 < K  # and no warp more than that
+
+
+def test_only_steps_of_few_rows(plan):
+    """More rows than one pass takes keep the geometry whose warps all stage."""
+    o = (ctypes.c_int * 3)()
+    assert [plan.small(SMS, n, 148, 512, 4, o) for n in (1, 2, 3, 4, 5, 8, 64, 256, 1024)] == [1, 1, 1, 1, 0, 0, 0, 0, 0]
