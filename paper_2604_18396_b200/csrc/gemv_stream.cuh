@@ -969,11 +969,14 @@ __global__ void __launch_bounds__(512) stream_proj_kernel(const P p, const ProjI
 // ---------------------------------------------------------------- a8: final norm + LM head + argmax partials
 // logits = W_lm . RMSNorm(h) for the rows that need them (all rows of a decode step; the last prompt position in
 // prefill), written as fp32 if the caller gave a buffer, and the greedy next token: every CTA keeps the best
-// (value, id) of its share of the vocabulary (ties -> lowest id), and the CTA that finishes last (atomic ticket, no spinning)
-// merges them.  In decode steps it also notes the last block's score - a diagnostic: no exit is taken there - and the final row
-// lists.  (Two launches fewer a step than with small kernels behind this one.)
+// (value, id) of its share of the vocabulary (ties -> lowest id), and for up to kHeadMergeRows rows the CTA that finishes last
+// (atomic ticket, no spinning) merges them; more rows are merged by argmax_final_kernel, a CTA each (by the last CTA, one row after
+// the other, a step of 1000 rows through two mini blocks took 17650 us, so 16570).  In decode steps it also notes the last block's
+// score - a diagnostic: no exit is taken there - and the final row lists.  (Two launches fewer a step than with small kernels behind
+// this one.)
+constexpr int kHeadMergeRows = 4;
 struct HeadEnd {
-    unsigned *ticket;                // zero between launches
+    unsigned *ticket;                // zero between launches; null: the last CTA does nothing
     unsigned long long *exit_hist;   // decode steps (else null): [L + 1] counters of the exit layers taken so far
     const float *h_prev;             // decode steps (else null): input of block L, fp32 [rows][d]
     const uint8_t *state_in;         // exit flags entering block L, and behind it
@@ -1114,6 +1117,7 @@ __global__ void __launch_bounds__(head_threads(N)) lm_head_kernel(const HeadArgs
     }
     // ---- the last CTA: the greedy tokens of all rows, the last block's scores, the final lists
     const HeadEnd &f = a.end;
+    if (!f.ticket) return;
     __shared__ bool s_last;
     __threadfence();
     __syncthreads();

@@ -100,8 +100,9 @@ cudaError_t launch_head_stream(river_ctx *c, const HeadArgs &a, int n_head) {
     const int n_sel = std::min(n_head, 4);
     const int xstride = xs_stride(a.d, 8);
     const size_t smem = sizeof(float) * (64 + (size_t)n_sel * xstride);
-    const int share = (a.V / (n_sel == 1 ? 2 : 4) + c->head_grid - 1) / c->head_grid;  // (as pick_geometry)
-    const int threads = std::min(head_threads(n_sel), 32 * std::max(4, share));
+    const int share = (a.V / (n_sel == 1 ? 2 : 4) + c->head_grid - 1) / c->head_grid;
+    const int few = n_head <= kStreamFewRows ? std::max(4, share) : 16;  // (as stream_small_share)
+    const int threads = std::min(head_threads(n_sel), 32 * few);
 #define HEAD_CASE(N_, R_)                                                                                          \
     if (n_sel == N_) {                                                                                             \
         const cudaError_t e = ensure_smem(c, lm_head_kernel<N_, R_>, smem);                                        \

@@ -552,6 +552,9 @@ cudaError_t launch_head(river_ctx *c, const float *h, int n_head, const float *p
         TcHeadEpi e{c->meta(), g.V, c->part_val, c->part_idx, n_parts};
         note(launch_tc(c, a.in, c->tc_map_head, c->tc_map_head, c->tc_map_head, d, n_parts, n_head, 0, 0, 0,
                        c->head_rows(), c->meta_dev + 2 /* StepMeta::n_head_rows */, e, false, nullptr));
+    } else if (n_head > kHeadMergeRows) {
+        LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
+        note(launch_head_stream(c, a, n_head));
     } else {
         LaunchScope ls(c, K_HEAD, 2.0 * g.V * d + 4.0 * n_head * g.V, 0, -1);
         a.end.ticket = c->tickets + 2;
