@@ -1026,7 +1026,7 @@ __global__ void __launch_bounds__(head_threads(N)) lm_head_kernel(const HeadArgs
     float *xs = stream_smem + 64;
     __shared__ float s_val[head_threads(N) / 32][N];
     __shared__ int s_idx[head_threads(N) / 32][N];
-    constexpr bool PIPE = N * R <= 2;
+    constexpr bool PIPE = N * R <= 2;  // (one head row: one pass)
     const int K = a.d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     pdl_launch();
@@ -1053,12 +1053,6 @@ __global__ void __launch_bounds__(head_threads(N)) lm_head_kernel(const HeadArgs
 #pragma unroll
         for (int n = 0; n < N; ++n) { best[n] = -CUDART_INF_F; besti[n] = 0x7fffffff; }
         const int nch = K >> 3, nit = (nch + 31) >> 5;
-        if (PIPE && i0 > 0 && t0 + warp < t1) {
-            const uint16_t *rows[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) rows[r] = a.w + ((size_t)(t0 + warp) * R + r) * K;
-            stream_issue_bf16<R>(rows, nch, 0, lane, pre);
-        }
         for (int t = t0 + warp; t < t1; t += nwarps) {
             const size_t o0 = (size_t)t * R;
             const uint16_t *rows[R];

@@ -78,7 +78,7 @@ const char *check_config(const river_config *c) {
     return nullptr;
 }
 
-int head_grid_for(const river_config *c) { return 148 * 2 > c->V / 4 ? std::max(1, c->V / 4) : 148 * 2; }
+int head_grid_for(const river_config *c) { return std::max(1, std::min(148, c->V / 4)); }  // one CTA fits an SM
 int head_parts_for(const river_config *c) { return std::max(head_grid_for(c), c->V / 128 + 1); }  // argmax partials per row
 
 // Row-indexed buffers are sized for the larger of a decode step and a prefill chunk; the logits staging only for the
@@ -730,11 +730,6 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         const int32_t *na = c->n_act + (l - 1), *nr = c->n_riv + (l - 1);
         const RowLists rl{ai, na, ri, nr, c->hint_act, c->meta_dev /* StepMeta::n_rows */, c->state_at(l - 1)};
         float *h_in = c->h[hi], *h_mid = c->h[(hi + 1) % 3], *h_out = c->h[(hi + 2) % 3];
-        // With more rows than one CUDA-core pass takes, the backbone rows go to the tensor-core GEMM and the stream
-        // kernel only serves the exit-layer rows of the same launch slot.
-        const bool tc = c->tc_ok && n >= 5 && n <= c->tc_max_pad;
-        const river_ctx::LayerMaps *tm = tc ? &c->tc_maps[l - 1] : nullptr;
-        const river_ctx::LayerMaps *wm = (tc && c->w4tc_ok && has_river) ? &c->w4_maps[l - 1] : nullptr;
         const int32_t *nrh = c->n_riv + std::max(0, l - 2);  // never above the count entering this block
         bool staged = false;
         if (c->off_first && l >= c->off_first)
@@ -1168,7 +1163,7 @@ int river_init(const river_config *cfg, const river_weights *w, void *kv_pool, s
         return bail("cudaDeviceGetAttribute failed");
     if (cc_major != 10) return bail("this library is built for sm_100a (B200) only");
     c->device = dev;
-    c->head_grid = std::min(c->head_grid, c->num_sms);  // (one CTA fits an SM)
+    c->head_grid = std::min(c->head_grid, c->num_sms);
     if (make_kv_tensor_map(c)) { river_destroy(c); return RIVER_E_DEVICE; }
     c->tc_ok = !(cfg->flags & RIVER_F_NO_TC) && tc_shape_ok(*cfg) && make_tc_maps(c);
     c->w4tc_ok = c->tc_ok && !(cfg->flags & RIVER_F_NO_W4TC) && make_w4_maps(c);
