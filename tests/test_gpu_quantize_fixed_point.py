@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("group", [32, 64, 128])
-@pytest.mark.parametrize("iters,std", [(1, 0.02), (3, 0.02), (60, 0.02), (300, 0.02), (60, 0.2), (300, 0.2)])
+@pytest.mark.parametrize("iters,std", [(1, 0.02), (3, 0.02), (60, 0.02), (300, 0.02), (60, 0.2), (300, 0.2), (5, 4.0), (20, 1.0)])
 def test_as_if_every_round_had_run(group, iters, std):
     from paper_2604_18396_b200 import binding
     w = synth.normal(31, group + iters, (67, group * 3), std, "cuda").bfloat16().contiguous()
