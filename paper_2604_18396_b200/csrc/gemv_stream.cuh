@@ -1016,8 +1016,8 @@ __device__ __forceinline__ void head_block_best(float &bv, int &bi, float *s_val
 
 // One row: two weight rows a task on sixteen warps, the next batch of loads under the current one's arithmetic, as in
 // stream_pass_bf16; more rows: four weight rows on eight warps, whose registers hold no second batch.  One CTA fits an SM, and the
-// grid is one CTA per SM (two, of which the second half of the CTAs waited for the first and staged the row again, and loads not
-// pipelined: 8B-class, one row 2343 us a step, so 2287; three rows, 8 blocks 1326 -> 1309).
+// grid is one CTA per SM.  (8B-class, event times, with two CTAs per SM, of which the second half waited for the first and staged
+// the row again, loads not pipelined, and two kernels behind it: one row 179 + 9 + 7 us, so 160; three rows 214 + 7 + 9, so 213.)
 __host__ __device__ constexpr int head_threads(int n) { return n == 1 ? 512 : 256; }
 template <int N, int R>
 __global__ void __launch_bounds__(head_threads(N)) lm_head_kernel(const HeadArgs a, int xstride) {

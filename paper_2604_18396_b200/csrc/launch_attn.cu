@@ -46,7 +46,7 @@ cudaError_t launch_attn_small(river_ctx *c, int n, int layer0, int early) {
     a.skip = c->attn_skip;
     a.pos_depth = c->attn_layer1 ? c->pos_depth : nullptr; a.depth_stride = g.max_pages_per_seq * kPage; a.layer1 = c->attn_layer1;
     if (a.skip) early = 0;  // the flags belong to this block: nothing may be fetched before the dependency resolves
-    const int S = small_attn_splits(c->num_sms, n, g.Hkv);  // as the step metadata says
+    const int S = small_attn_splits(c->num_sms, n, g.Hkv);  // the most that the step metadata may say, whatever the context
     const size_t smem = sizeof(float) * (size_t)kSmallAttnWarps * GQ * (DH + 2);
     const cudaError_t e = ensure_smem(c, attn_small_kernel<DH, GQ>, smem);
     if (e != cudaSuccess) return e;

@@ -1,5 +1,5 @@
-// Launches of the CUDA-core streaming kernels: projections of steps of up to four rows per pass, the LM head and
-// the merge of its argmax partials.
+// Launches of the CUDA-core streaming kernels: projections of steps of up to four rows per pass, the LM head, and the merge of
+// argmax partials (the tensor-core LM head's, and those of more rows than this one merges itself).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>

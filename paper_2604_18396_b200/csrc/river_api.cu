@@ -688,8 +688,8 @@ cudaError_t block_tail(river_ctx *c, int l, int n, const RowLists &rl, int sets,
 //
 // Steps of up to four rows: per block QKV, attention, O, gate/up, down - the exit decision of block l is taken by the
 // QKV kernel of block l + 1 (every CTA computes Eq. 1 for itself while it stages the rows, see gemv_stream.cuh), so
-// no kernel boundary is spent on it; one score kernel after the LM head records the last block's score and the final
-// row lists.  Steps of five and more rows: backbone rows on the tensor-core GEMM, exit-layer rows on its dequantising
+// no kernel boundary is spent on it; the LM head's last CTA records the last block's score and the final row lists (in prefill
+// chunks, which may have no head rows, a score kernel behind it).  Steps of five and more rows: backbone rows on the tensor-core GEMM, exit-layer rows on its dequantising
 // variant, and the score / compaction kernel after every block.
 int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool record_fail = false) {
     const river_config &g = c->cfg;

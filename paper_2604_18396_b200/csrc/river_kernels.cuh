@@ -67,8 +67,9 @@ __global__ void step_begin_kernel(const StepMeta *meta, const int32_t *upd, /* [
 }
 
 // ---------------------------------------------------------------- a6 + a7: exit score, decision, compaction
-// (Steps of five and more rows after every block; steps of up to four rows only after the last block - their
-// decisions are folded into the kernel that consumes the block output, see gemv_stream.cuh.)
+// (Steps of five and more rows after every block, and smaller ones with offloading or another KV strategy; the decisions of other
+// steps of up to four rows are folded into the kernel that consumes the block output, see gemv_stream.cuh - the last block's into
+// the LM head, or in prefill chunks into this kernel.)
 // One CTA per row of the step.  state_in / state_out: the sticky exit flags entering block l / block l + 1.  A row
 // still in the backbone gets s = <h_in, h_out> / (|h_in| |h_out|) (Eq. 1) in
 // fp32 with a fixed reduction order and the flag s > tau (strict; NaN fails; a zero norm gives s = 0).  The last
