@@ -290,7 +290,7 @@ int river_quantize_w4(const void *w, int out, int in, int group, int refine_iter
                       void *cuda_stream);
 
 int river_seq_len(const river_ctx *ctx, int slot);       /* tokens cached in the slot, or RIVER_E_BADSLOT */
-int river_release(river_ctx *ctx, int slot);             /* free the slot's pages */
+int river_release(river_ctx *ctx, int slot);             /* free the slot's pages, behind the work queued so far; does not wait */
 int river_stats(river_ctx *ctx, river_stats_t *host_out); /* synchronises the stream; fills host_out even when it
                                                              returns a device-error code */
 void river_destroy(river_ctx *ctx);

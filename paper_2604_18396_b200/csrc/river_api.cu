@@ -999,7 +999,7 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
     struct KeepMetaRows {  // the metadata block is laid out for the chunk under way, and for decode steps behind it
         river_ctx *c; int rows;
         explicit KeepMetaRows(river_ctx *c_) : c(c_), rows(c_->meta_rows) {}
-        ~KeepMetaRows() { c->meta_rows = rows; }
+        ~KeepMetaRows() { c->meta_rows = rows; c->prefill_attn_now = false; }
     } keep(c);
     // rows of the chunk that starts at position p of sequence s, if it may hold `most` (token ids are contiguous in tok, and it
     // has no more prompt ends than the logits staging has rows), and the least depth among them
@@ -1016,9 +1016,10 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
     {
         long long total = 0;
         for (int s = 0; s < n_seqs; ++s) total += offsets[s + 1] - offsets[s];
-        const std::vector<float> ta((size_t)std::min<long long>(total, c->list_rows), tau);
-        CUDA_TRY(c, cudaMemcpyAsync(c->tau_i, ta.data(), sizeof(float) * ta.size(), cudaMemcpyHostToDevice, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        const int rows = (int)std::min<long long>(total, c->list_rows);
+        fill_f32_kernel<<<(rows + 255) / 256, 256, 0, c->stream>>>(c->tau_i, rows, tau);
+        CUDA_TRY(c, cudaGetLastError());
+        c->st.launches_total += 1;
     }
     int s = 0, p = 0;  // next (sequence, position) to schedule
     while (s < n_seqs) {
@@ -1047,7 +1048,9 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
             if (++p == len) { c->seq_len[slots[s]] = len; ++s; p = 0; }
         }
         mh[0] = n; mh[1] = n_upd; mh[2] = n_head;
-        set_attn_meta(c, mh, n);
+        c->prefill_attn_now = n >= 5 && prefill_attn_supported(c);
+        if (c->prefill_attn_now) mh[5] = n;  // hint_act; the decode attention's geometry is for the rows that need it
+        else set_attn_meta(c, mh, n);
         // query tiles of the prefill attention: consecutive positions of one sequence, up to 16 - or as many as make 128
         // query rows, for the tcgen05 kernel, where the rows of a long pass look back at 128 positions and more on average
         // (below, its tiles are mostly padding: mini shape, prompts of 96 positions 20 against 17 us; 1B-class, 435: 30 against 32)
@@ -1073,7 +1076,6 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
                 mh[kMetaHdr + 9 * max_rows + n_tiles + i] = 1;
             }
         reinterpret_cast<StepMeta *>(mh)->pad2[0] = n_tiles + (head_tiles ? n_head : 0);
-        c->prefill_attn_now = n >= 5 && prefill_attn_supported(c);
         const bool want_logits = logits_last && n_head > 0;
         set_io_meta(mh, tok + tok0, c->tau_i, c->row_forced(), want_logits ? c->logits_i : nullptr, c->next_i, c->exit_i,
                     nullptr);
@@ -1573,21 +1575,23 @@ int river_seq_len(const river_ctx *c, int slot) {
     return c->seq_len[slot];
 }
 
+// Nothing here waits: whoever is given the pages next writes and reads them on the same stream.
 int river_release(river_ctx *c, int slot) {
     if (!c) return RIVER_E_BADARG;
     if (!check_slot(c, slot)) return fail(c, RIVER_E_BADSLOT, "slot out of range");
     const river_config &g = c->cfg;
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    CUDA_TRY(c, cudaMemsetAsync(c->page_tbl_dev + (size_t)slot * g.max_pages_per_seq, 0xff,
+                                sizeof(int32_t) * g.max_pages_per_seq, c->stream));
+    if (g.kv_strategy == RIVER_KV_MONO_DECREASING) {  // a new sequence in this slot may go to full depth again
+        const int32_t cap0 = g.L;
+        CUDA_TRY(c, cudaMemcpyAsync(c->slot_cap + slot, &cap0, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
+        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    }
     for (int i = g.max_pages_per_seq - 1; i >= 0; --i) {
         int32_t &e = c->page_tbl[(size_t)slot * g.max_pages_per_seq + i];
         if (e >= 0) { c->free_pages.push_back(e); e = -1; }
     }
     c->seq_len[slot] = 0;
-    CUDA_TRY(c, cudaMemsetAsync(c->page_tbl_dev + (size_t)slot * g.max_pages_per_seq, 0xff,
-                                sizeof(int32_t) * g.max_pages_per_seq, c->stream));
-    const int32_t cap0 = g.L;  // a new sequence in this slot may go to full depth again
-    CUDA_TRY(c, cudaMemcpyAsync(c->slot_cap + slot, &cap0, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
     return RIVER_OK;
 }
 

@@ -66,6 +66,11 @@ __global__ void step_begin_kernel(const StepMeta *meta, const int32_t *upd, /* [
     }
 }
 
+__global__ void fill_f32_kernel(float *out, int n, float v) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = v;
+}
+
 // ---------------------------------------------------------------- a6 + a7: exit score, decision, compaction
 // (Steps of five and more rows after every block, and smaller ones with offloading or another KV strategy; the decisions of other
 // steps of up to four rows are folded into the kernel that consumes the block output, see gemv_stream.cuh - the last block's into

@@ -1,0 +1,48 @@
+"""river_release and river_prefill wait for nothing: prompts whose pages go back, and out again, while the kernels that fill and read
+them are still queued, against the same calls with a synchronisation after each."""
+import pytest
+import torch
+
+from paper_2604_18396_b200 import River, make_config
+from tests.gpu_harness import draw_model
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+
+
+# long passes, several of them; short passes (the batch kernels; at four rows and fewer the decode attention); depths by Eq. 1
+@pytest.mark.parametrize("lens,depth,strategy", [([300, 9, 200], None, 0), ([1100, 40], 3, 0), ([20, 30], 4, 0), ([3, 1], None, 0),
+                                                 ([60, 45], -1, 0), ([20, 7], None, 2)])
+def test_pages_handed_on_while_in_use(lens, depth, strategy):
+    shape, _, (bb, rv) = draw_model("mini8")
+    pages = sum((n + 16) // 16 for n in lens)
+    offs = [0]
+    for n in lens:
+        offs.append(offs[-1] + n)
+    slots = list(range(len(lens)))
+    out = {}
+    for wait in (True, False):
+        r = River(make_config(shape, max_seqs=len(lens), max_pages_per_seq=80, n_pages=pages, max_batch=8, prefill_chunk=256,
+                              kv_strategy=strategy), bb, rv)
+        got = out[wait] = []
+        for turn in range(5):
+            tok = torch.cat([synth.tokens(71 + turn, b, n, shape.V) for b, n in enumerate(lens)]).int().cuda()
+            lg = torch.empty((len(lens), shape.V), device="cuda")
+            if turn:
+                for s in (slots if turn % 2 else slots[::-1]):
+                    r.release(s)
+            d = r.prefill(slots, tok, offs, depth, lg, tau=0.5 + 0.1 * turn if depth == -1 else float("inf"))
+            nxt, ex = torch.empty(len(lens), dtype=torch.int32, device="cuda"), torch.empty(len(lens), dtype=torch.int32, device="cuda")
+            lg2 = torch.empty_like(lg)
+            r.decode_step(slots, tok[:len(lens)].contiguous(), torch.full((len(lens),), 0.9, device="cuda"), None, lg2, nxt, ex)
+            kv = [x.clone() for b in slots for x in r.read_kv(b, shape.L, 0, 1)]
+            if wait:
+                torch.cuda.synchronize()
+            got.append((d, lg, lg2, nxt, ex, kv))
+        torch.cuda.synchronize()
+        assert r.stats().device_error == 0
+        r.close()
+    for a, b in zip(out[True], out[False]):
+        assert a[0] == b[0]
+        assert all(torch.equal(x, y) for x, y in zip(a[1:5], b[1:5]))
+        assert all(torch.equal(x, y) for x, y in zip(a[5], b[5]))
