@@ -113,11 +113,13 @@ __device__ __forceinline__ float refine_sum_plain(const unsigned long long (&d)[
 // Measured on 4096 x 14336, 64 inputs per group, 20 rounds: 5488 us with the general round everywhere, 295 us
 // with every round taken, 222 us with the rounds that change something - 8 us a round and 130 us around them, spent on the quotients
 // x / s, a power per round for the threshold, and the codes' rounding and conversion (16 a clock each): 142 us with the quotients
-// from the reciprocal, the threshold carried along and the codes rounded by an addition.
+// from the reciprocal, the threshold carried along and the codes rounded by an addition; 140 with the range taken over pairs of bf16
+// values (128 inputs per group 207 -> 193).  The FMA pipe is 75 % busy then.  Dealing a CTA's groups that still move out over its
+// threads, after 3 and 6 rounds or after 6, left 40 % of the rounds away and won nothing (140 and 137; 32 and 128 inputs slower): at 4
+// CTAs per SM the warps that wait at its barriers are missing beside the others' chains of additions.
 // Weights whose half step lies above the threshold (scales of 0.3 and more) go through general rounds only, and those read the
-// weights again: 4096 x 4096, standard deviation 4, groups of 32, 64 and 128, 1.30, 1.86 and 3.34 ms (1.44, 1.72 and 3.42 with the
-// weights kept in registers and a power per round).  At 64, where that is the slower way, registers give 1.67, but the ordinary
-// case above 148 us; a copy in shared memory 1.77 there and 1.91, not 1.84, where general and plain rounds mix (deviation 1).
+// weights again: 4096 x 4096, standard deviation 4, groups of 32, 64 and 128, 1.30, 1.56 and 3.3 ms (64: 1.84 before the
+// range was taken over pairs, which left registers for a fifth CTA per SM).
 template <int G>
 __global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w, long long n_groups, int refine_iters, float last_threshold,
                                                           uint8_t *codes, __nv_bfloat16 *scale, __nv_bfloat16 *zero) {
@@ -131,9 +133,19 @@ __global__ void __launch_bounds__(128) quantize_w4_kernel(const __nv_bfloat16 *w
         xp[4 * i] = v.x; xp[4 * i + 1] = v.y; xp[4 * i + 2] = v.z; xp[4 * i + 3] = v.w;
     }
     auto x_at = [&](int i) { return __uint_as_float((i & 1) ? (xp[i / 2] & 0xffff0000u) : (xp[i / 2] << 16)); };
-    float mn = x_at(0), mx = mn;
+    float mn, mx;
+    if constexpr (G >= 64) {  // two at a time (at 32 the compiler then keeps more registers, and general rounds lose 4 %)
+        auto pair_at = [&](int i) { return *reinterpret_cast<const __nv_bfloat162 *>(&xp[i]); };
+        __nv_bfloat162 mn2 = pair_at(0), mx2 = mn2;
 #pragma unroll
-    for (int i = 1; i < G; ++i) { mn = fminf(mn, x_at(i)); mx = fmaxf(mx, x_at(i)); }
+        for (int i = 1; i < G / 2; ++i) { mn2 = __hmin2(mn2, pair_at(i)); mx2 = __hmax2(mx2, pair_at(i)); }
+        mn = fminf(__low2float(mn2), __high2float(mn2));
+        mx = fmaxf(__low2float(mx2), __high2float(mx2));
+    } else {
+        mn = mx = x_at(0);
+#pragma unroll
+        for (int i = 1; i < G; ++i) { mn = fminf(mn, x_at(i)); mx = fmaxf(mx, x_at(i)); }
+    }
     const bool constant = mx == mn;
     float s = bf16_round(__fdiv_rn(__fsub_rn(mx, mn), 15.0f));
     if (constant || s == 0.f) s = 1.f;
