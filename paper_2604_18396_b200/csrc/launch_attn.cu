@@ -87,10 +87,10 @@ cudaError_t launch_attn_prefill_tc_t(river_ctx *c, int n_tiles, int layer0) {
     a.q = c->qbuf; a.out = c->obuf; a.kv = kv_addr(c, layer0); a.Hq = c->cfg.Hq;
     a.qscale = 1.4426950408889634f / std::sqrt((float)DH);
     a.dev_err = c->dev_err;
-    const size_t smem = attn_prefill_tc_smem_bytes(DH);
+    const size_t smem = attn_prefill_tc_smem_bytes();
     const cudaError_t e = ensure_smem(c, attn_prefill_tc_kernel<DH, GQ>, smem);
     if (e != cudaSuccess) return e;
-    return launch_k(attn_prefill_tc_kernel<DH, GQ>, dim3(n_tiles, c->cfg.Hkv), dim3(kPtThreads), smem, c->stream, true, c->kv_tmap, a);
+    return launch_k(attn_prefill_tc_kernel<DH, GQ>, dim3(n_tiles * c->cfg.Hkv), dim3(kPtThreads), smem, c->stream, true, c->kv_tmap, a);
 }
 }  // namespace
 
