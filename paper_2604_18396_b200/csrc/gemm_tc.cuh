@@ -178,7 +178,7 @@ struct TcGateUpEpi {  // tile rows 0..63: gate features f0.., rows 64..127: up f
     int omode = 0;
     __device__ int quad_row(int i, int q0, int nq) const { return i < nq ? 4 * (q0 + i) : 64 + 4 * (q0 + i - nq); }
     __device__ void run(const float *tile, int ld, int tile_idx, int n_live, const int32_t *rows, int tid, int nthr,
-                        int pr0, int pr1, int = 0) const {
+                        int pr0, int pr1, int n0 = 0) const {
         const int f0 = tile_idx * 64, np = pr1 - pr0;
         for (int t = tid; t < n_live * np; t += nthr) {
             const int n = t / np, r = pr0 + t % np;
@@ -187,13 +187,13 @@ struct TcGateUpEpi {  // tile rows 0..63: gate features f0.., rows 64..127: up f
             act[(size_t)rows[n] * F + f0 + r] = v;
             if (omode == 1) {
                 const __nv_bfloat16 h = __float2bfloat16_rn(v);
-                const size_t o = (size_t)n * F + f0 + r;
+                const size_t o = (size_t)(n0 + n) * F + f0 + r;
                 ohi[o] = __bfloat16_as_ushort(h);
                 olo[o] = __bfloat16_as_ushort(__float2bfloat16_rn(v - __bfloat162float(h)));
             } else if (omode == 2) {
                 const __half h = __float2half_rn(v);
                 const int f = f0 + r, j = f & 7;
-                const size_t o = (size_t)n * F + (f & ~7) + (j < 4 ? 2 * j : 2 * (j - 4) + 1);
+                const size_t o = (size_t)(n0 + n) * F + (f & ~7) + (j < 4 ? 2 * j : 2 * (j - 4) + 1);
                 ohi[o] = __half_as_ushort(h);
                 olo[o] = __half_as_ushort(__float2half_rn(v - __half2float(h)));
             }
@@ -307,7 +307,7 @@ struct TcHeadEpi {  // logits (optional) and the tile's (max, lowest id) per row
 // ---------------------------------------------------------------- the GEMM kernel
 struct TcArgs {
     int K;            // inner dimension (multiple of 64)
-    int n_pad;        // N operand rows (multiple of 16, <= 256)
+    int n_pad;        // N operand rows of a CTA (multiple of 16, <= 256): rows n_pad blockIdx.y and on
     int splits;       // K splits per tile = CTAs per cluster (<= 8)
     int n_stages;     // pipeline depth
     int late_release; // 1: dependent grids may start only once this grid's own dependency is met (see the kernel)
@@ -334,12 +334,13 @@ struct TcArgs {
 // sums replace its own partial values in place (peers only ever read the rows of THEIR slices).  A CTA may not
 // exit while a peer still reads its tile: it arrives at the second cluster barrier right after its own reads and waits
 // for it after its epilogue.  Even a CTA that gave up takes part in both barriers: a cluster barrier has no time-out.
+// n0: the list row behind column 0 (n_live: live columns).
 // `wide`: the accumulator has 2 NP columns, W hi^T in [0, NP) and W lo^T in [NP, 2 NP), to be added up here; `sets` 2: a second
 // one of the same form behind it.
 template <class Epi>
 __device__ __forceinline__ void tc_finish(const Epi &epi, float *tile, uint32_t tmem_d, uint32_t tmem_cols, int NP,
                                           int splits, int split, int tile_idx, int n_live, const int32_t *rows, bool ok,
-                                          const int *s_abort, int nthr, bool wide = false, int sets = 1) {
+                                          const int *s_abort, int nthr, int n0, bool wide = false, int sets = 1) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (warp >= 2 && warp < 6 && ok && n_live > 0) {
         const int q = warp & 3;  // TMEM lane quarter this warp may read
@@ -402,7 +403,7 @@ __device__ __forceinline__ void tc_finish(const Epi &epi, float *tile, uint32_t 
         asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
         __syncthreads();
     }
-    if (good) epi.run(tile, kTcLd, tile_idx, n_live, rows, tid, nthr, pr0, pr1);
+    if (good) epi.run(tile, kTcLd, tile_idx, n_live, rows + n0, tid, nthr, pr0, pr1, n0);
     if (splits > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -424,7 +425,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort, s_some;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tile_idx = blockIdx.x / a.splits, split = blockIdx.x % a.splits;
+    const int tile_idx = blockIdx.x / a.splits, split = blockIdx.x % a.splits, n0 = blockIdx.y * NP;
     const int kb_total = a.K / kTcBK;
     const int kb0 = (int)(((long long)kb_total * split) / a.splits), kb1 = (int)(((long long)kb_total * (split + 1)) / a.splits);
     const int nkb = kb1 - kb0;
@@ -490,8 +491,8 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     };
     auto load_b = [&](uint32_t s, int x) {
         const uint32_t full = full0 + 8 * s, dst = stage0 + s * stage_bytes + a_bytes;
-        tma_load_2d(dst, &map_bhi, x, 0, full);
-        if (!a.one_box) tma_load_2d(dst + b_bytes, &map_blo, x, 0, full);
+        tma_load_2d(dst, &map_bhi, x, n0, full);
+        if (!a.one_box) tma_load_2d(dst + b_bytes, &map_blo, x, n0, full);
     };
 
     // weights first: they depend on nothing
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
         for (int i = 0; i < pre; ++i) load_a((uint32_t)i);
     pdl_wait();
     if (a.late_release) pdl_launch();
-    const int n_live = *a.cnt;  // rows of the backbone list; the stream kernel serves the exit-layer rows
+    const int n_live = min(*a.cnt - n0, NP);  // rows of the backbone list here
     // even with no live row the requested weight tiles must land before the CTA may exit: run the pipeline once
     const int nkb_run = n_live > 0 ? nkb : pre;
 
@@ -549,13 +550,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     bool ok = mbar_wait_sleepy(smem_u32(&bars[2 * S]), 0, abortp, a.dev_err);
     tc_fence_after();
     __syncthreads();  // all TMA writes and MMA reads of the pipeline memory are over: it now holds the tile
-    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kTcThreads, wide, sets);
-}
-
-inline size_t tc_smem_bytes(int n_pad, int n_stages) {
-    const size_t stage = (size_t)kTcBM * kTcBK * 2 + 2 * (size_t)n_pad * kTcBK * 2;
-    const size_t pipe = (size_t)n_stages * stage;  // the finished tile reuses it (the host checks the fit)
-    return 1024 + pipe + sizeof(uint64_t) * (2 * n_stages + 1) + 64;
+    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kTcThreads, n0, wide, sets);
 }
 
 }  // namespace river

@@ -127,7 +127,7 @@ static __global__ void __launch_bounds__(256) tc_prep_pair_kernel(const ProjIn i
 // ---------------------------------------------------------------- the kernel
 struct TcW4Args {
     int K;             // inner dimension (multiple of 256)
-    int n_pad;         // N operand rows (multiple of 16, <= 256)
+    int n_pad;         // N operand rows of a CTA (multiple of 16, <= 256): rows n_pad blockIdx.y and on
     int splits;        // K splits per tile = CTAs per cluster (<= 8), in whole raw tiles
     int n_stages;      // stages: activation tiles in shared memory AND A tiles in tensor memory (even)
     int overlap;       // 1: runs beside the preceding grid (tc_gemm_kernel of the same projection, launched with
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort, s_early;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tile_idx = blockIdx.x / a.splits, split = blockIdx.x % a.splits;
+    const int tile_idx = blockIdx.x / a.splits, split = blockIdx.x % a.splits, n0 = blockIdx.y * NP;
     const int sb_total = a.K / (kTcBK * kW4Super);
     const int sb0 = (int)(((long long)sb_total * split) / a.splits), sb1 = (int)(((long long)sb_total * (split + 1)) / a.splits);
     const int nsb = sb1 - sb0, kb0 = sb0 * kW4Super, nkb = nsb * kW4Super;
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
     // block - nothing here depends on it.  Whoever comes next in the stream waits for THIS grid, so this grid must not
     // complete before that one: every CTA waits for it just before it exits.
     if (!a.overlap) pdl_wait();
-    const int n_live = *a.cnt;
+    const int n_live = min(*a.cnt - n0, NP);
     if (n_live <= 0 && pre == 0) {  // uniform over the CTA and the cluster (nobody reaches a cluster barrier)
         if (a.overlap) pdl_wait();
         return;
@@ -296,8 +296,8 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
                 if (i >= S && !mbar_wait(empty0 + 8 * s, epar, abortp, a.dev_err)) break;
                 const uint32_t full = bfull0 + 8 * s;
                 mbar_expect_tx(full, 2 * b_bytes);
-                tma_load_2d(dst, &map_bhi, x, 0, full);
-                if (!a.one_box) tma_load_2d(dst + b_bytes, &map_blo, x, 0, full);
+                tma_load_2d(dst, &map_bhi, x, n0, full);
+                if (!a.one_box) tma_load_2d(dst + b_bytes, &map_blo, x, n0, full);
                 x += kTcBK;
                 if (++s == (uint32_t)S) { s = 0; epar ^= 1u; dst = stage0; } else dst += stage_bytes;
             }
@@ -393,14 +393,8 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
     bool ok = n_live > 0 ? mbar_wait(smem_u32(b_acc), 0, abortp, a.dev_err) : true;
     tc_fence_after();
     __syncthreads();  // all copies into and MMA reads of the pipeline memory are over: it now holds the tile
-    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kW4Threads, wide, a.sets);
+    tc_finish(epi, tile, tmem_d, tmem_cols, NP, a.splits, split, tile_idx, n_live, a.rows, ok, &s_abort, kW4Threads, n0, wide, a.sets);
     if (a.overlap) pdl_wait();
-}
-
-inline size_t tc_w4_smem_bytes(int n_pad, int n_stages) {
-    const size_t stage = 2 * (size_t)n_pad * kTcBK * 2;
-    return 1024 + (size_t)n_stages * stage + (size_t)kW4RawBufs * kW4RawBytes +
-           sizeof(uint64_t) * (2 * n_stages + 2 * kW4RawBufs + 1) + 64;
 }
 
 }  // namespace river

@@ -6,15 +6,14 @@
 
 namespace river {
 
-const river_ctx::BMap *tc_bmap(river_ctx *c, int K, int np, bool w4 = false, bool alt = false);
+// box: operand rows per copy (0: all np)
+const river_ctx::BMap *tc_bmap(river_ctx *c, int K, int np, bool w4 = false, bool alt = false, int box = 0);
+// operand rows per CTA of a projection's tensor-core kernels when the step has np
+int row_tile(const river_ctx *c, int np);
 
 // Both kernels of a projection (backbone rows, exit-layer rows) are in flight together: `phase` says which part of a
 // launch function runs - the operand kernel, the GEMM, or both in a row.
 enum : int { kTcPrep = 1, kTcGemm = 2, kTcBoth = 3 };
-// Shared memory and tensor-memory columns per CTA of the configurations tc_gemm_kernel may run in for `np` operand
-// rows (two or three CTAs per SM): what a kernel that shares the SMs with it must budget against.
-struct TcFootprint { size_t smem; int cols; };
-int tc_footprints(int np, TcFootprint (&out)[2]);
 
 // launch_tc.cu: backbone rows, 5 <= rows <= 256
 template <class Epi>

@@ -48,7 +48,8 @@ struct river_ctx {
     CUtensorMap tc_map_head;
     // operand maps of the tensor-core projections for (K, padded rows): up to 128 rows the lo rows follow the hi rows
     // in one buffer (`lo_ptr` = tc_xhi + np K) and `hi` covers both (one copy per k-block); beyond, two buffers
-    struct BMap { int K, np; bool w4, alt, one; __nv_bfloat16 *base, *lo_ptr; CUtensorMap hi, lo; };
+    // (box: rows of a copy, np or a row tile's; `one`: one copy takes the hi and the lo rows)
+    struct BMap { int K, np, box; bool w4, alt, one; __nv_bfloat16 *base, *lo_ptr; CUtensorMap hi, lo; };
     std::vector<BMap> tc_bmaps;
     // long prefill passes (launch_tc_wide.cu): rows per pass (0: not for this context), operand rows (high parts, low parts
     // behind them) of the projections that read h / the attention output, and of the down projection; f16 exit-layer weights

@@ -133,6 +133,90 @@ inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode, int mo
     return p;
 }
 
+// Operand rows per CTA of a step with np of them, from its widest projection (`tiles` 128-feature tiles, K inputs).  A small model's weight
+// tiles and K-splits are CTAs for a fraction of the chip (mini shape: 24 for QKV), each of which then finishes all the rows alone; so
+// the rows are dealt out as well, 16 to 64 to a CTA, while all CTAs of the widest projection find a place at once, two to an SM.  (The
+// 1B and 8B shapes fill the chip with their weights: there every row tile would only stream them again.)  The K-splits, and so what
+// one accumulator sums, stay those of all rows together.  Mini shape, us a block of a 118-row prompt, one tile / tiles of 32: QKV 24 /
+// 11, O 12 / 10, gate/up 18 / 10, down 15 / 8; the prompt 587 / 409.
+inline int tc_row_tile(int num_sms, int np, int tiles, int K, bool decode) {
+    const int splits = tc_plan(num_sms, np, tiles, K, true, decode).splits;
+    for (int nt = 16; nt <= 64 && nt < np; nt *= 2)
+        if (tiles * splits * ((np + nt - 1) / nt) <= 2 * num_sms) return nt;
+    return np;
+}
+// The plan for np rows, in the shared and tensor memory of CTAs that take nt of them.
+inline W4Plan w4_row_plan(W4Plan p, int np, int nt) {
+    if (nt >= np) return p;
+    const size_t stage = 2 * (size_t)nt * kTcBK * 2, raw = (size_t)kW4RawBufs * kW4RawBytes;
+    p.occ = 2;
+    p.n_stages = (int)std::min<size_t>(4, (110 * 1024 - raw - 4096) / stage) & ~1;
+    p.wide = 1;
+    p.cols = 32;
+    while (p.cols < p.sets * 2 * nt + p.n_stages * (int)kW4ACols) p.cols <<= 1;
+    return p;
+}
+
+inline size_t tc_smem_bytes(int n_pad, int n_stages) {  // (the finished tile reuses the stages: the launch checks the fit)
+    return 1024 + (size_t)n_stages * tc_stage_bytes(n_pad) + sizeof(uint64_t) * (2 * n_stages + 1) + 64;
+}
+inline size_t tc_w4_smem_bytes(int n_pad, int n_stages) {
+    const size_t stage = 2 * (size_t)n_pad * kTcBK * 2;
+    return 1024 + (size_t)n_stages * stage + (size_t)kW4RawBufs * kW4RawBytes + sizeof(uint64_t) * (2 * n_stages + 2 * kW4RawBufs + 1) + 64;
+}
+
+// Tensor memory: every CTA that can be resident on an SM must get its columns at once, since a CTA stuck in the allocation while
+// its cluster waits for it could not be waited out.  So whatever mix of a step's launches fits into an SM's shared memory has to
+// fit into its 512 columns, and requests are padded until it does.
+struct TcFootprint { size_t smem; int cols; };
+constexpr size_t kTcTwoSmem = 90 * 1024;  // two such CTAs leave no room for a third of any launch
+// tc_gemm_kernel with np operand rows per CTA: two CTAs per SM, with one accumulator or two, three; or the one that fits.
+inline int tc_footprints(int np, TcFootprint *out /* [3] */) {
+    int n = 0, wide;
+    for (int occ = tc_stages_at(np, 2) ? 2 : 1; occ <= 3; ++occ) {
+        const int st = tc_stages_at(np, occ);
+        if (!st) break;
+        out[n].smem = tc_smem_bytes(np, st);
+        out[n++].cols = tc_cols(np, occ, &wide);
+        if (occ == 2 && np <= kTcHalvesRows) {
+            out[n].smem = std::max(out[n - 1].smem, kTcTwoSmem);
+            out[n].cols = 2 * out[n - 1].cols;
+            ++n;
+        }
+        if (occ == 1) break;
+    }
+    return n;
+}
+// The most columns that CTAs of these footprints may ask of one SM.
+inline int most_columns(const TcFootprint *fp, int n, size_t room = kSmSmem) {
+    if (!n) return 0;
+    int most = 0;
+    for (int i = 0; i * fp[0].smem <= room; ++i) most = std::max(most, i * fp[0].cols + most_columns(fp + 1, n - 1, room - i * fp[0].smem));
+    return most;
+}
+// What a step with np operand rows, nt per CTA, launches on tc_gemm_kernel (the LM head may have all rows in a CTA).
+inline int step_footprints(int np, int nt, TcFootprint *out /* [6] */) {
+    int n = tc_footprints(nt, out);
+    if (nt == np) return n;
+    const int n0 = n;
+    n += tc_footprints(np, out + n);
+    for (int i = n0; i < n; ++i) out[i].smem = std::max(out[i].smem, kTcTwoSmem);
+    return n;
+}
+// Shared memory that a CTA of tc_gemm_w4_kernel asks for: its own, no more than p.occ of them, and the rule above beside the CTAs of
+// tc_gemm_kernel of the same step; 0: there is none.
+inline size_t w4_smem_request(const W4Plan &p, int np, int nt) {
+    if (p.occ * p.cols > 512) return 0;
+    TcFootprint fp[7];
+    const int n = step_footprints(np, nt, fp);
+    TcFootprint &mine = fp[n] = {std::max(tc_w4_smem_bytes(nt, p.n_stages), kSmSmem / (p.occ + 1) + 1024), p.cols};
+    while (most_columns(fp, n + 1) > 512) {
+        mine.smem += 4096;
+        if (mine.smem > kSmSmem / p.occ - 1024) return 0;
+    }
+    return mine.smem;
+}
+
 // tc_gemm_wide_kernel: k-blocks per accumulation segment.  1024 inputs, 512 where K is short, and never more than the longest
 // sum that the batch kernels' K-splits make of the same projection in passes of `pass_rows` rows (1B-class shape: 256 inputs for
 // O and gate/up, 384 for QKV; 8B-class: 1024 for all), since the error of a sum inside the tensor cores grows with its length:
