@@ -469,28 +469,28 @@ cudaError_t tc_pair(river_ctx *c, bool with_river, const ProjIn &in, int K, int 
 }
 
 // a2 of block l for the n rows of the step: attention norm + QKV + RoPE + KV write, on the weight set(s) the row
-// lists name (small steps: from the exit flags).
-cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const DecideArgs &dec, double kv_write) {
+// lists name (small steps: from the exit flags).  at: the entry of the row lists and exit flags; sets: as in block_tail.
+cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const DecideArgs &dec, double kv_write, int at, int sets = 3) {
     const river_config &g = c->cfg;
     const int d = g.d, B = c->list_rows, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
     const double w4f = 0.25 + 2.0 / g.group;
     const river_layer_weights &w = c->layers[l - 1];
     const int strat = g.kv_strategy;
-    const int has_river = strat == RIVER_KV_RIVER && w.rq.codes != nullptr;
-    const int32_t *ai = c->act_idx + (size_t)(l - 1) * B, *ri = c->riv_idx + (size_t)(l - 1) * B;
-    const int32_t *na = c->n_act + (l - 1), *nr = c->n_riv + (l - 1);
-    const RowLists rl{ai, na, ri, nr, c->hint_act, c->meta_dev /* StepMeta::n_rows */, c->state_at(l - 1)};
+    const int has_river = (sets & 2) && strat == RIVER_KV_RIVER && w.rq.codes != nullptr;
+    const int32_t *ai = c->act_idx + (size_t)at * B, *ri = c->riv_idx + (size_t)at * B;
+    const int32_t *na = c->n_act + at, *nr = c->n_riv + at;
+    const RowLists rl{ai, na, ri, nr, c->hint_act, c->meta_dev /* StepMeta::n_rows */, c->state_at(at)};
     const bool tc = c->tc_ok && n >= 5 && n <= c->tc_max_pad;
     const river_ctx::LayerMaps *tm = tc ? &c->tc_maps[l - 1] : nullptr;
     const river_ctx::LayerMaps *wm = (tc && c->w4tc_ok && has_river) ? &c->w4_maps[l - 1] : nullptr;
-    const int32_t *nrh = c->n_riv + std::max(0, l - 2);  // never above the count entering this block
+    const int32_t *nrh = c->n_riv + std::max(0, at - 1);  // never above the count entering this block
     cudaError_t err = cudaSuccess;
     auto note = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
     const double wb = 2.0 * (qdim + 2.0 * kvdim) * d;
     // bytes the rows that have left cost here: the 4-bit copy; the bf16 K and V matrices (State Propagation); nothing
     const double riv_bytes = strat == RIVER_KV_RIVER ? wb * w4f + kv_write
                            : strat == RIVER_KV_STATE_PROPAGATION ? 2.0 * 2.0 * kvdim * d + kv_write : 0.0;
-    LaunchScope ls(c, K_QKV, wb + kv_write, riv_bytes, l - 1);
+    LaunchScope ls(c, K_QKV, wb + kv_write, riv_bytes, at);
     QkvProblem p{};
     p.wq = (const uint16_t *)w.wq; p.wk = (const uint16_t *)w.wk; p.wv = (const uint16_t *)w.wv;
     p.rq = w4_of(w.rq); p.rk = w4_of(w.rk); p.rv = w4_of(w.rv);
@@ -501,15 +501,17 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
         const TcQkvEpi e{g.Hq, g.Hkv, g.dh, c->rope_cs, c->qbuf, kv_addr(c, l - 1), c->dev_err};
         const CUtensorMap *const cm[3] = {wm ? &wm->q : nullptr, wm ? &wm->k : nullptr, wm ? &wm->v : nullptr};
         const river_w4 *const cw[3] = {&w.rq, &w.rk, &w.rv};
-        note(tc_pair(c, wm != nullptr, in, d, n, rl,
-                     [&](int phase, bool late) {
-                         return launch_tc(c, in, tm->q, tm->k, tm->v, d, (qdim + 2 * kvdim) / kTcBM, n, 0, qdim / kTcBM,
-                                          kvdim / kTcBM, ai, na, e, true, c->hint_act, phase, late);
-                     },
-                     [&](int phase, bool beside) {
-                         return launch_tc_w4(c, in, cm, cw, d, (qdim + 2 * kvdim) / kTcBM, n, 0, qdim / kTcBM, kvdim / kTcBM,
-                                             ri, nr, nrh, e, phase, beside);
-                     }));
+        const auto river = [&](int phase, bool beside) {
+            return launch_tc_w4(c, in, cm, cw, d, (qdim + 2 * kvdim) / kTcBM, n, 0, qdim / kTcBM, kvdim / kTcBM, ri, nr, nrh, e, phase, beside);
+        };
+        if (sets & 1)
+            note(tc_pair(c, wm != nullptr, in, d, n, rl,
+                         [&](int phase, bool late) {
+                             return launch_tc(c, in, tm->q, tm->k, tm->v, d, (qdim + 2 * kvdim) / kTcBM, n, 0, qdim / kTcBM,
+                                              kvdim / kTcBM, ai, na, e, true, c->hint_act, phase, late);
+                         },
+                         river));
+        else if (wm) note(river(kTcBoth, false));
     }
     if (!wm && (!tc || has_river)) {
         note(launch_stream(c, p, in, rl, d, (g.Hq + 2 * g.Hkv) * (g.dh / 2), n, has_river, true, tc ? 1 : 0, dec));
@@ -691,7 +693,10 @@ cudaError_t block_tail(river_ctx *c, int l, int n, const RowLists &rl, int sets,
 // no kernel boundary is spent on it; the LM head's last CTA records the last block's score and the final row lists (in prefill
 // chunks, which may have no head rows, a score kernel behind it).  Steps of five and more rows: backbone rows on the tensor-core GEMM, exit-layer rows on its dequantising
 // variant, and the score / compaction kernel after every block.
-int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool record_fail = false) {
+//
+// depth (prefill passes; null: not known here): backbone blocks row i runs.  The batch kernels are then launched for the weight sets
+// that have rows, and the score kernel behind the blocks that some row leaves at.
+int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool record_fail = false, const int32_t *depth = nullptr) {
     const river_config &g = c->cfg;
     const int L = g.L, d = g.d, B = c->list_rows;
     int32_t *fail_buf = record_fail ? c->prefill_fail : nullptr;
@@ -707,6 +712,13 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     // the decisions ride in the QKV kernels - unless the host has to see every decision before it stages a block
     // (offloading) or the rows that left take another route than the 4-bit copies (then: score kernel per block)
     const bool fold = n <= 4 && !c->off_first && strat == RIVER_KV_RIVER;
+    const bool known = depth && c->tc_ok && n >= 5 && n <= c->tc_max_pad && !c->off_first && strat == RIVER_KV_RIVER;
+    std::vector<int> leave;  // rows that leave after block l
+    if (known) {
+        leave.assign(L + 1, 0);
+        for (int i = 0; i < n; ++i) leave[depth[i]] += 1;
+    }
+    int at = 0, gone = known ? leave[0] : 0;  // entry `at` of the row lists and exit flags describes the rows of this block
 
     {
         LaunchScope ls(c, K_BEGIN, (double)n * d * 2.0, 0, -1);
@@ -714,10 +726,10 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
                       c->page_tbl_dev, g.max_pages_per_seq, c->meta_rows, c->embed, d, g.V, c->h[0], c->row_pos(), c->inv_freq,
                       g.dh / 2, c->rope_cs, L, g.entry_layer, c->state_at(0), c->dev_err, lists, c->hint_act, c->tickets));
     }
-    auto launch_score = [&](int l, const float *h_in, const float *h_out) {
+    auto launch_score = [&](int l, const float *h_in, const float *h_out, int from) {
         LaunchScope ls(c, K_SCORE, (double)n * d * 8.0, 0, -1);
         note(launch_k(score_compact_kernel, dim3(n), dim3(256), 0, c->stream, true, c->meta(), l, L, g.entry_layer,
-                      g.exit_mode, h_in, h_out, d, c->pass, (const uint8_t *)c->state_at(l - 1), c->state_at(l), lists,
+                      g.exit_mode, h_in, h_out, d, c->pass, (const uint8_t *)c->state_at(from), c->state_at(l), lists,
                       c->hint_act, c->tickets + 1, fail_buf, (const int32_t *)c->row_slot(),
                       strat == RIVER_KV_MONO_DECREASING ? c->slot_cap : (int32_t *)nullptr));
     };
@@ -725,12 +737,12 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     const float *prev_in = nullptr;  // input of the previous block (its output is h[hi])
     for (int l = 1; l <= L; ++l) {
         const river_layer_weights &w = c->layers[l - 1];
-        const int has_river = strat == RIVER_KV_RIVER && w.rq.codes != nullptr;
-        const int32_t *ai = c->act_idx + (size_t)(l - 1) * B, *ri = c->riv_idx + (size_t)(l - 1) * B;
-        const int32_t *na = c->n_act + (l - 1), *nr = c->n_riv + (l - 1);
-        const RowLists rl{ai, na, ri, nr, c->hint_act, c->meta_dev /* StepMeta::n_rows */, c->state_at(l - 1)};
+        const int sets = known ? (gone < n ? 1 : 0) | (gone ? 2 : 0) : 1 | (strat == RIVER_KV_RIVER && w.rq.codes ? 2 : 0);
+        const int32_t *ai = c->act_idx + (size_t)at * B, *ri = c->riv_idx + (size_t)at * B;
+        const int32_t *na = c->n_act + at, *nr = c->n_riv + at;
+        const RowLists rl{ai, na, ri, nr, c->hint_act, c->meta_dev /* StepMeta::n_rows */, c->state_at(at)};
         float *h_in = c->h[hi], *h_mid = c->h[(hi + 1) % 3], *h_out = c->h[(hi + 2) % 3];
-        const int32_t *nrh = c->n_riv + std::max(0, l - 2);  // never above the count entering this block
+        const int32_t *nrh = c->n_riv + std::max(0, at - 1);  // never above the count entering this block
         bool staged = false;
         if (c->off_first && l >= c->off_first)
             if (int rc = offload_before_layer(c, l, &staged)) return rc;
@@ -742,10 +754,10 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
                 dec.h_prev = prev_in; dec.state_in = c->state_at(l - 2); dec.state_out = c->state_at(l - 1);
                 dec.lists = lists; dec.hint_act = c->hint_act; dec.fail = fail_buf; dec.row_slot = c->row_slot();
             }
-            note(launch_qkv(c, l, n, h_in, dec, kv_write));
+            note(launch_qkv(c, l, n, h_in, dec, kv_write, at, known ? sets : 3));
         }
         // the other KV strategies (Section 3): a row that has left neither attends nor changes its hidden state
-        c->attn_skip = strat == RIVER_KV_RIVER ? nullptr : c->state_at(l - 1);
+        c->attn_skip = strat == RIVER_KV_RIVER ? nullptr : c->state_at(at);
         // (a prefill chunk needs no visibility test: a prompt starts in an empty slot and all its positions stop at one
         // depth, so whatever a row that still runs may look back at has an entry - and the chunk's own positions have
         // not been noted yet)
@@ -764,9 +776,13 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
             note(launch_attention(c, n, l - 1));
         }
         // ---- a4, a5
-        note(block_tail(c, l, n, rl, 1 | (has_river ? 2 : 0), l - 1, nrh, h_in, h_mid, h_out, c->act));
+        note(block_tail(c, l, n, rl, sets, at, nrh, h_in, h_mid, h_out, c->act));
         // ---- a6 + a7: exit score, decision, compaction -> row lists entering block l+1
-        if (!fold) launch_score(l, h_in, h_out);
+        if (!known || record_fail || (l < L && leave[l])) {
+            if (!fold) launch_score(l, h_in, h_out, at);
+            at = l;
+            if (known && l < L) gone += leave[l];
+        }
         if (staged) note(cudaEventRecord(c->off_freed[(l - c->off_first) & 1], c->stream));  // the slot may be refilled
         prev_in = h_in;
         hi = (hi + 2) % 3;
@@ -775,7 +791,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
     // LM head of a decode step (prefill chunks may have none)
     const bool head_notes = fold && c->rows_distinct && n_head == n;
     if (n_head > 0) note(launch_head(c, c->h[hi], n_head, head_notes ? prev_in : nullptr));
-    if (fold && !head_notes) launch_score(L, prev_in, c->h[hi]);
+    if (fold && !head_notes) launch_score(L, prev_in, c->h[hi], L - 1);
     if (strat == RIVER_KV_MASK) {  // what the later tokens' attention may see of this step's positions
         LaunchScope ls(c, K_SCORE, 0, 0, -1);
         note(launch_k(depth_note_kernel, dim3((n + 127) / 128), dim3(128), 0, c->stream, true, c->meta(),
@@ -1082,9 +1098,10 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         if (int rc = push_meta(c, mh)) return rc;
         c->rows_distinct = false;  // consecutive positions of one sequence share a chunk
         const int32_t *pos = mh + kMetaHdr + max_rows;
+        const int32_t *row_depth = mh + kMetaHdr + 7 * max_rows;
         const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, tc_attn, n_head, mh + kMetaHdr + 5 * max_rows, head_tiles, pos,
-                                                      mh + kMetaHdr + 7 * max_rows, record_fail)
-                                      : run_rows(c, n, n_head, pos, record_fail);
+                                                      row_depth, record_fail)
+                                      : run_rows(c, n, n_head, pos, record_fail, row_depth);
         c->rows_distinct = true;
         c->prefill_attn_now = false;
         if (rc_rows) return rc_rows;
@@ -1412,7 +1429,7 @@ int river_project_kv(river_ctx *c, int layer, int use_exit_layer, int n_rows, co
     float *q_keep = c->qbuf;
     if (q_out) c->qbuf = q_out;
     const int64_t launched = t_launches;
-    const cudaError_t e = launch_qkv(c, layer, n_rows, h, DecideArgs{}, (double)n_rows * 4.0 * c->cfg.Hkv * c->cfg.dh);
+    const cudaError_t e = launch_qkv(c, layer, n_rows, h, DecideArgs{}, (double)n_rows * 4.0 * c->cfg.Hkv * c->cfg.dh, layer - 1);
     c->qbuf = q_keep;
     if (e != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(e));
     if (!use_exit_layer && c->off_first && layer >= c->off_first)

@@ -45,3 +45,38 @@ def test_short_passes_match_oracle(models, lens, depth):
     for b, n in enumerate(lens):
         p.compare_kv(b, n)
     p.close()
+
+
+def test_mixed_depths(models):
+    """Depths chosen per prompt by Eq. 1: passes of 120 and of 250 rows with rows on both weight sets, whose kernels are launched for
+    the sets that have rows."""
+    import torch
+    shape = models["mini8"][0]
+    L, lo = shape.L, max(shape.entry_layer, 1)
+    for lens in ([50, 40, 30], [100, 90, 60]):
+        prompts = [synth.tokens(83, b, n, shape.V).numpy() for b, n in enumerate(lens)]
+        probe = Pair(models["mini8"], 1, max(lens) + 2, 4, kv_store=1)
+        mins = []
+        for pr in prompts:
+            sc = np.stack([probe.oracle.decode_step([0], [tk], INF)["scores"][0] for tk in pr])
+            probe.oracle.release(0)
+            mins.append(sc[:, lo - 1:L - 1].min(axis=0))
+        probe.close()
+        mins = np.stack(mins)
+        edges = np.sort(mins.ravel())
+        first = lambda t: [next((lo + i for i in range(L - lo) if m[i] > t), L) for m in mins]  # noqa: E731
+        taus = [float(t) for t in 0.5 * (edges[:-1] + edges[1:]) if np.abs(mins - t).min() > 2.5e-3 and len(set(first(t))) > 1]
+        assert taus, "no threshold separates the prompts"
+        for tau in taus[::max(1, len(taus) // 2)]:
+            # (kv_store: the cache as both store it, 16 bits; of this many positions its roundings alone pass the plain bound)
+            p = Pair(models["mini8"], 3, max(lens) + 2, 8, prefill_chunk=256, page_shuffle_seed=9, kv_store=1)
+            want = [p.oracle.prefill_auto(b, pr, tau) for b, pr in enumerate(prompts)]
+            offs = np.concatenate([[0], np.cumsum(lens)]).tolist()
+            lg = torch.empty((3, shape.V), device="cuda")
+            got = p.gpu.prefill([0, 1, 2], torch.from_numpy(np.concatenate(prompts)).int().cuda(), offs, -1, lg, tau=tau)
+            torch.cuda.synchronize()
+            assert got == [w[2] for w in want] and len(set(got)) > 1
+            p.compare_logits(lg.cpu().numpy(), np.stack([w[0] for w in want]), f"tau {tau}")
+            for b, n in enumerate(lens):
+                p.compare_kv(b, n, f"tau {tau}")
+            p.close()
