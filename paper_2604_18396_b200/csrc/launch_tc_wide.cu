@@ -10,29 +10,45 @@ namespace river {
 namespace {
 
 // ---------------------------------------------------------------- exit-layer weights in f16, for the same kernel
-// With hundreds of rows a 4-bit matrix is worth expanding once per pass: row r of the (up to three) matrices laid one after
-// the other becomes K f16 values (q - z) * s - one rounding, as in tc_gemm_w4_kernel - with the inputs of every group of
-// eight in the order (0,4,1,5,2,6,3,7) that the f16 operand rows have too.  A thread expands 32 codes.  Bound by HBM:
-// 0.56 bytes read and 2 written per weight.
-struct W4Expand { W4 m[3]; int rows[3]; };
-__global__ void __launch_bounds__(256) w4_expand_kernel(const W4Expand e, int K, __half *out) {
+// With hundreds of rows a 4-bit matrix is worth expanding once per pass: the (up to three) matrices laid one after the other
+// become f16 values (q - z) * s - one rounding, as in tc_gemm_w4_kernel - with the inputs of every group of eight in the order
+// (0,4,1,5,2,6,3,7) that the f16 operand rows have too.  A warp takes a run of 1024 codes, 16 bytes per lane; four lanes trade their
+// words, so that they store 64 bytes side by side.  Bound by HBM: 0.56 bytes read and 2 written per weight.
+// 1B-class gate / up 29 -> 15 us (a thread stored its own 32 codes' 64 bytes 16 at a time before, half a sector each).  What did not
+// help: the operand rows' kernel as part of this launch (its CTAs in front: mini shape, 1100 positions 622 -> 658 us), and an
+// expansion beside the GEMM before it, in two buffers and CTAs without shared memory: they are not put next to that kernel's
+// on an SM, find room on the idle ones only and finish late elsewhere (1B-class, 829 positions 1164 -> 1254).
+struct W4Expand { W4 m[3]; int runs[3]; };
+constexpr int kExpandRuns = 2;  // of a warp, under way at a time
+__global__ void __launch_bounds__(256) w4_expand_kernel(const W4Expand e, __half *out) {
     pdl_launch();
+    const int lane = threadIdx.x & 31, r0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * kExpandRuns, runs = e.runs[0] + e.runs[1] + e.runs[2];
+    uint4 v[kExpandRuns];
+    uint32_t sz[kExpandRuns];  // scale | zero
+#pragma unroll
+    for (int u = 0; u < kExpandRuns; ++u) {  // (weights depend on nothing)
+        int r = min(r0 + u, runs - 1), m = 0;
+        while (r >= e.runs[m]) { r -= e.runs[m]; ++m; }
+        const W4 w = m == 0 ? e.m[0] : m == 1 ? e.m[1] : e.m[2];
+        v[u] = ldg_stream16(w.codes + (size_t)r * 512 + 16 * lane);
+        const size_t g = (size_t)r * 16 + (lane >> 1);
+        sz[u] = (uint32_t)ldg_u16(w.scale + g) | (uint32_t)ldg_u16(w.zero + g) << 16;
+    }
     pdl_wait();  // the GEMM before may still read the previous projection's expansion
-    const int per_row = K >> 5;
-    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    int r = (int)(i / per_row), m = 0;
-    const int c = (int)(i % per_row);  // 32-input run of the row
-    if (r >= e.rows[0] + e.rows[1] + e.rows[2]) return;
-    uint4 *dst = reinterpret_cast<uint4 *>(out + (size_t)r * K + 32 * c);
-    while (r >= e.rows[m]) { r -= e.rows[m]; ++m; }
-    const W4 w = e.m[m];
-    const size_t g = (size_t)r * (K >> 6) + (c >> 1);
-    const __half2 s2 = __float2half2_rn(bf16f(w.scale[g])), z2 = __float2half2_rn(bf16f(w.zero[g]));
-    const uint4 v = ldg_stream16(w.codes + (size_t)r * (K >> 1) + 16 * c);
-    dst[0] = w4_word_to_f16(v.x, z2, s2);
-    dst[1] = w4_word_to_f16(v.y, z2, s2);
-    dst[2] = w4_word_to_f16(v.z, z2, s2);
-    dst[3] = w4_word_to_f16(v.w, z2, s2);
+#pragma unroll
+    for (int u = 0; u < kExpandRuns; ++u) {
+        if (r0 + u >= runs) break;  // (uniform over the warp)
+        uint4 *dst = reinterpret_cast<uint4 *>(out) + (size_t)(r0 + u) * 128 + 4 * (lane & ~3) + (lane & 3);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {  // lane (group, i) stores word i of lane (group, j)
+            const int from = (lane & ~3) | j;
+            const uint32_t a = __shfl_sync(0xffffffffu, v[u].x, from), b = __shfl_sync(0xffffffffu, v[u].y, from),
+                           c = __shfl_sync(0xffffffffu, v[u].z, from), d = __shfl_sync(0xffffffffu, v[u].w, from),
+                           t = __shfl_sync(0xffffffffu, sz[u], from);
+            const uint32_t word = lane & 2 ? (lane & 1 ? d : c) : (lane & 1 ? b : a);
+            dst[4 * j] = w4_word_to_f16(word, __float2half2_rn(bf16hi(t)), __float2half2_rn(bf16lo(t)));
+        }
+    }
 }
 
 // Rows per tile: the tiles go to `pairs` CTA pairs in whole rounds, so a size that leaves the last round nearly full can win
@@ -72,13 +88,13 @@ cudaError_t launch_wide_operand(river_ctx *c, const ProjIn &in, int K, int n_lis
 
 cudaError_t launch_w4_expand(river_ctx *c, const river_w4 *const (&w)[3], const int (&rows)[3], int K) {
     W4Expand e{};
-    long long threads = 0;
+    long long runs = 0;
     for (int i = 0; i < 3; ++i) {
-        e.rows[i] = rows[i];
         if (rows[i]) e.m[i] = w4_of(*w[i]);
-        threads += (long long)rows[i] * (K / 32);
+        e.runs[i] = (int)((long long)rows[i] * K / 1024);  // (whole: rows and inputs are multiples of 64 and 256)
+        runs += e.runs[i];
     }
-    return launch_k(w4_expand_kernel, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, c->stream, true, e, K, c->wide_w);
+    return launch_k(w4_expand_kernel, dim3((unsigned)((runs + 8 * kExpandRuns - 1) / (8 * kExpandRuns))), dim3(256), 0, c->stream, true, e, c->wide_w);
 }
 
 template <class Epi>
