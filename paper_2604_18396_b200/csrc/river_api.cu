@@ -1042,7 +1042,8 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         // A long pass if there are rows enough for one, else the layout and the kernels of a short pass: its metadata is 11 arrays
         // of max_batch entries, a long pass's of wide_rows (45 KB to fill and to copy, whatever the rows).
         const Chunk most = chunk_at(s, p, wide ? c->wide_rows : g.max_batch);
-        const bool long_pass = wide && most.rows >= tc_long_pass_rows(g.d, g.L, g.L - most.least, g.max_batch);
+        const int tiled = tc_tiled_pass_rows(c->num_sms, std::max((g.Hq + 2 * g.Hkv) * g.dh / kTcBM, g.F / 64), g.d);
+        const bool long_pass = wide && most.rows >= tc_long_pass_rows(g.d, g.L, g.L - most.least, g.max_batch) && most.rows > std::min(tiled, g.max_batch);
         const int max_rows = long_pass ? c->wide_rows : g.max_batch;
         c->meta_rows = max_rows;
         int32_t *mh = next_meta(c);

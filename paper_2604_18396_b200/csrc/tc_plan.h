@@ -275,4 +275,14 @@ inline int tc_long_pass_rows(int d, int L, int exit_blocks, int max_rows) {
     return std::min(base + more * exit_blocks / L, std::min(max_rows, 256)) + 1;
 }
 
+// Where the batch kernels' rows are dealt out over CTAs (tc_row_tile), a short pass is the faster one for longer: up to this many rows.
+// Batch / pair kernels, us, 1 prompt:
+//   tiny 0/4      145 rows 210 / 243   176: 214 / 247   224: 223 / 255   256: 230 / 248     3/4  145: 246 / 265   256: 264 / 271
+//   mini 0/6      145: 377 / 446   176: 378 / 452   200: 454 / 464   224: 463 / 474   256: 479 / 462
+//        5/6      145: 440 / 460   176: 443 / 463   200: 509 / 505   224: 532 / 487   256: 519 / 471
+constexpr int kTcTiledPassRows = 192;
+inline int tc_tiled_pass_rows(int num_sms, int tiles, int K) {
+    return tc_row_tile(num_sms, kTcTiledPassRows, tiles, K, false) < kTcTiledPassRows ? kTcTiledPassRows : 0;
+}
+
 }  // namespace river

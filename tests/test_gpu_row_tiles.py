@@ -37,10 +37,12 @@ def test_steps_match_oracle(models, name, rows):
     p.close()
 
 
-@pytest.mark.parametrize("lens,depth", [([40], None), ([16, 17], 3), ([100, 20], 2), ([128], None)])
-def test_short_passes_match_oracle(models, lens, depth):
+# (192 rows and one more: the last short passes, the first long ones)
+@pytest.mark.parametrize("lens,depth,chunk", [([40], None, 128), ([16, 17], 3, 128), ([100, 20], 2, 128), ([128], None, 128), ([192], None, 256),
+                                              ([170, 23], None, 256), ([90, 102], 1, 256), ([193], 1, 256), ([150, 30], 0, 256)])
+def test_short_passes_match_oracle(models, lens, depth, chunk):
     shape = models["mini8"][0]
-    p = Pair(models["mini8"], len(lens), max(lens) + 8, 8, prefill_chunk=128, kv_store=1, storage_yardstick=True, page_shuffle_seed=3)
+    p = Pair(models["mini8"], len(lens), max(lens) + 8, 8, entry_layer=0 if depth == 0 else None, prefill_chunk=chunk, kv_store=1, storage_yardstick=True, page_shuffle_seed=3)
     p.prefill(list(range(len(lens))), [synth.tokens(82, b, n, shape.V).numpy() for b, n in enumerate(lens)], depth, logits=True)
     for b, n in enumerate(lens):
         p.compare_kv(b, n)

@@ -13,6 +13,7 @@ SHIM = r"""
 extern "C" {
 int row_tile(int sms, int np, int tiles, int K, int decode) { return river::tc_row_tile(sms, np, tiles, K, decode != 0); }
 int tc_splits(int sms, int np, int tiles, int K, int decode) { return river::tc_plan(sms, np, tiles, K, true, decode != 0).splits; }
+int pass_rows(int sms, int tiles, int K) { return river::tc_tiled_pass_rows(sms, tiles, K); }
 int tc_columns(int np, int nt) { river::TcFootprint f[6]; return river::most_columns(f, river::step_footprints(np, nt, f)); }
 long w4_smem(int sms, int np, int nt, int tiles, int K, int decode, int *o) {
     const river::W4Plan all = river::w4_plan(sms, np, tiles, K, decode != 0), p = river::w4_row_plan(all, np, nt);
@@ -63,3 +64,7 @@ def test_row_tiles_of_the_shapes(plan):
                 nt = plan.row_tile(SMS, np, t, K, decode)
                 assert nt == np or t * plan.tc_splits(SMS, np, t, K, decode) * ceil_div(np, nt) <= 2 * SMS
     assert got["mini8"][:5] == [16, 16, 16, 32, 32] and got["tiny"][:5] == [16, 16, 16, 16, 16], got
+
+
+def test_short_passes_of_dealt_out_rows(plan):
+    assert [plan.pass_rows(SMS, t, K) for t, K in ((16, 256), (24, 512), (128, 2048), (224, 4096))] == [192, 192, 0, 0]
