@@ -315,7 +315,7 @@ struct TcArgs {
     int wide;         // 1: hi and lo operand rows as one operand of 2 n_pad rows (the host checks the TMEM budget)
     int halves;       // 1 (wide only): the second half of the k-blocks goes to a second accumulator, added at the end: the error
                       // of a sum inside the tensor cores grows with its length
-    int a_rows_per_map;  // a tile's 128 rows come from map tile_idx / (rows_per_map / 128) ... see tile_map()
+    int f16;          // 1: operands are f16 (expanded exit-layer weights), else bf16
     int gateup;       // 1: a tile is 64 rows of map 0 + 64 rows of map 1
     int qkv_q_tiles, qkv_k_tiles;  // QKV: tiles per matrix (0 otherwise)
     const int32_t *rows;   // step row id of operand row n
@@ -495,7 +495,8 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
         if (!a.one_box) tma_load_2d(dst + b_bytes, &map_blo, x, n0, full);
     };
 
-    // weights first: they depend on nothing
+    // weights first: they depend on nothing (an expansion's are the kernel's before this one)
+    if (a.f16) pdl_wait();
     const int pre = min(S, nkb);
     if (tid == 0)
         for (int i = 0; i < pre; ++i) load_a((uint32_t)i);
@@ -519,7 +520,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = tc_idesc(acc_n);
+            const uint32_t idesc = a.f16 ? tc_idesc(acc_n) & ~((1u << 7) | (1u << 10)) : tc_idesc(acc_n);
             const uint64_t dfix = tc_smem_desc(0);  // everything but the address field
             const uint32_t stage16 = stage_bytes >> 4, a16 = a_bytes >> 4, b16 = b_bytes >> 4;
             uint32_t s = 0, par = 0, addr16 = stage0 >> 4, d = tmem_d;

@@ -65,6 +65,21 @@ cudaError_t launch_tc(river_ctx *c, const ProjIn &in, const CUtensorMap &a0, con
     return launch_kc(tc_gemm_kernel<Epi>, dim3(tiles * a.splits, row_tiles), dim3(kTcThreads), smem, c->stream, true, a.splits, a0,
                      a1, a2, bm->hi, bm->lo, a, epi);
 }
+cudaError_t launch_tc_pass(river_ctx *c, const CUtensorMap &a0, int K, int tiles, int n_list, int splits, const int32_t *rows,
+                           const int32_t *cnt, const TcResidEpi &epi, bool f16, bool alt_operand) {
+    const river_ctx::WMap *bm = wide_map(c, K, 2 * kTcPassRows, alt_operand);
+    if (!bm) return cudaErrorInvalidValue;
+    TcArgs a{};
+    a.K = K; a.n_pad = kTcPassRows; a.splits = splits; a.halves = 1; a.wide = 1; a.f16 = f16 ? 1 : 0;
+    a.n_stages = tc_stages_at(kTcPassRows, 2);
+    a.rows = rows; a.cnt = cnt; a.dev_err = c->dev_err;
+    a.hint = c->meta_dev;  // StepMeta::n_rows (the host launches nothing for an empty list)
+    const size_t smem = std::max<size_t>(tc_smem_bytes(kTcPassRows, a.n_stages), kTcTwoSmem);
+    const cudaError_t e = ensure_smem(c, tc_gemm_kernel<TcResidEpi>, smem);
+    if (e != cudaSuccess) return e;
+    return launch_kc(tc_gemm_kernel<TcResidEpi>, dim3(tiles * splits, (n_list + kTcPassRows - 1) / kTcPassRows), dim3(kTcThreads), smem, c->stream,
+                     true, splits, a0, a0, a0, bm->hi, bm->lo, a, epi);
+}
 #define RIVER_TC_INST(E) \
     template cudaError_t launch_tc<E>(river_ctx *, const ProjIn &, const CUtensorMap &, const CUtensorMap &, const CUtensorMap &, \
                                       int, int, int, int, int, int, const int32_t *, const int32_t *, const E &, bool, const int32_t *, \

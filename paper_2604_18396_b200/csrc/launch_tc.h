@@ -52,6 +52,11 @@ RIVER_TCW4_DECL(TcQkvEpi) RIVER_TCW4_DECL(TcResidEpi) RIVER_TCW4_DECL(TcGateUpEp
 inline uint16_t *wide_operand(const river_ctx *c, bool alt) { return alt ? c->wide_xalt : c->wide_x; }
 cudaError_t launch_wide_operand(river_ctx *c, const ProjIn &in, int K, int n_list, const int32_t *rows, const int32_t *cnt, bool f16);
 cudaError_t launch_w4_expand(river_ctx *c, const river_w4 *const (&w)[3], const int (&rows)[3], int K);
+// map `hi` / `lo` of the wide operand rows in boxes of bn / 2 rows
+const river_ctx::WMap *wide_map(river_ctx *c, int K, int bn, bool alt);
+// launch_tc.cu: O and down of a long pass on tc_gemm_kernel (tc_pass_splits)
+cudaError_t launch_tc_pass(river_ctx *c, const CUtensorMap &a0, int K, int tiles, int n_list, int splits, const int32_t *rows,
+                           const int32_t *cnt, const TcResidEpi &epi, bool f16, bool alt_operand);
 template <class Epi>
 cudaError_t launch_tc_wide(river_ctx *c, const CUtensorMap &a0, const CUtensorMap &a1, const CUtensorMap &a2, int K, int tiles,
                            int n_list, int q_tiles, int k_tiles, int run_step, int head_step, const int32_t *rows, const int32_t *cnt,

@@ -65,6 +65,8 @@ int wide_bn(int feature_pairs, int n, int pairs) {
     return best;
 }
 
+}  // namespace
+
 const river_ctx::WMap *wide_map(river_ctx *c, int K, int bn, bool alt) {
     for (auto &b : c->wide_maps)
         if (b.K == K && b.bn == bn && b.alt == alt) return &b;
@@ -74,8 +76,6 @@ const river_ctx::WMap *wide_map(river_ctx *c, int K, int bn, bool alt) {
     c->wide_maps.push_back(b);
     return &c->wide_maps.back();
 }
-
-}  // namespace
 
 cudaError_t launch_wide_operand(river_ctx *c, const ProjIn &in, int K, int n_list, const int32_t *rows, const int32_t *cnt, bool f16) {
     uint16_t *hi = wide_operand(c, false), *lo = hi + (size_t)c->wide_rows * K;

@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "river_ctx.h"
@@ -852,6 +853,12 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
                            const auto &epi) {
             if (set == 1) note(launch_w4_expand(c, w4, w4_rows, K));
             if (in) note(launch_wide_operand(c, *in, K, n_of[set], rows_of[set], cnt_of[set], set == 1));
+            if constexpr (std::is_same_v<std::decay_t<decltype(epi)>, WdResidEpi>)
+                if (const int splits = tc_pass_splits(c->num_sms, g.max_batch, tiles, K, set == 1, n_of[set])) {
+                    note(launch_tc_pass(c, m0, K, tiles, n_of[set], splits, rows_of[set], cnt_of[set], TcResidEpi{epi.resid, epi.out, epi.out_dim}, set == 1,
+                                        in == nullptr));
+                    return;
+                }
             note(launch_tc_wide(c, m0, m1, m2, K, tiles, n_of[set], q_tiles, k_tiles, run_step, head_step, rows_of[set], cnt_of[set], epi,
                                 set == 1, in == nullptr));
         };

@@ -235,6 +235,18 @@ inline int tc_wide_segment(int num_sms, int pass_rows, int tiles, int K, bool f1
     return std::min(K >= 4096 ? 16 : 8, run);
 }
 
+// Long passes of small models: where a projection has few features (O and down) its tiles keep no more than half of the pairs busy,
+// each with the whole run of k-blocks; then it goes to tc_gemm_kernel instead, 64 rows to a CTA, in as many K-splits as keep every
+// sum as short as the pair kernel's (two accumulators per CTA) - if its CTAs all find a place at once.  0: not so.  us a prompt, all
+// projections on the pair kernel / so: mini, full depth 256 rows 463 / 418, 512 499 / 470, 1024 590 / 563; five of six blocks on the
+// exit layers 535 / 507, 608 / 563, 676 / 662; d 1024, full depth 256 rows 388 / 335, 512 436 / 396.  (Fewer than 16 k-blocks are
+// no run to split.)
+constexpr int kTcPassRows = 64;
+inline int tc_pass_splits(int num_sms, int pass_rows, int tiles, int K, bool f16, int n) {
+    const int row_tiles = (n + kTcPassRows - 1) / kTcPassRows, kb = K / kTcBK, splits = (kb - 1) / (2 * tc_wide_segment(num_sms, pass_rows, tiles, K, f16)) + 1;
+    return tiles <= 8 && kb >= 16 && tiles / 2 * row_tiles <= num_sms / 4 && splits <= kTcMostSplits && tiles * splits * row_tiles <= 2 * num_sms ? splits : 0;
+}
+
 // Whether the last block of a long pass runs behind QKV (O, gate / up, down; f16: on the exit layers) on the kernels of decode steps,
 // for `ends` prompt ends.  Those put every SM to work on a few rows, by K-splits, where the pair kernel has a pair per 256 features
 // and every exit-layer matrix is expanded for it first; their time grows with the rows sooner.  And only where every sum inside the

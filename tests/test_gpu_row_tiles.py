@@ -49,6 +49,18 @@ def test_short_passes_match_oracle(models, lens, depth, chunk):
     p.close()
 
 
+@pytest.mark.parametrize("name,lens,depth", [("mini8", [257], None), ("mini8", [320, 5], 1), ("tiny", [640], 1), ("tiny", [300, 33], None)])
+def test_long_passes_match_oracle(models, name, lens, depth):
+    """O and down of long passes on the batch kernel: last row tiles of one row, full ones, both weight sets."""
+    shape = models[name][0]
+    p = Pair(models[name], len(lens), max(lens) + 8, 8, prefill_chunk=256, kv_store=1, storage_yardstick=True, page_shuffle_seed=3)
+    p.prefill(list(range(len(lens))), [synth.tokens(84, b, n, shape.V).numpy() for b, n in enumerate(lens)], depth, logits=True)
+    for b, n in enumerate(lens):
+        p.compare_kv(b, n)
+    assert p.gpu.stats().device_error == 0
+    p.close()
+
+
 def test_mixed_depths(models):
     """Depths chosen per prompt by Eq. 1: passes of 120 and of 250 rows with rows on both weight sets, whose kernels are launched for
     the sets that have rows."""

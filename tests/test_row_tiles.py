@@ -14,6 +14,8 @@ extern "C" {
 int row_tile(int sms, int np, int tiles, int K, int decode) { return river::tc_row_tile(sms, np, tiles, K, decode != 0); }
 int tc_splits(int sms, int np, int tiles, int K, int decode) { return river::tc_plan(sms, np, tiles, K, true, decode != 0).splits; }
 int pass_rows(int sms, int tiles, int K) { return river::tc_tiled_pass_rows(sms, tiles, K); }
+int pass_splits(int sms, int pass_rows, int tiles, int K, int f16, int n) { return river::tc_pass_splits(sms, pass_rows, tiles, K, f16 != 0, n); }
+int segment(int sms, int pass_rows, int tiles, int K, int f16) { return river::tc_wide_segment(sms, pass_rows, tiles, K, f16 != 0); }
 int tc_columns(int np, int nt) { river::TcFootprint f[6]; return river::most_columns(f, river::step_footprints(np, nt, f)); }
 long w4_smem(int sms, int np, int nt, int tiles, int K, int decode, int *o) {
     const river::W4Plan all = river::w4_plan(sms, np, tiles, K, decode != 0), p = river::w4_row_plan(all, np, nt);
@@ -68,3 +70,21 @@ def test_row_tiles_of_the_shapes(plan):
 
 def test_short_passes_of_dealt_out_rows(plan):
     assert [plan.pass_rows(SMS, t, K) for t, K in ((16, 256), (24, 512), (128, 2048), (224, 4096))] == [192, 192, 0, 0]
+
+
+@pytest.mark.parametrize("n", [225, 256, 600, 830, 1024])
+def test_long_passes_on_the_batch_kernel_sum_no_longer(plan, n):
+    taken = []
+    for tiles, K in SHAPES:
+        for f16 in (0, 1):
+            if K % 256:
+                continue
+            s = plan.pass_splits(SMS, 256, tiles, K, f16, n)
+            if s:
+                taken.append((tiles, K))
+                kb = K // 64
+                per = [kb * (i + 1) // s - kb * i // s for i in range(s)]
+                assert s <= 8 and min(per) >= 2 and max(ceil_div(p, 2) for p in per) <= plan.segment(SMS, 256, tiles, K, f16), (tiles, K)
+                assert tiles * s * ceil_div(n, 64) <= 2 * SMS
+    assert (4, 1536) in taken and (4, 1024) in taken and (2, 1024) in taken  # O and down of the mini and the tiny shape
+    assert not any(t >= 16 for t, _ in taken)
