@@ -36,12 +36,12 @@ struct AttnArgs {
     const StepMeta *meta;
     const float *q;        // [rows][Hq*DH]
     const int32_t *page_tbl, *row_slot, *row_pos;
-    const int32_t *order;  // grid z -> row (longest context first), a permutation of the step's rows
+    const int32_t *order;  // grid z -> row (longest context first): the step's rows, or those of a pass that attend here
     int n_pages, max_pages_per_seq, Hkv, Hq, layer0;
     float qscale;          // log2(e) / sqrt(DH)
-    float *part_o;         // [(row*Hq + head)*splits + split][DH]  unnormalised
+    float *part_o;         // [(z*Hq + head)*splits + split][DH]  unnormalised
     float2 *part_ml;       // same index: (max, sum) in the base-2 domain
-    unsigned *tickets;     // [rows][Hkv], zero between launches: the last split of a (row, kv head) merges them all
+    unsigned *tickets;     // [z][Hkv], zero between launches: the last split of a (row, kv head) merges them all
     float *out;            // [rows][Hq*DH]
     int *dev_err;
     const uint8_t *skip;   // rows whose flag is set do not attend (they have left and run nothing here), or null
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(attn_threads(MMA)) attn_split_kernel(const __g
         if (ns == 1) {  // the only split of the row: this is the attention output
             a.out[((size_t)row * a.Hq + kvh * GQ + g) * DH + e] = num / den;
         } else {
-            const size_t idx = ((size_t)row * a.Hq + kvh * GQ + g) * n_splits + split;
+            const size_t idx = ((size_t)blockIdx.z * a.Hq + kvh * GQ + g) * n_splits + split;
             a.part_o[idx * DH + e] = num;
             if (e == 0) a.part_ml[idx] = make_float2(M, den);
         }
@@ -432,12 +432,12 @@ __global__ void __launch_bounds__(attn_threads(MMA)) attn_split_kernel(const __g
     // out = sum_s 2^(m_s - M) o_s / sum_s 2^(m_s - M) l_s  (atomic ticket, no spinning)
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = (atomicAdd(&a.tickets[row * a.Hkv + kvh], 1u) == (unsigned)(ns - 1));
+    if (tid == 0) s_last = (atomicAdd(&a.tickets[blockIdx.z * a.Hkv + kvh], 1u) == (unsigned)(ns - 1));
     __syncthreads();
     if (!s_last) return;
     __threadfence();
     float *wgt = sm;  // [GQ][ns] weights 2^(m_s - M) / sum, reusing the merge buffer (ns <= 64)
-    const size_t base0 = ((size_t)row * a.Hq + kvh * GQ) * n_splits;
+    const size_t base0 = ((size_t)blockIdx.z * a.Hq + kvh * GQ) * n_splits;
     for (int t = tid; t < GQ * ns; t += kAttnThreads) {
         const int g = t / ns, sidx = t % ns;
         const float2 ml = __ldcg(&a.part_ml[base0 + (size_t)g * n_splits + sidx]);
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(attn_threads(MMA)) attn_split_kernel(const __g
         for (int sidx = 0; sidx < ns; ++sidx) num = fmaf(wgt[g * 64 + sidx], __ldcg(po + (size_t)sidx * DH), num);
         a.out[((size_t)row * a.Hq + kvh * GQ + g) * DH + e] = num;
     }
-    if (tid == 0) a.tickets[row * a.Hkv + kvh] = 0;
+    if (tid == 0) a.tickets[blockIdx.z * a.Hkv + kvh] = 0;
 }
 
 inline size_t attn_smem_bytes(int DH, int GQ) {  // (both consumer kinds: the tensor-core one leaves sq / sp unused)

@@ -19,7 +19,6 @@ constexpr int kPfPad = 8;       // bf16 elements of padding per staged row (16 b
 
 struct PrefillAttnArgs {
     const StepMeta *meta;        // n_tiles
-    int tile0;                   // first tile of this launch
     const int32_t *tile_row0;    // first row of the chunk in the tile
     const int32_t *tile_rows;    // rows in the tile (1..16): same sequence, consecutive positions
     const float *q;              // [rows][Hq * DH] fp32
@@ -53,7 +52,7 @@ __global__ void __launch_bounds__(32 * GQ) attn_prefill_kernel(const PrefillAttn
     __nv_bfloat16 *vs = ks + 2 * kPfBN * LD;                         // [2][kPfBN][LD]
     pdl_launch();
     pdl_wait();  // q and the chunk's own K/V come from the kernel before this one
-    const int tile = a.tile0 + blockIdx.x, kvh = blockIdx.y;
+    const int tile = blockIdx.x, kvh = blockIdx.y;
     if (tile >= a.meta->pad2[0]) return;
     const int row0 = a.tile_row0[tile], n_rows = a.tile_rows[tile];
     if (a.skip && a.skip[row0]) return;  // (the rows of a chunk leave together: prefill exits at one depth)

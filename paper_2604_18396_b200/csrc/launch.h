@@ -17,9 +17,10 @@ cudaError_t launch_argmax_final(river_ctx *c, int n_head, int n_parts);
 
 // launch_attn.cu: paged GQA decode attention (TMA-fed split-KV kernel; small-step kernel for 1-4 rows)
 cudaError_t launch_attention(river_ctx *c, int n, int layer0);
+cudaError_t launch_attention_split(river_ctx *c, int n, int layer0);  // the split-KV kernel: the first n rows of the metadata's order
 bool prefill_attn_supported(const river_ctx *c);
-// tensor-core causal attention of a prefill chunk's query tiles [tile0, tile0 + n_tiles) (as the step metadata lists them)
-cudaError_t launch_attention_prefill(river_ctx *c, int tile0, int n_tiles, int layer0);
+// tensor-core causal attention of a prefill chunk's query tiles (as the step metadata lists them)
+cudaError_t launch_attention_prefill(river_ctx *c, int n_tiles, int layer0);
 // the same on tcgen05: the query tiles [0, n_tiles) hold up to prefill_tc_positions() positions (instead of kPfBM)
 int prefill_tc_positions(const river_ctx *c);
 cudaError_t launch_attention_prefill_tc(river_ctx *c, int n_tiles, int layer0);

@@ -63,10 +63,10 @@ bool prefill_attn_supported(const river_ctx *c) {
 
 namespace {
 template <int DH, int GQ>
-cudaError_t launch_attn_prefill_t(river_ctx *c, int tile0, int n_tiles, int layer0) {
+cudaError_t launch_attn_prefill_t(river_ctx *c, int n_tiles, int layer0) {
     const river_config &g = c->cfg;
     PrefillAttnArgs a{};
-    a.meta = c->meta(); a.tile0 = tile0; a.tile_row0 = c->tile_row0(); a.tile_rows = c->tile_rows();
+    a.meta = c->meta(); a.tile_row0 = c->tile_row0(); a.tile_rows = c->tile_rows();
     a.q = c->qbuf; a.out = c->obuf; a.kv = kv_addr(c, layer0); a.Hq = g.Hq;
     a.qscale = 1.4426950408889634f / std::sqrt((float)DH);
     a.dev_err = c->dev_err;
@@ -103,9 +103,9 @@ cudaError_t launch_attention_prefill_tc(river_ctx *c, int n_tiles, int layer0) {
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_attention_prefill(river_ctx *c, int tile0, int n_tiles, int layer0) {
+cudaError_t launch_attention_prefill(river_ctx *c, int n_tiles, int layer0) {
     const int gq = c->cfg.Hq / c->cfg.Hkv;
-#define ATTP(DH_, GQ_) if (c->cfg.dh == DH_ && gq == GQ_) return launch_attn_prefill_t<DH_, GQ_>(c, tile0, n_tiles, layer0);
+#define ATTP(DH_, GQ_) if (c->cfg.dh == DH_ && gq == GQ_) return launch_attn_prefill_t<DH_, GQ_>(c, n_tiles, layer0);
     ATTP(64, 1) ATTP(64, 2) ATTP(64, 4) ATTP(64, 8) ATTP(128, 1) ATTP(128, 2) ATTP(128, 4) ATTP(128, 8)
 #undef ATTP
     return cudaErrorInvalidValue;
@@ -118,6 +118,11 @@ cudaError_t launch_attention(river_ctx *c, int n, int layer0) {
         ATTS(64, 1) ATTS(64, 2) ATTS(64, 4) ATTS(64, 8) ATTS(128, 1) ATTS(128, 2) ATTS(128, 4) ATTS(128, 8)
 #undef ATTS
     }
+    return launch_attention_split(c, n, layer0);
+}
+
+cudaError_t launch_attention_split(river_ctx *c, int n, int layer0) {
+    const int gq = c->cfg.Hq / c->cfg.Hkv;
 #define ATT(DH_, GQ_) if (c->cfg.dh == DH_ && gq == GQ_) return launch_attn_split<DH_, GQ_>(c, n, layer0);
     ATT(64, 1) ATT(64, 2) ATT(64, 4) ATT(64, 8) ATT(128, 1) ATT(128, 2) ATT(128, 4) ATT(128, 8)
 #undef ATT

@@ -177,14 +177,14 @@ size_t carve(const river_config *c, river_ctx *x, char *base, int head_rows) {
 // equally long and outnumber the slots, a few when the lengths are mixed, and with few rows enough to fill three
 // quarters of the slots.  Splits are whole tiles, at least two.  The split count is part of a captured launch's key;
 // the chunk length lives in the step metadata.
-void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
+struct AttnSplits { int splits, chunk, max_pos; };
+AttnSplits attn_splits(const river_ctx *c, const int32_t *row_pos, int n) {
     const river_config &g = c->cfg;
     int max_pos = 0;
     double total = 0.0;
     for (int i = 0; i < n; ++i) {
-        const int pos = mh[kMetaHdr + c->meta_rows + i];
-        max_pos = std::max(max_pos, pos);
-        total += pos + 1;
+        max_pos = std::max(max_pos, row_pos[i]);
+        total += row_pos[i] + 1;
     }
     // three CTAs of the attention kernel fit per SM (registers; shared memory at head dim 128)
     const double slots = 3.0 * c->num_sms, ovh = 250.0 * 128.0 / g.dh, merge = 350.0 * 128.0 / g.dh;
@@ -202,7 +202,7 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
         int ch = (max_pos + 1 + s - 1) / s;
         ch = std::max(2 * kAttnTile, (ch + kAttnTile - 1) / kAttnTile * kAttnTile);
         double items = 0.0;
-        for (int i = 0; i < n; ++i) items += (mh[kMetaHdr + c->meta_rows + i] + ch) / ch;  // ceil((pos + 1) / ch)
+        for (int i = 0; i < n; ++i) items += (row_pos[i] + ch) / ch;  // ceil((pos + 1) / ch)
         items *= g.Hkv;
         const int longest = std::min(ch, max_pos + 1);
         // whole waves of items of the mean length bound it from below as well (equal lengths: 1.3 waves cost 2)
@@ -216,8 +216,15 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
         if (chunk == 0 || t < best * 0.97) { best = t; S = s; chunk = ch; }
         if (ch == 2 * kAttnTile) break;  // finer splits do not exist
     }
-    mh[3] = chunk;
-    mh[4] = S;
+    return AttnSplits{S, chunk, max_pos};
+}
+
+void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
+    const river_config &g = c->cfg;
+    const AttnSplits sp = attn_splits(c, mh + kMetaHdr + c->meta_rows, n);
+    const int max_pos = sp.max_pos;
+    mh[3] = sp.chunk;
+    mh[4] = sp.splits;
     mh[5] = n;  // hint_act: every row starts in the backbone
     // the attention grid takes its rows longest context first: CTA slots are handed out in launch order, and a long
     // item that starts last is what the step ends on
@@ -240,7 +247,7 @@ void set_attn_meta(river_ctx *c, int32_t *mh, int n) {
     // cache before the grid dependency resolves: in the replayed step it wins up to four batches per warp (contexts up
     // to ~4.6 K at one row: 3.84 -> 3.49 ms per step at 4 K), beyond that the TMA-fed kernel's staging pays
     c->attn_small_now = n <= 4 && cchunk <= 4 * 4 * kSmallAttnWarps && !(g.flags & RIVER_F_TMA_ATTN);
-    c->attn_splits_now = S;
+    c->attn_splits_now = sp.splits;
 }
 
 void set_io_meta(int32_t *mh, const int32_t *tok, const float *tau, const int32_t *forced, float *logits,
@@ -771,7 +778,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         // ---- a3: paged GQA decode attention
         if (c->prefill_attn_now) {
             LaunchScope ls(c, K_PREFILL_ATTN, kv_read, 0, -1);
-            note(launch_attention_prefill(c, 0, n, l - 1));
+            note(launch_attention_prefill(c, n, l - 1));
         } else {
             LaunchScope ls(c, K_ATTN, kv_read, 0, -1);
             note(launch_attention(c, n, l - 1));
@@ -812,10 +819,11 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
 // pass that looks for the unified depth).  Both weight sets go through tc_gemm_wide_kernel, one after the other.
 //
 // The last block owes the cache the K and V of every position, but its output is read at the n_head prompt ends only: what
-// follows QKV there runs on those rows (head[]: their row ids; head_tiles: their one-row query tiles follow the chunk's
-// n_tiles in the metadata) and on none in a pass without a prompt end.  (8B-class shape, 1024 rows: the rest of a block takes
-// 0.7-1.0 ms for all of them, 0.2 ms for one: the projections' weight streams.)
-int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, const int32_t *head, bool head_tiles, const int32_t *row_pos_host,
+// follows QKV there runs on those rows (head[]: their row ids, which the metadata's attention order and splits are for) and on none
+// in a pass without a prompt end.  (8B-class shape, 1024 rows: the rest of a block takes 0.7-1.0 ms for all of them, 0.2 ms for
+// one: the projections' weight streams.)  Their attention is a decode step's: one-row query tiles walked their prompt with a CTA
+// per KV head (8B-class, one end of 1024 positions 82 us, so 22; tiny shape, four passes 1329 -> 1222 us a prompt).
+int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, const int32_t *head, const int32_t *row_pos_host,
                   const int32_t *depth, bool record_fail) {
     const river_config &g = c->cfg;
     const int L = g.L, d = g.d, F = g.F, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
@@ -873,7 +881,7 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
                             {qdim, kvdim, kvdim}, e);
                 }
         }
-        bool heads_only = l == L && head_tiles;
+        bool heads_only = l == L;
         if (heads_only) {
             int on_backbone = 0;
             for (int i = 0; i < n_head; ++i) on_backbone += depth[head[i]] >= L ? 1 : 0;
@@ -894,8 +902,8 @@ int run_rows_wide(river_ctx *c, int n, int n_tiles, bool tc_attn, int n_head, co
                 for (int i = 0; i < n_head; ++i) kv_bytes += (double)(row_pos_host[head[i]] + 1) * 4.0 * kvdim;
             }
             LaunchScope ls(c, K_PREFILL_ATTN, kv_bytes, 0, -1);
-            note(heads_only ? launch_attention_prefill(c, n_tiles, n_head, l - 1)
-                 : tc_attn ? launch_attention_prefill_tc(c, n_tiles, l - 1) : launch_attention_prefill(c, 0, n_tiles, l - 1));
+            note(heads_only ? launch_attention_split(c, n_head, l - 1)
+                 : tc_attn ? launch_attention_prefill_tc(c, n_tiles, l - 1) : launch_attention_prefill(c, n_tiles, l - 1));
         }
         if (heads_only && tc_ends_fit(c->num_sms, g.max_batch, n_head, d, qdim, F, !n_of[0])) {  // one list: head[]
             c->short_sums = true;
@@ -1093,13 +1101,16 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
             ++n_tiles;
             i = j;
         }
-        const bool head_tiles = long_pass && n_tiles + n_head <= max_rows;
-        if (head_tiles)  // the last block attends at the prompt ends only: a one-row tile each, behind the others
-            for (int i = 0; i < n_head; ++i) {
-                mh[kMetaHdr + 8 * max_rows + n_tiles + i] = mh[kMetaHdr + 5 * max_rows + i];
-                mh[kMetaHdr + 9 * max_rows + n_tiles + i] = 1;
-            }
-        reinterpret_cast<StepMeta *>(mh)->pad2[0] = n_tiles + (head_tiles ? n_head : 0);
+        if (long_pass && n_head > 0) {  // the last block attends at the prompt ends only, on the split-KV kernel
+            const int32_t *pos = mh + kMetaHdr + max_rows, *head = mh + kMetaHdr + 5 * max_rows;
+            int32_t *order = mh + kMetaHdr + 10 * max_rows, end_pos[kMaxBatch];
+            for (int i = 0; i < n_head; ++i) { order[i] = head[i]; end_pos[i] = pos[head[i]]; }
+            std::stable_sort(order, order + n_head, [&](int32_t x, int32_t y) { return pos[x] > pos[y]; });
+            const AttnSplits sp = attn_splits(c, end_pos, n_head);
+            mh[3] = sp.chunk;
+            mh[4] = c->attn_splits_now = sp.splits;
+        }
+        reinterpret_cast<StepMeta *>(mh)->pad2[0] = n_tiles;
         const bool want_logits = logits_last && n_head > 0;
         set_io_meta(mh, tok + tok0, c->tau_i, c->row_forced(), want_logits ? c->logits_i : nullptr, c->next_i, c->exit_i,
                     nullptr);
@@ -1107,7 +1118,7 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         c->rows_distinct = false;  // consecutive positions of one sequence share a chunk
         const int32_t *pos = mh + kMetaHdr + max_rows;
         const int32_t *row_depth = mh + kMetaHdr + 7 * max_rows;
-        const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, tc_attn, n_head, mh + kMetaHdr + 5 * max_rows, head_tiles, pos,
+        const int rc_rows = long_pass ? run_rows_wide(c, n, n_tiles, tc_attn, n_head, mh + kMetaHdr + 5 * max_rows, pos,
                                                       row_depth, record_fail)
                                       : run_rows(c, n, n_head, pos, record_fail, row_depth);
         c->rows_distinct = true;
