@@ -20,7 +20,7 @@
 // and O of one are half of tensor memory, and a serial walk (S, softmax, P V) leaves the pipe idle for more than half of it.  us per
 // block and pass, one stream of 64-key tiles in each of two CTAs per SM against this: 8B-class, passes of 1024 positions of one
 // prompt 64 / 114 / 171 -> 43 / 71 / 100; two prompts of the 1B class 26 -> 24; tiny shape, up to 1245 positions 45 -> 21.  The
-// warp-level kernel (attn_prefill.cuh) stays for short passes and prompts and for tiles of a single row.
+// warp-level kernel (attn_prefill.cuh) stays for short passes and prompts.
 #pragma once
 #include "gemm_tc_w4.cuh"
 #include "attn_prefill.cuh"
