@@ -89,7 +89,6 @@ __global__ void __launch_bounds__(kPtThreads, 1) attn_prefill_tc_kernel(const __
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile int *abortp = &s_abort;
-    pdl_launch();
     if (tid == 0) {
         s_abort = 0;
         for (int i = 0; i < 6 * kPtStreams; ++i) mbar_init(smem_u32(&bars[i]), i % 6 == 3 || i % 6 == 4 ? 4 : 1);
@@ -100,6 +99,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) attn_prefill_tc_kernel(const __
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512u));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
         tc_fence_before();
+        pdl_launch();  // (behind the allocation: see tc_gemm_kernel)
     }
     // (the pass's own layout was on the device before its first kernel started)
     // tiles in descending order, the KV heads of a tile side by side: the longest prefixes first
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kPtThreads, 1) attn_prefill_tc_kernel(const __
 }
 
 // (the head dim of 64 asks for as much as 128 does: a CTA takes all of an SM's tensor memory, so that no CTA that wants some - they
-// all hold 50 KB and more - may share its SM: one stuck in the allocation while others wait for it could not be waited out)
+// all hold 50 KB and more - shares its SM and waits there)
 inline size_t attn_prefill_tc_smem_bytes() { return 1024 + 2 * (2 * kPtRows * 128 + 2 * kPtStreams * kPtKeys * 128); }
 
 }  // namespace river

@@ -438,13 +438,17 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     const int sets = a.halves ? 2 : 1;
     while ((int)tmem_cols < sets * acc_n) tmem_cols <<= 1;
 
+    // Dependent grids may start once every CTA has its tensor memory (pdl_launch behind the allocation, here and in the other kernels
+    // that allocate): a CTA that keeps columns while it waits for the grids before it then waits for none that could be waiting for
+    // those columns.  (The LM head of 5 prompt ends used to get ahead of the dequantising kernel of a 200-row pass, which asks for all
+    // 512 columns.)
     // `late_release`: the next grid in the stream is the dequantising kernel of the same projection, which runs beside
     // this one instead of behind it: it never waits for this grid at its start, so it may only start once everything
     // BOTH read (the operand kernels' output) is complete - that is when every CTA here is past its own wait.
-    if (!a.late_release) pdl_launch();
     if (tid == 0) s_some = *reinterpret_cast<const volatile int32_t *>(a.hint) > 0;  // one read for the whole CTA
     __syncthreads();
     if (!s_some) {  // every row has left the backbone: nothing to fetch, nothing to compute (uniform over the cluster:
+        if (!a.late_release) pdl_launch();
         pdl_wait();  // the hint only changes between layers); still order this grid behind its predecessor
         return;
     }
@@ -459,6 +463,7 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(tmem_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
         tc_fence_before();
+        if (!a.late_release) pdl_launch();
     }
     __syncthreads();
     tc_fence_after();

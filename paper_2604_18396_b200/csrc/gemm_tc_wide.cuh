@@ -254,7 +254,6 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
     __shared__ int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = wd_rank();
-    pdl_launch();
     if (tid == 0) {
         s_abort = 0;
         for (int s = 0; s < S; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
@@ -266,6 +265,7 @@ __global__ void __launch_bounds__(kWdThreads, 1) tc_gemm_wide_kernel(const __gri
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(512u));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::);
         tc_fence_before();
+        pdl_launch();  // (behind the allocation: see tc_gemm_kernel)
     }
     __syncthreads();
     wd_cluster_sync();  // the leader's barriers are ready before the other CTA's copies count on them

@@ -41,8 +41,8 @@ inline int tc_stages_at(int np, int occ) {
     const size_t stage = tc_stage_bytes(np), room = std::min<size_t>(kSmSmem / occ, 227 * 1024);
     return room < kCtaFixed + 2 * stage ? 0 : (int)std::min<size_t>(occ == 1 ? 8 : occ == 2 ? 4 : 3, (room - kCtaFixed) / stage);
 }
-// hi | lo as one operand doubles the accumulator columns; all CTAs that can be resident on an SM must get their
-// tensor memory at once (a CTA stuck in the allocation while its cluster waits for it could not be waited out)
+// hi | lo as one operand doubles the accumulator columns; all CTAs of a launch that can be resident on an SM get their tensor memory
+// at once
 inline int tc_cols(int np, int occ, int *wide) {
     int cols = 32;
     while (cols < 2 * np) cols <<= 1;
@@ -165,9 +165,10 @@ inline size_t tc_w4_smem_bytes(int n_pad, int n_stages) {
     return 1024 + (size_t)n_stages * stage + (size_t)kW4RawBufs * kW4RawBytes + sizeof(uint64_t) * (2 * n_stages + 2 * kW4RawBufs + 1) + 64;
 }
 
-// Tensor memory: every CTA that can be resident on an SM must get its columns at once, since a CTA stuck in the allocation while
-// its cluster waits for it could not be waited out.  So whatever mix of a step's launches fits into an SM's shared memory has to
-// fit into its 512 columns, and requests are padded until it does.
+// Tensor memory: a grid starts once the CTAs of the grids before it have their columns (tc_gemm_kernel), so an allocation that has to wait
+// is a delay and no more.  Inside a step it need not wait: whatever mix of its projections' launches fits into an SM's shared memory fits
+// into its 512 columns, and requests are padded until it does.  (The LM head of a prefill pass has the prompt ends' rows, not the
+// pass's: beside the dequantising CTAs of a pass of 193 to 224 rows its own may wait.)
 struct TcFootprint { size_t smem; int cols; };
 constexpr size_t kTcTwoSmem = 90 * 1024;  // two such CTAs leave no room for a third of any launch
 // tc_gemm_kernel with np operand rows per CTA: two CTAs per SM, with one accumulator or two, three; or the one that fits.
