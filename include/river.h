@@ -144,7 +144,8 @@ int river_init(const river_config *cfg, const river_weights *w, void *kv_pool, s
  * (token, layer).
  *   prefill_exit_layer  e in [entry_layer, L] for every prompt of the call, or -1: chosen per prompt by Eq. 1 with
  *       the prompt as the batch - the first block l in [max(entry_layer, 1), L-1] after which every position of the
- *       prompt has s > tau, else L (costs a second pass over the prompts whose depth comes out below L);
+ *       prompt has s > tau, else L (costs a second pass over the prompts whose depth comes out below L, and waits for the
+ *       first pass, whose scores the host reads; with a given depth the call only queues its work);
  *   tau     threshold of the -1 rule (unused otherwise);
  *   slots   [host] n_seqs empty sequence slots;   tok [dev] int32 token ids, all prompts concatenated;
  *   offsets [host] n_seqs+1 prefix offsets into tok;
@@ -173,7 +174,7 @@ int river_decode_step(river_ctx *ctx, int batch, const int32_t *slots, const int
  * Device-side errors (a token id or page id out of range, a forced exit layer out of range, a bounded wait that
  * ran out) are recorded in a sticky error word and the offending access is skipped or redirected; the kernels always
  * return.  This call, river_stats and river_selftest_wait_timeout read the word back and return RIVER_E_TIMEOUT for
- * a wait that ran out, RIVER_E_DEVICE otherwise; river_decode_step and river_prefill (which do not synchronise) report
+ * a wait that ran out, RIVER_E_DEVICE otherwise; river_decode_step and river_prefill (which do not read it) report
  * it at the next such call.  Once the host has seen the word the context refuses further steps with the same code
  * until river_clear_device_error. */
 int river_decode_step_host(river_ctx *ctx, int batch, const int32_t *slots, const int32_t *tok, const float *tau,

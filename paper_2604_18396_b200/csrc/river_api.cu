@@ -1215,8 +1215,9 @@ int river_init(const river_config *cfg, const river_weights *w, void *kv_pool, s
         c->meta_host_rows[i] = c->meta_rows;  // entries past a step's rows stay valid row ids
         if (cudaEventCreateWithFlags(&c->meta_ev[i], cudaEventDisableTiming) != cudaSuccess) return bail("cudaEventCreate failed");
     }
-    c->pin_io_bytes = (size_t)cfg->max_batch * (4 * sizeof(int32_t) + sizeof(float)) + sizeof(int32_t);
+    c->pin_io_bytes = (size_t)cfg->max_batch * (4 * sizeof(int32_t) + sizeof(float)) + 2 * sizeof(int32_t);
     if (cudaMallocHost(&c->pin_io, c->pin_io_bytes) != cudaSuccess) return bail("cudaMallocHost failed");
+    *c->pin_full_depth() = cfg->L;
     c->page_tbl.assign((size_t)cfg->max_seqs * cfg->max_pages_per_seq, -1);
     c->seq_len.assign(cfg->max_seqs, 0);
     c->free_pages.resize(cfg->n_pages);
@@ -1307,7 +1308,7 @@ int river_decode_step_host(river_ctx *c, int batch, const int32_t *slots, const 
     const size_t B = g.max_batch;
     int32_t *p_tok = (int32_t *)c->pin_io, *p_forced = p_tok + B, *p_next = p_forced + B, *p_exit = p_next + B;
     float *p_tau = (float *)(p_exit + B);
-    int32_t *p_err = (int32_t *)(p_tau + B);  // pin_io holds 5 arrays of max_batch entries and this word
+    int32_t *p_err = (int32_t *)(p_tau + B);  // pin_io holds 5 arrays of max_batch entries, this word and pin_full_depth's
     std::memcpy(p_tok, tok, sizeof(int32_t) * batch);
     std::memcpy(p_tau, tau, sizeof(float) * batch);
     if (forced_exit) std::memcpy(p_forced, forced_exit, sizeof(int32_t) * batch);
@@ -1620,11 +1621,8 @@ int river_release(river_ctx *c, int slot) {
     const river_config &g = c->cfg;
     CUDA_TRY(c, cudaMemsetAsync(c->page_tbl_dev + (size_t)slot * g.max_pages_per_seq, 0xff,
                                 sizeof(int32_t) * g.max_pages_per_seq, c->stream));
-    if (g.kv_strategy == RIVER_KV_MONO_DECREASING) {  // a new sequence in this slot may go to full depth again
-        const int32_t cap0 = g.L;
-        CUDA_TRY(c, cudaMemcpyAsync(c->slot_cap + slot, &cap0, sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
-        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    }
+    if (g.kv_strategy == RIVER_KV_MONO_DECREASING)  // a new sequence in this slot may go to full depth again
+        CUDA_TRY(c, cudaMemcpyAsync(c->slot_cap + slot, c->pin_full_depth(), sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     for (int i = g.max_pages_per_seq - 1; i >= 0; --i) {
         int32_t &e = c->page_tbl[(size_t)slot * g.max_pages_per_seq + i];
         if (e >= 0) { c->free_pages.push_back(e); e = -1; }

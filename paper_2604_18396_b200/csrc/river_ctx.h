@@ -89,6 +89,7 @@ struct river_ctx {
     int meta_next = 0;
     void *pin_io = nullptr;  // pinned staging for the *_host entry point
     size_t pin_io_bytes = 0;
+    int32_t *pin_full_depth() const { return reinterpret_cast<int32_t *>(static_cast<char *>(pin_io) + pin_io_bytes) - 1; }  // holds L, for copies that nobody waits for
     std::vector<int32_t> last_pos;  // positions of the rows of the last decode step
     int head_grid = 0;
 

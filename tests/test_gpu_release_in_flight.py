@@ -9,36 +9,56 @@ from workloads import synth
 
 pytestmark = pytest.mark.gpu
 
+HOLD = 60_000_000  # cycles (30 ms) that a kernel of torch's keeps the context's stream busy: the host is far ahead meanwhile
 
-# long passes, several of them; short passes (the batch kernels; at four rows and fewer the decode attention); depths by Eq. 1
+
+def hold(r):
+    with torch.cuda.stream(r.stream):
+        torch.cuda._sleep(HOLD)
+        ev = torch.cuda.Event()
+        ev.record()
+    return ev
+
+
+# long passes, several of them; short passes (the batch kernels; at four rows and fewer the decode attention); depths by Eq. 1; the
+# strategy that gives a released slot its full depth back
 @pytest.mark.parametrize("lens,depth,strategy", [([300, 9, 200], None, 0), ([1100, 40], 3, 0), ([20, 30], 4, 0), ([3, 1], None, 0),
-                                                 ([60, 45], -1, 0), ([20, 7], None, 2)])
+                                                       ([60, 45], -1, 0), ([20, 7], None, 2), ([20, 7], None, 3)])
 def test_pages_handed_on_while_in_use(lens, depth, strategy):
     shape, _, (bb, rv) = draw_model("mini8")
     pages = sum((n + 16) // 16 for n in lens)
     offs = [0]
     for n in lens:
         offs.append(offs[-1] + n)
-    slots = list(range(len(lens)))
+    slots, B = list(range(len(lens))), len(lens)
+    toks = [torch.cat([synth.tokens(71 + turn, b, n, shape.V) for b, n in enumerate(lens)]).int().cuda() for turn in range(5)]
+    first = [t[:B].contiguous() for t in toks]
+    tau = torch.full((B,), 0.9, device="cuda")
     out = {}
     for wait in (True, False):
-        r = River(make_config(shape, max_seqs=len(lens), max_pages_per_seq=80, n_pages=pages, max_batch=8, prefill_chunk=256,
+        r = River(make_config(shape, max_seqs=B, max_pages_per_seq=80, n_pages=pages, max_batch=8, prefill_chunk=256,
                               kv_strategy=strategy), bb, rv)
         got = out[wait] = []
+        torch.cuda.synchronize()
+        held = None
         for turn in range(5):
-            tok = torch.cat([synth.tokens(71 + turn, b, n, shape.V) for b, n in enumerate(lens)]).int().cuda()
-            lg = torch.empty((len(lens), shape.V), device="cuda")
+            lg = torch.empty((B, shape.V), device="cuda")
             if turn:
                 for s in (slots if turn % 2 else slots[::-1]):
                     r.release(s)
-            d = r.prefill(slots, tok, offs, depth, lg, tau=0.5 + 0.1 * turn if depth == -1 else float("inf"))
-            nxt, ex = torch.empty(len(lens), dtype=torch.int32, device="cuda"), torch.empty(len(lens), dtype=torch.int32, device="cuda")
+                assert wait or not held.query(), "release waited for the device"
+            d = r.prefill(slots, toks[turn], offs, depth, lg, tau=0.5 + 0.1 * turn if depth == -1 else float("inf"))
+            if turn and depth != -1:  # (a depth that the device finds is waited for)
+                assert wait or not held.query(), "prefill waited for the device"
+            if not wait:
+                held = hold(r)  # what follows is queued behind it when the next turn's releases come
+            nxt, ex = torch.empty(B, dtype=torch.int32, device="cuda"), torch.empty(B, dtype=torch.int32, device="cuda")
             lg2 = torch.empty_like(lg)
-            r.decode_step(slots, tok[:len(lens)].contiguous(), torch.full((len(lens),), 0.9, device="cuda"), None, lg2, nxt, ex)
-            kv = [x.clone() for b in slots for x in r.read_kv(b, shape.L, 0, 1)]
+            r.decode_step(slots, first[turn], tau, None, lg2, nxt, ex)
+            kv = [r.read_kv(b, shape.L, 0, 1) for b in slots]
             if wait:
                 torch.cuda.synchronize()
-            got.append((d, lg, lg2, nxt, ex, kv))
+            got.append((d, lg, lg2, nxt, ex, [x for pair in kv for x in pair]))
         torch.cuda.synchronize()
         assert r.stats().device_error == 0
         r.close()
@@ -46,3 +66,4 @@ def test_pages_handed_on_while_in_use(lens, depth, strategy):
         assert a[0] == b[0]
         assert all(torch.equal(x, y) for x, y in zip(a[1:5], b[1:5]))
         assert all(torch.equal(x, y) for x, y in zip(a[5], b[5]))
+
