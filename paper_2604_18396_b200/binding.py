@@ -233,6 +233,13 @@ class River:
         if cur != self.stream:
             self.stream.wait_stream(cur)
 
+    def _order_current_after(self):
+        """What the context has queued so far precedes whatever torch's current stream is given next: its outputs may be read there,
+        and memory that its inputs leave may be handed out again."""
+        cur = torch.cuda.current_stream(self.device)
+        if cur != self.stream:
+            cur.wait_stream(self.stream)
+
     def _check(self, rc: int):
         if rc:
             raise RiverError(rc, load().river_last_error(self.h).decode())
@@ -256,9 +263,14 @@ class River:
         Returns the depth each prompt left the backbone at."""
         e = self.cfg.L if prefill_exit_layer is None else prefill_exit_layer
         depth = (C.c_int32 * len(slots))()
+        self._order_current_after()  # (the call waits for nothing: the steps before it may still be under way when it returns)
         self._order_after_current()
         self._check(load().river_prefill(self.h, len(slots), _i32_host(slots), _dp(tok), _i32_host(offsets), e,
                                          C.c_float(tau), _dp(logits_last), _dp(next_tok), depth))
+        if torch.cuda.current_stream(self.device) != self.stream:  # (the buffers' memory stays theirs until the prompt is through)
+            for t in (tok, logits_last, next_tok):
+                if t is not None:
+                    t.record_stream(self.stream)
         return list(depth)
 
     def decode_step(self, slots: Sequence[int], tok: torch.Tensor, tau: torch.Tensor,
@@ -349,7 +361,9 @@ class River:
         return load().river_seq_len(self.h, slot)
 
     def release(self, slot: int):
+        """river_release.  The host does not wait; torch's current stream does, for what the context has queued."""
         self._check(load().river_release(self.h, slot))
+        self._order_current_after()
 
     def profile(self, enable: bool):
         self._check(load().river_profile(self.h, int(enable)))
