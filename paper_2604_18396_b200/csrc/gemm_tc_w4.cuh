@@ -243,12 +243,14 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
     const int pre = early ? min(kW4RawBufs, nsb) : 0;
     if (tid == 0)
         for (int sb = 0; sb < pre; ++sb) load_raw(sb);
-    // Tensor memory before anything is waited for, and before the row count is known to be zero: behind the count, dependent grids start
-    // too late (8B-class, 8 blocks, 64 rows, none on the exit layers: 1927 -> 1957 us a step; so 1939 / 1940).
     // Beside the backbone kernel of the same projection (`overlap`): that grid let this one start only after the
     // operand kernels of both had completed, the two write disjoint rows, and the row count dates from the previous
     // block - nothing here depends on it.  Whoever comes next in the stream waits for THIS grid, so this grid must not
     // complete before that one: every CTA waits for it just before it exits.
+    if (!a.overlap) pdl_wait();
+    // Tensor memory behind that wait, if there is one: kept through it, it costs short passes 10 % (mini shape, 118 positions on the exit
+    // layers 399 -> 441 us).  And before the row count is known to be zero: behind the count, dependent grids start too late (8B-class,
+    // 8 blocks, 64 rows, none on the exit layers: 1927 -> 1957 us a step; so level).
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(tmem_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::);
@@ -256,7 +258,6 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
         __syncwarp();
         pdl_launch();  // (behind the allocation: see tc_gemm_kernel)
     }
-    if (!a.overlap) pdl_wait();
     const int n_live = min(*a.cnt - n0, NP);
     if (n_live <= 0 && pre == 0) {  // uniform over the CTA and the cluster (nobody reaches a cluster barrier)
         if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*reinterpret_cast<volatile uint32_t *>(&s_tmem)), "r"(tmem_cols));
