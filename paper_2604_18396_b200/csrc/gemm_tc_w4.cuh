@@ -140,7 +140,7 @@ struct TcW4Args {
     const uint16_t *scale[3], *zero[3];  // bf16 [rows][K/64] of the up to three matrices behind the code maps
     const int32_t *rows;
     const int32_t *cnt;
-    const int32_t *hint;  // a count of exit-layer rows that is never too high (an earlier layer's): > 0 means rows exist
+    const int32_t *hint;  // > 0: rows exist, and the codes are requested early (exit_rows_hint; a wrong one costs time, no more)
     int *dev_err;
 };
 
@@ -237,8 +237,8 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
             tma_load_2d(dst, maps[m0], x, ay, full);
         }
     };
-    // codes first: they depend on nothing - if an earlier layer already had rows on its exit layer (the count only
-    // grows inside a step); otherwise wait for the real count and leave at once if it is zero
+    // codes first: they depend on nothing - if rows are known to exist (exit_rows_hint; the count only grows inside a step); otherwise
+    // wait for the real count and leave at once if it is zero
     const bool early = s_early != 0;
     const int pre = early ? min(kW4RawBufs, nsb) : 0;
     if (tid == 0)

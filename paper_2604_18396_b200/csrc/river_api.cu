@@ -477,8 +477,8 @@ cudaError_t tc_pair(river_ctx *c, bool with_river, const ProjIn &in, int K, int 
 }
 
 // a2 of block l for the n rows of the step: attention norm + QKV + RoPE + KV write, on the weight set(s) the row
-// lists name (small steps: from the exit flags).  at: the entry of the row lists and exit flags; sets: as in block_tail.
-cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const DecideArgs &dec, double kv_write, int at, int sets = 3) {
+// lists name (small steps: from the exit flags).  at: the entry of the row lists and exit flags; hint_riv, sets: as in block_tail.
+cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const DecideArgs &dec, double kv_write, int at, const int32_t *hint_riv, int sets = 3) {
     const river_config &g = c->cfg;
     const int d = g.d, B = c->list_rows, qdim = g.Hq * g.dh, kvdim = g.Hkv * g.dh;
     const double w4f = 0.25 + 2.0 / g.group;
@@ -491,7 +491,6 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
     const bool tc = c->tc_ok && n >= 5 && n <= c->tc_max_pad;
     const river_ctx::LayerMaps *tm = tc ? &c->tc_maps[l - 1] : nullptr;
     const river_ctx::LayerMaps *wm = (tc && c->w4tc_ok && has_river) ? &c->w4_maps[l - 1] : nullptr;
-    const int32_t *nrh = c->n_riv + std::max(0, at - 1);  // never above the count entering this block
     cudaError_t err = cudaSuccess;
     auto note = [&](cudaError_t e) { if (err == cudaSuccess) err = e; };
     const double wb = 2.0 * (qdim + 2.0 * kvdim) * d;
@@ -510,7 +509,7 @@ cudaError_t launch_qkv(river_ctx *c, int l, int n, const float *h_in, const Deci
         const CUtensorMap *const cm[3] = {wm ? &wm->q : nullptr, wm ? &wm->k : nullptr, wm ? &wm->v : nullptr};
         const river_w4 *const cw[3] = {&w.rq, &w.rk, &w.rv};
         const auto river = [&](int phase, bool beside) {
-            return launch_tc_w4(c, in, cm, cw, d, (qdim + 2 * kvdim) / kTcBM, n, 0, qdim / kTcBM, kvdim / kTcBM, ri, nr, nrh, e, phase, beside);
+            return launch_tc_w4(c, in, cm, cw, d, (qdim + 2 * kvdim) / kTcBM, n, 0, qdim / kTcBM, kvdim / kTcBM, ri, nr, hint_riv, e, phase, beside);
         };
         if (sets & 1)
             note(tc_pair(c, wm != nullptr, in, d, n, rl,
@@ -586,7 +585,7 @@ cudaError_t launch_head(river_ctx *c, const float *h, int n_head, const float *p
 
 // What follows attention in block l (a4, a5: O, gate/up and down projections, with their residuals) for the rows of `rl`, n at most,
 // on the kernels of decode steps.  sets: 1 = the backbone's rows, 2 = the exit layers', 3 = both.  list_idx: the list whose counts
-// say which weights were read (timing), -1: all of `sets`.  hint_riv: a count that is never above the exit layers' rows.
+// say which weights were read (timing), -1: all of `sets`.  hint_riv: exit_rows_hint.
 cudaError_t block_tail(river_ctx *c, int l, int n, const RowLists &rl, int sets, int list_idx, const int32_t *hint_riv, const float *h_in, float *h_mid,
                        float *h_out, float *act) {
     const river_config &g = c->cfg;
@@ -726,7 +725,8 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         leave.assign(L + 1, 0);
         for (int i = 0; i < n; ++i) leave[depth[i]] += 1;
     }
-    int at = 0, gone = known ? leave[0] : 0;  // entry `at` of the row lists and exit flags describes the rows of this block
+    const auto hint_of = [&](int entry) { return entry < 0 ? c->meta_dev /* StepMeta::n_rows */ : c->n_riv + entry; };
+    int at = 0, at_before = 0, gone = known ? leave[0] : 0;  // entry `at` of the row lists and exit flags describes the rows of this block
 
     {
         LaunchScope ls(c, K_BEGIN, (double)n * d * 2.0, 0, -1);
@@ -750,7 +750,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         const int32_t *na = c->n_act + at, *nr = c->n_riv + at;
         const RowLists rl{ai, na, ri, nr, c->hint_act, c->meta_dev /* StepMeta::n_rows */, c->state_at(at)};
         float *h_in = c->h[hi], *h_mid = c->h[(hi + 1) % 3], *h_out = c->h[(hi + 2) % 3];
-        const int32_t *nrh = c->n_riv + std::max(0, at - 1);  // never above the count entering this block
+        const int32_t *nrh = hint_of(exit_rows_hint(sets == 2, at, at_before, at < l - 1));
         bool staged = false;
         if (c->off_first && l >= c->off_first)
             if (int rc = offload_before_layer(c, l, &staged)) return rc;
@@ -762,7 +762,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
                 dec.h_prev = prev_in; dec.state_in = c->state_at(l - 2); dec.state_out = c->state_at(l - 1);
                 dec.lists = lists; dec.hint_act = c->hint_act; dec.fail = fail_buf; dec.row_slot = c->row_slot();
             }
-            note(launch_qkv(c, l, n, h_in, dec, kv_write, at, known ? sets : 3));
+            note(launch_qkv(c, l, n, h_in, dec, kv_write, at, nrh, known ? sets : 3));
         }
         // the other KV strategies (Section 3): a row that has left neither attends nor changes its hidden state
         c->attn_skip = strat == RIVER_KV_RIVER ? nullptr : c->state_at(at);
@@ -788,6 +788,7 @@ int run_rows(river_ctx *c, int n, int n_head, const int32_t *row_pos_host, bool 
         // ---- a6 + a7: exit score, decision, compaction -> row lists entering block l+1
         if (!known || record_fail || (l < L && leave[l])) {
             if (!fold) launch_score(l, h_in, h_out, at);
+            at_before = at;
             at = l;
             if (known && l < L) gone += leave[l];
         }
@@ -1451,7 +1452,8 @@ int river_project_kv(river_ctx *c, int layer, int use_exit_layer, int n_rows, co
     float *q_keep = c->qbuf;
     if (q_out) c->qbuf = q_out;
     const int64_t launched = t_launches;
-    const cudaError_t e = launch_qkv(c, layer, n_rows, h, DecideArgs{}, (double)n_rows * 4.0 * c->cfg.Hkv * c->cfg.dh, layer - 1);
+    const cudaError_t e = launch_qkv(c, layer, n_rows, h, DecideArgs{}, (double)n_rows * 4.0 * c->cfg.Hkv * c->cfg.dh, layer - 1,
+                                     use_exit_layer ? c->meta_dev : c->n_riv + std::max(0, layer - 2));
     c->qbuf = q_keep;
     if (e != cudaSuccess) return fail(c, RIVER_E_DEVICE, std::string("kernel launch failed: ") + cudaGetErrorString(e));
     if (!use_exit_layer && c->off_first && layer >= c->off_first)

@@ -133,6 +133,15 @@ inline W4Plan w4_plan(int num_sms, int np, int tiles, int K, bool decode, int mo
     return p;
 }
 
+// Where tc_gemm_w4_kernel looks, before the grids before it are through, whether it will have rows (and may request its codes at once):
+// the entry of n_riv to read, or -1 for the rows of the pass.  `at`: the entry that describes the rows of this block; `settled`: it was
+// written before the block before this one, so it may be read; `before`: the entry before it, whose count is no higher; `all`: the host
+// knows that every row is on the exit layers.  Steps write an entry per block (at = l - 1, never settled), passes whose depths the host
+// knows only those behind blocks that rows leave at: every other entry holds whatever an earlier step left there.  Short passes in a
+// context that had not decoded, entry at - 1 / this, us: mini shape, 118 positions, depth 3 of 6 388 / 381, tiny shape, 100 positions,
+// depth 3 of 4 213 / 210.
+inline int exit_rows_hint(bool all, int at, int before, bool settled) { return all ? -1 : settled ? at : before; }
+
 // Operand rows per CTA of a step with np of them, from its widest projection (`tiles` 128-feature tiles, K inputs).  A small model's weight
 // tiles and K-splits are CTAs for a fraction of the chip (mini shape: 24 for QKV), each of which then finishes all the rows alone; so
 // the rows are dealt out as well, 16 to 64 to a CTA, while all CTAs of the widest projection find a place at once, two to an SM.  (The
