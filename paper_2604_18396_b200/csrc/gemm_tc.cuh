@@ -320,7 +320,7 @@ struct TcArgs {
     int qkv_q_tiles, qkv_k_tiles;  // QKV: tiles per matrix (0 otherwise)
     const int32_t *rows;   // step row id of operand row n
     const int32_t *cnt;    // live operand rows (device)
-    const int32_t *hint;   // a count of those rows that is never too low: 0 means there are certainly none
+    const int32_t *hint;   // a count of those rows that is never too low: a row tile behind it certainly has none
     int *dev_err;
 };
 
@@ -445,11 +445,11 @@ __global__ void __launch_bounds__(kTcThreads) tc_gemm_kernel(const __grid_consta
     // `late_release`: the next grid in the stream is the dequantising kernel of the same projection, which runs beside
     // this one instead of behind it: it never waits for this grid at its start, so it may only start once everything
     // BOTH read (the operand kernels' output) is complete - that is when every CTA here is past its own wait.
-    if (tid == 0) s_some = *reinterpret_cast<const volatile int32_t *>(a.hint) > 0;  // one read for the whole CTA
+    if (tid == 0) s_some = *reinterpret_cast<const volatile int32_t *>(a.hint) > n0;  // one read for the whole CTA
     __syncthreads();
-    if (!s_some) {  // every row has left the backbone: nothing to fetch, nothing to compute (uniform over the cluster:
-        if (!a.late_release) pdl_launch();
-        pdl_wait();  // the hint only changes between layers); still order this grid behind its predecessor
+    if (!s_some) {  // every row here has left the backbone: nothing to fetch or compute (a CTA of the cluster that read an older hint finds
+        if (!a.late_release) pdl_launch();  // no live row either, and waits for nobody); still order this grid behind its predecessor
+        pdl_wait();
         return;
     }
     if (tid == 0) {

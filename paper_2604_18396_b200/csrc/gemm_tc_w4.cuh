@@ -140,7 +140,7 @@ struct TcW4Args {
     const uint16_t *scale[3], *zero[3];  // bf16 [rows][K/64] of the up to three matrices behind the code maps
     const int32_t *rows;
     const int32_t *cnt;
-    const int32_t *hint;  // > 0: rows exist, and the codes are requested early (exit_rows_hint; a wrong one costs time, no more)
+    const int32_t *hint;  // a row tile in front of it has rows, and requests its codes early (exit_rows_hint; a wrong one costs time, no more)
     int *dev_err;
 };
 
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kW4Threads, 2) tc_gemm_w4_kernel(const __grid_
 
     if (tid == 0) {
         s_abort = 0;
-        s_early = *reinterpret_cast<const volatile int32_t *>(a.hint) > 0;  // one read for the whole CTA
+        s_early = *reinterpret_cast<const volatile int32_t *>(a.hint) > n0;  // one read for the whole CTA
         for (int s = 0; s < S; ++s) {
             // a stage is full when its A tile is written (one arrival per lane quarter) AND its activation tile has
             // landed (the producer's arrival with the byte count): ONE barrier, one poll per k-block for the MMA lane
