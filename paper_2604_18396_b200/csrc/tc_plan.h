@@ -297,11 +297,13 @@ inline int tc_long_pass_rows(int d, int L, int exit_blocks, int max_rows) {
     return std::min(base + more * exit_blocks / L, std::min(max_rows, 256)) + 1;
 }
 
-// Where the batch kernels' rows are dealt out over CTAs (tc_row_tile), a short pass is the faster one for longer: up to this many rows.
-// Batch / pair kernels, us, 1 prompt:
-//   tiny 0/4      145 rows 210 / 243   176: 214 / 247   224: 223 / 255   256: 230 / 248     3/4  145: 246 / 265   256: 264 / 271
-//   mini 0/6      145: 377 / 446   176: 378 / 452   200: 454 / 464   224: 463 / 474   256: 479 / 462
-//        5/6      145: 440 / 460   176: 443 / 463   200: 509 / 505   224: 532 / 487   256: 519 / 471
+// Where the batch kernels' rows are dealt out over CTAs (tc_row_tile), a short pass is the faster one for longer: up to this many rows,
+// where the mini shape's tiles become wider than 32 rows.  (The tiny shape's stay narrow, and its short passes ahead up to 256.)
+// Batch / pair kernels (O and down of the latter by tc_pass_splits), us, 1 prompt:
+//   tiny 0/4   129 rows 209 / 239   145: 206 / 239   176: 209 / 237   192: 209 / 236   200: 216 / 242   224: 218 / 241   256: 224 / 240
+//        3/4   129: 231 / 275       145: 224 / 277   176: 231 / 276   192: 232 / 276   200: 239 / 279   224: 240 / 277   256: 246 / 278
+//   mini 0/6   129: 365 / 396       145: 372 / 396   176: 377 / 399   192: 384 / 402   200: 453 / 406   224: 462 / 409   256: 476 / 410
+//        5/6   129: 411 / 486       145: 408 / 485   176: 417 / 486   192: 421 / 488   200: 479 / 493   224: 489 / 494   256: 494 / 497
 constexpr int kTcTiledPassRows = 192;
 inline int tc_tiled_pass_rows(int num_sms, int tiles, int K) {
     return tc_row_tile(num_sms, kTcTiledPassRows, tiles, K, false) < kTcTiledPassRows ? kTcTiledPassRows : 0;
