@@ -1085,13 +1085,10 @@ int prefill_pass(river_ctx *c, int n_seqs, const int32_t *slots, const int32_t *
         if (c->prefill_attn_now) mh[5] = n;  // hint_act; the decode attention's geometry is for the rows that need it
         else set_attn_meta(c, mh, n);
         // query tiles of the prefill attention: consecutive positions of one sequence, up to 16 - or as many as make 128
-        // query rows, for the tcgen05 kernel, where the rows of a long pass look back far enough on average: at 128 positions (below, its
-        // tiles are mostly padding: 1B-class, 5 prompts of 160 positions 1017 against 995 us, 4 of 240 level), at 64 where the other
-        // kernel's CTAs, 16 positions and a KV head each, are one per SM at most, so that one's walk over the keys is the time it takes
-        // (mini shape, 5 prompts of 160 479 against 505, 4 of 240 500 against 550; of 90 460 against 456)
+        // query rows, for the tcgen05 kernel of long passes
         long long seen = 0;
         for (int i = 0; i < n; ++i) seen += mh[kMetaHdr + max_rows + i] + 1;
-        const bool tc_attn = long_pass && seen >= ((n + kPfBM - 1) / kPfBM * g.Hkv <= c->num_sms ? 64LL : 128LL) * n;
+        const bool tc_attn = long_pass && tc_long_attention(c->num_sms, (n + kPfBM - 1) / kPfBM * g.Hkv, n, seen);
         const int tile_max = tc_attn ? prefill_tc_positions(c) : kPfBM;
         int n_tiles = 0;
         for (int i = 0; i < n;) {

@@ -309,4 +309,10 @@ inline int tc_tiled_pass_rows(int num_sms, int tiles, int K) {
     return tc_row_tile(num_sms, kTcTiledPassRows, tiles, K, false) < kTcTiledPassRows ? kTcTiledPassRows : 0;
 }
 
+// Attention of a long pass's n rows, which see `seen` positions in all: the tcgen05 kernel where they look back far enough on average, at
+// 128 positions (below, its tiles are mostly padding: 1B-class, 5 prompts of 160 positions 1017 against 995 us, 4 of 240 level), at 64
+// where the warp-level kernel's CTAs, 16 positions and a KV head each, are one per SM at most, so that one's walk over the keys is the
+// time it takes (mini shape, 5 prompts of 160 479 against 505, 4 of 240 500 against 550; of 90 460 against 456).
+inline bool tc_long_attention(int num_sms, int warp_ctas, int n, long long seen) { return seen >= (warp_ctas <= num_sms ? 64LL : 128LL) * n; }
+
 }  // namespace river
