@@ -36,11 +36,13 @@ def test_decode_steps(rows, flags, strategy):
     r.close()
 
 
-@pytest.mark.parametrize("lens,tau", [([20], 0.0), ([150], 0.0), ([60, 45, 40], 0.9), ([60, 45, 40], 2.0)])
+@pytest.mark.parametrize("lens,tau", [([20], 0.0), ([150], 0.0), ([60, 45, 40], 0.9), ([60, 45, 40], 2.0),
+                                      ([200], 0.0), ([90, 65, 60], 0.9), ([90, 65, 60], 2.0)])
 def test_prefill_passes(lens, tau):
-    """tau 0.9 lies between the prompts' scores often enough for rows on both weight sets; 2: every row on the backbone."""
+    """Short passes and (200 rows and more) long ones.  tau 0.9 lies between the prompts' scores often enough for rows on both weight
+    sets; 2: every row on the backbone."""
     shape, _, (bb, rv) = draw_model("mini8")
-    r = River(make_config(shape, max_seqs=3, max_pages_per_seq=10, n_pages=30, max_batch=8, prefill_chunk=256), bb, rv)
+    r = River(make_config(shape, max_seqs=3, max_pages_per_seq=13, n_pages=39, max_batch=8, prefill_chunk=256), bb, rv)
     tok = torch.cat([synth.tokens(43, b, n, shape.V) for b, n in enumerate(lens)]).int().cuda()
     offs = np.concatenate([[0], np.cumsum(lens)]).tolist()
     before = r.stats().launches_total

@@ -22,7 +22,7 @@ def mini8():
 
 def test_steps_in_a_graph_around_long_and_short_passes(mini8):
     shape = mini8[0]
-    lens = [21, 7, 300, 4, 140, 33]
+    lens = [21, 7, 300, 4, 170, 33]
     p = Pair(mini8, 6, 320, 6, prefill_chunk=256, kv_store=1, storage_yardstick=True, page_shuffle_seed=2, flags=binding.RIVER_F_GRAPH)
     prompts = [synth.tokens(61, b, n, shape.V).numpy() for b, n in enumerate(lens)]
     t = 0
@@ -43,7 +43,7 @@ def test_steps_in_a_graph_around_long_and_short_passes(mini8):
     p.prefill([2], prompts[2:3])                 # a long pass: the other layout, on the device and in the staging blocks
     steps([0, 1], 2)                             # the graph from before it
     steps([0, 1, 2], 3)
-    p.prefill([3, 4, 5], prompts[3:], 4)         # 177 rows of three prompts, leaving after block 4
+    p.prefill([3, 4, 5], prompts[3:], 4)         # 207 rows of three prompts, a long pass, leaving after block 4
     steps([3, 4, 5, 0, 1, 2], 3)                 # six rows: the batch kernels
     steps([0, 1], 1)
     for b in range(6):

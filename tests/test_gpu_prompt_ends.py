@@ -19,7 +19,7 @@ def mini8():
 
 
 @pytest.mark.parametrize("depth", [6, 2])
-@pytest.mark.parametrize("lens", [[150], [1030], [90, 3, 40, 31], [40, 30, 30, 20, 30], [17] * 20, [5] * 64, [4] * 65, [3] * 96, [3] * 97, [2, 1] * 100])
+@pytest.mark.parametrize("lens", [[200], [1030], [120, 3, 40, 31], [60, 40, 30, 50, 30], [17] * 20, [5] * 64, [4] * 65, [3] * 96, [3] * 97, [2, 1] * 100])
 def test_logits_and_cache(mini8, lens, depth):
     shape = mini8[0]
     p = Pair(mini8, len(lens), max(lens) + 8, len(lens), kv_store=1, storage_yardstick=True, prefill_chunk=256)

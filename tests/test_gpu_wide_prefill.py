@@ -14,9 +14,9 @@ def mini8():
     return draw_model("mini8")
 
 
-# 129 rows: the shortest long pass; 225 / 300: last tiles of a few rows; several prompts in one pass and across two passes;
+# 193 rows: the shortest long pass; 225 / 300: last tiles of a few rows; several prompts in one pass and across two passes;
 # 1150: a full pass and a rest of 126 rows for the batch kernels
-@pytest.mark.parametrize("lens,depth", [([129], None), ([225], 2), ([40, 300, 9, 200], None), ([300, 17], 4), ([1150], None),
+@pytest.mark.parametrize("lens,depth", [([193], None), ([225], 2), ([40, 300, 9, 200], None), ([300, 17], 4), ([1150], None),
                                         ([700, 600], 3)])
 def test_long_passes_match_oracle(mini8, lens, depth):
     shape = mini8[0]
@@ -35,7 +35,8 @@ def test_long_passes_match_oracle(mini8, lens, depth):
 
 def test_mixed_depths_in_one_pass(mini8):
     """Depth chosen per prompt by Eq. 1, thresholds between the per-block minima of the oracle's scores (never within 2.5e-3 of
-    one, so the depths are unambiguous): one pass of 145 rows holds rows on both weight sets; depths, logits and cache."""
+    one, so the depths are unambiguous): one pass of 145 rows (a long one: short passes end at prefill_chunk) holds rows on both weight
+    sets; depths, logits and cache."""
     shape = mini8[0]
     lens, L, lo = [60, 45, 40], shape.L, max(shape.entry_layer, 1)
     prompts = [synth.tokens(43, b, n, shape.V).numpy() for b, n in enumerate(lens)]
@@ -53,7 +54,7 @@ def test_mixed_depths_in_one_pass(mini8):
     mixed = [t for t in taus if len(set(first(t))) > 1]
     assert mixed, "no threshold separates the prompts"
     for tau in mixed[::max(1, len(mixed) // 4)]:
-        p = Pair(mini8, 3, max(lens) + 2, 8, prefill_chunk=256, page_shuffle_seed=9)
+        p = Pair(mini8, 3, max(lens) + 2, 8, prefill_chunk=128, page_shuffle_seed=9)
         want = [p.oracle.prefill_auto(b, pr, tau) for b, pr in enumerate(prompts)]
         offs = np.concatenate([[0], np.cumsum(lens)]).tolist()
         lg = torch.empty((3, shape.V), device="cuda")
@@ -71,8 +72,8 @@ def test_mixed_depths_in_one_pass(mini8):
 def test_long_pass_from_the_first_block_on(mini8, depth, exit_mode):
     """Every row on the exit layers from block 1 on (depth 0), from block 3 on, never; both exit modes, and steps behind them."""
     shape = mini8[0]
-    lens = [170, 3]
-    p = Pair(mini8, 2, 180, 4, exit_mode, entry_layer=0, prefill_chunk=256, kv_store=1, storage_yardstick=True)
+    lens = [200, 3]
+    p = Pair(mini8, 2, 210, 4, exit_mode, entry_layer=0, prefill_chunk=256, kv_store=1, storage_yardstick=True)
     p.prefill([0, 1], [synth.tokens(44, b, n, shape.V).numpy() for b, n in enumerate(lens)], depth, logits=True)
     for t in range(2):
         tk = synth.tokens(44, 90 + t, 2, shape.V).numpy()
@@ -110,7 +111,7 @@ def test_gate_and_up_in_either_order_in_memory(mini8):
 @pytest.mark.parametrize("dh,gq", [(64, 1), (64, 2), (64, 4), (64, 8), (128, 1), (128, 2), (128, 4), (128, 8)])
 def test_long_pass_attention_geometries(dh, gq):
     """Every head dim and group size of the attention kernel, prompts that end inside and on the edges of its query tiles
-    (128 / gq positions), key tiles (64) and pages (16): the second block's cache shows the attention of every position."""
+    (128 / gq positions), key tiles (128, in two streams) and pages (16): the second block's cache shows the attention of every position."""
     hkv = max(1, 512 // dh // gq, 128 // dh)
     shape = synth.ModelShape("a", 2, 256, hkv * gq, hkv, dh, 256, 1024, seed=7, resid_decay=1.0)
     bb = synth.make_backbone(shape, "cpu")
