@@ -17,7 +17,9 @@
 // What bounds it: the tensor pipe (64 MMAs of 79 cycles per 128 keys of each stream, 6300 cycles of which 5100 are theirs) once a CTA
 // is under way, and before that its start: 4 us until Q, K and V of the first tiles are there, as many again for the first pass over
 // the code on every SM.  128 keys per tile because an MMA of M = 128 takes 75-85 cycles whatever its N up to 128; two streams because S
-// and O of one are half of tensor memory, and a serial walk (S, softmax, P V) leaves the pipe idle for more than half of it.  us per
+// and O of one are half of tensor memory, and a serial walk (S, softmax, P V) leaves the pipe idle for more than half of it.  (ncu, 8B
+// class, 1024 positions: 46.5 us cold, pipe active 24 % of the SMs' time - it counts the 32 cycles of mathematics in an MMA's 79 -, DRAM 21
+// MB.)  us per
 // block and pass, one stream of 64-key tiles in each of two CTAs per SM against this: 8B-class, passes of 1024 positions of one
 // prompt 64 / 114 / 171 -> 43 / 71 / 100; two prompts of the 1B class 26 -> 24; tiny shape, up to 1245 positions 45 -> 21.  The
 // warp-level kernel (attn_prefill.cuh) stays for short passes and prompts.

@@ -17,7 +17,7 @@
 //
 // What bounds it: the tensor pipe for gate/up and down (81 and 76 % of the kernel's time busy under ncu), and the power cap
 // when passes follow each other; QKV and O (65 and 63 %) have too few tiles for whole rounds.  8B-class shape, 1024 rows, inside
-// passes that follow each other, operand kernel included: QKV 100 us, O 63, gate/up 331, down 158 - 1.03, 1.09, 1.45 and 1.52 PFLOP/s of
+// passes that follow each other, operand kernel included: QKV 94 us, O 59, gate/up 321, down 154 - 1.10, 1.16, 1.50 and 1.56 PFLOP/s of
 // bf16 MMAs, half of them for the low parts - against 4 x (108, 42, 191, 81) us in passes of 256 rows on tc_gemm_kernel.
 #pragma once
 #include "gemm_tc.cuh"
